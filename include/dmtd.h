@@ -248,7 +248,7 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *ctx, float temperature, uint64_t seed);
  *   "tc_attention" 0/1  attention of the per-step kernels by the tiled split-KV kernels for
  *                       head_dim 128 (tensor cores with a bf16 cache, FMAs with an fp32 cache)
  *                       instead of the one-warp-per-key-group kernel (default 1)
- *   "tcgen05_gemm" 0/1  projections of more than 4 rows (prefill chunks included) on the tcgen05
+ *   "tcgen05_gemm" 0/1  projections outside the pass kernel (prefill chunks included) on the tcgen05
  *                       tensor cores; bf16 contexts whose hidden, query and intermediate sizes
  *                       are multiples of 64 hold the second weight copy it reads, which doubles
  *                       the weight memory of the context (default 1)
@@ -272,8 +272,8 @@ dmtd_status dmtd_debug_set_error_word(dmtd_ctx *ctx, int32_t word);
 
 /* Device memory the context holds, by purpose.  A bf16 context whose hidden, query and
  * intermediate sizes are multiples of 64 keeps its weights twice: as the atom stream the
- * mma.sync kernels and the pass kernel read (passes of up to 4 rows) and as the 16 KiB blocks
- * the tcgen05 GEMM reads (more rows, and every prefill): 2 x 8.04 GB for the Qwen3-4B shape.
+ * pass kernel reads (passes of up to 4 rows) and as the 16 KiB blocks
+ * the tcgen05 GEMM reads (everything else): 2 x 8.04 GB for the Qwen3-4B shape.
  * With DMTD_WEIGHT_COPIES=1 in the environment at create only the first is kept. */
 typedef struct {
   size_t weight_stream_bytes, weight_block_bytes, kv_cache_bytes, workspace_bytes;

@@ -55,7 +55,7 @@ struct dmtd_ctx {
   std::vector<LayerDev> layers;
   PackedMat embed{};
   UmmaMat embed_u{};
-  bool umma_ok = false, use_umma = true;    // tcgen05 GEMM for projections of more than 4 rows
+  bool umma_ok = false, use_umma = true;    // tcgen05 GEMM for the projections
   int gemm_stages = 0;                      // pipeline stages of its blocks; 0: chosen per launch
   uint4 *act_blocks = nullptr;
   float *w_final = nullptr;
@@ -276,9 +276,11 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // With `norm_w` the activations are RMSNorm(act rows) * norm_w, computed while the blocks are written, and
-// the output rows are cleared first (the projections after a norm write a fresh buffer).
+// the output rows are cleared first (the projections after a norm write a fresh buffer); the rows of `act` may
+// then come in segments (RowSegments).
 dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, int lda, int M, float *out, int ldo,
-                             int gate_up_I = 0, const float *norm_w = nullptr, int merge_nsplit = 0) {
+                             int gate_up_I = 0, const float *norm_w = nullptr, int merge_nsplit = 0, int seg_rows = 0,
+                             int seg_stride = 0) {
   const int SET = TG_MAX_COLS / 2;                       // rows per sweep
   for (int m0 = 0; m0 < M; m0 += TG_MAX_SWEEPS * SET) {
     GemmTcParams P{};
@@ -318,12 +320,12 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, in
       LAUNCH_OK(c, "merge_act_blocks_kernel");
     } else if (norm_w) {
       const int n_groups = P.n_sweeps * (P.n_cols / 2 / NAB_ROWS);
-      const size_t zero_n4 = (size_t)P.rows * ldo / 4;                  // ldo is a multiple of 4 (checked by the caller)
-      const int n_zero = (int)std::min<size_t>((zero_n4 + 1023) / 1024, 2 * c->n_sms);
+      const size_t zero_n = (size_t)P.rows * ldo;
+      const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
       const int ky = std::max(1, std::min(W.n_kb, 4 * c->n_sms / std::max(1, n_groups)));
       CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
-                             act + (size_t)m0 * lda, lda, norm_w, c->s.rms_eps, P.rows, W.K, P.n_cols, c->act_blocks, n_groups,
-                             reinterpret_cast<float4 *>(out + (size_t)m0 * ldo), zero_n4));
+                             act, lda, RowSegments{m0, seg_rows, seg_stride}, norm_w, c->s.rms_eps, P.rows, W.K, P.n_cols,
+                             c->act_blocks, n_groups, P.out, zero_n));
       LAUNCH_OK(c, "norm_act_blocks_kernel");
     } else {
       long long units = (long long)W.n_kb * 8 * P.n_cols;
@@ -350,7 +352,10 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, in
 // out[m][n] += sum_k W[n][k] act[m][k]
 dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const float *act, int lda, int M, float *out,
                         int ldo) {
-  if (U.w && c->use_umma && M > 4) return launch_gemm_tc05(c, U, act, lda, M, out, ldo);
+  // the tcgen05 GEMM at every row count: the mma.sync kernel, whose warps load their weights through registers,
+  // streams the tied head of the Qwen3-4B shape (778 MB, 1 - 4 rows) at 3.6 TB/s, the tcgen05 kernel at 5.9, and a
+  // layer's projections at 3 rows in 82 us against 58 (kernel times)
+  if (U.w && c->use_umma) return launch_gemm_tc05(c, U, act, lda, M, out, ldo);
   if (W.wf) {
     gemv_f32_kernel<<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo);
     LAUNCH_OK(c, "gemv_f32_kernel");
@@ -466,7 +471,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   const LayerDev &lw = c->layers[l];
   int M = B * R, H = s.hidden, I = s.intermediate, QD = s.n_q_heads * s.head_dim;
   // the tcgen05 path normalises while it writes its activation blocks
-  const bool tc = lw.qkv_u.w && c->use_umma && M > 4 && c->ldqkv % 4 == 0 && c->ldgu % 4 == 0;
+  const bool tc = lw.qkv_u.w && c->use_umma;
   if (tc) {
     TRY(launch_gemm_tc05(c, lw.qkv_u, x, H, M, c->qkv, c->ldqkv, 0, lw.w_in));
   } else {
@@ -490,7 +495,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, lw.gu, lw.gu_u, c->act, c->lda, M, c->gu, c->ldgu));
   }
-  if (lw.down_u.w && c->use_umma && M > 4) {
+  if (tc) {
     // the tcgen05 path gates while it writes its activation blocks
     TRY(launch_gemm_tc05(c, lw.down_u, c->gu, c->ldgu, M, x, H, I));
   } else {
@@ -510,9 +515,9 @@ SampleParams sample_params(const dmtd_ctx *c) {
 }
 
 // Step a9/a10: final norm, tied LM head, greedy pick, token feedback.
-dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits, size_t out_pitch_floats = 0) {
+dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits) {
   const dmtd_model_shape &s = c->s;
-  if (c->embed_u.w && c->use_umma && B > 4 && c->ldl % 4 == 0) {
+  if (c->embed_u.w && c->use_umma) {
     TRY(launch_gemm_tc05(c, c->embed_u, c->x_up, s.hidden, B, c->logits, c->ldl, 0, c->w_final));
   } else {
     prep_norm_kernel<<<dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
@@ -522,8 +527,8 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
     TRY(launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, B, c->logits, c->ldl));
   }
   if (out_logits)
-    CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (out_pitch_floats ? out_pitch_floats : (size_t)s.vocab) * 4, c->logits,
-                                  (size_t)c->ldl * 4, (size_t)s.vocab * 4, B, cudaMemcpyDeviceToDevice, c->stream));
+    CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (size_t)s.vocab * 4, c->logits, (size_t)c->ldl * 4, (size_t)s.vocab * 4, B,
+                                  cudaMemcpyDeviceToDevice, c->stream));
   argmax_slices_kernel<<<dim3(B, ARGMAX_SLICES), 256, 0, c->stream>>>(c->logits, c->ldl, s.vocab, c->pick_val, c->pick_idx,
                                                                       c->dstate, sample_params(c));
   LAUNCH_OK(c, "argmax_slices_kernel");
@@ -531,6 +536,24 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
                                               write_token ? 1 : 0, out_argmax);
   LAUNCH_OK(c, "argmax_pick_kernel");
   return DMTD_OK;
+}
+
+// The LM head over many positions (the scoring pass): final norm and tied head of n_seg segments of seg_rows rows,
+// segment i starting at row i * seg_stride of x; row m of them all to out[m][vocab].  One GEMM over all rows: a
+// head launch per position streams the whole head again (Qwen3-4B shape, 2 x 187 of 2 x 250 positions: 187 x 0.25 ms
+// of 59.1 ms a call; 13.4 ms now).
+dmtd_status run_head_rows(dmtd_ctx *c, const float *x, int n_seg, int seg_rows, int seg_stride, float *out) {
+  const dmtd_model_shape &s = c->s;
+  const int M = n_seg * seg_rows;
+  if (c->embed_u.w && c->use_umma)
+    return launch_gemm_tc05(c, c->embed_u, x, s.hidden, M, out, s.vocab, 0, c->w_final, 0, seg_rows, seg_stride);
+  for (int i = 0; i < n_seg; ++i) {
+    prep_norm_kernel<<<dim3(seg_rows, (s.vocab + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
+        x + (size_t)i * seg_stride * s.hidden, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda,
+        c->lda, out + (size_t)i * seg_rows * s.vocab, s.vocab, s.vocab);
+    LAUNCH_OK(c, "prep_norm_kernel");
+  }
+  return launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, M, out, s.vocab);
 }
 
 // Kernels that need more than 48 KiB of dynamic shared memory must be told so once per device
@@ -846,7 +869,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   const int H = s.hidden, D = s.head_dim, QD = s.n_q_heads * D, KVD = s.n_kv_heads * D, I = s.intermediate;
 
   // weights; every bf16 context whose dimensions fit also gets the copy the tcgen05 GEMM reads:
-  // passes of more than 4 rows (batch x cycle length) and the prefill of every context use it
+  // every pass outside the pass kernel uses it
   c->umma_ok = s.weight_dtype == DMTD_BF16 && H % TG_KB == 0 && QD % TG_KB == 0 && I % TG_KB == 0;
   // DMTD_WEIGHT_COPIES=1 in the environment keeps only the atom stream (half the weight memory):
   // every projection then runs on the mma.sync kernels, the prefill included (slower from 5 rows up)
@@ -1120,10 +1143,16 @@ dmtd_status dmtd_masked_forward(dmtd_ctx *c, const int32_t *tokens, int32_t B, i
     masked_select_kernel<<<B * R, 256, 0, c->stream>>>(c->x_lo, c->h_base, R, H, p0, P, c->tau, c->literal_sum ? 1 : 0);   // Eq. 3-4
     LAUNCH_OK(c, "masked_select_kernel");
     for (int l = lo; l < L; ++l) TRY(run_layer(c, l, c->x_lo, B, R, &c->dstate->scratch, p0 + R));   // Eq. 5: decoding layers
-    for (int r = std::max(0, P - 1 - p0); r < R; ++r) {                                                // ... and the LM head
-      select_row_kernel<<<B, 256, 0, c->stream>>>(c->x_lo, R, r, H, c->x_up);
-      LAUNCH_OK(c, "select_row_kernel");
-      TRY(run_head(c, B, false, nullptr, out_logits + (size_t)(p0 + r - (P - 1)) * c->s.vocab, n_out * c->s.vocab));
+    // ... and the LM head on the chunk's rows from position P - 1 on
+    const int r0 = std::max(0, P - 1 - p0);
+    if (r0 >= R) continue;
+    const float *x0 = c->x_lo + (size_t)r0 * H;
+    float *out = out_logits + (size_t)(p0 + r0 - (P - 1)) * c->s.vocab;
+    if (R - r0 == (int)n_out) {
+      TRY(run_head_rows(c, x0, B, R - r0, R, out));                                  // all positions of all sequences
+    } else {
+      for (int b = 0; b < B; ++b)
+        TRY(run_head_rows(c, x0 + (size_t)b * R * H, 1, R - r0, R, out + (size_t)b * n_out * c->s.vocab));
     }
   }
   // the cache now holds this forward's K and V; the schedule state is untouched (still "no sequence")

@@ -1,5 +1,5 @@
 // Skinny GEMM on the 5th-generation tensor cores (tcgen05, sm_100a) for projections with many
-// activation rows: out[m][n] += sum_k W[n][k] act[m][k] for 5..128 rows m.
+// activation rows: out[m][n] += sum_k W[n][k] act[m][k] for 1..128 rows m.
 //
 // Operands are swapped against the usual orientation: the 128 weight rows of a tile are the M
 // axis of the MMA, the activation rows its N axis (each row as two columns, the bf16 hi and lo
@@ -243,11 +243,21 @@ __global__ void act_blocks_kernel(const float *__restrict__ act_all, int lda, in
 // path): block g < n_groups takes 4 rows (a sweep of the GEMM is n_cols / 2 rows, padded with zero
 // rows), sums their squares, and writes their hi and lo columns of every k block; the blocks
 // behind them clear the buffer the GEMM accumulates into.  x [rows][ldx] fp32; K values per row.
+// Row m of the launch is row m0 + m of the activations, whose rows come in segments of seg_rows every
+// seg_stride rows of x (the rows of a chunk that the LM head reads when logits of many positions are asked for);
+// seg_rows = 0: one segment.
 constexpr int NAB_ROWS = 4;
-__global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, const float *__restrict__ w,
-                                                              float eps, int rows_all, int K, int n_cols,
-                                                              uint4 *__restrict__ blocks_all, int n_groups,
-                                                              float4 *__restrict__ zero, size_t zero_n4) {
+struct RowSegments {
+  int m0, seg_rows, seg_stride;
+  __host__ __device__ __forceinline__ size_t row(int m) const {
+    m += m0;
+    return seg_rows > 0 ? (size_t)(m / seg_rows) * seg_stride + m % seg_rows : (size_t)m;
+  }
+};
+__global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, RowSegments seg,
+                                                              const float *__restrict__ w, float eps, int rows_all, int K,
+                                                              int n_cols, uint4 *__restrict__ blocks_all, int n_groups,
+                                                              float *__restrict__ zero, size_t zero_n) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
@@ -255,9 +265,13 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if ((int)blockIdx.x >= n_groups) {
     const size_t n_z = (size_t)(gridDim.x - n_groups) * gridDim.y;
-    for (size_t i = ((size_t)(blockIdx.x - n_groups) * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x; i < zero_n4;
-         i += n_z * blockDim.x)
-      zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const size_t i0 = ((size_t)(blockIdx.x - n_groups) * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x;
+    const size_t head = min(zero_n, (size_t)((16 - (reinterpret_cast<uintptr_t>(zero) & 15)) & 15) / 4);   // up to the first 16-byte boundary
+    float4 *z4 = reinterpret_cast<float4 *>(zero + head);
+    const size_t n4 = (zero_n - head) / 4;
+    for (size_t i = i0; i < n4; i += n_z * blockDim.x) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i0 < head) zero[i0] = 0.f;
+    if (i0 < zero_n - head - n4 * 4) zero[head + n4 * 4 + i0] = 0.f;
     return;
   }
   const int sweep_rows = n_cols / 2, groups_per_sweep = sweep_rows / NAB_ROWS;
@@ -272,7 +286,7 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
     const int r = warp >> 1, m = m0 + r;
     float ss = 0.f;
     if (m < rows_all) {
-      const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)m * ldx);
+      const float4 *xr = reinterpret_cast<const float4 *>(x + seg.row(m) * ldx);
       for (int k4 = (warp & 1) * 32 + lane; k4 < K / 4; k4 += 64) {
         const float4 v = xr[k4];
         ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
@@ -293,8 +307,9 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
     const int m = m0 + r, k = kb * TG_KB + c * 8;
     uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
     if (m < rows_all) {
-      const float4 a = *reinterpret_cast<const float4 *>(x + (size_t)m * ldx + k);
-      const float4 b = *reinterpret_cast<const float4 *>(x + (size_t)m * ldx + k + 4);
+      const float *xr = x + seg.row(m) * ldx;
+      const float4 a = *reinterpret_cast<const float4 *>(xr + k);
+      const float4 b = *reinterpret_cast<const float4 *>(xr + k + 4);
       const float4 wa = __ldg(reinterpret_cast<const float4 *>(w + k)), wb = __ldg(reinterpret_cast<const float4 *>(w + k + 4));
       const float s = inv[r];
       const float f[8] = {a.x * s * wa.x, a.y * s * wa.y, a.z * s * wa.z, a.w * s * wa.w,

@@ -92,7 +92,7 @@ __global__ void prep_norm_kernel(const float *__restrict__ x, int ldx, const flo
   if (zero_buf) {
     const int c0 = blockIdx.y * PREP_ZERO_COLS, c1 = min(zero_cols, c0 + PREP_ZERO_COLS);
     float *row = zero_buf + (size_t)m * zero_ld;
-    const bool aligned = (zero_ld & 3) == 0;              // then every row starts on a 16-byte boundary
+    const bool aligned = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
     for (int k = c0 + threadIdx.x * 4; k < c1; k += blockDim.x * 4) {
       if (aligned && k + 4 <= c1) *reinterpret_cast<float4 *>(row + k) = make_float4(0.f, 0.f, 0.f, 0.f);
       else for (int j = k; j < c1; ++j) row[j] = 0.f;
@@ -583,13 +583,6 @@ __global__ void masked_select_kernel(float *__restrict__ x, const float *__restr
   const float *br = base + (size_t)blockIdx.x * H;
   if (m && !literal_sum) return;
   for (int k = threadIdx.x; k < H; k += blockDim.x) xr[k] = m ? br[k] + xr[k] : br[k];
-}
-
-// x_up[b][:] = x[b][r][:]
-__global__ void select_row_kernel(const float *__restrict__ x, int R, int r, int H, float *__restrict__ x_up) {
-  const int b = blockIdx.x;
-  const float *src = x + ((size_t)b * R + r) * H;
-  for (int k = threadIdx.x; k < H; k += blockDim.x) x_up[(size_t)b * H + k] = src[k];
 }
 
 // ------------------------------------------------------------------------------------

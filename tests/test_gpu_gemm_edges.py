@@ -1,0 +1,55 @@
+"""Projections on the tcgen05 GEMM at the sizes where its tiles, row counts and work shares end: the scoring pass
+(its LM head takes all positions in one GEMM) and teacher-forced decoding against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from synthetic import SHAPES, make_prompts, make_weights
+
+from helpers import check_logits, gpu_forced, oracle_forced, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+# every K a multiple of 64, so that the tcgen05 GEMM runs; a vocabulary that no 4-value load divides
+SHAPE = SHAPES["mid"].with_(n_layers=4, intermediate=1856, vocab=5001)
+
+
+@pytest.fixture(scope="module")
+def dmtd():
+    import paper_2510_11958_b200 as pkg
+    pkg.load_library()
+    return pkg
+
+
+@pytest.mark.parametrize("B,P,n", [
+    (1, 1, 1),              # a single row
+    (1, 3, 6),              # 4 rows: fewer than the mma.sync kernels' limit
+    (2, 7, 71),             # rows of two sequences, in one segment each
+    (1, 5, 133),            # 129 rows in the head: one more than a sweep
+    (3, 40, 400),           # several chunks of the workspace (256 rows of three sequences each)
+])
+def test_scoring_pass(dmtd, B, P, n):
+    w = make_weights(SHAPE, seed=0, norm_jitter=0.1)
+    tokens = make_prompts(SHAPE.vocab, B, n, seed=5).numpy()
+    eng = dmtd.Dmtd(SHAPE, to_cuda(w), L_d=2, tau=3, max_batch=B, max_seq=n + 2, kv_dtype="f32")
+    got = eng.masked_forward(torch.from_numpy(tokens).cuda(), P).double().cpu().numpy()
+    for b in range(B):
+        ref = oracle.masked_parallel_forward(SHAPE, w, 2, 3, tokens[b], P)
+        # fp32 cache and sums, bf16 hi + lo activations (2^-17): the bound of the other fp32-cache tests
+        assert np.abs(got[b] - ref).max() < 1e-3
+
+
+@pytest.mark.parametrize("B,tau", [(1, 1), (1, 3), (3, 1), (4, 1), (5, 3), (17, 4), (43, 3)])
+def test_decode_rows(dmtd, B, tau):
+    """1 to 129 rows a pass on the per-step kernels."""
+    w = make_weights(SHAPE, seed=0, norm_jitter=0.1)
+    prompts = make_prompts(SHAPE.vocab, B, 9, seed=1).numpy()
+    forced = make_prompts(SHAPE.vocab, B, 2 * tau + 2, seed=2).numpy()
+    ref_logits, ref_am, o = oracle_forced(SHAPE, w, 2, tau, prompts, forced)
+    eng = dmtd.Dmtd(SHAPE, to_cuda(w), L_d=2, tau=tau, max_batch=B, max_seq=9 + forced.shape[1] + 1, kv_dtype="f32")
+    eng.set_option("fused_pass", 0)
+    got_logits, got_am = gpu_forced(eng, prompts, forced)
+    err, _ = check_logits(got_logits, ref_logits, got_am, ref_am)
+    assert err < 1e-3
+    assert eng.device_state() == o.state()

@@ -221,7 +221,7 @@ dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs,
   int N = 0;
   for (int i = 0; i < n_src; ++i) N += Ns[i];
   UmmaMat m{};
-  m.N = N; m.K = K; m.n_tiles = (N + TG_ROWS - 1) / TG_ROWS; m.n_kb = K / TG_KB;
+  m.N = N; m.K = K; m.n_tiles = (N + 2 * TG_ROWS - 1) / (2 * TG_ROWS) * 2; m.n_kb = K / TG_KB;
   uint4 *dst = nullptr;
   size_t units = (size_t)m.n_tiles * m.n_kb * (TG_WBLOCK / 16);
   c->mem_kind = 1;
@@ -257,10 +257,6 @@ dmtd_status launch_gemv_nt(dmtd_ctx *c, const PackedMat &W, const float *act, in
   return DMTD_OK;
 }
 
-// out[m][n] += sum_k W[n][k] act[m][k] on the tcgen05 tensor cores.  A block multiplies a 128-row
-// weight tile with up to 128 activation rows (a sweep); prefill chunks of more rows are several
-// sweeps in one launch (up to TG_MAX_SWEEPS), ordered so that the sweeps of one weight tile run
-// together and share it through L2.
 // Launch with programmatic stream serialisation: the kernel's blocks may become resident while the
 // kernel before it in the stream is still running; it calls griddepcontrol.wait before it touches
 // anything that kernel (or one before it) writes.
@@ -275,77 +271,50 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// With `norm_w` the activations are RMSNorm(act rows) * norm_w, computed while the blocks are written, and
+// out[m][n] += sum_k W[n][k] act[m][k] on the tcgen05 tensor cores: the kernel that writes the activation blocks, then
+// the GEMM.  With `norm_w` the activations are RMSNorm(act rows) * norm_w, computed while the blocks are written, and
 // the output rows are cleared first (the projections after a norm write a fresh buffer); the rows of `act` may
-// then come in segments (RowSegments).
+// then come in segments (RowSegments).  With merge_nsplit > 0 they are the attention's key slices, merged on the way.
 dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, int lda, int M, float *out, int ldo,
                              int gate_up_I = 0, const float *norm_w = nullptr, int merge_nsplit = 0, int seg_rows = 0,
                              int seg_stride = 0) {
-  const int SET = TG_MAX_COLS / 2;                       // rows per sweep
-  for (int m0 = 0; m0 < M; m0 += TG_MAX_SWEEPS * SET) {
-    GemmTcParams P{};
-    P.W = W; P.act_blocks = c->act_blocks;
-    P.rows = std::min(TG_MAX_SWEEPS * SET, M - m0);
-    P.n_sweeps = (P.rows + SET - 1) / SET;
-    P.n_cols = P.n_sweeps > 1 ? TG_MAX_COLS : (2 * P.rows + 15) / 16 * 16;
-    P.out = out + (size_t)m0 * ldo; P.ldo = ldo;
-    P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
-    // Every block of a launch should be resident at once (a block streams at the rate its own
-    // stages allow, so a second round of blocks doubles the time): blocks per SM follow from
-    // shared memory and tensor memory; with more row tiles than that, two-stage blocks make room
-    // for two per SM.  Row tiles are then split along k over as many blocks as still fit.
-    // (Several sweeps fill the SMs by themselves: no k split then.)
-    int tmem_cols = 32;
-    while (tmem_cols < P.n_cols) tmem_cols <<= 1;
-    auto smem_of = [&](int st) { return st * (TG_WBLOCK + P.n_cols * 128) + 128; };
-    auto per_sm_of = [&](int st) { return std::max(1, std::min((227 * 1024) / (smem_of(st) + 1024), 512 / tmem_cols)); };
-    // stages: what keeps the most weight blocks in flight per SM (stages x resident blocks: a block streams at the
-    // rate its bytes in flight allow), more resident blocks on a tie (their fill and epilogue overlap)
-    const int max_stages = std::min(TG_STAGES, (227 * 1024 - 1024 - 128) / (TG_WBLOCK + P.n_cols * 128));
-    P.stages = 2;
-    for (int st = 2; st <= max_stages; ++st)
-      if (st * per_sm_of(st) > P.stages * per_sm_of(P.stages)) P.stages = st;
-    if (c->gemm_stages >= 2) P.stages = std::min(c->gemm_stages, max_stages);
-    if (P.n_sweeps == 1 && W.n_tiles > c->n_sms * per_sm_of(P.stages) && W.n_tiles <= c->n_sms * per_sm_of(2)) P.stages = 2;
-    const int slots = c->n_sms * per_sm_of(P.stages);
-    P.ksplit = std::max(1, std::min(W.n_kb, slots / (W.n_tiles * P.n_sweeps)));
-    if (merge_nsplit > 0) {
-      // `act` is unused: the activations are the attention's key slices, merged on the way
-      const int n_groups = P.n_sweeps * (P.n_cols / 2 / NAB_ROWS);
-      const int ky = std::max(1, std::min(W.n_kb, 4 * c->n_sms / std::max(1, n_groups)));
-      CUDA_TRY(c, launch_pdl(merge_act_blocks_kernel, dim3(n_groups, ky), dim3(256), 0, c->stream,
-                             c->part_o + (size_t)m0 * c->s.n_q_heads * merge_nsplit * c->s.head_dim,
-                             c->part_ml + (size_t)m0 * c->s.n_q_heads * merge_nsplit * 2, merge_nsplit, c->s.n_q_heads,
-                             c->s.head_dim, P.rows, P.n_cols, c->act_blocks));
-      LAUNCH_OK(c, "merge_act_blocks_kernel");
-    } else if (norm_w) {
-      const int n_groups = P.n_sweeps * (P.n_cols / 2 / NAB_ROWS);
-      const size_t zero_n = (size_t)P.rows * ldo;
-      const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
-      const int ky = std::max(1, std::min(W.n_kb, 4 * c->n_sms / std::max(1, n_groups)));
-      CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
-                             act, lda, RowSegments{m0, seg_rows, seg_stride}, norm_w, c->s.rms_eps, P.rows, W.K, P.n_cols,
-                             c->act_blocks, n_groups, P.out, zero_n));
-      LAUNCH_OK(c, "norm_act_blocks_kernel");
-    } else {
-      long long units = (long long)W.n_kb * 8 * P.n_cols;
-      CUDA_TRY(c, launch_pdl(act_blocks_kernel, dim3((int)std::min<long long>((units + 255) / 256, 4096), P.n_sweeps), dim3(256), 0,
-                             c->stream, act + (size_t)m0 * lda, lda, P.rows, W.K, P.n_cols, c->act_blocks, gate_up_I));
-      LAUNCH_OK(c, "act_blocks_kernel");
-    }
-    int smem = smem_of(P.stages);
-    // launched with programmatic stream serialisation: its blocks may start (allocate tensor
-    // memory, request their first weight blocks) while act_blocks_kernel is still running
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(W.n_tiles * P.ksplit * P.n_sweeps); cfg.blockDim = dim3(TG_THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = c->stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
-    CUDA_TRY(c, cudaLaunchKernelEx(&cfg, gemm_tc05_kernel, P));
-    LAUNCH_OK(c, "gemm_tc05_kernel");
+  GemmTcParams P{};
+  P.W = W; P.act_blocks = c->act_blocks;
+  P.rows = M;
+  P.T = act_tiles_for(M, W.n_kb);
+  P.out = out; P.ldo = ldo;
+  P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
+  const int n_groups = (M + NAB_ROWS - 1) / NAB_ROWS, ky = std::max(1, std::min(W.n_kb, 4 * c->n_sms / n_groups));
+  if (merge_nsplit > 0) {
+    CUDA_TRY(c, launch_pdl(merge_act_blocks_kernel, dim3(n_groups, ky), dim3(256), 0, c->stream, c->part_o, c->part_ml,
+                           merge_nsplit, c->s.n_q_heads, c->s.head_dim, M, P.T, c->act_blocks));
+    LAUNCH_OK(c, "merge_act_blocks_kernel");
+  } else if (norm_w) {
+    const size_t zero_n = (size_t)M * ldo;
+    const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
+    CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
+                           act, lda, RowSegments{seg_rows, seg_stride}, norm_w, c->s.rms_eps, M, W.K, P.T,
+                           c->act_blocks, n_groups, out, zero_n));
+    LAUNCH_OK(c, "norm_act_blocks_kernel");
+  } else {
+    const int units = W.n_kb * 8 * M;
+    CUDA_TRY(c, launch_pdl(act_blocks_kernel, dim3(std::min((units + 255) / 256, 8 * c->n_sms)), dim3(256), 0, c->stream, act, lda,
+                           M, P.T, c->act_blocks, gate_up_I));
+    LAUNCH_OK(c, "act_blocks_kernel");
   }
+  // as many stages as shared memory holds, two accumulators where tensor memory does.  (Half of both for decode launches,
+  // so that the next projection's blocks become resident beside this one's and fetch their first weights, was no
+  // faster at 8-32 rows and slower at 96: fewer stages are in flight while a launch streams.)
+  const int n_cols = P.T.split ? 2 * P.T.tile_rows : P.T.tile_rows, stage_bytes = TG_WBLOCK + P.T.tile_rows * 128;
+  P.stages = std::max(2, std::min(TG_MAX_STAGES, (TG_MAX_SMEM - TG_TAIL_BYTES) / stage_bytes));
+  if (c->gemm_stages >= 2) P.stages = std::min(P.stages, c->gemm_stages);
+  int cols = 32;
+  while (cols < n_cols) cols <<= 1;
+  P.n_acc = 2 * cols <= 512 ? 2 : 1;
+  P.tmem_cols = P.n_acc * cols;
+  CUDA_TRY(c, launch_pdl(gemm_tc05_kernel, dim3(c->n_sms / 2 * 2), dim3(TG_THREADS), (size_t)P.stages * stage_bytes + TG_TAIL_BYTES,
+                         c->stream, P));
+  LAUNCH_OK(c, "gemm_tc05_kernel");
   return DMTD_OK;
 }
 
@@ -564,7 +533,7 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<1>, dyn, 100 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<2>, dyn, 100 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<4>, dyn, 100 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_kernel, dyn, 227 * 1024 - 1024));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_kernel, dyn, TG_MAX_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpBf16>, dyn, ATTN_TC_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpF16>, dyn, ATTN_TC_SMEM));
@@ -965,7 +934,11 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   c->pend_cap = std::max(1, c->ws_rows / max_batch);
   CTRY(dev_alloc(c, &c->h_pend, (size_t)max_batch * c->pend_cap * H));
   CTRY(dev_alloc(c, &c->h_base, (size_t)c->ws_rows * H));
-  if (c->umma_ok) CTRY(dev_alloc(c, &c->act_blocks, (size_t)TG_MAX_SWEEPS * (c->lda / TG_KB) * 8 * TG_MAX_COLS));
+  // activation blocks: hi and lo units of every row, the rows rounded up to whole column tiles
+  if (c->umma_ok) {
+    const size_t rows = (size_t)c->ws_rows + 16 * (c->ws_rows / TG_TILE_ROWS + 1);
+    CTRY(dev_alloc(c, &c->act_blocks, rows * (c->lda / 8) * 2));
+  }
   CTRY(configure_kernels(c));
   CTRY(setup_fused(c));
   CTRY(dmtd_reset(c));
@@ -1238,7 +1211,7 @@ dmtd_status dmtd_set_option(dmtd_ctx *c, const char *name, int64_t value) {
     c->L_e = (int)value; drop_graphs(c); return DMTD_OK;
   }
   if (!strcmp(name, "tcgen05_gemm_stages")) {
-    if (value != 0 && (value < 2 || value > TG_STAGES)) return fail(c, DMTD_ERR_INVALID_ARG, "tcgen05_gemm_stages takes 0 (chosen per launch) or 2..%d", TG_STAGES);
+    if (value != 0 && (value < 2 || value > 6)) return fail(c, DMTD_ERR_INVALID_ARG, "tcgen05_gemm_stages takes 0 (chosen per launch) or 2..6");
     c->gemm_stages = (int)value; drop_graphs(c); return DMTD_OK;
   }
   if (value != 0 && value != 1) return fail(c, DMTD_ERR_INVALID_ARG, "option %s takes 0 or 1", name);

@@ -1,55 +1,101 @@
-// Skinny GEMM on the 5th-generation tensor cores (tcgen05, sm_100a) for projections with many
-// activation rows: out[m][n] += sum_k W[n][k] act[m][k] for 1..128 rows m.
+// GEMM on the 5th-generation tensor cores (tcgen05, sm_100a) for every projection outside the pass kernel:
+// out[m][n] += sum_k W[n][k] act[m][k], one row m up to the rows of a prefill chunk.
 //
-// Operands are swapped against the usual orientation: the 128 weight rows of a tile are the M
-// axis of the MMA, the activation rows its N axis (each row as two columns, the bf16 hi and lo
-// parts of the fp32 activation, summed in the epilogue), so that every weight byte is read from
-// HBM once whatever the batch is.  Both operands are K-major in shared memory in the interleaved
-// (no swizzle) canonical form: 8 rows x 16 bytes per core matrix, core matrices of a 64-k block
-// ordered [k chunk of 8][row group of 8].  The weights are stored in global memory in exactly
-// that order (one 16 KiB block per (row tile, k block)), the activations are written that way by
-// act_blocks_kernel, so a pipeline stage is two bulk copies.  Accumulators live in tensor memory
-// (128 lanes x N columns of fp32), read back with tcgen05.ld for the epilogue.
+// Operands are swapped against the usual orientation: weight rows are the M axis of the MMA, activation rows its N
+// axis, so that every weight byte is read from HBM once whatever the batch is.  The fp32 activations enter as two
+// bf16 parts, hi + lo (error 2^-17 relative), one MMA each.  Two SMs work as a pair (cta_group::2): M = 256 weight
+// rows, 128 from each SM's shared memory, and each SM holds one half of the columns, which halves the activation
+// traffic per weight byte.
 //
-// Warp roles: warp 0 issues the bulk copies, warp 1 owns the tensor memory and issues the MMAs,
-// warps 2-5 run the epilogue (each reads the 32 lanes of its quarter).  Every wait is bounded and
-// reports through an error word; tensor memory is freed on every path.
+// Two forms of a column tile:
+//   up to 128 rows (decode):  hi and lo parts are columns of their own (N = 2 x rows): SM 0 of the pair holds the hi
+//     columns, SM 1 the lo columns, the epilogue adds them.  Four MMAs per 64-deep k block: one thread issues an MMA
+//     every 80 cycles or more whatever N is.
+//   more rows (prefill):      hi and lo MMAs add into the same columns (N = rows, up to 256 per tile): a weight block
+//     is multiplied with 256 rows x 2 parts for one copy into shared memory, 47 bytes per cycle and SM at full rate.
+//
+// Both operands are K-major in shared memory in the interleaved (no swizzle) canonical form: 8 rows x 16 bytes per
+// core matrix.  The weights are stored in global memory in exactly that order (16 KiB blocks, one per 128-row tile and
+// k block), the activations are written that way by the kernels below, so a pipeline stage is two bulk copies.
+//
+// Persistent: one pair of blocks per two SMs.  The work of a launch (row-tile pairs x column tiles x k blocks) is one
+// line of units, cut into equal shares whatever the shape is; a share that ends inside a tile adds its partial sums,
+// so every output is added with fp32 reductions (measured at 3.9 TB/s into L2; plain stores 4.8).  The accumulators
+// of a tile are read back while the next tile is multiplied where tensor memory holds two.
+//
+// Measured (Qwen3-4B shapes, launches back to back, against the kernel before this one: 128-row sweeps, one MMA-issuing
+// block per tile, hi and lo columns always apart): gate+up at 512 rows 139 -> 75 us (1350 TFLOP/s counting both
+// parts, at the clock the power cap leaves), QKV 50 -> 29 us; head at 512 rows 541 us (1470 TFLOP/s); decode is bound by
+// HBM and by what a launch costs: head at 32 rows 127 us (6.1 TB/s), gate+up at 96 rows 44 -> 27 us, at 8 rows 24 us.
+//
+// Warp roles: warp 0 issues the bulk copies, warp 1 issues the MMAs (first SM of the pair) or passes on to the first
+// SM that a stage has landed (second SM), warps 2-9 run the epilogue (each the 32 lanes of its quarter, every second 16 columns).  Every wait is
+// bounded and reports through an error word; tensor memory is freed on every path.
 #pragma once
 
 #include "pass_stream.cuh"
 
 namespace dmtd {
 
-constexpr int TG_THREADS = 192;
-constexpr int TG_STAGES = 6;                 // most pipeline stages a block may be given
-constexpr int TG_ROWS = 128;                 // weight rows per tile (MMA M)
-constexpr int TG_KB = 64;                    // k per pipeline stage: four MMAs of K = 16
+constexpr int TG_EPI_WARPS = 8;              // epilogue warps: two per quarter of the tensor-memory lanes
+constexpr int TG_THREADS = 64 + 32 * TG_EPI_WARPS;
+constexpr int TG_MAX_STAGES = 8;             // most pipeline stages of a block
+constexpr int TG_ROWS = 128;                 // weight rows per tile; a pair of blocks takes two tiles (MMA M = 256)
+constexpr int TG_KB = 64;                    // k per pipeline stage: four MMAs of K = 16 (per part)
 constexpr int TG_WBLOCK = TG_ROWS * TG_KB * 2;      // 16384 bytes
-constexpr int TG_MAX_COLS = 256;             // MMA N: two columns per activation row
-constexpr int TG_MAX_SWEEPS = 8;             // sweeps of 128 activation rows in one launch
+constexpr int TG_SPLIT_ROWS = 128;           // most rows of a column tile with hi and lo in columns of their own
+constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
+constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
+constexpr int TG_MAX_SMEM = 226 * 1024;      // dynamic shared memory of a block: it has its SM to itself
 enum { TG_ERR_WAIT = 4 };
 
 // A weight matrix [N][K] as 16 KiB blocks [row tile][k block][k chunk 8][row group 16][row 8][8 values].
 struct UmmaMat {
   const uint4 *w;
   int N, K;
-  int n_tiles;       // ceil(N / 128)
+  int n_tiles;       // ceil(N / 128), rounded up to even (the last tile may be all zero)
   int n_kb;          // K / 64
 };
 
+// How a launch's activation rows are cut into column tiles, and where their 16-byte units (8 values of k of one row,
+// hi or lo part) lie: per column tile and k block the two SMs' shares one after the other, each in the canonical
+// K-major order [part][k chunk 8][column].
+struct ActTiles {
+  int n_kb;
+  int n_ctiles;      // column tiles
+  int tile_rows;     // activation rows per column tile: a multiple of 8 (split parts) or 16
+  int split;         // 1: SM 0 holds the hi columns of all rows, SM 1 the lo columns; 0: each SM holds half of the rows, both parts
+  __host__ __device__ __forceinline__ size_t units_per_sm() const { return (size_t)tile_rows * 8; }      // of one k block
+  // unit of (row m, k block kb, k chunk c): hi part; the lo part lies lo_offset() further
+  __device__ __forceinline__ size_t unit(int m, int kb, int c) const {
+    const int ct = m / tile_rows, col = m - ct * tile_rows;
+    const size_t base = ((size_t)ct * n_kb + kb) * 2 * units_per_sm();
+    if (split) return base + c * tile_rows + col;
+    const int half = tile_rows / 2, sm = col >= half ? 1 : 0;
+    return base + sm * units_per_sm() + c * half + (col - sm * half);
+  }
+  __device__ __forceinline__ size_t lo_offset() const { return split ? units_per_sm() : units_per_sm() / 2; }
+};
+
+inline ActTiles act_tiles_for(int rows, int n_kb) {
+  ActTiles t;
+  t.n_kb = n_kb;
+  t.split = rows <= TG_SPLIT_ROWS;
+  t.n_ctiles = t.split ? 1 : (rows + TG_TILE_ROWS - 1) / TG_TILE_ROWS;
+  const int per = (rows + t.n_ctiles - 1) / t.n_ctiles, unit = t.split ? 8 : 16;
+  t.tile_rows = (per + unit - 1) / unit * unit;
+  return t;
+}
+
 struct GemmTcParams {
   UmmaMat W;
-  const uint4 *act_blocks;   // [k block][N_cols * 128 bytes], see act_blocks_kernel
-  int n_cols;                // MMA N: multiple of 16, >= 2 * rows
+  const uint4 *act_blocks;
+  ActTiles T;
   int rows;                  // activation rows of this launch
-  float *out;                // [rows][ldo], accumulated into
+  float *out;                // [rows][ldo], added into
   int ldo;
-  int ksplit;                // blocks per row tile, each taking a share of the k blocks
-  int stages;                // pipeline stages of a block, 2 .. TG_STAGES
-  int n_sweeps;              // sets of up to 128 activation rows in this launch (prefill chunks); set s has its
-                             // activation blocks s * n_kb blocks further and its output rows 128 s further.
-                             // Consecutive blocks of the grid are the sweeps of one (row tile, k share): they
-                             // run together, and all but the first find the weight blocks in L2.
+  int stages;                // pipeline stages of a block, 2 .. TG_MAX_STAGES
+  int n_acc, tmem_cols;      // accumulators in tensor memory (1 or 2), tmem_cols / n_acc columns apart
   int *error;
   long long wait_limit;
 };
@@ -61,202 +107,342 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t smem_addr, uint32_t 
          (1ull << 46);
 }
 
-// kind::f16 instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, M = 128, N = n_cols
-__device__ __forceinline__ uint32_t umma_instr_desc(int n_cols) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_cols >> 3) << 17) | ((uint32_t)(TG_ROWS >> 4) << 24);
+// kind::f16 instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, M x N
+__device__ __forceinline__ uint32_t umma_instr_desc(int m, int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-__device__ __forceinline__ bool tg_wait(uint32_t bar, uint32_t parity, const GemmTcParams &P) {
-  if (mbar_try_wait(bar, parity)) return true;
+// Bounded wait.  The error word (another block gave up) is looked at only after the wait has lasted half a
+// millisecond: a read of global memory inside the spin takes a microsecond under load, which made every wait that
+// long (head at 8 rows 2.2 TB/s instead of 6).
+__device__ __noinline__ bool tg_wait_slow(uint32_t bar, uint32_t parity, const GemmTcParams &P) {
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > P.wait_limit || *reinterpret_cast<volatile int *>(P.error) >= TG_ERR_WAIT) {
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i)
+      if (mbar_try_wait(bar, parity)) return true;
+    const long long dt = clock64() - t0;
+    if (dt > (1 << 20) && (dt > P.wait_limit || *reinterpret_cast<volatile int *>(P.error) >= TG_ERR_WAIT)) {
       atomicMax(P.error, TG_ERR_WAIT);
       return false;
     }
   }
-  return true;
 }
-
-__global__ void __launch_bounds__(TG_THREADS, 1) gemm_tc05_kernel(const __grid_constant__ GemmTcParams P) {
+__device__ __forceinline__ bool tg_wait(uint32_t bar, uint32_t parity, const GemmTcParams &P) {
+  return mbar_try_wait(bar, parity) || tg_wait_slow(bar, parity, P);
+}
+// Arrive on the barrier at the same place in the first SM of the pair.  Without a scope: what is handed over is the
+// completion of bulk copies and of tensor-memory loads, not this thread's stores, and an arrive that releases at
+// cluster scope waits for a fence of about 2000 cycles under load, once per stage.
+__device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
+  asm volatile(
+      "{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, 0;\n"
+      " mbarrier.arrive.shared::cluster.b64 _, [a];\n}\n" ::"r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+  // arrives on the barrier at this place in both SMs once the MMAs issued so far are complete
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+}
+__device__ __forceinline__ void red_add(float *p, float v) {
+  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_tc05_kernel(const __grid_constant__ GemmTcParams P) {
   extern __shared__ __align__(1024) unsigned char tg_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int act_block = P.n_cols * 128, stage_bytes = TG_WBLOCK + act_block;
-  const int S = P.stages;
-  uint64_t *bars = reinterpret_cast<uint64_t *>(tg_smem + S * stage_bytes);    // full[S], empty[S], done
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
-  volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 1);   // a wait of this block ran out: no epilogue
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S), done = smem_u32(bars + 2 * S);
+  const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int S = P.stages, n_kb = P.W.n_kb, tile_rows = P.T.tile_rows;
+  const uint32_t act_bytes = (uint32_t)tile_rows * 128, stage_bytes = TG_WBLOCK + act_bytes;
+  unsigned char *const tail = tg_smem + (size_t)S * stage_bytes;
+  const uint32_t full0 = smem_u32(tail), empty0 = full0 + 8 * TG_MAX_STAGES, acc_full0 = empty0 + 8 * TG_MAX_STAGES,
+                 acc_empty0 = acc_full0 + 16;
+  uint32_t *const tmem_slot = reinterpret_cast<uint32_t *>(tail + 16 * TG_MAX_STAGES + 32);
+  volatile int *const gave_up = reinterpret_cast<volatile int *>(tmem_slot + 1);   // a wait of this block ran out: no more output
 
-  const int sweep = blockIdx.x % P.n_sweeps, unit = blockIdx.x / P.n_sweeps;
-  const int tile = unit / P.ksplit, ks = unit % P.ksplit;
-  const int rows = min(TG_MAX_COLS / 2, P.rows - sweep * (TG_MAX_COLS / 2));        // rows of this sweep
-  const uint4 *act_blocks = P.act_blocks + (size_t)sweep * P.W.n_kb * (P.n_cols * 8);
-  float *out = P.out + (size_t)sweep * (TG_MAX_COLS / 2) * P.ldo;
-  const int kb0 = P.W.n_kb * ks / P.ksplit, kb1 = P.W.n_kb * (ks + 1) / P.ksplit, n_it = kb1 - kb0;
-  int tmem_cols = 32;
-  while (tmem_cols < P.n_cols) tmem_cols <<= 1;
+  // this pair's share of the units (row-tile pair, column tile, k block), k fastest, then the column tile
+  const long long n_units = (long long)(P.W.n_tiles / 2) * P.T.n_ctiles * n_kb;
+  const int u0 = (int)(n_units * pair / n_pairs), u1 = (int)(n_units * (pair + 1) / n_pairs);
 
   // the kernel after this one (the next projection's activation-block kernel, launched the same way) may become
   // resident now; it waits for this grid's completion before it reads or writes anything, and the GEMM behind it
   // can then request its first weight blocks while this grid's last blocks finish
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // producer's position in the share (thread 0)
+  int kb_w = u0 % n_kb, ct_w = (u0 / n_kb) % P.T.n_ctiles, rt_w = u0 / n_kb / P.T.n_ctiles;
+  int kb_a = kb_w, ct_a = ct_w;
+  auto copy_w = [&](int st) {
+    bulk_g2s(smem_u32(tg_smem) + st * stage_bytes, P.W.w + ((size_t)(2 * rt_w + rank) * n_kb + kb_w) * (TG_WBLOCK / 16), TG_WBLOCK,
+             full0 + st * 8);
+    if (++kb_w == n_kb) {
+      kb_w = 0;
+      if (++ct_w == P.T.n_ctiles) { ct_w = 0; ++rt_w; }
+    }
+  };
+  auto copy_act = [&](int st) {
+    bulk_g2s(smem_u32(tg_smem) + st * stage_bytes + TG_WBLOCK,
+             P.act_blocks + (((size_t)ct_a * n_kb + kb_a) * 2 + rank) * P.T.units_per_sm(), act_bytes, full0 + st * 8);
+    if (++kb_a == n_kb) {
+      kb_a = 0;
+      if (++ct_a == P.T.n_ctiles) ct_a = 0;
+    }
+  };
+  const int n_it = u1 - u0, n_first = min(S, n_it);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2 * S + 1; ++s) mbar_init(smem_u32(bars + s), 1);
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full0 + s * 8, rank == 0 ? 2 : 1);       // this block's copies; on the first SM also the other's
+      mbar_init(empty0 + s * 8, 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(acc_full0 + a * 8, 1);
+      mbar_init(acc_empty0 + a * 8, 2 * TG_EPI_WARPS);   // the epilogue warps of both blocks
+    }
     *gave_up = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(P.tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if (threadIdx.x == 0) {
+    // the weight blocks of the first stages are requested before the other block is waited for: they touch this
+    // block's barriers only, and eight copies take the issuing thread some thousand cycles
+    for (int i = 0; i < n_first; ++i) {
+      mbar_expect_tx(full0 + i * 8, stage_bytes);
+      copy_w(i);
+    }
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  const int acc_cols = P.tmem_cols / P.n_acc;
 
-  if (warp == 0 && lane == 0) {
-    // ---- producer: two bulk copies per k block.  The kernel is launched so that it may start
-    // while the kernel before it (which writes the activation blocks) is still running: the
-    // weight blocks of the first stages are requested at once, the activation blocks only after
-    // that kernel has completed and its writes are visible.
-    const int n_first = min(S, n_it);
-    for (int i = 0; i < n_first; ++i) {
-      mbar_expect_tx(full0 + i * 8, (uint32_t)stage_bytes);
-      bulk_g2s(smem_u32(tg_smem + i * stage_bytes), P.W.w + ((size_t)tile * P.W.n_kb + kb0 + i) * (TG_WBLOCK / 16), TG_WBLOCK,
-               full0 + i * 8);
-    }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = 0; i < n_first; ++i)
-      bulk_g2s(smem_u32(tg_smem + i * stage_bytes) + TG_WBLOCK, act_blocks + (size_t)(kb0 + i) * (act_block / 16),
-               (uint32_t)act_block, full0 + i * 8);
-    for (int i = n_first; i < n_it; ++i) {
-      const int st = i % S;
-      if (!tg_wait(empty0 + st * 8, ((i / S) - 1) & 1, P)) break;
-      const uint32_t dst = smem_u32(tg_smem + st * stage_bytes);
-      mbar_expect_tx(full0 + st * 8, (uint32_t)stage_bytes);
-      bulk_g2s(dst, P.W.w + ((size_t)tile * P.W.n_kb + kb0 + i) * (TG_WBLOCK / 16), TG_WBLOCK, full0 + st * 8);
-      bulk_g2s(dst + TG_WBLOCK, act_blocks + (size_t)(kb0 + i) * (act_block / 16), (uint32_t)act_block, full0 + st * 8);
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer: four K = 16 MMAs per k block, then release the stage
-    const uint32_t idesc = umma_instr_desc(P.n_cols);
-    const uint32_t b_lbo = (uint32_t)(P.n_cols / 8) * 128;
-    bool ok = true;
-    for (int i = 0; i < n_it && ok; ++i) {
-      const int st = i % S;
-      ok = tg_wait(full0 + st * 8, (i / S) & 1, P);
-      if (!ok) { *gave_up = 1; __threadfence_block(); break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_base = smem_u32(tg_smem + st * stage_bytes), b_base = a_base + TG_WBLOCK;
-#pragma unroll
-      for (int kk = 0; kk < TG_KB / 16; ++kk) {
-        const uint64_t da = umma_smem_desc(a_base + kk * 2 * (TG_ROWS / 8) * 128, (TG_ROWS / 8) * 128, 128);
-        const uint64_t db = umma_smem_desc(b_base + kk * 2 * b_lbo, b_lbo, 128);
-        const uint32_t accumulate = (i > 0 || kk > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n}\n" ::"r"(tmem),
-            "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(0u)
-            : "memory");
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- producer: two bulk copies per unit; the activation blocks only after the kernel that writes them has
+      // completed and its writes are visible
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      for (int i = 0; i < n_first; ++i) copy_act(i);
+      int st = 0, issued = n_first;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int i = n_first; i < n_it; ++i) {
+        ok = tg_wait(empty0 + st * 8, ph, P);
+        if (!ok) break;
+        mbar_expect_tx(full0 + st * 8, stage_bytes);
+        copy_w(st);
+        copy_act(st);
+        ++issued;
+        if (++st == S) { st = 0; ph ^= 1; }
       }
-      // arrives on the stage's empty barrier once the MMAs issued so far have read shared memory
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty0 + st * 8) : "memory");
-    }
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done) : "memory");
-  } else if (warp >= 2) {
-    // ---- epilogue: thread = weight row (lane of tensor memory), registers = columns
-    const int quarter = warp & 3;
-    const int n = tile * TG_ROWS + quarter * 32 + lane;
-    // the accumulators are complete only if no wait of this block ran out
-    if (tg_wait(done, 0, P) && !*gave_up) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int c0 = 0; c0 < P.n_cols && c0 < 2 * rows; c0 += 16) {
-        uint32_t r[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + c0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int m = (c0 >> 1) + j;                  // columns 2m (hi) and 2m + 1 (lo) belong to activation row m
-          if (m < rows && n < P.W.N) atomicAdd(out + (size_t)m * P.ldo + n, __uint_as_float(r[2 * j]) + __uint_as_float(r[2 * j + 1]));
+      if (!ok) {
+        // leave no copy in flight: each stage's last copies get a bounded wait
+        for (int i = max(0, issued - S); i < issued; ++i) {
+          const long long t0 = clock64();
+          while (!mbar_try_wait(full0 + (i % S) * 8, (i / S) & 1))
+            if (clock64() - t0 > P.wait_limit) break;
         }
       }
     }
+  } else if (warp == 1 && rank == 0) {
+    // ---- MMA issuer
+    const int n_cols = P.T.split ? 2 * tile_rows : tile_rows;         // MMA N
+    const uint32_t idesc = umma_instr_desc(2 * TG_ROWS, n_cols);
+    const uint32_t b_lbo = (uint32_t)(n_cols / 2) * 16, part_bytes = b_lbo * 8;
+    int kb = u0 % n_kb, st = 0, acc = 0;
+    uint32_t ph = 0, acc_ph = 1;                                      // the accumulators start free
+    bool first = true, ok = true;
+    for (int u = u0; u < u1; ++u) {
+      if (first) {
+        ok = __all_sync(0xffffffffu, tg_wait(acc_empty0 + acc * 8, acc_ph, P));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      }
+      ok = __all_sync(0xffffffffu, tg_wait(full0 + st * 8, ph, P));
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const bool last = ++kb == n_kb || u + 1 == u1;
+      if (elect_one()) {
+        const uint32_t a_base = smem_u32(tg_smem) + st * stage_bytes, b_base = a_base + TG_WBLOCK;
+        const uint32_t d = tmem + acc * acc_cols;
+        uint64_t da = umma_smem_desc(a_base, (TG_ROWS / 8) * 128, 128), db = umma_smem_desc(b_base, b_lbo, 128);
+        const uint64_t da_step = 2 * (TG_ROWS / 8) * 128 / 16, db_step = 2 * b_lbo / 16, part_step = part_bytes / 16;
+        uint32_t accumulate = first ? 0u : 1u;
+#pragma unroll
+        for (int kk = 0; kk < TG_KB / 16; ++kk) {
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+              "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+              : "memory");
+          accumulate = 1u;
+          if (!P.T.split)                                             // the lo part into the same columns
+            asm volatile(
+                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                "l"(da), "l"(db + part_step), "r"(idesc), "r"(1u)
+                : "memory");
+          da += da_step;
+          db += db_step;
+        }
+        umma_commit_pair(empty0 + st * 8);
+        if (last) umma_commit_pair(acc_full0 + acc * 8);
+      }
+      __syncwarp();
+      first = last;
+      if (last) {
+        kb = 0;
+        if (++acc == P.n_acc) { acc = 0; acc_ph ^= 1; }
+      }
+      if (++st == S) { st = 0; ph ^= 1; }
+    }
+    if (!ok && lane == 0) { *gave_up = 1; __threadfence_block(); }
+  } else if (warp == 1) {
+    // ---- second SM: pass every landed stage on to the issuer
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 0;
+      for (int u = u0; u < u1; ++u) {
+        if (!tg_wait(full0 + st * 8, ph, P)) break;
+        mbar_arrive_leader(full0 + st * 8);
+        if (++st == S) { st = 0; ph ^= 1; }
+      }
+    }
+  } else {
+    // ---- epilogue: thread = weight row (lane of tensor memory), registers = columns
+    const int quarter = warp & 3;
+    int u = u0, acc = 0;
+    uint32_t ph = 0;
+    while (u < u1) {
+      const int tile = u / n_kb, ct = tile % P.T.n_ctiles, rt = tile / P.T.n_ctiles;
+      u = min(u1, (tile + 1) * n_kb);
+      const bool ok = __all_sync(0xffffffffu, tg_wait(acc_full0 + acc * 8, ph, P)) && !*gave_up;
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int n = (2 * rt + rank) * TG_ROWS + quarter * 32 + lane;
+      const int m0 = ct * tile_rows, n_rows = min(tile_rows, P.rows - m0);
+      const uint32_t t_base = tmem + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols;
+      const int c_first = warp < 6 ? 0 : 16;
+      float *dst = P.out + (size_t)(m0 + c_first) * P.ldo + n;
+#pragma unroll 1
+      for (int c0 = c_first; c0 < n_rows; c0 += 32) {
+        uint32_t r[16];
+        tmem_ld16(t_base + c0, r);
+        if (P.T.split) {                                              // the lo columns
+          uint32_t q[16];
+          tmem_ld16(t_base + tile_rows + c0, q);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(q[j]));
+        } else {
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        }
+        // straight-line code for whole groups of 16 rows: a warp has its scheduler to itself, every instruction counts
+        if (n < P.W.N) {
+          if (c0 + 16 <= n_rows) {
+            float *d = dst;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              red_add(d, __uint_as_float(r[j]));
+              d += P.ldo;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 15; ++j)
+              if (c0 + j < n_rows) red_add(dst + (size_t)j * P.ldo, __uint_as_float(r[j]));
+          }
+        }
+        dst += (size_t)32 * P.ldo;
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_leader(acc_empty0 + acc * 8);
+      if (++acc == P.n_acc) { acc = 0; ph ^= 1; }
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  // the other block is done with this one's shared and tensor memory (no release: it would wait for the reductions)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.tmem_cols) : "memory");
   }
 }
 
-// Activations [rows][lda] fp32 -> bf16 hi/lo columns in the canonical K-major block order:
-// block kb holds k = 64 kb .. 64 kb + 63 as [k chunk 8][column group n_cols/8][column 8][8 values];
-// column 2m is the hi part of row m, column 2m + 1 its lo part; columns beyond 2 * rows are zero.
-// blockIdx.y = set of up to 128 rows (a sweep of the GEMM): its rows start 128 y further, its
-// blocks n_kb blocks further.
+// Activations [rows][lda] fp32 -> bf16 hi/lo units in the order of ActTiles.  One thread per unit: 8 values of k of a
+// row, both parts; neighbouring threads take neighbouring rows (consecutive 16-byte stores, 32-byte reads).
 // With gate_up_I > 0 the source rows hold gate | up values (gate at k, up at gate_up_I + k) and the
 // activation is the SwiGLU gate silu(gate) * up (step a6, second half), computed on the way.
-__global__ void act_blocks_kernel(const float *__restrict__ act_all, int lda, int rows_all, int K, int n_cols,
-                                  uint4 *__restrict__ blocks_all, int gate_up_I) {
-  const int rows = min(TG_MAX_COLS / 2, rows_all - (int)blockIdx.y * (TG_MAX_COLS / 2));
-  const float *act = act_all + (size_t)blockIdx.y * (TG_MAX_COLS / 2) * lda;
-  uint4 *blocks = blocks_all + (size_t)blockIdx.y * (K / TG_KB) * (n_cols * 8);
+__device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, size_t lo_offset) {
+  uint32_t hi[4], lo[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    hi[j] = pack_bf16x2(f[2 * j], f[2 * j + 1]);
+    lo[j] = pack_bf16x2(f[2 * j] - __uint_as_float(hi[j] << 16), f[2 * j + 1] - __uint_as_float(hi[j] & 0xffff0000u));
+  }
+  dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  dst[lo_offset] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+__global__ void act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T, uint4 *__restrict__ blocks,
+                                  int gate_up_I) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int n_kb = K / TG_KB;
-  const long long total = (long long)n_kb * 8 * n_cols;            // 16-byte units
-  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += (long long)gridDim.x * blockDim.x) {
-    const int col = (int)(u % n_cols), c = (int)((u / n_cols) % 8), kb = (int)(u / n_cols / 8);
-    const int m = col >> 1, k = kb * TG_KB + c * 8;
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    if (m < rows) {
-      const float4 a = *reinterpret_cast<const float4 *>(act + (size_t)m * lda + k);
-      const float4 b = *reinterpret_cast<const float4 *>(act + (size_t)m * lda + k + 4);
-      float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-      if (gate_up_I > 0) {
-        const float4 ua = *reinterpret_cast<const float4 *>(act + (size_t)m * lda + gate_up_I + k);
-        const float4 ub = *reinterpret_cast<const float4 *>(act + (size_t)m * lda + gate_up_I + k + 4);
-        const float u[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
+  const int total = T.n_kb * 8 * rows;
+  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
+    const int m = u % rows, kc = u / rows, k = kc * 8;
+    const float *src = act + (size_t)m * lda + k;
+    const float4 a = *reinterpret_cast<const float4 *>(src), b = *reinterpret_cast<const float4 *>(src + 4);
+    float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    if (gate_up_I > 0) {
+      const float4 ua = *reinterpret_cast<const float4 *>(src + gate_up_I);
+      const float4 ub = *reinterpret_cast<const float4 *>(src + gate_up_I + 4);
+      const float up[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) f[j] = f[j] / (1.f + expf(-f[j])) * u[j];
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t h = pack_bf16x2(f[2 * j], f[2 * j + 1]);
-        w[j] = (col & 1) ? pack_bf16x2(f[2 * j] - __uint_as_float(h << 16), f[2 * j + 1] - __uint_as_float(h & 0xffff0000u)) : h;
-      }
+      for (int j = 0; j < 8; ++j) f[j] = f[j] / (1.f + expf(-f[j])) * up[j];
     }
-    // column group = col / 8, column in group = col % 8
-    blocks[((size_t)kb * 8 + c) * n_cols + col] = make_uint4(w[0], w[1], w[2], w[3]);
+    store_hi_lo(f, blocks + T.unit(m, kc >> 3, kc & 7), T.lo_offset());
   }
 }
 
 // RMSNorm and the activation blocks in one kernel (steps a2 / a6 / a9, first half, on the tcgen05
-// path): block g < n_groups takes 4 rows (a sweep of the GEMM is n_cols / 2 rows, padded with zero
-// rows), sums their squares, and writes their hi and lo columns of every k block; the blocks
-// behind them clear the buffer the GEMM accumulates into.  x [rows][ldx] fp32; K values per row.
-// Row m of the launch is row m0 + m of the activations, whose rows come in segments of seg_rows every
-// seg_stride rows of x (the rows of a chunk that the LM head reads when logits of many positions are asked for);
-// seg_rows = 0: one segment.
+// path): block g < n_groups takes 4 rows, sums their squares, and writes their hi and lo parts of
+// every k block; the blocks behind them clear the buffer the GEMM accumulates into.  x [rows][ldx]
+// fp32; K values per row.
+// The rows come in segments of seg_rows every seg_stride rows of x (the rows of a chunk that the LM head
+// reads when logits of many positions are asked for); seg_rows = 0: one segment.
 constexpr int NAB_ROWS = 4;
 struct RowSegments {
-  int m0, seg_rows, seg_stride;
+  int seg_rows, seg_stride;
   __host__ __device__ __forceinline__ size_t row(int m) const {
-    m += m0;
     return seg_rows > 0 ? (size_t)(m / seg_rows) * seg_stride + m % seg_rows : (size_t)m;
   }
 };
 __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, RowSegments seg,
                                                               const float *__restrict__ w, float eps, int rows_all, int K,
-                                                              int n_cols, uint4 *__restrict__ blocks_all, int n_groups,
+                                                              ActTiles T, uint4 *__restrict__ blocks, int n_groups,
                                                               float *__restrict__ zero, size_t zero_n) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -274,11 +460,7 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
     if (i0 < zero_n - head - n4 * 4) zero[head + n4 * 4 + i0] = 0.f;
     return;
   }
-  const int sweep_rows = n_cols / 2, groups_per_sweep = sweep_rows / NAB_ROWS;
-  const int sweep = blockIdx.x / groups_per_sweep, m_in0 = (blockIdx.x % groups_per_sweep) * NAB_ROWS;
-  const int m0 = sweep * (TG_MAX_COLS / 2) + m_in0;                 // first row of the group (sweeps are 128 rows apart)
-  const int n_kb = K / TG_KB;
-  uint4 *blocks = blocks_all + (size_t)sweep * n_kb * (n_cols * 8);
+  const int m0 = blockIdx.x * NAB_ROWS, n_kb = T.n_kb;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ float part[8], inv[NAB_ROWS];
   {
@@ -305,24 +487,14 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
   for (int u = threadIdx.x; u < total; u += blockDim.x) {
     const int r = u % NAB_ROWS, c = (u / NAB_ROWS) % 8, kb = kb_lo + u / (NAB_ROWS * 8);
     const int m = m0 + r, k = kb * TG_KB + c * 8;
-    uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
-    if (m < rows_all) {
-      const float *xr = x + seg.row(m) * ldx;
-      const float4 a = *reinterpret_cast<const float4 *>(xr + k);
-      const float4 b = *reinterpret_cast<const float4 *>(xr + k + 4);
-      const float4 wa = __ldg(reinterpret_cast<const float4 *>(w + k)), wb = __ldg(reinterpret_cast<const float4 *>(w + k + 4));
-      const float s = inv[r];
-      const float f[8] = {a.x * s * wa.x, a.y * s * wa.y, a.z * s * wa.z, a.w * s * wa.w,
-                          b.x * s * wb.x, b.y * s * wb.y, b.z * s * wb.z, b.w * s * wb.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        hi[j] = pack_bf16x2(f[2 * j], f[2 * j + 1]);
-        lo[j] = pack_bf16x2(f[2 * j] - __uint_as_float(hi[j] << 16), f[2 * j + 1] - __uint_as_float(hi[j] & 0xffff0000u));
-      }
-    }
-    uint4 *dst = blocks + ((size_t)kb * 8 + c) * n_cols + 2 * (m_in0 + r);
-    dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    dst[1] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    if (m >= rows_all) continue;
+    const float *xr = x + seg.row(m) * ldx;
+    const float4 a = *reinterpret_cast<const float4 *>(xr + k), b = *reinterpret_cast<const float4 *>(xr + k + 4);
+    const float4 wa = __ldg(reinterpret_cast<const float4 *>(w + k)), wb = __ldg(reinterpret_cast<const float4 *>(w + k + 4));
+    const float s = inv[r];
+    const float f[8] = {a.x * s * wa.x, a.y * s * wa.y, a.z * s * wa.z, a.w * s * wa.w,
+                        b.x * s * wb.x, b.y * s * wb.y, b.z * s * wb.z, b.w * s * wb.w};
+    store_hi_lo(f, blocks + T.unit(m, kb, c), T.lo_offset());
   }
 }
 
@@ -332,17 +504,13 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
 // part_o [(row * nq + head) * nsplit + slice][D], part_ml the same with (max, sum); K = nq * D.
 constexpr int MAB_MAX_SLOTS = 2048;            // (rows of a group) x heads x slices the weights of a group may take
 __global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml,
-                                                               int nsplit, int nq, int D, int rows_all, int n_cols,
-                                                               uint4 *__restrict__ blocks_all) {
+                                                               int nsplit, int nq, int D, int rows_all, ActTiles T,
+                                                               uint4 *__restrict__ blocks) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int K = nq * D, n_kb = K / TG_KB;
-  const int sweep_rows = n_cols / 2, groups_per_sweep = sweep_rows / NAB_ROWS;
-  const int sweep = blockIdx.x / groups_per_sweep, m_in0 = (blockIdx.x % groups_per_sweep) * NAB_ROWS;
-  const int m0 = sweep * (TG_MAX_COLS / 2) + m_in0;
-  uint4 *blocks = blocks_all + (size_t)sweep * n_kb * (n_cols * 8);
+  const int m0 = blockIdx.x * NAB_ROWS, n_kb = T.n_kb;
   __shared__ float wgt[MAB_MAX_SLOTS];
   // weights: one thread per (row, head)
   for (int i = threadIdx.x; i < NAB_ROWS * nq; i += blockDim.x) {
@@ -369,29 +537,20 @@ __global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__re
   for (int u = threadIdx.x; u < total; u += blockDim.x) {
     const int r = u % NAB_ROWS, c = (u / NAB_ROWS) % 8, kb = kb_lo + u / (NAB_ROWS * 8);
     const int m = m0 + r, k = kb * TG_KB + c * 8, h = k / D, d0 = k - h * D;
-    uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
-    if (m < rows_all) {
-      float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      const float *wr = wgt + (size_t)(r * nq + h) * nsplit;
-      const float *po = part_o + ((size_t)m * nq + h) * nsplit * D + d0;
-      for (int s = 0; s < nsplit; ++s) {
-        const float ws = wr[s];
-        if (ws != 0.f) {                                   // empty slices hold nothing that may be read
-          const float4 a = *reinterpret_cast<const float4 *>(po + (size_t)s * D);
-          const float4 b = *reinterpret_cast<const float4 *>(po + (size_t)s * D + 4);
-          f[0] += ws * a.x; f[1] += ws * a.y; f[2] += ws * a.z; f[3] += ws * a.w;
-          f[4] += ws * b.x; f[5] += ws * b.y; f[6] += ws * b.z; f[7] += ws * b.w;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        hi[j] = pack_bf16x2(f[2 * j], f[2 * j + 1]);
-        lo[j] = pack_bf16x2(f[2 * j] - __uint_as_float(hi[j] << 16), f[2 * j + 1] - __uint_as_float(hi[j] & 0xffff0000u));
+    if (m >= rows_all) continue;
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float *wr = wgt + (size_t)(r * nq + h) * nsplit;
+    const float *po = part_o + ((size_t)m * nq + h) * nsplit * D + d0;
+    for (int s = 0; s < nsplit; ++s) {
+      const float ws = wr[s];
+      if (ws != 0.f) {                                     // empty slices hold nothing that may be read
+        const float4 a = *reinterpret_cast<const float4 *>(po + (size_t)s * D);
+        const float4 b = *reinterpret_cast<const float4 *>(po + (size_t)s * D + 4);
+        f[0] += ws * a.x; f[1] += ws * a.y; f[2] += ws * a.z; f[3] += ws * a.w;
+        f[4] += ws * b.x; f[5] += ws * b.y; f[6] += ws * b.z; f[7] += ws * b.w;
       }
     }
-    uint4 *dst = blocks + ((size_t)kb * 8 + c) * n_cols + 2 * (m_in0 + r);
-    dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    dst[1] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    store_hi_lo(f, blocks + T.unit(m, kb, c), T.lo_offset());
   }
 }
 

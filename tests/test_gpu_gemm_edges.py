@@ -26,8 +26,10 @@ def dmtd():
     (1, 1, 1),              # a single row
     (1, 3, 6),              # 4 rows: fewer than the mma.sync kernels' limit
     (2, 7, 71),             # rows of two sequences, in one segment each
-    (1, 5, 133),            # 129 rows in the head: one more than a sweep
-    (3, 40, 400),           # several chunks of the workspace (256 rows of three sequences each)
+    (1, 6, 133),            # 128 rows in the head, 133 in the layers: both forms of a column tile
+    (1, 5, 133),            # 129 rows in the head
+    (1, 2, 257),            # two column tiles
+    (3, 40, 400),           # several chunks of the workspace, four column tiles each
 ])
 def test_scoring_pass(dmtd, B, P, n):
     w = make_weights(SHAPE, seed=0, norm_jitter=0.1)

@@ -20,6 +20,7 @@
 #include "pass_kernel.cuh"
 #include "attention_kernel.cuh"
 #include "gemm_tc05.cuh"
+#include "attention_tc05.cuh"
 
 using namespace dmtd;
 
@@ -73,7 +74,8 @@ struct dmtd_ctx {
   int B = 0;
 
   // workspace
-  int ws_rows = 0, lda = 0, ldqkv = 0, ldgu = 0, ldl = 0, CH = 0, nsplit_max = 0;
+  int ws_rows = 0, part_rows = 0;           // rows of a chunk; ... of a chunk whose attention runs over key slices
+  int lda = 0, ldqkv = 0, ldgu = 0, ldl = 0, CH = 0, nsplit_max = 0;
   float *x_lo = nullptr, *x_up = nullptr, *act = nullptr, *qkv = nullptr, *gu = nullptr,
         *logits = nullptr, *part_o = nullptr, *part_ml = nullptr;
   float2 *rope_tab = nullptr;
@@ -274,7 +276,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // out[m][n] += sum_k W[n][k] act[m][k] on the tcgen05 tensor cores: the kernel that writes the activation blocks, then
 // the GEMM.  With `norm_w` the activations are RMSNorm(act rows) * norm_w, computed while the blocks are written, and
 // the output rows are cleared first (the projections after a norm write a fresh buffer); the rows of `act` may
-// then come in segments (RowSegments).  With merge_nsplit > 0 they are the attention's key slices, merged on the way.
+// then come in segments (RowSegments).  With merge_nsplit > 0 they are the attention's key slices, merged on the way;
+// with merge_nsplit < 0 the blocks have been written already.
 dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, int lda, int M, float *out, int ldo,
                              int gate_up_I = 0, const float *norm_w = nullptr, int merge_nsplit = 0, int seg_rows = 0,
                              int seg_stride = 0) {
@@ -289,6 +292,7 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, in
     CUDA_TRY(c, launch_pdl(merge_act_blocks_kernel, dim3(n_groups, ky), dim3(256), 0, c->stream, c->part_o, c->part_ml,
                            merge_nsplit, c->s.n_q_heads, c->s.head_dim, M, P.T, c->act_blocks));
     LAUNCH_OK(c, "merge_act_blocks_kernel");
+  } else if (merge_nsplit < 0) {
   } else if (norm_w) {
     const size_t zero_n = (size_t)M * ldo;
     const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
@@ -353,11 +357,18 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
   }
   if constexpr (D == PK_D && !std::is_same<KVT, float>::value) {
     if (flash) {
-      // a chunk of many positions per sequence (the prefill): the causal kernel, rows straight into `act`
+      // a chunk of many positions per sequence (the prefill): the causal kernel on the tcgen05 tensor cores
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
-      const int QB = PK_WARPS * (PK_QR / G);
-      attn_prefill_kernel<Op><<<dim3((R + QB - 1) / QB, s.n_kv_heads, B), PK_THREADS, ATTN_PF_SMEM, c->stream>>>(
-          c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, pos0, c->act, c->lda);
+      const int QB = AP_M / G;
+      AttnPrefillParams A{};
+      A.qkv = c->qkv; A.kc = kc; A.vc = vc; A.ldq = c->ldqkv; A.max_seq = c->max_seq; A.nq = s.n_q_heads; A.nkv = s.n_kv_heads;
+      A.R = R; A.pos0 = pos0; A.out = c->act; A.ld = c->lda;
+      if (!merge) {                         // straight into the O projection's activation blocks
+        A.blocks = c->act_blocks;
+        A.T = act_tiles_for(M, s.n_q_heads * D / TG_KB);
+      }
+      A.error = &c->dstate->error; A.wait_limit = kDeviceWaitLimitTicks;
+      attn_prefill_kernel<Op><<<dim3((R + QB - 1) / QB, s.n_kv_heads, B), AP_THREADS, AP_SMEM, c->stream>>>(A);
       LAUNCH_OK(c, "attn_prefill_kernel");
       return DMTD_OK;
     }
@@ -397,7 +408,12 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
 constexpr int kFlashMinRows = 16;
 bool flash_attention_ok(const dmtd_ctx *c, int R) {
   const int G = c->s.n_q_heads / c->s.n_kv_heads;
-  return c->use_tc_attention && c->s.head_dim == PK_D && c->s.kv_dtype != DMTD_F32 && R >= kFlashMinRows && PK_QR % G == 0;
+  return c->use_tc_attention && c->s.head_dim == PK_D && c->s.kv_dtype != DMTD_F32 && R >= kFlashMinRows && AP_M % G == 0;
+}
+
+// Positions per sequence of one prefill chunk of B sequences.
+int chunk_positions(const dmtd_ctx *c, int B) {
+  return std::max(1, (flash_attention_ok(c, c->ws_rows / B) ? c->ws_rows : c->part_rows) / B);
 }
 
 dmtd_status launch_attention(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge = true,
@@ -438,7 +454,7 @@ int splits_for(const dmtd_ctx *c, int pos_end) {
 dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos0, int pos_end) {
   const dmtd_model_shape &s = c->s;
   const LayerDev &lw = c->layers[l];
-  int M = B * R, H = s.hidden, I = s.intermediate, QD = s.n_q_heads * s.head_dim;
+  int M = B * R, H = s.hidden, I = s.intermediate;
   // the tcgen05 path normalises while it writes its activation blocks
   const bool tc = lw.qkv_u.w && c->use_umma;
   if (tc) {
@@ -451,10 +467,11 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   }
   const int nsplit = splits_for(c, pos_end);
   const bool flash = flash_attention_ok(c, R);
-  const bool fuse_merge = tc && !flash && NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS;
+  // on the tcgen05 path the O projection's activation blocks come from the prefill attention itself, or from the
+  // kernel that merges the key slices
+  const bool fuse_merge = tc && (flash || NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS);
   TRY(launch_attention(c, l, B, R, pos0, nsplit, !fuse_merge, flash));
-  (void)QD;
-  if (fuse_merge) TRY(launch_gemm_tc05(c, lw.o_u, nullptr, 0, M, x, H, 0, nullptr, nsplit));
+  if (fuse_merge) TRY(launch_gemm_tc05(c, lw.o_u, nullptr, 0, M, x, H, 0, nullptr, flash ? -1 : nsplit));
   else TRY(launch_gemv(c, lw.o, lw.o_u, c->act, c->lda, M, x, H));
   if (tc) {
     TRY(launch_gemm_tc05(c, lw.gu_u, x, H, M, c->gu, c->ldgu, 0, lw.w_post));
@@ -539,8 +556,8 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpF16>, dyn, ATTN_TC_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpBf16, true>, dyn, ATTN_TC_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpF16, true>, dyn, ATTN_TC_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, ATTN_PF_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, ATTN_PF_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, __half>, dyn, 64 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __half>, dyn, 64 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, float>, dyn, 64 * 1024));
@@ -916,10 +933,10 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
     c->CH = std::max(64, ((max_seq + want - 1) / want + 63) / 64 * 64);
   }
   c->nsplit_max = (max_seq + c->CH - 1) / c->CH;
-  // Rows of the workspace = rows of one prefill chunk: up to 1024 (fewer, larger launches, and the
-  // row blocks of one sequence find its K and V in L2), less where many key slices would make
-  // the slices' partial results large; never fewer than a decode pass needs.
-  c->ws_rows = std::max(std::max(256, max_batch * std::max(tau, 8)), std::min(1024, 16384 / std::max(1, c->nsplit_max)));
+  // Rows of the workspace = rows of one prefill chunk: up to 1024.  Chunks whose attention runs over key slices take
+  // less where many slices would make the slices' partial results large; never fewer than a decode pass needs.
+  c->part_rows = std::max(std::max(256, max_batch * std::max(tau, kFlashMinRows)), std::min(1024, 16384 / std::max(1, c->nsplit_max)));
+  c->ws_rows = std::max(1024, c->part_rows);
   CTRY(dev_alloc(c, &c->x_lo, (size_t)c->ws_rows * H));
   CTRY(dev_alloc(c, &c->x_up, (size_t)max_batch * H));
   CTRY(dev_alloc(c, &c->act, (size_t)c->ws_rows * c->lda));
@@ -928,10 +945,10 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   CTRY(dev_alloc(c, &c->logits, (size_t)max_batch * c->ldl));
   CTRY(dev_alloc(c, &c->pick_val, (size_t)max_batch * ARGMAX_SLICES));
   CTRY(dev_alloc(c, &c->pick_idx, (size_t)max_batch * ARGMAX_SLICES));
-  CTRY(dev_alloc(c, &c->part_o, (size_t)c->ws_rows * s.n_q_heads * c->nsplit_max * D));
-  CTRY(dev_alloc(c, &c->part_ml, (size_t)c->ws_rows * s.n_q_heads * c->nsplit_max * 2));
+  CTRY(dev_alloc(c, &c->part_o, (size_t)c->part_rows * s.n_q_heads * c->nsplit_max * D));
+  CTRY(dev_alloc(c, &c->part_ml, (size_t)c->part_rows * s.n_q_heads * c->nsplit_max * 2));
   CTRY(dev_alloc(c, &c->rope_tab, (size_t)c->ws_rows * (D / 2)));
-  c->pend_cap = std::max(1, c->ws_rows / max_batch);
+  c->pend_cap = std::max(1, c->part_rows / max_batch);
   CTRY(dev_alloc(c, &c->h_pend, (size_t)max_batch * c->pend_cap * H));
   CTRY(dev_alloc(c, &c->h_base, (size_t)c->ws_rows * H));
   // activation blocks: hi and lo units of every row, the rows rounded up to whole column tiles
@@ -986,7 +1003,7 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
                                 cudaMemcpyDeviceToDevice, c->stream));
   // All prompt rows through all layers (Section 2.2: the prefill is pass 1 of cycle 1), in
   // causal chunks of rows that fit the workspace.
-  const int Rc_max = std::max(1, c->ws_rows / B);
+  const int Rc_max = chunk_positions(c, B);
   int last_R = 0;
   for (int p0 = 0; p0 < P; p0 += Rc_max) {
     int R = std::min(Rc_max, P - p0);
@@ -1079,8 +1096,9 @@ dmtd_status dmtd_step_layers(dmtd_ctx *c, int32_t l0, int32_t l1, float *hidden,
   if (!hidden || l0 < 0 || l1 > c->s.n_layers || l0 > l1 || B < 1 || R < 1 || pos0 < 0)
     return fail(c, DMTD_ERR_INVALID_ARG, "step_layers: bad layer range, sizes or null hidden");
   CHECK_NOT_FAILED(c);
-  if (B > c->max_batch || R > c->max_seq || pos0 > c->max_seq - R || (long long)B * R > c->ws_rows)
-    return fail(c, DMTD_ERR_CAPACITY, "step_layers: B=%d R=%d pos0=%d exceed max_batch=%d max_seq=%d rows=%d", B, R, pos0, c->max_batch, c->max_seq, c->ws_rows);
+  if (B > c->max_batch || R > c->max_seq || pos0 > c->max_seq - R || (long long)B * R > (flash_attention_ok(c, R) ? c->ws_rows : c->part_rows))
+    return fail(c, DMTD_ERR_CAPACITY, "step_layers: B=%d R=%d pos0=%d exceed max_batch=%d max_seq=%d rows=%d", B, R, pos0, c->max_batch, c->max_seq,
+                flash_attention_ok(c, R) ? c->ws_rows : c->part_rows);
   set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->scratch, pos0);
   LAUNCH_OK(c, "set_int_kernel");
   TRY(launch_rope_table(c, &c->dstate->scratch, R));
@@ -1100,7 +1118,7 @@ dmtd_status dmtd_masked_forward(dmtd_ctx *c, const int32_t *tokens, int32_t B, i
                                 cudaMemcpyDeviceToDevice, c->stream));
   // Eq. 1-5 chunk by chunk: a chunk of rows goes through every layer before the next one starts
   // (each layer is causal and the earlier chunks' K and V are in the cache by then).
-  const int Rc_max = std::max(1, c->ws_rows / B);
+  const int Rc_max = chunk_positions(c, B);
   const size_t n_out = (size_t)(n - (P - 1));
   for (int p0 = 0; p0 < n; p0 += Rc_max) {
     const int R = std::min(Rc_max, n - p0);
@@ -1187,7 +1205,7 @@ dmtd_status dmtd_set_tau(dmtd_ctx *c, int32_t tau) {
   if (!c) return DMTD_ERR_INVALID_ARG;
   if (tau < 1) return fail(c, DMTD_ERR_SHAPE, "set_tau: tau must be >= 1");
   if (c->prefilled && c->h.slot != 0) return fail(c, DMTD_ERR_STATE, "set_tau: only at a cycle boundary");
-  if (c->max_batch * tau > c->ws_rows) return fail(c, DMTD_ERR_CAPACITY, "set_tau: workspace too small for tau=%d", tau);
+  if (c->max_batch * tau > c->part_rows) return fail(c, DMTD_ERR_CAPACITY, "set_tau: workspace too small for tau=%d", tau);
   c->tau = tau; c->h.tau = tau;
   CUDA_TRY(c, cudaMemcpyAsync(&c->dstate->tau, &c->tau, sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));

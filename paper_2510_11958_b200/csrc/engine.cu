@@ -339,6 +339,17 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   return launch_gemv_nt<4>(c, W, act, lda, M, out, ldo);
 }
 
+// Does the attention of R new rows per sequence run on attn_decode_kernel?
+bool tc_decode_attention(const dmtd_ctx *c) { return c->use_tc_attention && c->s.head_dim == PK_D && c->s.kv_dtype != DMTD_F32; }
+
+// Its blocks and slots: as many slots as the partial results' buffer holds (and, up to four rows at a time, the merge
+// inside the O projection's activation-block kernel).
+AttnDecodePlan tc_attention_plan(const dmtd_ctx *c, int B, int R, int max_slots) {
+  const dmtd_model_shape &s = c->s;
+  const int RB = std::max(1, ATTN_QR / (s.n_q_heads / s.n_kv_heads)), n_rb = (R + RB - 1) / RB;
+  return attn_decode_plan(c->n_sms, B * s.n_kv_heads * n_rb, (c->max_seq + AD_UNIT - 1) / AD_UNIT, max_slots);
+}
+
 template <int D, typename KVT>
 dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge, bool flash) {
   const dmtd_model_shape &s = c->s;
@@ -348,7 +359,7 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
   const LayerDev &lw = c->layers[layer];
   // a3 inside the attention kernel (16-bit cache, head_dim 128, decode-sized chunks): one launch less per layer
   const bool fused_a3 = D == PK_D && !std::is_same<KVT, float>::value && c->use_tc_attention && c->fuse_qk_rope && !flash &&
-                        R <= ATTN_TC_MAX_NEW;
+                        R <= AD_MAX_NEW;
   if (!fused_a3) {
     qk_norm_rope_append_kernel<D, KVT><<<dim3(M, (heads + 3) / 4), 128, 0, c->stream>>>(
         c->qkv, c->ldqkv, s.n_q_heads, s.n_kv_heads, R, lw.w_qn, lw.w_kn, s.rms_eps, c->rope_tab, pos0, kc, vc,
@@ -381,13 +392,14 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
           c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, c->part_o, c->part_ml, nsplit);
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
+      const int n_blocks = tc_attention_plan(c, B, R, nsplit).n_blocks;
       if (fused_a3)
-        attn_tc_kernel<Op, true><<<dim3(nsplit, s.n_kv_heads * n_rb, B), PK_THREADS, ATTN_TC_SMEM, c->stream>>>(
-            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, c->part_o, c->part_ml, nsplit,
+        attn_decode_kernel<Op, true><<<n_blocks, AD_THREADS, AD_SMEM, c->stream>>>(
+            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, c->part_o, c->part_ml, nsplit,
             AttnFuse{lw.w_qn, lw.w_kn, c->rope_tab, s.rms_eps});
       else
-        attn_tc_kernel<Op><<<dim3(nsplit, s.n_kv_heads * n_rb, B), PK_THREADS, ATTN_TC_SMEM, c->stream>>>(
-            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, c->part_o, c->part_ml, nsplit);
+        attn_decode_kernel<Op><<<n_blocks, AD_THREADS, AD_SMEM, c->stream>>>(
+            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, c->part_o, c->part_ml, nsplit);
     }
   } else {
   size_t smem = (size_t)ATTN_WARPS * ATTN_QR * D * sizeof(float);
@@ -442,11 +454,19 @@ dmtd_status launch_embed(dmtd_ctx *c, const int *pos0, int B, int R, float *x, b
   return DMTD_OK;
 }
 
-// Number of key slices to launch: all of them while capturing a graph (the graph must stay
+// Number of key slices of fixed length to launch: all of them while capturing a graph (the graph must stay
 // valid as the context grows), else just enough for keys [0, pos_end).
 int splits_for(const dmtd_ctx *c, int pos_end) {
   if (c->capturing) return c->nsplit_max;
   return std::max(1, std::min(c->nsplit_max, (pos_end + c->CH - 1) / c->CH));
+}
+
+// Key slices (slots of partial results per row and head) of a launch of B x R rows that ends at position pos_end.
+int slices_for(const dmtd_ctx *c, int B, int R, int pos_end) {
+  if (!tc_decode_attention(c)) return splits_for(c, pos_end);
+  const long long room = (long long)c->part_rows * c->nsplit_max / ((long long)B * R);
+  const int fused_merge = MAB_MAX_SLOTS / (NAB_ROWS * c->s.n_q_heads);
+  return tc_attention_plan(c, B, R, (int)std::max(1ll, std::min<long long>(room, std::max(1, fused_merge)))).nsplit;
 }
 
 // One decoder layer (steps a2-a7) on x [B*R][hidden]; rows of sequence b sit at positions
@@ -465,8 +485,8 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, lw.qkv, lw.qkv_u, c->act, c->lda, M, c->qkv, c->ldqkv));
   }
-  const int nsplit = splits_for(c, pos_end);
   const bool flash = flash_attention_ok(c, R);
+  const int nsplit = flash ? 1 : slices_for(c, B, R, pos_end);
   // on the tcgen05 path the O projection's activation blocks come from the prefill attention itself, or from the
   // kernel that merges the key slices
   const bool fuse_merge = tc && (flash || NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS);
@@ -552,10 +572,10 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<4>, dyn, 100 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_kernel, dyn, TG_MAX_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpBf16>, dyn, ATTN_TC_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpF16>, dyn, ATTN_TC_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpBf16, true>, dyn, ATTN_TC_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_tc_kernel<OpF16, true>, dyn, ATTN_TC_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16>, dyn, AD_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16>, dyn, AD_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16, true>, dyn, AD_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, __half>, dyn, 64 * 1024));
@@ -1329,6 +1349,7 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
   float *part_ml = reinterpret_cast<float *>(scratch + p.ml_off);
   float *part_o = reinterpret_cast<float *>(scratch + p.o_off);
   const int G = nq / nkv, RB = std::max(1, ATTN_QR / G), n_rb = (R + RB - 1) / RB, ld = nq * D;
+  int nsplit = p.nsplit;                    // slots per (row, head)
   set_int_kernel<<<1, 1, 0, stream>>>(pos_dev, pos0);
   cudaError_t e;
   if (D == PK_D) {
@@ -1340,10 +1361,15 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
           part_ml, p.nsplit);
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
-      e = cudaFuncSetAttribute(attn_tc_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, ATTN_TC_SMEM);
+      e = cudaFuncSetAttribute(attn_decode_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
-      attn_tc_kernel<Op><<<dim3(p.nsplit, nkv * n_rb, B), PK_THREADS, ATTN_TC_SMEM, stream>>>(
-          q, ld, k, v, max_seq, nq, nkv, R, RB, p.CH, pos_dev, part_o, part_ml, p.nsplit);
+      int dev = 0, n_sms = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fail(nullptr, DMTD_ERR_CUDA, "attention: device query failed");
+      const AttnDecodePlan dp = attn_decode_plan(n_sms, B * nkv * n_rb, (pos0 + R + AD_UNIT - 1) / AD_UNIT, p.nsplit);
+      nsplit = dp.nsplit;
+      attn_decode_kernel<Op><<<dp.n_blocks, AD_THREADS, AD_SMEM, stream>>>(q, ld, k, v, max_seq, nq, nkv, B, R, RB, pos_dev, part_o,
+                                                                          part_ml, nsplit);
     }
   } else {
     size_t smem = (size_t)ATTN_WARPS * ATTN_QR * D * sizeof(float);
@@ -1354,7 +1380,7 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
         part_ml, p.nsplit);
   }
   int n_rh = B * R * nq;
-  attn_merge_kernel<D><<<(n_rh + 3) / 4, 128, 0, stream>>>(part_o, part_ml, p.nsplit, n_rh, nq, out, ld);
+  attn_merge_kernel<D><<<(n_rh + 3) / 4, 128, 0, stream>>>(part_o, part_ml, nsplit, n_rh, nq, out, ld);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
   return DMTD_OK;

@@ -1,0 +1,47 @@
+"""Split-KV attention of a few new rows per sequence (dmtd_attention_decode) where its key shares, pieces and tiles
+end, against softmax(Q K^T / sqrt(d)) V in fp64."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dmtd():
+    import paper_2510_11958_b200 as pkg
+    pkg.load_library()
+    return pkg
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("B,R,nq,nkv,n_keys", [
+    (1, 1, 8, 2, 1),            # one key
+    (1, 1, 8, 2, 16),           # one warp's tile
+    (1, 3, 8, 2, 65),           # one key in the second unit, 12 query rows
+    (1, 1, 32, 8, 1000),        # fewer units than blocks
+    (2, 4, 8, 2, 129),          # 16 query rows
+    (3, 5, 8, 2, 200),          # two row blocks
+    (1, 1, 16, 1, 4097),        # one item, many pieces
+    (5, 2, 32, 8, 777),         # shares that cross item boundaries
+    (40, 1, 32, 8, 333),        # more items than blocks
+    (37, 3, 8, 8, 70),          # one query head per kv head
+    (150, 1, 8, 2, 515),
+])
+def test_attention_decode_pieces(dmtd, dtype, B, R, nq, nkv, n_keys):
+    D, G, pos0 = 128, nq // nkv, n_keys - R
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q = torch.randn(B, R, nq, D, generator=g, device="cuda") * 2
+    k, v = (torch.randn(B, nkv, n_keys + 3, D, generator=g, device="cuda").to(dtype) for _ in range(2))
+    k[:, :, n_keys:] = float("nan")                          # nothing behind the last key may be used
+    v[:, :, n_keys:] = float("nan")
+    out = dmtd.attention_decode(q, k, v, pos0)
+    kd, vd = (x[:, :, :n_keys].double().repeat_interleave(G, 1) for x in (k, v))
+    s = torch.einsum("brhd,bhkd->bhrk", q.double(), kd) / D ** 0.5
+    hidden = torch.arange(n_keys, device="cuda")[None] > (pos0 + torch.arange(R, device="cuda"))[:, None]
+    p = torch.softmax(s.masked_fill(hidden, float("-inf")), -1)
+    ref = torch.einsum("bhrk,bhkd->brhd", p, vd)
+    # the query is rounded once (relative 2^-9 or 2^-12, which moves a score of size |s| by as much) and the
+    # probabilities once; |s| stays below 12 here
+    u = 2.0 ** -9 if dtype == torch.bfloat16 else 2.0 ** -12
+    err = (out.double() - ref).abs().max().item()
+    assert err <= 4 * u * max(1.0, ref.abs().max().item()), err

@@ -293,8 +293,8 @@ def attention_decode(q, k, v, pos0, scratch=None):
     assert k.is_cuda and v.is_cuda and k.is_contiguous() and v.is_contiguous() and k.dtype == v.dtype
     B, R, nq, D = q.shape
     _, nkv, max_seq, _ = k.shape
-    need = dll.dmtd_attention_scratch_bytes(B, R, nq, D, pos0 + R)
     if scratch is None:
+        need = dll.dmtd_attention_scratch_bytes(B, R, nq, D, pos0 + R)
         scratch = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
     out = torch.empty_like(q)
     rc = dll.dmtd_attention_decode(_ptr(q), _ptr(k), _ptr(v), _kv_code(k), B, R, nq, nkv, D, max_seq, pos0,

@@ -4,6 +4,7 @@
 // results of the key slices are merged by attn_merge_kernel or by the O projection's activation-block kernel.
 #pragma once
 
+#include "kernels.cuh"
 #include "pass_attention_f32.cuh"
 
 namespace dmtd {
@@ -270,17 +271,26 @@ struct AttnShares {
 template <class Op, bool FUSED = false>
 __global__ void __launch_bounds__(AD_THREADS, 2)
 attn_decode_kernel(const float *__restrict__ qkv, int ldq, const void *__restrict__ kc, const void *__restrict__ vc, int max_seq,
-                   int nq, int nkv, int B, int R, int RB, const int *__restrict__ pos0_ptr, float *__restrict__ part_o,
+                   int nq, int nkv, int B, int R, int RB, const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
                    float *__restrict__ part_ml, int nsplit, AttnFuse F = AttnFuse{nullptr, nullptr, nullptr, 0.f}) {
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int G = nq / nkv, n_rb = (R + RB - 1) / RB;
-  const int pos0 = *pos0_ptr;
+  // The next kernel may become resident (see pdl_enter).  With the fused step a3 the keys in front of the new rows come from
+  // earlier passes: the first tiles are requested before the projection in front is waited for.  The position is older
+  // than the last plainly launched kernel (the rotary table's).
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!FUSED) asm volatile("griddepcontrol.wait;" ::: "memory");
+  bool waited = !FUSED;
+  const int pos0 = pos0_ptr ? *pos0_ptr : pos0_val;
   AttnShares sh;
   sh.per_item = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
   sh.total = (long long)B * nkv * n_rb * sh.per_item;
   sh.n_blocks = (int)min((long long)gridDim.x, sh.total);             // no empty shares: pieces of an item are consecutive blocks
-  if ((int)blockIdx.x >= sh.n_blocks) return;
+  if ((int)blockIdx.x >= sh.n_blocks) {
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");    // this grid's end stands for the end of those before it
+    return;
+  }
   const int u_end = sh.begin(blockIdx.x + 1);
   const uint32_t ring = smem_u32(sc + AD_RING) + warp * AD_STAGES * AD_SLOT, q_t = smem_u32(sc + AD_Q);
   float *const o_s = reinterpret_cast<float *>(sc + AD_OS), *const red_m = reinterpret_cast<float *>(sc + AD_RED);
@@ -319,6 +329,10 @@ attn_decode_kernel(const float *__restrict__ qkv, int ldq, const void *__restric
     };
 #pragma unroll
     for (int s = 0; s < AD_STAGES; ++s) fetch(t0 + s, s);
+    if (!waited) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      waited = true;
+    }
 
     // query rows (beyond nQ zero): row qi = (position r0 + qi / G, head kvh*G + qi % G), scaled by 1/sqrt(d)
     for (int qi = warp; qi < PK_QR; qi += AD_WARPS) {
@@ -475,14 +489,15 @@ constexpr int ATTN_F32_SMEM = StepF32Map::NEW;           // K and V tile, Q, par
 
 __global__ void __launch_bounds__(PK_THREADS, 2)
 attn_f32_kernel(const float *__restrict__ qkv, int ldq, const float *__restrict__ kc, const float *__restrict__ vc, int max_seq,
-                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, float *__restrict__ part_o,
+                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
                 float *__restrict__ part_ml, int nsplit) {
+  pdl_enter();
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = nq / nkv, n_rb = (R + RB - 1) / RB;
   const int split = blockIdx.x, kvh = blockIdx.y / n_rb, rb = blockIdx.y % n_rb, b = blockIdx.z;
   const int r0 = rb * RB, r1 = min(R, r0 + RB), nQ = (r1 - r0) * G;
-  const int pos0 = *pos0_ptr;
+  const int pos0 = pos0_ptr ? *pos0_ptr : pos0_val;
   const int j0 = split * CH, j1 = min(j0 + CH, pos0 + r1);      // the last row of the block sees position pos0 + r1 - 1
   if (j0 >= j1) {                                                 // empty slice: mark and leave
     for (int qi = threadIdx.x; qi < nQ; qi += PK_THREADS) {

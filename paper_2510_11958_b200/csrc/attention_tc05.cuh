@@ -23,6 +23,7 @@
 #pragma once
 
 #include "gemm_tc05.cuh"
+#include "kernels.cuh"
 #include "pass_attention.cuh"
 
 namespace dmtd {
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
   const int G = P.nq / P.nkv, QB = AP_M / G;                          // positions per block
   const int kvh = blockIdx.y, b = blockIdx.z;
   const int r0 = blockIdx.x * QB, r1 = min(P.R, r0 + QB);
+  pdl_enter();
   const int pos0 = *P.pos0;
   const int n_keys = pos0 + r1, n_tiles = (n_keys + AP_TK - 1) / AP_TK;     // the block's last position sees keys [0, pos0 + r1)
   const uint32_t smem = smem_u32(sc);

@@ -245,20 +245,6 @@ dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs,
 
 // ---------------------------------------------------------------------------- launches
 
-int gemv_smem_bytes(const PackedMat &W, int NT) {
-  int KS = W.aps * 32;
-  int row_bytes = ((KS * 2) % 128 == 64) ? KS * 2 : KS * 2 + 64;
-  return 8 * NT * row_bytes;
-}
-
-template <int NT>
-dmtd_status launch_gemv_nt(dmtd_ctx *c, const PackedMat &W, const float *act, int lda, int M, float *out, int ldo) {
-  int smem = gemv_smem_bytes(W, NT);
-  gemv_bf16_kernel<NT><<<2 * c->n_sms, GEMV_THREADS, smem, c->stream>>>(W, act, lda, M, out, ldo);
-  LAUNCH_OK(c, "gemv_bf16_kernel");
-  return DMTD_OK;
-}
-
 // Launch with programmatic stream serialisation: the kernel's blocks may become resident while the
 // kernel before it in the stream is still running; it calls griddepcontrol.wait before it touches
 // anything that kernel (or one before it) writes.
@@ -271,6 +257,21 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+int gemv_smem_bytes(const PackedMat &W, int NT) {
+  int KS = W.aps * 32;
+  int row_bytes = ((KS * 2) % 128 == 64) ? KS * 2 : KS * 2 + 64;
+  return 8 * NT * row_bytes;
+}
+
+template <int NT>
+dmtd_status launch_gemv_nt(dmtd_ctx *c, const PackedMat &W, const float *act, int lda, int M, float *out, int ldo) {
+  int smem = gemv_smem_bytes(W, NT);
+  CUDA_TRY(c, launch_pdl(gemv_bf16_kernel<NT>, dim3(2 * c->n_sms), dim3(GEMV_THREADS), (size_t)(smem), c->stream,
+                          W, act, lda, M, out, ldo));
+  LAUNCH_OK(c, "gemv_bf16_kernel");
+  return DMTD_OK;
 }
 
 // out[m][n] += sum_k W[n][k] act[m][k] on the tcgen05 tensor cores: the kernel that writes the activation blocks, then
@@ -330,13 +331,27 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   // layer's projections at 3 rows in 82 us against 58 (kernel times)
   if (U.w && c->use_umma) return launch_gemm_tc05(c, U, act, lda, M, out, ldo);
   if (W.wf) {
-    gemv_f32_kernel<<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo);
+    CUDA_TRY(c, launch_pdl(gemv_f32_kernel, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream,
+                            W, act, lda, M, out, ldo));
     LAUNCH_OK(c, "gemv_f32_kernel");
     return DMTD_OK;
   }
   if (M <= 4) return launch_gemv_nt<1>(c, W, act, lda, M, out, ldo);
   if (M <= 8) return launch_gemv_nt<2>(c, W, act, lda, M, out, ldo);
   return launch_gemv_nt<4>(c, W, act, lda, M, out, ldo);
+}
+
+// attn_partial_kernel compiled for the fewest query rows that hold n_rows.
+template <typename KVT>
+struct AttnPartialKernel {
+  void (*kernel)(const float *, int, const KVT *, const KVT *, int, int, int, int, int, int, const int *, int, float *, float *, int);
+  size_t smem;
+};
+template <int D, typename KVT>
+AttnPartialKernel<KVT> attn_partial_for(int n_rows) {
+  const int nq = n_rows <= 4 ? 4 : n_rows <= 8 ? 8 : 16;
+  return {nq == 4 ? attn_partial_kernel<D, KVT, 4> : nq == 8 ? attn_partial_kernel<D, KVT, 8> : attn_partial_kernel<D, KVT, 16>,
+          (size_t)ATTN_WARPS * nq * D * sizeof(float)};
 }
 
 // Does the attention of R new rows per sequence run on attn_decode_kernel?
@@ -361,9 +376,8 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
   const bool fused_a3 = D == PK_D && !std::is_same<KVT, float>::value && c->use_tc_attention && c->fuse_qk_rope && !flash &&
                         R <= AD_MAX_NEW;
   if (!fused_a3) {
-    qk_norm_rope_append_kernel<D, KVT><<<dim3(M, (heads + 3) / 4), 128, 0, c->stream>>>(
-        c->qkv, c->ldqkv, s.n_q_heads, s.n_kv_heads, R, lw.w_qn, lw.w_kn, s.rms_eps, c->rope_tab, pos0, kc, vc,
-        c->max_seq);
+    CUDA_TRY(c, launch_pdl(qk_norm_rope_append_kernel<D, KVT>, dim3(M, (heads + 3) / 4), dim3(128), (size_t)(0), c->stream,
+                             c->qkv, c->ldqkv, s.n_q_heads, s.n_kv_heads, R, lw.w_qn, lw.w_kn, s.rms_eps, c->rope_tab, pos0, kc, vc, c->max_seq));
     LAUNCH_OK(c, "qk_norm_rope_append_kernel");
   }
   if constexpr (D == PK_D && !std::is_same<KVT, float>::value) {
@@ -379,7 +393,8 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
         A.T = act_tiles_for(M, s.n_q_heads * D / TG_KB);
       }
       A.error = &c->dstate->error; A.wait_limit = kDeviceWaitLimitTicks;
-      attn_prefill_kernel<Op><<<dim3((R + QB - 1) / QB, s.n_kv_heads, B), AP_THREADS, AP_SMEM, c->stream>>>(A);
+      CUDA_TRY(c, launch_pdl(attn_prefill_kernel<Op>, dim3((R + QB - 1) / QB, s.n_kv_heads, B), dim3(AP_THREADS), (size_t)(AP_SMEM), c->stream,
+                              A));
       LAUNCH_OK(c, "attn_prefill_kernel");
       return DMTD_OK;
     }
@@ -388,30 +403,26 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
   if (D == PK_D && c->use_tc_attention) {
     // head_dim 128: the tensor-core kernel with a bf16 cache, the FMA kernel with an fp32 cache
     if constexpr (std::is_same<KVT, float>::value) {
-      attn_f32_kernel<<<dim3(nsplit, s.n_kv_heads * n_rb, B), PK_THREADS, ATTN_F32_SMEM, c->stream>>>(
-          c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, c->part_o, c->part_ml, nsplit);
+      CUDA_TRY(c, launch_pdl(attn_f32_kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(PK_THREADS), ATTN_F32_SMEM, c->stream,
+                             c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, 0, c->part_o,
+                             c->part_ml, nsplit));
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
       const int n_blocks = tc_attention_plan(c, B, R, nsplit).n_blocks;
-      if (fused_a3)
-        attn_decode_kernel<Op, true><<<n_blocks, AD_THREADS, AD_SMEM, c->stream>>>(
-            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, c->part_o, c->part_ml, nsplit,
-            AttnFuse{lw.w_qn, lw.w_kn, c->rope_tab, s.rms_eps});
-      else
-        attn_decode_kernel<Op><<<n_blocks, AD_THREADS, AD_SMEM, c->stream>>>(
-            c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, c->part_o, c->part_ml, nsplit);
+      CUDA_TRY(c, launch_pdl(fused_a3 ? attn_decode_kernel<Op, true> : attn_decode_kernel<Op, false>, dim3(n_blocks), dim3(AD_THREADS),
+                             AD_SMEM, c->stream, c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, 0,
+                             c->part_o, c->part_ml, nsplit, AttnFuse{lw.w_qn, lw.w_kn, c->rope_tab, s.rms_eps}));
     }
   } else {
-  size_t smem = (size_t)ATTN_WARPS * ATTN_QR * D * sizeof(float);
-  attn_partial_kernel<D, KVT><<<dim3(nsplit, s.n_kv_heads * n_rb, B), ATTN_WARPS * 32, smem, c->stream>>>(
-      c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, c->part_o, c->part_ml,
-      nsplit);
+    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT>(std::min(R, RB) * G);
+    CUDA_TRY(c, launch_pdl(ap.kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(ATTN_WARPS * 32), ap.smem, c->stream, c->qkv, c->ldqkv,
+                           kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, 0, c->part_o, c->part_ml, nsplit));
   }
   LAUNCH_OK(c, "attn_partial_kernel");
   if (!merge) return DMTD_OK;               // the O projection's activation-block kernel merges the slices
   int n_rh = M * s.n_q_heads;
-  attn_merge_kernel<D><<<(n_rh + 3) / 4, 128, 0, c->stream>>>(c->part_o, c->part_ml, nsplit, n_rh, s.n_q_heads,
-                                                             c->act, c->lda);
+  CUDA_TRY(c, launch_pdl(attn_merge_kernel<D>, dim3((n_rh + 3) / 4), dim3(128), (size_t)(0), c->stream,
+                          c->part_o, c->part_ml, nsplit, n_rh, s.n_q_heads, c->act, c->lda));
   LAUNCH_OK(c, "attn_merge_kernel");
   return DMTD_OK;
 }
@@ -480,8 +491,8 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   if (tc) {
     TRY(launch_gemm_tc05(c, lw.qkv_u, x, H, M, c->qkv, c->ldqkv, 0, lw.w_in));
   } else {
-    prep_norm_kernel<<<dim3(M, (c->ldqkv + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
-        x, H, lw.w_in, H, s.rms_eps, c->act, c->lda, c->qkv, c->ldqkv, c->ldqkv);
+    CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldqkv + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
+                             x, H, lw.w_in, H, s.rms_eps, c->act, c->lda, c->qkv, c->ldqkv, c->ldqkv));
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, lw.qkv, lw.qkv_u, c->act, c->lda, M, c->qkv, c->ldqkv));
   }
@@ -496,8 +507,8 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   if (tc) {
     TRY(launch_gemm_tc05(c, lw.gu_u, x, H, M, c->gu, c->ldgu, 0, lw.w_post));
   } else {
-    prep_norm_kernel<<<dim3(M, (c->ldgu + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
-        x, H, lw.w_post, H, s.rms_eps, c->act, c->lda, c->gu, c->ldgu, c->ldgu);
+    CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldgu + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
+                             x, H, lw.w_post, H, s.rms_eps, c->act, c->lda, c->gu, c->ldgu, c->ldgu));
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, lw.gu, lw.gu_u, c->act, c->lda, M, c->gu, c->ldgu));
   }
@@ -505,7 +516,8 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     // the tcgen05 path gates while it writes its activation blocks
     TRY(launch_gemm_tc05(c, lw.down_u, c->gu, c->ldgu, M, x, H, I));
   } else {
-    prep_swiglu_kernel<<<dim3((I + 255) / 256, M), 256, 0, c->stream>>>(c->gu, c->ldgu, I, c->act, c->lda);
+    CUDA_TRY(c, launch_pdl(prep_swiglu_kernel, dim3((I + 255) / 256, M), dim3(256), (size_t)(0), c->stream,
+                            c->gu, c->ldgu, I, c->act, c->lda));
     LAUNCH_OK(c, "prep_swiglu_kernel");
     TRY(launch_gemv(c, lw.down, lw.down_u, c->act, c->lda, M, x, H));
   }
@@ -526,20 +538,19 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
   if (c->embed_u.w && c->use_umma) {
     TRY(launch_gemm_tc05(c, c->embed_u, c->x_up, s.hidden, B, c->logits, c->ldl, 0, c->w_final));
   } else {
-    prep_norm_kernel<<<dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
-        c->x_up, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act, c->lda,
-                                               c->logits, c->ldl, c->ldl);
+    CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
+                             c->x_up, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act, c->lda, c->logits, c->ldl, c->ldl));
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, B, c->logits, c->ldl));
   }
   if (out_logits)
     CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (size_t)s.vocab * 4, c->logits, (size_t)c->ldl * 4, (size_t)s.vocab * 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
-  argmax_slices_kernel<<<dim3(B, ARGMAX_SLICES), 256, 0, c->stream>>>(c->logits, c->ldl, s.vocab, c->pick_val, c->pick_idx,
-                                                                      c->dstate, sample_params(c));
+  CUDA_TRY(c, launch_pdl(argmax_slices_kernel, dim3(B, ARGMAX_SLICES), dim3(256), (size_t)(0), c->stream,
+                          c->logits, c->ldl, s.vocab, c->pick_val, c->pick_idx, c->dstate, sample_params(c)));
   LAUNCH_OK(c, "argmax_slices_kernel");
-  argmax_pick_kernel<<<B, 32, 0, c->stream>>>(c->pick_val, c->pick_idx, ARGMAX_SLICES, c->tokens, c->max_seq, c->dstate,
-                                              write_token ? 1 : 0, out_argmax);
+  CUDA_TRY(c, launch_pdl(argmax_pick_kernel, dim3(B), dim3(32), (size_t)(0), c->stream,
+                          c->pick_val, c->pick_idx, ARGMAX_SLICES, c->tokens, c->max_seq, c->dstate, write_token ? 1 : 0, out_argmax));
   LAUNCH_OK(c, "argmax_pick_kernel");
   return DMTD_OK;
 }
@@ -554,9 +565,8 @@ dmtd_status run_head_rows(dmtd_ctx *c, const float *x, int n_seg, int seg_rows, 
   if (c->embed_u.w && c->use_umma)
     return launch_gemm_tc05(c, c->embed_u, x, s.hidden, M, out, s.vocab, 0, c->w_final, 0, seg_rows, seg_stride);
   for (int i = 0; i < n_seg; ++i) {
-    prep_norm_kernel<<<dim3(seg_rows, (s.vocab + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), 256, 0, c->stream>>>(
-        x + (size_t)i * seg_stride * s.hidden, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda,
-        c->lda, out + (size_t)i * seg_rows * s.vocab, s.vocab, s.vocab);
+    CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(seg_rows, (s.vocab + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
+                             x + (size_t)i * seg_stride * s.hidden, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda, c->lda, out + (size_t)i * seg_rows * s.vocab, s.vocab, s.vocab));
     LAUNCH_OK(c, "prep_norm_kernel");
   }
   return launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, M, out, s.vocab);
@@ -578,12 +588,10 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, __half>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __half>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, float>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<64, __nv_bfloat16>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, float>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __nv_bfloat16>, dyn, 64 * 1024));
+  // 16 query rows of 128 dimensions: a little over 48 KiB with the kernel's static arrays
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, float, 16>, dyn, 64 * 1024));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __nv_bfloat16, 16>, dyn, 64 * 1024));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __half, 16>, dyn, 64 * 1024));
   return DMTD_OK;
 }
 
@@ -713,12 +721,14 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
       TRY(launch_rope_table(c, &c->dstate->lo_len, R_lower));
       for (int l = Le; l < lo; ++l) TRY(run_layer(c, l, c->x_lo, B, R_lower, &c->dstate->lo_len, c->h.n_known));
       if (c->literal_sum) {
-        select_last_kernel<<<B, 256, 0, c->stream>>>(c->x_lo, R_lower, H, c->h_base);
+        CUDA_TRY(c, launch_pdl(select_last_kernel, dim3(B), dim3(256), (size_t)(0), c->stream,
+                                c->x_lo, R_lower, H, c->h_base));
         LAUNCH_OK(c, "select_last_kernel");
         copy_rows_kernel<<<64, 256, 0, c->stream>>>(c->h_base, c->x_up, (size_t)B * H / 4, 1);
         LAUNCH_OK(c, "copy_rows_kernel");
       } else {
-        select_last_kernel<<<B, 256, 0, c->stream>>>(c->x_lo, R_lower, H, c->x_up);
+        CUDA_TRY(c, launch_pdl(select_last_kernel, dim3(B), dim3(256), (size_t)(0), c->stream,
+                                c->x_lo, R_lower, H, c->x_up));
         LAUNCH_OK(c, "select_last_kernel");
       }
     } else if (kind == 2) {
@@ -729,7 +739,8 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
     TRY(launch_embed(c, &c->dstate->lo_len, B, R_lower, c->x_lo, false));
     TRY(launch_rope_table(c, &c->dstate->lo_len, R_lower));
     for (int l = 0; l < lo; ++l) TRY(run_layer(c, l, c->x_lo, B, R_lower, &c->dstate->lo_len, c->h.n_known));
-    select_last_kernel<<<B, 256, 0, c->stream>>>(c->x_lo, R_lower, H, c->x_up);
+    CUDA_TRY(c, launch_pdl(select_last_kernel, dim3(B), dim3(256), (size_t)(0), c->stream,
+                            c->x_lo, R_lower, H, c->x_up));
     LAUNCH_OK(c, "select_last_kernel");
     if (c->literal_sum) TRY(launch_embed(c, &c->dstate->newest, B, 1, c->x_up, true));
   } else {
@@ -738,7 +749,8 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
   TRY(launch_rope_table(c, &c->dstate->newest, 1));
   for (int l = lo; l < L; ++l) TRY(run_layer(c, l, c->x_up, B, 1, &c->dstate->newest, newest + 1));
   TRY(run_head(c, B, write_token, out_argmax, out_logits));
-  advance_state_kernel<<<1, 1, 0, c->stream>>>(c->dstate, kind, 0);
+  CUDA_TRY(c, launch_pdl(advance_state_kernel, dim3(1), dim3(1), (size_t)(0), c->stream,
+                          c->dstate, kind, 0));
   LAUNCH_OK(c, "advance_state_kernel");
   return DMTD_OK;
 }
@@ -1049,7 +1061,8 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
     }
     last_R = R;
   }
-  select_last_kernel<<<B, 256, 0, c->stream>>>(c->x_lo, last_R, c->s.hidden, c->x_up);
+  CUDA_TRY(c, launch_pdl(select_last_kernel, dim3(B), dim3(256), (size_t)(0), c->stream,
+                          c->x_lo, last_R, c->s.hidden, c->x_up));
   LAUNCH_OK(c, "select_last_kernel");
   // n_known must read P when the head writes the token
   set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->n_known, P);
@@ -1058,7 +1071,8 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
   if (forced_first)
     CUDA_TRY(c, cudaMemcpy2DAsync(c->tokens + P, (size_t)c->max_seq * 4, forced_first, 4, 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
-  advance_state_kernel<<<1, 1, 0, c->stream>>>(c->dstate, 0, P);
+  CUDA_TRY(c, launch_pdl(advance_state_kernel, dim3(1), dim3(1), (size_t)(0), c->stream,
+                          c->dstate, 0, P));
   LAUNCH_OK(c, "advance_state_kernel");
   c->h.n_known = P + 1; c->h.lo_len = P; c->h.up_len = P; c->h.cycle = 1;
   c->h.slot = 1 % c->tau; c->h.n_emitted = 1;
@@ -1314,8 +1328,7 @@ namespace {
 
 struct AttnPlan { int CH, nsplit; size_t ml_off, o_off, bytes; };
 
-// Scratch layout: [0, 256) the first position as a device int, then the running (max, sum)
-// pairs, then the unnormalised partial outputs, one set per (row, head, key slice).
+// Scratch layout: [0, 256) unused, then the running (max, sum) pairs, then the unnormalised partial outputs, one set per (row, head, key slice).
 AttnPlan attn_plan(int B, int R, int nq, int D, int n_keys) {
   AttnPlan p{};
   // slices enough to fill a GPU of about 150 SMs four times over (the call does not know the
@@ -1345,19 +1358,17 @@ dmtd_status attention_check(const float *q, const void *k, const void *v, int kv
 template <int D, typename KVT>
 dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int B, int R, int nq, int nkv, int max_seq,
                                int pos0, unsigned char *scratch, const AttnPlan &p, float *out, cudaStream_t stream) {
-  int *pos_dev = reinterpret_cast<int *>(scratch);
   float *part_ml = reinterpret_cast<float *>(scratch + p.ml_off);
   float *part_o = reinterpret_cast<float *>(scratch + p.o_off);
   const int G = nq / nkv, RB = std::max(1, ATTN_QR / G), n_rb = (R + RB - 1) / RB, ld = nq * D;
   int nsplit = p.nsplit;                    // slots per (row, head)
-  set_int_kernel<<<1, 1, 0, stream>>>(pos_dev, pos0);
   cudaError_t e;
   if (D == PK_D) {
     if constexpr (std::is_same<KVT, float>::value) {
       e = cudaFuncSetAttribute(attn_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATTN_F32_SMEM);
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
       attn_f32_kernel<<<dim3(p.nsplit, nkv * n_rb, B), PK_THREADS, ATTN_F32_SMEM, stream>>>(
-          q, ld, static_cast<const float *>(k), static_cast<const float *>(v), max_seq, nq, nkv, R, RB, p.CH, pos_dev, part_o,
+          q, ld, static_cast<const float *>(k), static_cast<const float *>(v), max_seq, nq, nkv, R, RB, p.CH, nullptr, pos0, part_o,
           part_ml, p.nsplit);
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
@@ -1368,20 +1379,21 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
         return fail(nullptr, DMTD_ERR_CUDA, "attention: device query failed");
       const AttnDecodePlan dp = attn_decode_plan(n_sms, B * nkv * n_rb, (pos0 + R + AD_UNIT - 1) / AD_UNIT, p.nsplit);
       nsplit = dp.nsplit;
-      attn_decode_kernel<Op><<<dp.n_blocks, AD_THREADS, AD_SMEM, stream>>>(q, ld, k, v, max_seq, nq, nkv, B, R, RB, pos_dev, part_o,
-                                                                          part_ml, nsplit);
+      e = launch_pdl(attn_decode_kernel<Op, false>, dim3(dp.n_blocks), dim3(AD_THREADS), AD_SMEM, stream, q, ld, k, v, max_seq, nq, nkv, B,
+                     R, RB, nullptr, pos0, part_o, part_ml, nsplit, AttnFuse{});
+      if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
     }
   } else {
-    size_t smem = (size_t)ATTN_WARPS * ATTN_QR * D * sizeof(float);
-    e = cudaFuncSetAttribute(attn_partial_kernel<D, KVT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT>(std::min(R, RB) * G);
+    e = cudaFuncSetAttribute(ap.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ap.smem);
     if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
-    attn_partial_kernel<D, KVT><<<dim3(p.nsplit, nkv * n_rb, B), ATTN_WARPS * 32, smem, stream>>>(
-        q, ld, static_cast<const KVT *>(k), static_cast<const KVT *>(v), max_seq, nq, nkv, R, RB, p.CH, pos_dev, part_o,
+    ap.kernel<<<dim3(p.nsplit, nkv * n_rb, B), ATTN_WARPS * 32, ap.smem, stream>>>(
+        q, ld, static_cast<const KVT *>(k), static_cast<const KVT *>(v), max_seq, nq, nkv, R, RB, p.CH, nullptr, pos0, part_o,
         part_ml, p.nsplit);
   }
   int n_rh = B * R * nq;
-  attn_merge_kernel<D><<<(n_rh + 3) / 4, 128, 0, stream>>>(part_o, part_ml, nsplit, n_rh, nq, out, ld);
-  e = cudaGetLastError();
+  e = launch_pdl(attn_merge_kernel<D>, dim3((n_rh + 3) / 4), dim3(128), 0, stream, part_o, part_ml, nsplit, n_rh, nq, out, ld);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
   return DMTD_OK;
 }

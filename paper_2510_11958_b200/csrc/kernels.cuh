@@ -8,6 +8,15 @@
 
 namespace dmtd {
 
+// First statement of a kernel that is launched with programmatic stream serialisation: the kernel after it may become
+// resident now (it does the same, or touches nothing but weights and the cache rows of earlier passes before it waits);
+// nothing is read or written here before the kernels in front are complete.  Kernels without it are launched
+// plainly: they start when everything before them is complete.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int GEMV_THREADS = 256;
 constexpr int GEMV_WARPS = GEMV_THREADS / 32;
 
@@ -88,6 +97,7 @@ constexpr int PREP_ZERO_COLS = 4096;
 __global__ void prep_norm_kernel(const float *__restrict__ x, int ldx, const float *__restrict__ w,
                                  int K, float eps, float *__restrict__ act, int lda,
                                  float *__restrict__ zero_buf, int zero_ld, int zero_cols) {
+  pdl_enter();
   const int m = blockIdx.x;
   if (zero_buf) {
     const int c0 = blockIdx.y * PREP_ZERO_COLS, c1 = min(zero_cols, c0 + PREP_ZERO_COLS);
@@ -119,6 +129,7 @@ __global__ void prep_norm_kernel(const float *__restrict__ x, int ldx, const flo
 // act[m][i] = silu(g) * u with g = gu[m][i], u = gu[m][I + i]  (the SwiGLU gate).
 __global__ void prep_swiglu_kernel(const float *__restrict__ gu, int ldgu, int I,
                                    float *__restrict__ act, int lda) {
+  pdl_enter();
   int m = blockIdx.y;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= I) return;
@@ -141,6 +152,7 @@ template <int NT>
 __global__ void __launch_bounds__(GEMV_THREADS)
 gemv_bf16_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
                  float *__restrict__ out, int ldo) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int KS = W.aps * 32;
   const int row_bytes = ((KS * 2) % 128 == 64) ? KS * 2 : KS * 2 + 64;   // conflict-free LDS.128
@@ -226,6 +238,7 @@ gemv_bf16_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
 // Projection, fp32 weights (small verification models only): one warp per output row.
 __global__ void gemv_f32_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
                                 float *__restrict__ out, int ldo) {
+  pdl_enter();
   int lane = threadIdx.x & 31;
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
   for (int n = warp; n < W.N; n += n_warps) {
@@ -282,6 +295,7 @@ __global__ void qk_norm_rope_append_kernel(float *__restrict__ qkv, int ldq, int
                                            float eps, const float2 *__restrict__ table,
                                            const int *__restrict__ pos0, KVT *__restrict__ kc,
                                            KVT *__restrict__ vc, int max_seq) {
+  pdl_enter();
   constexpr int E = D / 32;                 // values per lane; value j pairs with j + E/2
   int lane = threadIdx.x & 31;
   int head = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -359,25 +373,29 @@ template <> __device__ __forceinline__ void load8<__half>(const __half *p, float
     f[2 * j + 1] = x.y;
   }
 }
-template <int D, typename KVT>
+// NQ: query rows the block is compiled for, 4, 8 or 16 (the scores, the probabilities and the outputs of all NQ rows are
+// worked out); the loads of eight keys are in flight at a time.  36 keys of one head, 2 query rows: 27 us with 16 rows
+// and one load at a time.
+template <int D, typename KVT, int NQ>
 __global__ void __launch_bounds__(ATTN_WARPS * 32)
 attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restrict__ kc,
                     const KVT *__restrict__ vc, int max_seq, int nq, int nkv, int R, int RB, int CH,
-                    const int *__restrict__ pos0_ptr, float *__restrict__ part_o,
+                    const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
                     float *__restrict__ part_ml, int nsplit) {
+  pdl_enter();
   constexpr int E = D / 32;
   const int G = nq / nkv;
   const int split = blockIdx.x, n_rb = (R + RB - 1) / RB;
   const int kvh = blockIdx.y / n_rb, rb = blockIdx.y % n_rb, b = blockIdx.z;
   const int r0 = rb * RB, r1 = min(R, r0 + RB), nQ = (r1 - r0) * G;
-  const int pos0 = *pos0_ptr;
+  const int pos0 = pos0_ptr ? *pos0_ptr : pos0_val;
   const int j0 = split * CH, j1 = min(j0 + CH, pos0 + r1);      // keys [j0, j1); last row sees pos0+r1-1
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  __shared__ float q_s[ATTN_QR][D];
-  __shared__ float p_s[ATTN_WARPS][ATTN_QR][32];
-  __shared__ float red_m[ATTN_WARPS][ATTN_QR], red_l[ATTN_WARPS][ATTN_QR];
-  extern __shared__ __align__(16) float o_s[];                   // [ATTN_WARPS][ATTN_QR][D]
+  __shared__ float q_s[NQ][D];
+  __shared__ float p_s[ATTN_WARPS][NQ][32];
+  __shared__ float red_m[ATTN_WARPS][NQ], red_l[ATTN_WARPS][NQ];
+  extern __shared__ __align__(16) float o_s[];                   // [ATTN_WARPS][NQ][D]
 
   if (j0 >= j1) {                                                 // empty slice: mark and leave
     for (int qi = threadIdx.x; qi < nQ; qi += blockDim.x) {
@@ -389,7 +407,7 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     return;
   }
   const float scale = rsqrtf((float)D);
-  for (int idx = threadIdx.x; idx < ATTN_QR * D; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < NQ * D; idx += blockDim.x) {
     int qi = idx / D, dd = idx % D;
     float v = 0.f;
     if (qi < nQ) {
@@ -402,9 +420,9 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
 
   const KVT *kbase = kc + ((size_t)b * nkv + kvh) * max_seq * D;
   const KVT *vbase = vc + ((size_t)b * nkv + kvh) * max_seq * D;
-  float m_run[ATTN_QR], l_run[ATTN_QR], o_acc[ATTN_QR][E];
+  float m_run[NQ], l_run[NQ], o_acc[NQ][E];
 #pragma unroll
-  for (int qi = 0; qi < ATTN_QR; ++qi) {
+  for (int qi = 0; qi < NQ; ++qi) {
     m_run[qi] = -INFINITY; l_run[qi] = 0.f;
 #pragma unroll
     for (int e = 0; e < E; ++e) o_acc[qi][e] = 0.f;
@@ -412,16 +430,17 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
 
   for (int jb = j0 + warp * 32; jb < j1; jb += ATTN_WARPS * 32) {
     const int j = jb + lane;
-    float s[ATTN_QR];
+    float s[NQ];
 #pragma unroll
-    for (int qi = 0; qi < ATTN_QR; ++qi) s[qi] = 0.f;
+    for (int qi = 0; qi < NQ; ++qi) s[qi] = 0.f;
     if (j < j1) {
       const KVT *kr = kbase + (size_t)j * D;
+#pragma unroll 4
       for (int c = 0; c < D / 8; ++c) {
         float kf[8];
         load8<KVT>(kr + c * 8, kf);
 #pragma unroll
-        for (int qi = 0; qi < ATTN_QR; ++qi) {
+        for (int qi = 0; qi < NQ; ++qi) {
           const float4 qa = *reinterpret_cast<const float4 *>(&q_s[qi][c * 8]);
           const float4 qb = *reinterpret_cast<const float4 *>(&q_s[qi][c * 8 + 4]);
           s[qi] += kf[0] * qa.x + kf[1] * qa.y + kf[2] * qa.z + kf[3] * qa.w + kf[4] * qb.x +
@@ -430,7 +449,7 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
       }
     }
 #pragma unroll
-    for (int qi = 0; qi < ATTN_QR; ++qi) {
+    for (int qi = 0; qi < NQ; ++qi) {
       if (qi < nQ) {                                  // uniform across the warp
         const int pos = pos0 + r0 + qi / G;
         const bool ok = (j < j1) && (j <= pos);
@@ -450,17 +469,23 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     }
     __syncwarp();
     const int n_here = min(32, j1 - jb);
-    for (int jj = 0; jj < n_here; ++jj) {
-      const KVT *vr = vbase + (size_t)(jb + jj) * D + lane * E;
-      float vf[E];
+    for (int j8 = 0; j8 < n_here; j8 += 8) {
+      float vf[8][E];
 #pragma unroll
-      for (int e = 0; e < E; ++e) vf[e] = (float)vr[e];
+      for (int jj = 0; jj < 8; ++jj) {                  // past the last key: its row again, with probability 0
+        const KVT *vr = vbase + (size_t)(jb + min(j8 + jj, n_here - 1)) * D + lane * E;
 #pragma unroll
-      for (int qi = 0; qi < ATTN_QR; ++qi) {
+        for (int e = 0; e < E; ++e) vf[jj][e] = (float)vr[e];
+      }
+#pragma unroll
+      for (int qi = 0; qi < NQ; ++qi) {
         if (qi < nQ) {
-          const float p = p_s[warp][qi][jj];
 #pragma unroll
-          for (int e = 0; e < E; ++e) o_acc[qi][e] += p * vf[e];
+          for (int jj = 0; jj < 8; ++jj) {
+            const float p = p_s[warp][qi][j8 + jj];
+#pragma unroll
+            for (int e = 0; e < E; ++e) o_acc[qi][e] += p * vf[jj][e];
+          }
         }
       }
     }
@@ -469,10 +494,10 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
 
   // combine the warps of the block
 #pragma unroll
-  for (int qi = 0; qi < ATTN_QR; ++qi) {
+  for (int qi = 0; qi < NQ; ++qi) {
     if (lane == 0) { red_m[warp][qi] = m_run[qi]; red_l[warp][qi] = l_run[qi]; }
 #pragma unroll
-    for (int e = 0; e < E; ++e) o_s[((size_t)warp * ATTN_QR + qi) * D + lane * E + e] = o_acc[qi][e];
+    for (int e = 0; e < E; ++e) o_s[((size_t)warp * NQ + qi) * D + lane * E + e] = o_acc[qi][e];
   }
   __syncthreads();
   for (int idx = threadIdx.x; idx < nQ * D; idx += blockDim.x) {
@@ -485,7 +510,7 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     for (int w = 0; w < ATTN_WARPS; ++w) {
       float f = red_m[w][qi] > -INFINITY ? __expf(red_m[w][qi] - m) : 0.f;
       l += red_l[w][qi] * f;
-      o += o_s[((size_t)w * ATTN_QR + qi) * D + dd] * f;
+      o += o_s[((size_t)w * NQ + qi) * D + dd] * f;
     }
     int r = r0 + qi / G, h = kvh * G + qi % G;
     size_t slot = ((size_t)(b * R + r) * nq + h) * nsplit + split;
@@ -498,6 +523,7 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
 template <int D>
 __global__ void attn_merge_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml,
                                   int nsplit, int n_rows_heads, int nq, float *__restrict__ act, int lda) {
+  pdl_enter();
   constexpr int E = D / 32;
   int lane = threadIdx.x & 31;
   int idx = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -530,6 +556,7 @@ __global__ void attn_merge_kernel(const float *__restrict__ part_o, const float 
 // on into the decoding layers (Section 2.2); the refill rows' outputs are dropped.
 // ------------------------------------------------------------------------------------
 __global__ void select_last_kernel(const float *__restrict__ x_lo, int R, int H, float *__restrict__ x_up) {
+  pdl_enter();
   int b = blockIdx.x;
   const float *src = x_lo + ((size_t)b * R + (R - 1)) * H;
   for (int k = threadIdx.x; k < H; k += blockDim.x) x_up[(size_t)b * H + k] = src[k];
@@ -592,7 +619,7 @@ __global__ void masked_select_kernel(float *__restrict__ x, const float *__restr
 // n_known of the token buffer unless a forced token already sits there (teacher forcing), and
 // to out_argmax if given.
 // ------------------------------------------------------------------------------------
-constexpr int ARGMAX_SLICES = 16;
+constexpr int ARGMAX_SLICES = 64;       // 151 936 logits of one sequence: 16 slices 10 us, 64 slices 3
 
 __device__ __forceinline__ void argmax_block_reduce(float best, int bi, float *sv, int *si) {
   sv[threadIdx.x] = best; si[threadIdx.x] = bi;
@@ -611,6 +638,7 @@ __device__ __forceinline__ void argmax_block_reduce(float best, int bi, float *s
 // grid (sequences, ARGMAX_SLICES), 256 threads
 __global__ void argmax_slices_kernel(const float *__restrict__ logits, int ldl, int V, float *__restrict__ part_val,
                                      int *__restrict__ part_idx, const DevState *__restrict__ st, SampleParams sp) {
+  pdl_enter();
   const int b = blockIdx.x, per = (V + gridDim.y - 1) / gridDim.y;
   const int i0 = blockIdx.y * per, i1 = min(V, i0 + per);
   const float *z = logits + (size_t)b * ldl;
@@ -655,6 +683,7 @@ __global__ void argmax_slices_kernel(const float *__restrict__ logits, int ldl, 
 __global__ void argmax_pick_kernel(const float *__restrict__ part_val, const int *__restrict__ part_idx, int n_slices,
                                    int *__restrict__ tokens, int max_seq, const DevState *__restrict__ st, int write_token,
                                    int *__restrict__ out_argmax) {
+  pdl_enter();
   const int b = blockIdx.x;
   float best = -INFINITY;
   int bi = 0x7fffffff;
@@ -676,6 +705,7 @@ __global__ void argmax_pick_kernel(const float *__restrict__ part_val, const int
 // a0: schedule counters after a pass (Section 2.2).  kind: 0 = prefill of P rows, 1 = full
 // pass, 2 = decoding-layers-only pass.
 __global__ void advance_state_kernel(DevState *st, int kind, int P) {
+  pdl_enter();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   if (kind == 0) {
     st->n_known = P + 1; st->lo_len = P; st->up_len = P; st->cycle = 1;

@@ -315,6 +315,7 @@ __global__ void __launch_bounds__(PK_THREADS, 1) dmtd_pass_kernel(const __grid_c
     float *x = lower ? P.x_lo : P.x_up;
     const int nsplit = lower ? nsplit_lo : nsplit_up, CH = lower ? CH_lo : CH_up;      // key slices of the attention stage
     const PassLayer &Ly = S.layers[head ? 0 : li];
+    const int pf_chunks = attn_prefetch_chunks((int)gridDim.x - P.B * P.nkv * nsplit);           // asked for during the attention stage
     const PackedMat *W = nullptr;
     float *out = nullptr;
     int ldo = 0;
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(PK_THREADS, 1) dmtd_pass_kernel(const __grid_c
       else attention_stage<OpBf16>(P, Ly, R, pos0, nsplit, CH);
       if (PK_ATTN_PF_ATOMS > 0) {
         const int items = P.B * P.nkv * nsplit;
-        if ((int)blockIdx.x >= items) prefetch_matrix_part(Ly.gu, (int)blockIdx.x - items, (int)gridDim.x - items);
+        if ((int)blockIdx.x >= items && pf_chunks > 0) prefetch_matrix_part(Ly.gu, (int)blockIdx.x - items, (int)gridDim.x - items);
       }
     } else if (ph == 2) {
       // a4 merge of the key slices + a5: O projection into the residual rows
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(PK_THREADS, 1) dmtd_pass_kernel(const __grid_c
     // the prologue's own loads are done: ask L2 for the next atoms of the warp's stream (HBM is idle until the
     // projection has drained the ring)
     if (PK_PRO_PF_ATOMS > 0 && lane == 0 && ph != 1 && ph != 2)
-      prefetch_own_stream(S.pipes[warp].cur, (!head && ph == 3) ? PK_ATTN_PF_ATOMS : 0);
+      prefetch_own_stream(S.pipes[warp].cur, (!head && ph == 3) ? pf_chunks * PK_CHUNK_ATOMS : 0);
     PK_STAMP();
 #ifdef DMTD_PASS_TIMING
     const int chunk_log = (!head && li == nL - 1 && ph != 1) ? 2048 + 64 * (ph - (ph > 1)) : -1;

@@ -69,13 +69,26 @@ __device__ __forceinline__ void stream_ranges(const PackedMat &W, int warp, int 
 #endif
 constexpr int PK_ATTN_PF_ATOMS = DMTD_PASS_ATTN_PF;
 constexpr int PK_ATTN_PF_SKIP = PK_SLOTS * PK_CHUNK_ATOMS;
-__device__ __forceinline__ void prefetch_matrix_part(const PackedMat &W, int idle_rank, int n_idle) {
+// Requests an idle block can work off while the others are in the attention stage: with 4 idle blocks (3 sequences:
+// 144 items) the whole 32 KiB per warp were 1184 requests a block, and every layer waited 30 us for them.  So the part
+// that is asked for is whole chunks per warp, as many as the idle blocks have time for.  Requests per idle block
+// 100 / 136 / 200: 25.5 / 25.35 / 25.8 ms for 8 cycles of one sequence (context 520 - 2500), 26.05 without the limit;
+// three sequences 24.0 ms for 6 cycles at each, 26.8 without.
+#ifndef DMTD_PASS_PF_PER_BLOCK
+#define DMTD_PASS_PF_PER_BLOCK 136
+#endif
+constexpr int PK_ATTN_PF_PER_BLOCK = DMTD_PASS_PF_PER_BLOCK;
+__device__ __forceinline__ int attn_prefetch_chunks(int n_idle) {
   constexpr int REQ = (PK_ATTN_PF_ATOMS + PK_CHUNK_ATOMS - 1) / PK_CHUNK_ATOMS;      // requests per warp
+  return max(0, min(REQ, n_idle * PK_ATTN_PF_PER_BLOCK / ((int)gridDim.x * PK_WARPS)));
+}
+__device__ __forceinline__ void prefetch_matrix_part(const PackedMat &W, int idle_rank, int n_idle) {
+  const int chunks = attn_prefetch_chunks(n_idle);
   const unsigned A = (unsigned)(W.n_slabs * W.n_tiles * W.aps);
-  const int total = (int)gridDim.x * PK_WARPS * REQ;
+  const int total = (int)gridDim.x * PK_WARPS * chunks;
 #pragma unroll 1
   for (int j = (int)threadIdx.x * n_idle + idle_rank; j < total; j += n_idle * PK_THREADS) {     // spread evenly over the idle blocks
-    const int k = j % REQ, wg = j / REQ, warp = wg % PK_WARPS, blk = wg / PK_WARPS;
+    const int k = j % chunks, wg = j / chunks, warp = wg % PK_WARPS, blk = wg / PK_WARPS;
     const int c0 = (int)(A * (unsigned)blk / gridDim.x), c1 = (int)(A * (unsigned)(blk + 1) / gridDim.x);
     const int w0 = c0 + (c1 - c0) * warp / PK_WARPS, w1 = c0 + (c1 - c0) * (warp + 1) / PK_WARPS;
     const int start = w0 + PK_ATTN_PF_SKIP + k * PK_CHUNK_ATOMS;

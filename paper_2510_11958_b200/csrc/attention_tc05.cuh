@@ -15,11 +15,12 @@
 // conflicts), K of the next tile under the softmax of this one, V under the next S.  One tile of each and half of the
 // tensor memory (S 128 columns, P over them, O 128): two blocks per SM, one's products under the other's softmax.
 //
-// Bound: the tensor pipe and the softmax's exponentials together (S + P V take 1350 cycles of the pipe per tile,
-// 128 x 128 exponentials 1024 cycles of the special-function units).  The kernel before this one ran the same tiles on
-// mma.sync, each warp re-reading K and V from shared memory for 16 rows.
+// Bound: the chain of one tile, 4030 cycles (S 770, softmax 1870, hand-over 550, P V 850) with two blocks per SM beside
+// each other, i.e. 2015 per tile and SM against 1350 of the tensor pipe.  1024 positions behind 8000 keys: 209 us
+// (680 TFLOP/s); one sequence of 512 tokens (32 query and 8 kv heads): 18 us per layer, 69 us with the kernel
+// before this one, which ran the same tiles on mma.sync, each warp re-reading K and V from shared memory for 16 rows.
 //
-// Warps 0-3 load Q, run the softmax and store; warp 4 issues the MMAs; warps 5 and 6 copy K and V.  All waits bounded.
+// Warps 0-3 load Q, run the softmax and store; warp 4 issues the MMAs; warp 5 copies K and V.  All waits bounded.
 #pragma once
 
 #include "gemm_tc05.cuh"
@@ -30,7 +31,7 @@ namespace dmtd {
 
 constexpr int AP_M = 128;                        // query rows per block
 constexpr int AP_TK = 128;                       // keys per tile
-constexpr int AP_LOADERS = 64;                   // copying threads
+constexpr int AP_LOADERS = 32;                   // copying threads (six warps a block: 168 registers a thread, seven would leave 128)
 constexpr int AP_THREADS = AP_M + 32 + AP_LOADERS;
 constexpr int AP_HALF = 128 * 128;               // bytes of one half (64 of the 128 dimensions) of 128 rows
 constexpr int AP_Q = 0, AP_K = 2 * AP_HALF, AP_V = 4 * AP_HALF, AP_BARS = 6 * AP_HALF;
@@ -103,11 +104,29 @@ __device__ __forceinline__ float exp2_approx(float x) {
   return y;
 }
 
+// two floats at a time (a scheduler has one softmax warp of each block: issue slots count)
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 template <class Op>
 __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __grid_constant__ AttnPrefillParams P) {
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = P.nq / P.nkv, QB = AP_M / G;                          // positions per block
+  const int G = P.nq / P.nkv, lgG = 31 - __clz(G), QB = AP_M >> lgG;  // G is a power of two (it divides 128); positions per block
   const int kvh = blockIdx.y, b = blockIdx.z;
   const int r0 = blockIdx.x * QB, r1 = min(P.R, r0 + QB);
   pdl_enter();
@@ -117,8 +136,9 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
   // tile i completes phase i of every barrier
   const uint32_t bar_k = smem + AP_BARS, bar_v = bar_k + 8;           // K / V tile in shared memory
   const uint32_t bar_s = bar_k + 16, bar_p = bar_k + 24, bar_o = bar_k + 32;   // S computed; P stored; P V computed
-  uint32_t *const tmem_slot = reinterpret_cast<uint32_t *>(sc + AP_BARS + 40);
-  volatile int *const gave_up = reinterpret_cast<volatile int *>(sc + AP_BARS + 44);
+  const uint32_t bar_q = bar_k + 40;                                  // Q in shared memory (once)
+  uint32_t *const tmem_slot = reinterpret_cast<uint32_t *>(sc + AP_BARS + 48);
+  volatile int *const gave_up = reinterpret_cast<volatile int *>(sc + AP_BARS + 52);
 
   if (threadIdx.x == 0) {
     mbar_init(bar_k, AP_LOADERS);
@@ -126,25 +146,13 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     mbar_init(bar_s, 1);
     mbar_init(bar_p, AP_M);
     mbar_init(bar_o, 1);
+    mbar_init(bar_q, AP_M);
     *gave_up = 0;
     fence_mbar_init();
   }
   if (warp == 4) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(AP_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  if (warp < 4) {
-    // Q tile: row i = (position r0 + i / G, head kvh * G + i % G), scaled by 1/sqrt(d); rows past the chunk zero
-    const float scale = rsqrtf(128.f);
-#pragma unroll 4
-    for (int j = 0; j < 32; ++j) {
-      const int row = warp * 32 + j, r = r0 + row / G;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (r < P.R) v = reinterpret_cast<const float4 *>(P.qkv + (size_t)(b * P.R + r) * P.ldq + (size_t)(kvh * G + row % G) * 128)[lane];
-      *reinterpret_cast<uint2 *>(sc + AP_Q + ap_part(row, lane >> 1) + (lane & 1) * 8) =
-          make_uint2(Op::pack2(v.x * scale, v.y * scale), Op::pack2(v.z * scale, v.w * scale));
-    }
-    fence_proxy_async();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -198,8 +206,8 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     constexpr uint32_t fmt = std::is_same<typename Op::T, __half>::value ? 0u : 1u;       // A and B of one type
     const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
     const uint32_t idesc_pv = idesc | (1u << 16);                                         // B is N-major
-    bool ok = true;
-    for (int i = 0; i < n_tiles; ++i) {
+    bool ok = __all_sync(0xffffffffu, ap_wait(bar_q, 0, P));
+    for (int i = 0; i < n_tiles && ok; ++i) {
       ok = __all_sync(0xffffffffu, ap_wait(bar_k, i & 1, P));
       if (i > 0) ok = __all_sync(0xffffffffu, ok && ap_wait(bar_o, (i - 1) & 1, P));      // P lies over S
       if (!ok) break;
@@ -240,7 +248,22 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     if (!ok && lane == 0) { *gave_up = 1; __threadfence_block(); }
   } else {
     // ---- softmax: thread = query row = lane of tensor memory
-    const int row = threadIdx.x, r = r0 + row / G, my_pos = pos0 + r;
+    {
+      // Q tile: row i = (position r0 + i / G, head kvh * G + i % G), scaled by 1/sqrt(d); rows past the chunk zero
+      const float scale = rsqrtf(128.f);
+#pragma unroll 8
+      for (int j = 0; j < 32; ++j) {
+        const int qrow = warp * 32 + j, qr = r0 + (qrow >> lgG);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (qr < P.R)
+          v = reinterpret_cast<const float4 *>(P.qkv + (size_t)(b * P.R + qr) * P.ldq + (size_t)(kvh * G + (qrow & (G - 1))) * 128)[lane];
+        *reinterpret_cast<uint2 *>(sc + AP_Q + ap_part(qrow, lane >> 1) + (lane & 1) * 8) =
+            make_uint2(Op::pack2(v.x * scale, v.y * scale), Op::pack2(v.z * scale, v.w * scale));
+      }
+      fence_proxy_async();
+      mbar_arrive(bar_q);
+    }
+    const int row = threadIdx.x, r = r0 + (row >> lgG), my_pos = pos0 + r;
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     const uint32_t t_s = tmem_s + lane_off, t_o = tmem_o + lane_off;
     float m_ref = -INFINITY, l = 0.f;                                 // reference maximum (times log2 e) and running sum
@@ -252,20 +275,22 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
       // keys of the tile this row sees: [0, lim); only the block's last tiles are cut
       const int lim = min(min(my_pos + 1, n_keys) - i * AP_TK, AP_TK);
       const bool cut = (i + 1) * AP_TK > pos0 + r0 + 1;                 // the same for all rows of the block
-      float mx = -INFINITY;
+      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four chains: a dependent maximum takes four cycles
 #pragma unroll
-      for (int c0 = 0; c0 < AP_TK; c0 += 32) {
-        uint32_t s[32];
-        tmem_ld32(t_s + c0, s);
+      for (int c0 = 0; c0 < AP_TK; c0 += 64) {
+        uint32_t s[64];
+        tmem_ld32(t_s + c0, *reinterpret_cast<uint32_t(*)[32]>(s));
+        tmem_ld32(t_s + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(s + 32));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if (cut) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) mx = fmaxf(mx, c0 + j < lim ? __uint_as_float(s[j]) : -INFINITY);
+          for (int j = 0; j < 64; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], c0 + j < lim ? __uint_as_float(s[j]) : -INFINITY);
         } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) mx = fmaxf(mx, __uint_as_float(s[j]));
+          for (int j = 0; j < 64; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], __uint_as_float(s[j]));
         }
       }
+      float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
       mx *= AP_LOG2E;
       float alpha = 1.f;
       if (i == 0) {
@@ -288,38 +313,48 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
           }
         }
       }
+      const uint64_t log2e2 = f2_pack(AP_LOG2E, AP_LOG2E), neg_m2 = f2_pack(-m_ref, -m_ref);
+      uint64_t sum2[2] = {0ull, 0ull};
       // P over S: columns 16 q .. + 15 of P (keys 32 q ..) lie over columns of S that have been read by then
 #pragma unroll
-      for (int c0 = 0; c0 < AP_TK; c0 += 32) {
-        uint32_t s[32];
-        tmem_ld32(t_s + c0, s);
+      for (int c0 = 0; c0 < AP_TK; c0 += 64) {
+        uint32_t s[64];
+        tmem_ld32(t_s + c0, *reinterpret_cast<uint32_t(*)[32]>(s));
+        tmem_ld32(t_s + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(s + 32));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        uint32_t p[16];
-        float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float a = exp2_approx(fmaf(__uint_as_float(s[2 * j]), AP_LOG2E, -m_ref));
-          float c = exp2_approx(fmaf(__uint_as_float(s[2 * j + 1]), AP_LOG2E, -m_ref));
-          if (cut) {
-            a = c0 + 2 * j < lim ? a : 0.f;
-            c = c0 + 2 * j + 1 < lim ? c : 0.f;
+        for (int h = 0; h < 2; ++h) {
+          uint32_t p[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int k = 32 * h + 2 * j;
+            float a, c;
+            f2_unpack(f2_fma(f2_pack(__uint_as_float(s[k]), __uint_as_float(s[k + 1])), log2e2, neg_m2), a, c);
+            a = exp2_approx(a);
+            c = exp2_approx(c);
+            if (cut) {
+              a = c0 + k < lim ? a : 0.f;
+              c = c0 + k + 1 < lim ? c : 0.f;
+            }
+            sum2[j & 1] = f2_add(sum2[j & 1], f2_pack(a, c));
+            p[j] = Op::pack2(a, c);
           }
-          sum0 += a; sum1 += c;
-          p[j] = Op::pack2(a, c);
+          tmem_st16(t_s + c0 / 2 + 16 * h, p);
         }
-        l += sum0 + sum1;
-        tmem_st16(t_s + c0 / 2, p);
       }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(bar_p);
+      float l0, l1;
+      f2_unpack(f2_add(sum2[0], sum2[1]), l0, l1);
+      l += l0 + l1;
     }
     // ---- O / l: fp32 rows, or hi and lo units of the O projection's activations
     if (ok && n_tiles > 0) ok = __all_sync(0xffffffffu, ap_wait(bar_o, (n_tiles - 1) & 1, P)) && !*gave_up;
     if (ok) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const float inv = 1.f / l;
-      const int m = b * P.R + r, k0 = (kvh * G + row % G) * 128;
+      const int m = b * P.R + r, k0 = (kvh * G + (row & (G - 1))) * 128;
 #pragma unroll 1
       for (int c0 = 0; c0 < 128; c0 += 16) {
         uint32_t o[16];

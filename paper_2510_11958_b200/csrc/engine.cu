@@ -58,7 +58,8 @@ struct dmtd_ctx {
   UmmaMat embed_u{};
   bool umma_ok = false, use_umma = true;    // tcgen05 GEMM for the projections
   int gemm_stages = 0;                      // pipeline stages of its blocks; 0: chosen per launch
-  uint4 *act_blocks = nullptr;
+  uint4 *act_blocks = nullptr;              // activation blocks of the projection at hand
+  uint4 *gated_blocks = nullptr;            // ... of the down projection, where gate+up writes them
   float *w_final = nullptr;
   double *inv_freq = nullptr;
 
@@ -218,8 +219,9 @@ dmtd_status vec_to_float(dmtd_ctx *c, float **out, const void *src, int n) {
   return DMTD_OK;
 }
 
-// Second copy of a (fused) matrix in the block order of the tcgen05 GEMM.
-dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs, const int *Ns, int n_src) {
+// Second copy of a (fused) matrix in the block order of the tcgen05 GEMM; in_turn: the rows of the sources (of equal
+// size) one after the other instead of source after source.
+dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs, const int *Ns, int n_src, bool in_turn = false) {
   int N = 0;
   for (int i = 0; i < n_src; ++i) N += Ns[i];
   UmmaMat m{};
@@ -234,9 +236,10 @@ dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs,
   for (int i = 0; i < n_src; ++i) {
     long long total = (long long)Ns[i] * (K / 8);
     int grid = (int)std::min<long long>((total + 255) / 256, 65535);
-    pack_umma_kernel<<<grid, 256, 0, c->stream>>>(static_cast<const __nv_bfloat16 *>(srcs[i]), Ns[i], K, row0, m.n_kb, dst);
+    pack_umma_kernel<<<grid, 256, 0, c->stream>>>(static_cast<const __nv_bfloat16 *>(srcs[i]), Ns[i], K, row0, in_turn ? n_src : 1,
+                                                  m.n_kb, dst);
     LAUNCH_OK(c, "pack_umma_kernel");
-    row0 += Ns[i];
+    row0 += in_turn ? 1 : Ns[i];
   }
   m.w = dst;
   *out = m;
@@ -274,37 +277,68 @@ dmtd_status launch_gemv_nt(dmtd_ctx *c, const PackedMat &W, const float *act, in
   return DMTD_OK;
 }
 
-// out[m][n] += sum_k W[n][k] act[m][k] on the tcgen05 tensor cores: the kernel that writes the activation blocks, then
-// the GEMM.  With `norm_w` the activations are RMSNorm(act rows) * norm_w, computed while the blocks are written, and
-// the output rows are cleared first (the projections after a norm write a fresh buffer); the rows of `act` may
-// then come in segments (RowSegments).  With merge_nsplit > 0 they are the attention's key slices, merged on the way;
-// with merge_nsplit < 0 the blocks have been written already.
-dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, int lda, int M, float *out, int ldo,
-                             int gate_up_I = 0, const float *norm_w = nullptr, int merge_nsplit = 0, int seg_rows = 0,
-                             int seg_stride = 0) {
+using GemmTcKernel = void (*)(GemmTcParams);
+GemmTcKernel gemm_tc05_for(bool split, int whole) {
+  if (split) return whole == TG_STORE ? gemm_tc05_kernel<true, TG_STORE> : gemm_tc05_kernel<true, TG_ADD>;
+  return whole == TG_STORE ? gemm_tc05_kernel<false, TG_STORE> : whole == TG_SWIGLU ? gemm_tc05_kernel<false, TG_SWIGLU>
+                                                                                   : gemm_tc05_kernel<false, TG_ADD>;
+}
+
+// Where the activation blocks of a projection on the tcgen05 tensor cores come from.
+struct GemmInput {
+  enum Kind { ROWS, NORM, SWIGLU, SLICES, READY } kind = ROWS;
+  const float *act = nullptr;               // ROWS, NORM: [rows][lda]; SWIGLU: gate and up values in turn
+  int lda = 0;
+  const float *norm_w = nullptr;            // NORM: RMSNorm(row) * norm_w
+  int seg_rows = 0, seg_stride = 0;         // NORM: the rows come in segments (RowSegments)
+  int nsplit = 0;                           // SLICES: the attention's key slices, merged on the way
+  int kb0 = 0;                              // SWIGLU: the first k block that is not written yet
+  uint4 *blocks = nullptr;                  // READY (and SWIGLU, for the rest): the blocks' own buffer
+};
+
+// out[m][n] (+)= sum_k W[n][k] act[m][k]: the kernel that writes the activation blocks, then the GEMM.  After a norm the
+// outputs are new: what the GEMM adds into is cleared beside the norm, the rest is stored (`whole`).  With `gated` the
+// matrix is gate+up and the gate's result goes to the down projection's activation blocks there; `out` takes the
+// values of the weight rows behind the tiles dealt out whole, [M][ldo] from row tg_whole_pairs * 256 on.
+dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in, int M, float *out, int ldo, uint4 *gated = nullptr) {
   GemmTcParams P{};
-  P.W = W; P.act_blocks = c->act_blocks;
+  P.W = W;
   P.rows = M;
   P.T = act_tiles_for(M, W.n_kb);
   P.out = out; P.ldo = ldo;
   P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
+  uint4 *blocks = in.blocks ? in.blocks : c->act_blocks;
+  P.act_blocks = blocks;
+  const int n_pairs = c->n_sms / 2;
+  // Tiles dealt out whole: gate+up where it gates, and matrices of many rounds of tiles (the head).  With one round (gate+up
+  // of a decode pass) the part of a tile in front of it costs an epilogue more than the clearing it saves: batch 32
+  // 23.3 ms for 4 cycles instead of 22.8, batch 3 24.3 instead of 24.0 for 6.
+  const int whole = in.kind != GemmInput::NORM ? TG_ADD : gated ? TG_SWIGLU : W.n_tiles / 2 >= 4 * n_pairs ? TG_STORE : TG_ADD;
+  P.rt_whole = tg_whole_pairs(W, whole, n_pairs);
+  P.whole_units = P.rt_whole / n_pairs * P.T.n_ctiles * W.n_kb;
+  const int n_line = (W.n_tiles / 2 - P.rt_whole) * P.T.n_ctiles * W.n_kb;
+  P.line_q = n_line / n_pairs; P.line_r = n_line % n_pairs;
+  const int n_whole = P.rt_whole * 2 * TG_ROWS;                                   // weight rows dealt out whole
+  if (gated) { P.gated = gated; P.gated_kb = W.N / 2 / TG_KB; P.out_n0 = n_whole; }
   const int n_groups = (M + NAB_ROWS - 1) / NAB_ROWS, ky = std::max(1, std::min(W.n_kb, 4 * c->n_sms / n_groups));
-  if (merge_nsplit > 0) {
+  if (in.kind == GemmInput::SLICES) {
     CUDA_TRY(c, launch_pdl(merge_act_blocks_kernel, dim3(n_groups, ky), dim3(256), 0, c->stream, c->part_o, c->part_ml,
-                           merge_nsplit, c->s.n_q_heads, c->s.head_dim, M, P.T, c->act_blocks));
+                           in.nsplit, c->s.n_q_heads, c->s.head_dim, M, P.T, blocks));
     LAUNCH_OK(c, "merge_act_blocks_kernel");
-  } else if (merge_nsplit < 0) {
-  } else if (norm_w) {
-    const size_t zero_n = (size_t)M * ldo;
+  } else if (in.kind == GemmInput::NORM) {
+    const int n_rest = std::max(0, W.N - n_whole);
+    ZeroArea zero{gated ? out : out + n_whole, M, n_rest, (size_t)ldo};
+    if (n_whole == 0) zero.cols = ldo;                                            // whole rows, padding included
+    const size_t zero_n = (size_t)zero.rows * zero.cols;
     const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
     CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
-                           act, lda, RowSegments{seg_rows, seg_stride}, norm_w, c->s.rms_eps, M, W.K, P.T,
-                           c->act_blocks, n_groups, out, zero_n));
+                           in.act, in.lda, RowSegments{in.seg_rows, in.seg_stride}, in.norm_w, c->s.rms_eps, M, W.K, P.T,
+                           blocks, n_groups, zero));
     LAUNCH_OK(c, "norm_act_blocks_kernel");
-  } else {
-    const int units = W.n_kb * 8 * M;
-    CUDA_TRY(c, launch_pdl(act_blocks_kernel, dim3(std::min((units + 255) / 256, 8 * c->n_sms)), dim3(256), 0, c->stream, act, lda,
-                           M, P.T, c->act_blocks, gate_up_I));
+  } else if (in.kind != GemmInput::READY && in.kb0 < W.n_kb) {
+    const int units = (W.n_kb - in.kb0) * 8 * M;
+    CUDA_TRY(c, launch_pdl(act_blocks_kernel, dim3(std::min((units + 255) / 256, 8 * c->n_sms)), dim3(256), 0, c->stream, in.act,
+                           in.lda, M, P.T, blocks, in.kind == GemmInput::SWIGLU ? 1 : 0, in.kb0));
     LAUNCH_OK(c, "act_blocks_kernel");
   }
   // as many stages as shared memory holds, two accumulators where tensor memory does.  (Half of both for decode launches,
@@ -317,10 +351,21 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const float *act, in
   while (cols < n_cols) cols <<= 1;
   P.n_acc = 2 * cols <= 512 ? 2 : 1;
   P.tmem_cols = P.n_acc * cols;
-  CUDA_TRY(c, launch_pdl(gemm_tc05_kernel, dim3(c->n_sms / 2 * 2), dim3(TG_THREADS), (size_t)P.stages * stage_bytes + TG_TAIL_BYTES,
+  CUDA_TRY(c, launch_pdl(gemm_tc05_for(P.T.split != 0, whole), dim3(2 * n_pairs), dim3(TG_THREADS), (size_t)P.stages * stage_bytes + TG_TAIL_BYTES,
                          c->stream, P));
   LAUNCH_OK(c, "gemm_tc05_kernel");
   return DMTD_OK;
+}
+
+GemmInput rows_input(const float *act, int lda) {
+  GemmInput in;
+  in.act = act; in.lda = lda;
+  return in;
+}
+GemmInput norm_input(const float *x, int ldx, const float *w) {
+  GemmInput in = rows_input(x, ldx);
+  in.kind = GemmInput::NORM; in.norm_w = w;
+  return in;
 }
 
 // out[m][n] += sum_k W[n][k] act[m][k]
@@ -329,7 +374,7 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   // the tcgen05 GEMM at every row count: the mma.sync kernel, whose warps load their weights through registers,
   // streams the tied head of the Qwen3-4B shape (778 MB, 1 - 4 rows) at 3.6 TB/s, the tcgen05 kernel at 5.9, and a
   // layer's projections at 3 rows in 82 us against 58 (kernel times)
-  if (U.w && c->use_umma) return launch_gemm_tc05(c, U, act, lda, M, out, ldo);
+  if (U.w && c->use_umma) return launch_gemm_tc05(c, U, rows_input(act, lda), M, out, ldo);
   if (W.wf) {
     CUDA_TRY(c, launch_pdl(gemv_f32_kernel, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream,
                             W, act, lda, M, out, ldo));
@@ -489,7 +534,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   // the tcgen05 path normalises while it writes its activation blocks
   const bool tc = lw.qkv_u.w && c->use_umma;
   if (tc) {
-    TRY(launch_gemm_tc05(c, lw.qkv_u, x, H, M, c->qkv, c->ldqkv, 0, lw.w_in));
+    TRY(launch_gemm_tc05(c, lw.qkv_u, norm_input(x, H, lw.w_in), M, c->qkv, c->ldqkv));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldqkv + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              x, H, lw.w_in, H, s.rms_eps, c->act, c->lda, c->qkv, c->ldqkv, c->ldqkv));
@@ -502,20 +547,33 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   // kernel that merges the key slices
   const bool fuse_merge = tc && (flash || NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS);
   TRY(launch_attention(c, l, B, R, pos0, nsplit, !fuse_merge, flash));
-  if (fuse_merge) TRY(launch_gemm_tc05(c, lw.o_u, nullptr, 0, M, x, H, 0, nullptr, flash ? -1 : nsplit));
+  if (fuse_merge) {
+    GemmInput in;
+    in.kind = flash ? GemmInput::READY : GemmInput::SLICES;
+    in.nsplit = nsplit;
+    TRY(launch_gemm_tc05(c, lw.o_u, in, M, x, H));
+  }
   else TRY(launch_gemv(c, lw.o, lw.o_u, c->act, c->lda, M, x, H));
   if (tc) {
-    TRY(launch_gemm_tc05(c, lw.gu_u, x, H, M, c->gu, c->ldgu, 0, lw.w_post));
+    // more rows than a decode pass has: the GEMM gates its outputs and writes the down projection's activation blocks
+    // itself, but for the few row tiles it has to share between blocks (their values go through `gu`)
+    GemmInput down;
+    down.kind = GemmInput::SWIGLU;
+    down.act = c->gu;
+    if (M > TG_SPLIT_ROWS) {
+      const int n_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, c->n_sms / 2) * 2 * TG_ROWS, n_rest = std::max(0, 2 * I - n_whole);
+      down.lda = std::max(4, n_rest); down.kb0 = n_whole / 2 / TG_KB; down.blocks = c->gated_blocks;
+      TRY(launch_gemm_tc05(c, lw.gu_u, norm_input(x, H, lw.w_post), M, c->gu, down.lda, c->gated_blocks));
+    } else {
+      down.lda = c->ldgu;
+      TRY(launch_gemm_tc05(c, lw.gu_u, norm_input(x, H, lw.w_post), M, c->gu, c->ldgu));
+    }
+    TRY(launch_gemm_tc05(c, lw.down_u, down, M, x, H));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldgu + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              x, H, lw.w_post, H, s.rms_eps, c->act, c->lda, c->gu, c->ldgu, c->ldgu));
     LAUNCH_OK(c, "prep_norm_kernel");
     TRY(launch_gemv(c, lw.gu, lw.gu_u, c->act, c->lda, M, c->gu, c->ldgu));
-  }
-  if (tc) {
-    // the tcgen05 path gates while it writes its activation blocks
-    TRY(launch_gemm_tc05(c, lw.down_u, c->gu, c->ldgu, M, x, H, I));
-  } else {
     CUDA_TRY(c, launch_pdl(prep_swiglu_kernel, dim3((I + 255) / 256, M), dim3(256), (size_t)(0), c->stream,
                             c->gu, c->ldgu, I, c->act, c->lda));
     LAUNCH_OK(c, "prep_swiglu_kernel");
@@ -536,7 +594,7 @@ SampleParams sample_params(const dmtd_ctx *c) {
 dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits) {
   const dmtd_model_shape &s = c->s;
   if (c->embed_u.w && c->use_umma) {
-    TRY(launch_gemm_tc05(c, c->embed_u, c->x_up, s.hidden, B, c->logits, c->ldl, 0, c->w_final));
+    TRY(launch_gemm_tc05(c, c->embed_u, norm_input(c->x_up, s.hidden, c->w_final), B, c->logits, c->ldl));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              c->x_up, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act, c->lda, c->logits, c->ldl, c->ldl));
@@ -562,8 +620,11 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
 dmtd_status run_head_rows(dmtd_ctx *c, const float *x, int n_seg, int seg_rows, int seg_stride, float *out) {
   const dmtd_model_shape &s = c->s;
   const int M = n_seg * seg_rows;
-  if (c->embed_u.w && c->use_umma)
-    return launch_gemm_tc05(c, c->embed_u, x, s.hidden, M, out, s.vocab, 0, c->w_final, 0, seg_rows, seg_stride);
+  if (c->embed_u.w && c->use_umma) {
+    GemmInput in = norm_input(x, s.hidden, c->w_final);
+    in.seg_rows = seg_rows; in.seg_stride = seg_stride;
+    return launch_gemm_tc05(c, c->embed_u, in, M, out, s.vocab);
+  }
   for (int i = 0; i < n_seg; ++i) {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(seg_rows, (s.vocab + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              x + (size_t)i * seg_stride * s.hidden, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda, c->lda, out + (size_t)i * seg_rows * s.vocab, s.vocab, s.vocab));
@@ -580,7 +641,8 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<1>, dyn, 100 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<2>, dyn, 100 * 1024));
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<4>, dyn, 100 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_kernel, dyn, TG_MAX_SMEM));
+  for (int whole : {TG_ADD, TG_STORE, TG_SWIGLU})
+    for (bool split : {false, true}) CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_for(split, whole), dyn, TG_MAX_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16>, dyn, AD_SMEM));
@@ -917,7 +979,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
     if (c->umma_ok) {
       CTRY(pack_umma(c, &ld.qkv_u, H, qkv_src, qkv_n, 3));
       CTRY(pack_umma(c, &ld.o_u, QD, o_src, o_n, 1));
-      CTRY(pack_umma(c, &ld.gu_u, H, gu_src, gu_n, 2));
+      CTRY(pack_umma(c, &ld.gu_u, H, gu_src, gu_n, 2, true));        // gate and up of one index side by side: the epilogue gates
       CTRY(pack_umma(c, &ld.down_u, I, d_src, d_n, 1));
     }
     CTRY(vec_to_float(c, &ld.w_in, lw.input_norm, H));
@@ -987,6 +1049,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   if (c->umma_ok) {
     const size_t rows = (size_t)c->ws_rows + 16 * (c->ws_rows / TG_TILE_ROWS + 1);
     CTRY(dev_alloc(c, &c->act_blocks, rows * (c->lda / 8) * 2));
+    CTRY(dev_alloc(c, &c->gated_blocks, rows * (I / 8) * 2));
   }
   CTRY(configure_kernels(c));
   CTRY(setup_fused(c));

@@ -18,15 +18,20 @@
 // core matrix.  The weights are stored in global memory in exactly that order (16 KiB blocks, one per 128-row tile and
 // k block), the activations are written that way by the kernels below, so a pipeline stage is two bulk copies.
 //
-// Persistent: one pair of blocks per two SMs.  The work of a launch (row-tile pairs x column tiles x k blocks) is one
-// line of units, cut into equal shares whatever the shape is; a share that ends inside a tile adds its partial sums,
-// so every output is added with fp32 reductions (measured at 3.9 TB/s into L2; plain stores 4.8).  The accumulators
-// of a tile are read back while the next tile is multiplied where tensor memory holds two.
+// Persistent: one pair of blocks per two SMs.  The units of a launch (row-tile pairs x column tiles x k blocks) are cut
+// into equal shares whatever the shape is: the row-tile pairs that are not a multiple of the block pairs (all of them,
+// where there are fewer) form one line of units cut into equal parts, and a part that ends inside a tile adds its
+// partial sums with fp32 reductions (measured at 3.9 TB/s into L2; plain stores 4.8).  The other row-tile pairs are
+// dealt out whole: their outputs can be stored (nothing to clear, nothing to add), or, for gate+up, gated and written
+// as the down projection's activation blocks by the epilogue.  The accumulators of a tile are read back while the next
+// tile is multiplied where tensor memory holds two.
 //
 // Measured (Qwen3-4B shapes, launches back to back, against the kernel before this one: 128-row sweeps, one MMA-issuing
 // block per tile, hi and lo columns always apart): gate+up at 512 rows 139 -> 75 us (1350 TFLOP/s counting both
 // parts, at the clock the power cap leaves), QKV 50 -> 29 us; head at 512 rows 541 us (1470 TFLOP/s); decode is bound by
 // HBM and by what a launch costs: head at 32 rows 127 us (6.1 TB/s), gate+up at 96 rows 44 -> 27 us, at 8 rows 24 us.
+// Gating in gate+up's epilogue instead of clearing, adding and reading 40 MB per 512 rows: prefill of 512 tokens
+// 8.8 -> 8.1 ms, of 32 x 1024 tokens 539 -> 469 ms.
 //
 // Warp roles: warp 0 issues the bulk copies, warp 1 issues the MMAs (first SM of the pair) or passes on to the first
 // SM that a stage has landed (second SM), warps 2-9 run the epilogue (each the 32 lanes of its quarter, every second 16 columns).  Every wait is
@@ -48,6 +53,7 @@ constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
 constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
 constexpr int TG_MAX_SMEM = 226 * 1024;      // dynamic shared memory of a block: it has its SM to itself
 enum { TG_ERR_WAIT = 4 };
+enum { TG_ADD = 0, TG_STORE = 1, TG_SWIGLU = 2 };           // tiles dealt out whole: none; stored; gated
 
 // A weight matrix [N][K] as 16 KiB blocks [row tile][k block][k chunk 8][row group 16][row 8][8 values].
 struct UmmaMat {
@@ -94,6 +100,12 @@ struct GemmTcParams {
   int rows;                  // activation rows of this launch
   float *out;                // [rows][ldo], added into
   int ldo;
+  int rt_whole;              // row-tile pairs dealt out whole, a multiple of the block pairs: the first ones
+  int whole_units;           // units of a block pair's whole tiles
+  int line_q, line_r;        // a block pair's part of the units of the others: line_q, one more for the first line_r pairs
+  int out_n0;                // first weight row of out's columns (TG_SWIGLU: out holds the remaining row-tile pairs only)
+  uint4 *gated;              // TG_SWIGLU: units of the next projection, in the tiles of T (k = half of the interleaved weight row)
+  int gated_kb;              // ... and its k blocks
   int stages;                // pipeline stages of a block, 2 .. TG_MAX_STAGES
   int n_acc, tmem_cols;      // accumulators in tensor memory (1 or 2), tmem_cols / n_acc columns apart
   int *error;
@@ -161,6 +173,69 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
 __device__ __forceinline__ void red_add(float *p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
+// Row-tile pairs dealt out whole: the largest multiple of the block pairs.
+inline int tg_whole_pairs(const UmmaMat &W, int whole, int n_pairs) {
+  return whole == TG_ADD ? 0 : W.n_tiles / 2 / n_pairs * n_pairs;
+}
+
+// The units of a block pair in order: its part of the line of units of the remaining row-tile pairs, then its whole
+// tiles; k fastest, then the column tile.
+struct TgCursor {
+  int kb, ct, rt;            // k block, column tile, row-tile pair
+  int left;                  // units left of the line; then 0
+  int step;                  // row-tile pairs from one tile row to the next
+  __device__ __forceinline__ void next(int n_kb, int n_ct, int pair, int n_pairs) {
+    if (left > 0 && --left == 0) {
+      kb = 0; ct = 0; rt = pair; step = n_pairs;
+      return;
+    }
+    if (++kb == n_kb) {
+      kb = 0;
+      if (++ct == n_ct) { ct = 0; rt += step; }
+    }
+  }
+};
+
+// TG_SWIGLU epilogue: the lane's weight row is 2 i (gate) or 2 i + 1 (up) of intermediate index i, r its values for 16
+// activation rows.  Even lanes gate the even columns, odd lanes the odd ones; the 8 x 8 transposes between the lanes of
+// eight indices then leave every lane with one 16-byte unit (8 indices of one activation row), hi and lo part.
+// On return hi / lo are the unit of column 2 * ((lane >> 1) & 7) + (lane & 1) and of the indices 8 * (lane >> 4) .. + 7 of
+// the warp's 16.
+__device__ __forceinline__ void swiglu_units(const uint32_t (&r)[16], uint4 &hi, uint4 &lo) {
+  const int lane = threadIdx.x & 31, odd = lane & 1, p = lane >> 1;
+  uint32_t w[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float send = __uint_as_float(odd ? r[2 * q] : r[2 * q + 1]);
+    const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
+    const float g = odd ? recv : __uint_as_float(r[2 * q]), u = odd ? __uint_as_float(r[2 * q + 1]) : recv;
+    const float a = g / (1.f + expf(-g)) * u;
+    const __nv_bfloat16 h = __float2bfloat16_rn(a), l = __float2bfloat16_rn(a - __bfloat162float(h));
+    w[q] = (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
+  }
+#pragma unroll
+  for (int b = 1; b < 8; b <<= 1) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (q & b) continue;
+      const bool up = (p & b) != 0;
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? w[q] : w[q | b], b << 1);
+      if (up) w[q] = got; else w[q | b] = got;
+    }
+  }
+  uint32_t h4[4], l4[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    h4[j] = __byte_perm(w[2 * j], w[2 * j + 1], 0x5410);
+    l4[j] = __byte_perm(w[2 * j], w[2 * j + 1], 0x7632);
+  }
+  hi = make_uint4(h4[0], h4[1], h4[2], h4[3]);
+  lo = make_uint4(l4[0], l4[1], l4[2], l4[3]);
+}
+
+// SPLIT: the form of the column tiles (one tile of up to 128 rows); WHOLE: what becomes of the tiles dealt out whole.  (Forms
+// of their own: the code that a decode launch does not run cost it 2 us per layer, a launch fetches its instructions anew.)
+template <bool SPLIT, int WHOLE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_tc05_kernel(const __grid_constant__ GemmTcParams P) {
   extern __shared__ __align__(1024) unsigned char tg_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -173,34 +248,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   uint32_t *const tmem_slot = reinterpret_cast<uint32_t *>(tail + 16 * TG_MAX_STAGES + 32);
   volatile int *const gave_up = reinterpret_cast<volatile int *>(tmem_slot + 1);   // a wait of this block ran out: no more output
 
-  // this pair's share of the units (row-tile pair, column tile, k block), k fastest, then the column tile
-  const long long n_units = (long long)(P.W.n_tiles / 2) * P.T.n_ctiles * n_kb;
-  const int u0 = (int)(n_units * pair / n_pairs), u1 = (int)(n_units * (pair + 1) / n_pairs);
+  // this pair's share of the units
+  const int n_ct = SPLIT ? 1 : P.T.n_ctiles;
+  const int u0 = pair * P.line_q + min(pair, P.line_r), n_part = P.line_q + (pair < P.line_r ? 1 : 0);
+  const int n_it = n_part + (WHOLE == TG_ADD ? 0 : P.whole_units);
+  TgCursor start;
+  if (n_part > 0) {
+    const int tile = u0 / n_kb, row = n_ct == 1 ? tile : tile / n_ct;
+    start = TgCursor{u0 - tile * n_kb, tile - row * n_ct, P.rt_whole + row, n_part, 1};
+  } else {
+    start = TgCursor{0, 0, pair, 0, n_pairs};
+  }
 
   // the kernel after this one (the next projection's activation-block kernel, launched the same way) may become
   // resident now; it waits for this grid's completion before it reads or writes anything, and the GEMM behind it
   // can then request its first weight blocks while this grid's last blocks finish
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // producer's position in the share (thread 0)
-  int kb_w = u0 % n_kb, ct_w = (u0 / n_kb) % P.T.n_ctiles, rt_w = u0 / n_kb / P.T.n_ctiles;
-  int kb_a = kb_w, ct_a = ct_w;
+  TgCursor cur_w = start, cur_a = start;               // producer's positions (thread 0)
   auto copy_w = [&](int st) {
-    bulk_g2s(smem_u32(tg_smem) + st * stage_bytes, P.W.w + ((size_t)(2 * rt_w + rank) * n_kb + kb_w) * (TG_WBLOCK / 16), TG_WBLOCK,
-             full0 + st * 8);
-    if (++kb_w == n_kb) {
-      kb_w = 0;
-      if (++ct_w == P.T.n_ctiles) { ct_w = 0; ++rt_w; }
-    }
+    bulk_g2s(smem_u32(tg_smem) + st * stage_bytes, P.W.w + ((size_t)(2 * cur_w.rt + rank) * n_kb + cur_w.kb) * (TG_WBLOCK / 16),
+             TG_WBLOCK, full0 + st * 8);
+    cur_w.next(n_kb, n_ct, pair, n_pairs);
   };
   auto copy_act = [&](int st) {
     bulk_g2s(smem_u32(tg_smem) + st * stage_bytes + TG_WBLOCK,
-             P.act_blocks + (((size_t)ct_a * n_kb + kb_a) * 2 + rank) * P.T.units_per_sm(), act_bytes, full0 + st * 8);
-    if (++kb_a == n_kb) {
-      kb_a = 0;
-      if (++ct_a == P.T.n_ctiles) ct_a = 0;
-    }
+             P.act_blocks + (((size_t)cur_a.ct * n_kb + cur_a.kb) * 2 + rank) * P.T.units_per_sm(), act_bytes, full0 + st * 8);
+    cur_a.next(n_kb, n_ct, pair, n_pairs);
   };
-  const int n_it = u1 - u0, n_first = min(S, n_it);
+  const int n_first = min(S, n_it);
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full0 + s * 8, rank == 0 ? 2 : 1);       // this block's copies; on the first SM also the other's
@@ -263,13 +338,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     }
   } else if (warp == 1 && rank == 0) {
     // ---- MMA issuer
-    const int n_cols = P.T.split ? 2 * tile_rows : tile_rows;         // MMA N
+    const int n_cols = SPLIT ? 2 * tile_rows : tile_rows;         // MMA N
     const uint32_t idesc = umma_instr_desc(2 * TG_ROWS, n_cols);
     const uint32_t b_lbo = (uint32_t)(n_cols / 2) * 16, part_bytes = b_lbo * 8;
-    int kb = u0 % n_kb, st = 0, acc = 0;
+    int kb = start.kb, st = 0, acc = 0;
     uint32_t ph = 0, acc_ph = 1;                                      // the accumulators start free
     bool first = true, ok = true;
-    for (int u = u0; u < u1; ++u) {
+    for (int i = 0; i < n_it; ++i) {
       if (first) {
         ok = __all_sync(0xffffffffu, tg_wait(acc_empty0 + acc * 8, acc_ph, P));
         if (!ok) break;
@@ -278,7 +353,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
       ok = __all_sync(0xffffffffu, tg_wait(full0 + st * 8, ph, P));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const bool last = ++kb == n_kb || u + 1 == u1;
+      const bool last = ++kb == n_kb || i + 1 == n_part;
       if (elect_one()) {
         const uint32_t a_base = smem_u32(tg_smem) + st * stage_bytes, b_base = a_base + TG_WBLOCK;
         const uint32_t d = tmem + acc * acc_cols;
@@ -293,7 +368,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
               "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
               : "memory");
           accumulate = 1u;
-          if (!P.T.split)                                             // the lo part into the same columns
+          if (!SPLIT)                                             // the lo part into the same columns
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                 " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
@@ -319,7 +394,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     if (lane == 0) {
       int st = 0;
       uint32_t ph = 0;
-      for (int u = u0; u < u1; ++u) {
+      for (int i = 0; i < n_it; ++i) {
         if (!tg_wait(full0 + st * 8, ph, P)) break;
         mbar_arrive_leader(full0 + st * 8);
         if (++st == S) { st = 0; ph ^= 1; }
@@ -328,24 +403,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   } else {
     // ---- epilogue: thread = weight row (lane of tensor memory), registers = columns
     const int quarter = warp & 3;
-    int u = u0, acc = 0;
+    int acc = 0, kb = start.kb, ct = start.ct, rt = start.rt, left = n_part;
     uint32_t ph = 0;
-    while (u < u1) {
-      const int tile = u / n_kb, ct = tile % P.T.n_ctiles, rt = tile / P.T.n_ctiles;
-      u = min(u1, (tile + 1) * n_kb);
+    for (int i = 0; i < n_it;) {
+      // the next tile of the share, or part of one
+      const bool whole = WHOLE != TG_ADD && left == 0;
+      const int units = whole ? n_kb : min(n_kb - kb, left), this_ct = ct, this_rt = rt;
+      i += units;
+      kb = 0;
+      if (!whole && (left -= units) == 0) { ct = 0; rt = pair; }
+      else if (++ct == n_ct) { ct = 0; rt += whole ? n_pairs : 1; }
       const bool ok = __all_sync(0xffffffffu, tg_wait(acc_full0 + acc * 8, ph, P)) && !*gave_up;
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int n = (2 * rt + rank) * TG_ROWS + quarter * 32 + lane;
-      const int m0 = ct * tile_rows, n_rows = min(tile_rows, P.rows - m0);
+      const int n = (2 * this_rt + rank) * TG_ROWS + quarter * 32 + lane;
+      const int m0 = this_ct * tile_rows, n_rows = min(tile_rows, P.rows - m0);
       const uint32_t t_base = tmem + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols;
       const int c_first = warp < 6 ? 0 : 16;
-      float *dst = P.out + (size_t)(m0 + c_first) * P.ldo + n;
+      float *dst = P.out + (size_t)(m0 + c_first) * P.ldo + (n - (WHOLE == TG_SWIGLU ? P.out_n0 : 0));
 #pragma unroll 1
       for (int c0 = c_first; c0 < n_rows; c0 += 32) {
         uint32_t r[16];
         tmem_ld16(t_base + c0, r);
-        if (P.T.split) {                                              // the lo columns
+        if (SPLIT) {                                              // the lo columns
           uint32_t q[16];
           tmem_ld16(t_base + tile_rows + c0, q);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -355,8 +435,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         }
         // straight-line code for whole groups of 16 rows: a warp has its scheduler to itself, every instruction counts
-        if (n < P.W.N) {
-          if (c0 + 16 <= n_rows) {
+        if (n >= P.W.N) {                                             // rows that pad the last tile (gate+up: whole tiles of them)
+        } else if (WHOLE == TG_SWIGLU && whole) {
+          uint4 hi, lo;
+          swiglu_units(r, hi, lo);
+          const int col = c0 + 2 * ((lane >> 1) & 7) + (lane & 1), half = tile_rows / 2, sm = col >= half ? 1 : 0;
+          if (col < n_rows) {
+            uint4 *u = P.gated + (((size_t)this_ct * P.gated_kb + 2 * this_rt + rank) * 2 + sm) * P.T.units_per_sm() +
+                       (2 * quarter + (lane >> 4)) * half + (col - sm * half);
+            u[0] = hi;
+            u[P.T.lo_offset()] = lo;
+          }
+        } else {
+          if (whole) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < n_rows) dst[(size_t)j * P.ldo] = __uint_as_float(r[j]);
+          } else if (c0 + 16 <= n_rows) {
             float *d = dst;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
@@ -390,8 +485,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
 
 // Activations [rows][lda] fp32 -> bf16 hi/lo units in the order of ActTiles.  One thread per unit: 8 values of k of a
 // row, both parts; neighbouring threads take neighbouring rows (consecutive 16-byte stores, 32-byte reads).
-// With gate_up_I > 0 the source rows hold gate | up values (gate at k, up at gate_up_I + k) and the
-// activation is the SwiGLU gate silu(gate) * up (step a6, second half), computed on the way.
+// With `gated` the source rows hold gate and up values in turn and the activation is the SwiGLU gate silu(gate) * up
+// (step a6, second half), computed on the way; the source's first column then belongs to k block kb0.
 __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, size_t lo_offset) {
   uint32_t hi[4], lo[4];
 #pragma unroll
@@ -404,26 +499,29 @@ __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, siz
 }
 
 __global__ void act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T, uint4 *__restrict__ blocks,
-                                  int gate_up_I) {
+                                  int gated, int kb0) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int total = T.n_kb * 8 * rows;
+  const int total = (T.n_kb - kb0) * 8 * rows;
   for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
-    const int m = u % rows, kc = u / rows, k = kc * 8;
-    const float *src = act + (size_t)m * lda + k;
-    const float4 a = *reinterpret_cast<const float4 *>(src), b = *reinterpret_cast<const float4 *>(src + 4);
-    float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    if (gate_up_I > 0) {
-      const float4 ua = *reinterpret_cast<const float4 *>(src + gate_up_I);
-      const float4 ub = *reinterpret_cast<const float4 *>(src + gate_up_I + 4);
-      const float up[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
+    const int m = u % rows, kc = u / rows;
+    const float4 *src = reinterpret_cast<const float4 *>(act + (size_t)m * lda + (size_t)kc * (gated ? 16 : 8));
+    float f[8];
+    if (gated) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) f[j] = f[j] / (1.f + expf(-f[j])) * up[j];
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = src[j];
+        f[2 * j] = v.x / (1.f + expf(-v.x)) * v.y;
+        f[2 * j + 1] = v.z / (1.f + expf(-v.z)) * v.w;
+      }
+    } else {
+      const float4 a = src[0], b = src[1];
+      f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
     }
-    store_hi_lo(f, blocks + T.unit(m, kc >> 3, kc & 7), T.lo_offset());
+    store_hi_lo(f, blocks + T.unit(m, kb0 + (kc >> 3), kc & 7), T.lo_offset());
   }
 }
 
@@ -434,6 +532,12 @@ __global__ void act_blocks_kernel(const float *__restrict__ act, int lda, int ro
 // The rows come in segments of seg_rows every seg_stride rows of x (the rows of a chunk that the LM head
 // reads when logits of many positions are asked for); seg_rows = 0: one segment.
 constexpr int NAB_ROWS = 4;
+// `cols` columns of `rows` rows that lie ld floats apart
+struct ZeroArea {
+  float *p;
+  int rows, cols;
+  size_t ld;
+};
 struct RowSegments {
   int seg_rows, seg_stride;
   __host__ __device__ __forceinline__ size_t row(int m) const {
@@ -443,7 +547,7 @@ struct RowSegments {
 __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, RowSegments seg,
                                                               const float *__restrict__ w, float eps, int rows_all, int K,
                                                               ActTiles T, uint4 *__restrict__ blocks, int n_groups,
-                                                              float *__restrict__ zero, size_t zero_n) {
+                                                              ZeroArea zero_area) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
@@ -451,7 +555,13 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if ((int)blockIdx.x >= n_groups) {
     const size_t n_z = (size_t)(gridDim.x - n_groups) * gridDim.y;
+    const size_t zero_n = (size_t)zero_area.rows * zero_area.cols;
+    float *zero = zero_area.p;
     const size_t i0 = ((size_t)(blockIdx.x - n_groups) * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x;
+    if (zero_area.cols < zero_area.ld) {               // columns of longer rows
+      for (size_t i = i0; i < zero_n; i += n_z * blockDim.x) zero[i / zero_area.cols * zero_area.ld + i % zero_area.cols] = 0.f;
+      return;
+    }
     const size_t head = min(zero_n, (size_t)((16 - (reinterpret_cast<uintptr_t>(zero) & 15)) & 15) / 4);   // up to the first 16-byte boundary
     float4 *z4 = reinterpret_cast<float4 *>(zero + head);
     const size_t n4 = (zero_n - head) / 4;
@@ -555,14 +665,15 @@ __global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__re
 }
 
 // Weights [N][K] bf16 row-major (rows [row0, row0 + N_src) of the fused matrix) -> 16 KiB blocks.
-__global__ void pack_umma_kernel(const __nv_bfloat16 *__restrict__ src, int N_src, int K, int row0, int n_kb,
+// Source row r becomes row row0 + r * row_step (gate and up rows in turn: step 2).
+__global__ void pack_umma_kernel(const __nv_bfloat16 *__restrict__ src, int N_src, int K, int row0, int row_step, int n_kb,
                                  uint4 *__restrict__ dst) {
   const long long total = (long long)N_src * (K / 8);              // 16-byte units of the source
   for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += (long long)gridDim.x * blockDim.x) {
-    const int kc = (int)(u % (K / 8)), row = row0 + (int)(u / (K / 8));
+    const int kc = (int)(u % (K / 8)), src_row = (int)(u / (K / 8)), row = row0 + src_row * row_step;
     const int tile = row / TG_ROWS, rg = (row % TG_ROWS) / 8, j = row % 8, kb = kc / 8, c = kc % 8;
     dst[(((size_t)tile * n_kb + kb) * 8 + c) * TG_ROWS + rg * 8 + j] =
-        *reinterpret_cast<const uint4 *>(src + (size_t)(row - row0) * K + kc * 8);
+        *reinterpret_cast<const uint4 *>(src + (size_t)src_row * K + kc * 8);
   }
 }
 

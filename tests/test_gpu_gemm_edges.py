@@ -55,3 +55,20 @@ def test_decode_rows(dmtd, B, tau):
     err, _ = check_logits(got_logits, ref_logits, got_am, ref_am)
     assert err < 1e-3
     assert eng.device_state() == o.state()
+
+
+@pytest.mark.parametrize("intermediate", [
+    9472,       # 74 pairs of row tiles of gate+up: all dealt out whole on 148 SMs
+    9536,       # one pair more, half of it padding
+    9728,       # two pairs more
+])
+@pytest.mark.parametrize("n", [90, 129, 300])
+def test_gated_epilogue(dmtd, intermediate, n):
+    """Gate+up wide enough for whole tiles: below 129 rows a pass of its own gates, above the epilogue does."""
+    shape = SHAPE.with_(n_layers=2, hidden=256, intermediate=intermediate, vocab=600)
+    w = make_weights(shape, seed=4, norm_jitter=0.1)
+    tokens = make_prompts(shape.vocab, 1, n, seed=6).numpy()
+    ref = oracle.masked_parallel_forward(shape, w, 1, 2, tokens[0], 5)
+    eng = dmtd.Dmtd(shape, to_cuda(w), L_d=1, tau=2, max_batch=1, max_seq=n + 2, kv_dtype="f32")
+    got = eng.masked_forward(torch.from_numpy(tokens).cuda(), 5).double().cpu().numpy()
+    assert np.abs(got[0] - ref).max() < 1e-3

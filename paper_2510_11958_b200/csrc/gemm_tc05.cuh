@@ -544,6 +544,57 @@ struct RowSegments {
     return seg_rows > 0 ? (size_t)(m / seg_rows) * seg_stride + m % seg_rows : (size_t)m;
   }
 };
+// Rows m0 .. m0 + 3 by 256 threads (tid), k blocks [kb_lo, kb_hi): a share of the k blocks needs the whole rows' sums of
+// squares.  What a thread's first unit needs is requested beside the rows, so that the whole costs one trip to memory
+// (as two, and with the rows' loads in small batches, 5.5 us a launch instead of 4.5).  part: 8 floats of shared memory.
+__device__ __forceinline__ void norm_group(const float *x, int ldx, RowSegments seg, const float *__restrict__ w, float eps, int rows_all,
+                                           int K, const ActTiles &T, uint4 *__restrict__ blocks, int m0, int kb_lo, int kb_hi, float *part,
+                                           int tid) {
+  const int warp = tid >> 5, lane = tid & 31;
+  // unit = (k block, k chunk of 8, row of the group): this thread writes the row's hi and lo parts
+  const int r = tid % NAB_ROWS, c = (tid / NAB_ROWS) % 8, total = (kb_hi - kb_lo) * 8 * NAB_ROWS;
+  const bool row_ok = m0 + r < rows_all;
+  const float *xu = x + seg.row(row_ok ? m0 + r : 0) * ldx + c * 8;
+  float4 ua = make_float4(0.f, 0.f, 0.f, 0.f), ub = ua, wa = ua, wb = ua;
+  auto load_unit = [&](int u) {
+    const int k0 = (kb_lo + u / (NAB_ROWS * 8)) * TG_KB;
+    ua = __ldcg(reinterpret_cast<const float4 *>(xu + k0));
+    ub = __ldcg(reinterpret_cast<const float4 *>(xu + k0 + 4));
+    wa = __ldg(reinterpret_cast<const float4 *>(w + k0 + c * 8));
+    wb = __ldg(reinterpret_cast<const float4 *>(w + k0 + c * 8 + 4));
+  };
+  if (tid < total && row_ok) load_unit(tid);
+  {
+    // two warps per row
+    const int m = m0 + (warp >> 1);
+    float ss = 0.f;
+    if (m < rows_all) {
+      const float4 *xr = reinterpret_cast<const float4 *>(x + seg.row(m) * ldx);
+      const int n4 = K / 4;
+#pragma unroll 1
+      for (int k4 = (warp & 1) * 32 + lane; k4 < n4; k4 += 64 * 10) {
+        float4 v[10];
+#pragma unroll
+        for (int j = 0; j < 10; ++j) v[j] = k4 + 64 * j < n4 ? __ldcg(xr + k4 + 64 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 10; ++j) ss += v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
+      }
+    }
+    ss = warp_sum(ss);
+    if (lane == 0) part[warp] = ss;
+  }
+  __syncthreads();
+  const float s = rsqrtf((part[2 * r] + part[2 * r + 1]) / (float)K + eps);
+  if (!row_ok) return;
+#pragma unroll 1
+  for (int u = tid; u < total; u += 256) {
+    if (u != tid) load_unit(u);
+    const float f[8] = {ua.x * s * wa.x, ua.y * s * wa.y, ua.z * s * wa.z, ua.w * s * wa.w,
+                        ub.x * s * wb.x, ub.y * s * wb.y, ub.z * s * wb.z, ub.w * s * wb.w};
+    store_hi_lo(f, blocks + T.unit(m0 + r, kb_lo + u / (NAB_ROWS * 8), c), T.lo_offset());
+  }
+}
+
 __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, RowSegments seg,
                                                               const float *__restrict__ w, float eps, int rows_all, int K,
                                                               ActTiles T, uint4 *__restrict__ blocks, int n_groups,
@@ -570,42 +621,9 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
     if (i0 < zero_n - head - n4 * 4) zero[head + n4 * 4 + i0] = 0.f;
     return;
   }
-  const int m0 = blockIdx.x * NAB_ROWS, n_kb = T.n_kb;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ float part[8], inv[NAB_ROWS];
-  {
-    // two warps per row
-    const int r = warp >> 1, m = m0 + r;
-    float ss = 0.f;
-    if (m < rows_all) {
-      const float4 *xr = reinterpret_cast<const float4 *>(x + seg.row(m) * ldx);
-      for (int k4 = (warp & 1) * 32 + lane; k4 < K / 4; k4 += 64) {
-        const float4 v = xr[k4];
-        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-      }
-    }
-    ss = warp_sum(ss);
-    if (lane == 0) part[warp] = ss;
-  }
-  __syncthreads();
-  if (threadIdx.x < NAB_ROWS) inv[threadIdx.x] = rsqrtf((part[2 * threadIdx.x] + part[2 * threadIdx.x + 1]) / (float)K + eps);
-  __syncthreads();
-  // unit = (k block, k chunk of 8, row of the group): this thread writes the row's hi and lo columns;
-  // blockIdx.y takes a share of the k blocks (every share needs the whole row's sum of squares)
-  const int kb_lo = n_kb * blockIdx.y / gridDim.y, kb_hi = n_kb * (blockIdx.y + 1) / gridDim.y;
-  const int total = (kb_hi - kb_lo) * 8 * NAB_ROWS;
-  for (int u = threadIdx.x; u < total; u += blockDim.x) {
-    const int r = u % NAB_ROWS, c = (u / NAB_ROWS) % 8, kb = kb_lo + u / (NAB_ROWS * 8);
-    const int m = m0 + r, k = kb * TG_KB + c * 8;
-    if (m >= rows_all) continue;
-    const float *xr = x + seg.row(m) * ldx;
-    const float4 a = *reinterpret_cast<const float4 *>(xr + k), b = *reinterpret_cast<const float4 *>(xr + k + 4);
-    const float4 wa = __ldg(reinterpret_cast<const float4 *>(w + k)), wb = __ldg(reinterpret_cast<const float4 *>(w + k + 4));
-    const float s = inv[r];
-    const float f[8] = {a.x * s * wa.x, a.y * s * wa.y, a.z * s * wa.z, a.w * s * wa.w,
-                        b.x * s * wb.x, b.y * s * wb.y, b.z * s * wb.z, b.w * s * wb.w};
-    store_hi_lo(f, blocks + T.unit(m, kb, c), T.lo_offset());
-  }
+  __shared__ float part[8];
+  norm_group(x, ldx, seg, w, eps, rows_all, K, T, blocks, blockIdx.x * NAB_ROWS, T.n_kb * blockIdx.y / gridDim.y,
+             T.n_kb * (blockIdx.y + 1) / gridDim.y, part, threadIdx.x);
 }
 
 // The merge of the attention's key slices (step a4, second half) and the activation blocks of the O
@@ -613,6 +631,73 @@ __global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__res
 // from the slices' running max and sum, and writes the merged head outputs as hi and lo columns.
 // part_o [(row * nq + head) * nsplit + slice][D], part_ml the same with (max, sum); K = nq * D.
 constexpr int MAB_MAX_SLOTS = 2048;            // (rows of a group) x heads x slices the weights of a group may take
+// Rows m0 .. m0 + 3, k blocks [kb_lo, kb_hi), by 256 threads: the weight of every (row, head, slice) from the slices' max and
+// sum (one thread per row and head, into wgt), then the merged values.  A thread's first unit has its first slices
+// requested beside the weights' inputs: one trip to memory for up to four slices.
+constexpr int MERGE_AHEAD = 4;
+__device__ __forceinline__ void merge_group(const float *__restrict__ part_o, const float *__restrict__ part_ml, int nsplit, int nq, int D,
+                                            int rows_all, const ActTiles &T, uint4 *__restrict__ blocks, int m0, int kb_lo, int kb_hi,
+                                            float *wgt, int tid) {
+  const int r = tid % NAB_ROWS, c = (tid / NAB_ROWS) % 8, m = m0 + r, total = (kb_hi - kb_lo) * 8 * NAB_ROWS;
+  const bool row_ok = m < rows_all;
+  float4 va[MERGE_AHEAD], vb[MERGE_AHEAD];
+  const float *po = nullptr;
+  int h = 0;
+  auto load_unit = [&](int u) {
+    const int k = (kb_lo + u / (NAB_ROWS * 8)) * TG_KB + c * 8;
+    h = k / D;
+    po = part_o + ((size_t)m * nq + h) * nsplit * D + (k - h * D);
+    // (slots that no slice was written to are loaded too, but not used)
+#pragma unroll
+    for (int s = 0; s < MERGE_AHEAD; ++s)
+      if (s < nsplit) {
+        va[s] = *reinterpret_cast<const float4 *>(po + (size_t)s * D);
+        vb[s] = *reinterpret_cast<const float4 *>(po + (size_t)s * D + 4);
+      }
+  };
+  if (tid < total && row_ok) load_unit(tid);
+#pragma unroll 1
+  for (int i = tid; i < NAB_ROWS * nq; i += 256) {
+    const int wr_row = i / nq, wr_h = i - wr_row * nq, wm = m0 + wr_row;
+    if (wm >= rows_all) continue;
+    float *wr = wgt + (size_t)i * nsplit;
+    const float2 *ml = reinterpret_cast<const float2 *>(part_ml) + ((size_t)wm * nq + wr_h) * nsplit;
+    float mx = -INFINITY;
+    for (int s = 0; s < nsplit; ++s) {
+      const float2 v = ml[s];
+      if (v.y > 0.f) mx = fmaxf(mx, v.x);
+    }
+    float l = 0.f;
+    for (int s = 0; s < nsplit; ++s) {
+      const float2 v = ml[s];
+      const float f = v.y > 0.f ? __expf(v.x - mx) : 0.f;
+      wr[s] = f;
+      l += v.y * f;
+    }
+    const float inv = 1.f / l;
+    for (int s = 0; s < nsplit; ++s) wr[s] *= inv;
+  }
+  __syncthreads();
+  if (!row_ok) return;
+#pragma unroll 1
+  for (int u = tid; u < total; u += 256) {
+    if (u != tid) load_unit(u);
+    const float *wr = wgt + (size_t)(r * nq + h) * nsplit;
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    auto add = [&](float ws, const float4 &a, const float4 &b) {
+      if (ws != 0.f) {                                     // empty slices hold nothing that may be used
+        f[0] += ws * a.x; f[1] += ws * a.y; f[2] += ws * a.z; f[3] += ws * a.w;
+        f[4] += ws * b.x; f[5] += ws * b.y; f[6] += ws * b.z; f[7] += ws * b.w;
+      }
+    };
+#pragma unroll
+    for (int s = 0; s < MERGE_AHEAD; ++s)
+      if (s < nsplit) add(wr[s], va[s], vb[s]);
+    for (int s = MERGE_AHEAD; s < nsplit; ++s)
+      add(wr[s], *reinterpret_cast<const float4 *>(po + (size_t)s * D), *reinterpret_cast<const float4 *>(po + (size_t)s * D + 4));
+    store_hi_lo(f, blocks + T.unit(m, kb_lo + u / (NAB_ROWS * 8), c), T.lo_offset());
+  }
+}
 __global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml,
                                                                int nsplit, int nq, int D, int rows_all, ActTiles T,
                                                                uint4 *__restrict__ blocks) {
@@ -620,48 +705,9 @@ __global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__re
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int m0 = blockIdx.x * NAB_ROWS, n_kb = T.n_kb;
   __shared__ float wgt[MAB_MAX_SLOTS];
-  // weights: one thread per (row, head)
-  for (int i = threadIdx.x; i < NAB_ROWS * nq; i += blockDim.x) {
-    const int r = i / nq, h = i % nq, m = m0 + r;
-    float *wr = wgt + (size_t)i * nsplit;
-    if (m >= rows_all) { for (int s = 0; s < nsplit; ++s) wr[s] = 0.f; continue; }
-    const float *ml = part_ml + ((size_t)m * nq + h) * nsplit * 2;
-    float mx = -INFINITY;
-    for (int s = 0; s < nsplit; ++s)
-      if (ml[2 * s + 1] > 0.f) mx = fmaxf(mx, ml[2 * s]);
-    float l = 0.f;
-    for (int s = 0; s < nsplit; ++s) {
-      const float ls = ml[2 * s + 1];
-      const float f = ls > 0.f ? __expf(ml[2 * s] - mx) : 0.f;
-      wr[s] = f;
-      l += ls * f;
-    }
-    const float inv = 1.f / l;
-    for (int s = 0; s < nsplit; ++s) wr[s] *= inv;
-  }
-  __syncthreads();
-  const int kb_lo = n_kb * blockIdx.y / gridDim.y, kb_hi = n_kb * (blockIdx.y + 1) / gridDim.y;   // this block's share of the k blocks
-  const int total = (kb_hi - kb_lo) * 8 * NAB_ROWS;
-  for (int u = threadIdx.x; u < total; u += blockDim.x) {
-    const int r = u % NAB_ROWS, c = (u / NAB_ROWS) % 8, kb = kb_lo + u / (NAB_ROWS * 8);
-    const int m = m0 + r, k = kb * TG_KB + c * 8, h = k / D, d0 = k - h * D;
-    if (m >= rows_all) continue;
-    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float *wr = wgt + (size_t)(r * nq + h) * nsplit;
-    const float *po = part_o + ((size_t)m * nq + h) * nsplit * D + d0;
-    for (int s = 0; s < nsplit; ++s) {
-      const float ws = wr[s];
-      if (ws != 0.f) {                                     // empty slices hold nothing that may be read
-        const float4 a = *reinterpret_cast<const float4 *>(po + (size_t)s * D);
-        const float4 b = *reinterpret_cast<const float4 *>(po + (size_t)s * D + 4);
-        f[0] += ws * a.x; f[1] += ws * a.y; f[2] += ws * a.z; f[3] += ws * a.w;
-        f[4] += ws * b.x; f[5] += ws * b.y; f[6] += ws * b.z; f[7] += ws * b.w;
-      }
-    }
-    store_hi_lo(f, blocks + T.unit(m, kb, c), T.lo_offset());
-  }
+  merge_group(part_o, part_ml, nsplit, nq, D, rows_all, T, blocks, blockIdx.x * NAB_ROWS, T.n_kb * blockIdx.y / gridDim.y,
+              T.n_kb * (blockIdx.y + 1) / gridDim.y, wgt, threadIdx.x);
 }
 
 // Weights [N][K] bf16 row-major (rows [row0, row0 + N_src) of the fused matrix) -> 16 KiB blocks.

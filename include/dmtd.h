@@ -255,8 +255,8 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *ctx, float temperature, uint64_t seed);
  *   "tcgen05_gemm_stages" n  pipeline stages of a block of that GEMM, 2..6; 0 = as many as
  *                       shared memory holds (default 0)
  *   "fused_qk_rope" 0/1 QK-norm, rotary embedding and the KV append (Section 3.1's Qwen3 block) inside
- *                       the tensor-core attention kernel of the per-step path (16-bit cache, head_dim
- *                       128, chunks of fewer than 16 positions) instead of a launch of their own (default 1)
+ *                       the decode attention kernels of the per-step path (chunks of fewer than 16 positions; not
+ *                       an fp32 cache with head_dim 128) instead of a launch of their own (default 1)
  * Errors: INVALID_ARG for an unknown name or value; SHAPE / STATE for encoding_layers as above. */
 dmtd_status dmtd_set_option(dmtd_ctx *ctx, const char *name, int64_t value);
 

@@ -47,32 +47,6 @@ __device__ __forceinline__ uint32_t ad_part(int row, int part) {
   return (uint32_t)(row * 256 + ((part & 8) | ((part & 7) ^ (((row & 1) << 2) | ((row >> 1) & 3)))) * 16);
 }
 
-// What the fused form of attn_decode_kernel needs for step a3 (QK-norm, rotary embedding, KV append): with these the
-// kernel reads the raw q | k | v rows of the QKV projection itself; every block normalises and rotates its own
-// query rows and the new K rows that fall into its keys (a few rows, recomputed by the blocks that share
-// them), and the block that owns a position appends its K and V rows to the cache.  w_qn == nullptr: the rows in
-// qkv are finished already and the new K / V rows are in the cache (the stand-alone attention call).
-struct AttnFuse {
-  const float *w_qn, *w_kn;        // QK-norm weights [128]
-  const float2 *table;             // (cos, sin) of the pass's positions [R][64]
-  float eps;
-};
-// QK-norm and rotary embedding of one head vector, one value per lane and quarter (v[j] = element lane + 32 j).
-__device__ __forceinline__ void head_norm_rope_table(const float *w, const float2 *cs_row, float eps, int lane, float (&v)[4]) {
-  float ss = v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
-  ss = warp_sum(ss);
-  const float inv = rsqrtf(ss / (float)PK_D + eps);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = v[j] * inv * w[lane + 32 * j];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float2 cs = cs_row[lane + 32 * j];
-    const float a = v[j], bb = v[j + 2];
-    v[j] = a * cs.x - bb * cs.y;
-    v[j + 2] = bb * cs.x + a * cs.y;
-  }
-}
-
 // One warp tile (16 keys, K at k_t, V at v_t) against up to 8 query rows, operands swapped: the keys are the M axis of
 // S^T = K Q^T and the 128 output dimensions the M axis of O^T = V^T P^T, the query rows the 8 columns (with the rows on
 // the M axis an m16 tile would be half padding or more).  Thread (g, t) holds columns (query rows) 2t, 2t + 1 of rows
@@ -342,7 +316,7 @@ attn_decode_kernel(const float *__restrict__ qkv, int ldq, const void *__restric
         const float *src = qkv + (size_t)(b * R + r0 + qi / G) * ldq + (size_t)(kvh * G + qi % G) * PK_D;
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = src[lane + 32 * j];
-        if (FUSED) head_norm_rope_table(F.w_qn, F.table + (size_t)(r0 + qi / G) * (PK_D / 2), F.eps, lane, v);
+        if (FUSED) head_norm_rope<PK_D>(F.w_qn, F.table + (size_t)(r0 + qi / G) * (PK_D / 2), F.eps, lane, v);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) qh[lane + 32 * j] = Op::from_float(v[j] * scale);
@@ -357,7 +331,7 @@ attn_decode_kernel(const float *__restrict__ qkv, int ldq, const void *__restric
         float v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = src[lane + 32 * j];
-        if (!is_v) head_norm_rope_table(F.w_kn, F.table + (size_t)r * (PK_D / 2), F.eps, lane, v);
+        if (!is_v) head_norm_rope<PK_D>(F.w_kn, F.table + (size_t)r * (PK_D / 2), F.eps, lane, v);
         typename Op::T *row = reinterpret_cast<typename Op::T *>(sc + AD_NEW) + ((is_v ? AD_MAX_NEW : 0) + r - r_lo) * PK_D;
         typename Op::T *cache = const_cast<typename Op::T *>(is_v ? vb : kb) + (size_t)(pos0 + r) * PK_D;
 #pragma unroll

@@ -80,6 +80,7 @@ struct dmtd_ctx {
   float *x_lo = nullptr, *x_up = nullptr, *act = nullptr, *qkv = nullptr, *gu = nullptr,
         *logits = nullptr, *part_o = nullptr, *part_ml = nullptr;
   float2 *rope_tab = nullptr;
+  const float2 *rope_rows = nullptr;       // rows of rope_tab of the positions the next layers work on
   float *h_pend = nullptr;                  // [max_batch][pend_cap][hidden]: h_enc of positions the thinking layers have not seen
   float *h_base = nullptr;                  // [ws_rows][hidden]: h_emb / h_enc of a chunk of rows (literal sum, masked forward)
   int pend_cap = 0;
@@ -98,6 +99,7 @@ struct dmtd_ctx {
   unsigned int *grid_bar = nullptr;
   float *pick_val = nullptr;                // per-step greedy pick: best of every vocabulary slice, [max_batch][ARGMAX_SLICES]
   int *pick_idx = nullptr;
+  unsigned int *pick_arrived = nullptr;
   long long *pass_timing = nullptr;         // profiling builds only
 
   // graphs: [kind 1 = full, 2 = upper-only]
@@ -388,17 +390,26 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   return launch_gemv_nt<4>(c, W, act, lda, M, out, ldo);
 }
 
-// attn_partial_kernel compiled for the fewest query rows that hold n_rows.
+// attn_partial_kernel compiled for the fewest query rows that hold n_rows, for slices of CH keys.
 template <typename KVT>
 struct AttnPartialKernel {
-  void (*kernel)(const float *, int, const KVT *, const KVT *, int, int, int, int, int, int, const int *, int, float *, float *, int);
+  void (*kernel)(const float *, int, const KVT *, const KVT *, int, int, int, int, int, int, const int *, int, float *, float *, int, AttnFuse);
+  int threads;
   size_t smem;
 };
-template <int D, typename KVT>
-AttnPartialKernel<KVT> attn_partial_for(int n_rows) {
-  const int nq = n_rows <= 4 ? 4 : n_rows <= 8 ? 8 : 16;
-  return {nq == 4 ? attn_partial_kernel<D, KVT, 4> : nq == 8 ? attn_partial_kernel<D, KVT, 8> : attn_partial_kernel<D, KVT, 16>,
-          (size_t)ATTN_WARPS * nq * D * sizeof(float)};
+template <int D, typename KVT, bool FUSED, int T>
+AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R) {
+  const int nq = n_rows <= 4 ? 4 : n_rows <= 8 ? 8 : 16, warps = attn_warps(T);
+  return {nq == 4   ? attn_partial_kernel<D, KVT, 4, FUSED, T>
+          : nq == 8 ? attn_partial_kernel<D, KVT, 8, FUSED, T>
+                    : attn_partial_kernel<D, KVT, 16, FUSED, T>,
+          warps * 32, (size_t)warps * nq * D * sizeof(float) + (FUSED ? 2 * (size_t)R * D * sizeof(KVT) : 0)};
+}
+template <int D, typename KVT, bool FUSED>
+AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R, int CH) {
+  if constexpr (D == 64)                    // head_dim 128: only with "tensor_core_attention" off
+    if (CH <= 64) return attn_partial_for<D, KVT, FUSED, 1>(n_rows, R);
+  return attn_partial_for<D, KVT, FUSED, 4>(n_rows, R);
 }
 
 // Does the attention of R new rows per sequence run on attn_decode_kernel?
@@ -419,12 +430,12 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
   KVT *kc = static_cast<KVT *>(c->kc) + (size_t)layer * c->kv_layer_elems;
   KVT *vc = static_cast<KVT *>(c->vc) + (size_t)layer * c->kv_layer_elems;
   const LayerDev &lw = c->layers[layer];
-  // a3 inside the attention kernel (16-bit cache, head_dim 128, decode-sized chunks): one launch less per layer
-  const bool fused_a3 = D == PK_D && !std::is_same<KVT, float>::value && c->use_tc_attention && c->fuse_qk_rope && !flash &&
-                        R <= AD_MAX_NEW;
+  // a3 inside the attention kernel (decode-sized chunks): one launch less per layer
+  const bool tiled = D == PK_D && c->use_tc_attention;                 // attn_decode_kernel or attn_f32_kernel
+  const bool fused_a3 = (tiled ? !std::is_same<KVT, float>::value : D == 64) && c->fuse_qk_rope && !flash && R <= AD_MAX_NEW;
   if (!fused_a3) {
     CUDA_TRY(c, launch_pdl(qk_norm_rope_append_kernel<D, KVT>, dim3(M, (heads + 3) / 4), dim3(128), (size_t)(0), c->stream,
-                             c->qkv, c->ldqkv, s.n_q_heads, s.n_kv_heads, R, lw.w_qn, lw.w_kn, s.rms_eps, c->rope_tab, pos0, kc, vc, c->max_seq));
+                             c->qkv, c->ldqkv, s.n_q_heads, s.n_kv_heads, R, lw.w_qn, lw.w_kn, s.rms_eps, c->rope_rows, pos0, kc, vc, c->max_seq));
     LAUNCH_OK(c, "qk_norm_rope_append_kernel");
   }
   if constexpr (D == PK_D && !std::is_same<KVT, float>::value) {
@@ -447,7 +458,7 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
     }
   }
   int RB = std::max(1, ATTN_QR / G), n_rb = (R + RB - 1) / RB;
-  if (D == PK_D && c->use_tc_attention) {
+  if (tiled) {
     // head_dim 128: the tensor-core kernel with a bf16 cache, the FMA kernel with an fp32 cache
     if constexpr (std::is_same<KVT, float>::value) {
       CUDA_TRY(c, launch_pdl(attn_f32_kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(PK_THREADS), ATTN_F32_SMEM, c->stream,
@@ -458,12 +469,14 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
       const int n_blocks = tc_attention_plan(c, B, R, nsplit).n_blocks;
       CUDA_TRY(c, launch_pdl(fused_a3 ? attn_decode_kernel<Op, true> : attn_decode_kernel<Op, false>, dim3(n_blocks), dim3(AD_THREADS),
                              AD_SMEM, c->stream, c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, 0,
-                             c->part_o, c->part_ml, nsplit, AttnFuse{lw.w_qn, lw.w_kn, c->rope_tab, s.rms_eps}));
+                             c->part_o, c->part_ml, nsplit, AttnFuse{lw.w_qn, lw.w_kn, c->rope_rows, s.rms_eps}));
     }
   } else {
-    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT>(std::min(R, RB) * G);
-    CUDA_TRY(c, launch_pdl(ap.kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(ATTN_WARPS * 32), ap.smem, c->stream, c->qkv, c->ldqkv,
-                           kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, 0, c->part_o, c->part_ml, nsplit));
+    const AttnPartialKernel<KVT> ap =
+        fused_a3 ? attn_partial_for<D, KVT, D == 64>(std::min(R, RB) * G, R, c->CH) : attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, c->CH);
+    CUDA_TRY(c, launch_pdl(ap.kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(ap.threads), ap.smem, c->stream, c->qkv, c->ldqkv,
+                           kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, 0, c->part_o, c->part_ml, nsplit,
+                           AttnFuse{lw.w_qn, lw.w_kn, c->rope_rows, s.rms_eps}));
   }
   LAUNCH_OK(c, "attn_partial_kernel");
   if (!merge) return DMTD_OK;               // the O projection's activation-block kernel merges the slices
@@ -498,17 +511,23 @@ dmtd_status launch_attention(dmtd_ctx *c, int layer, int B, int R, const int *po
                         : launch_attention_t<64, float>(c, layer, B, R, pos0, nsplit, merge, flash);
 }
 
+RopeTable rope_table(const dmtd_ctx *c) { return RopeTable{c->inv_freq, c->rope_tab, c->s.head_dim / 2}; }
+int rope_blocks(const dmtd_ctx *c, int R) { return (R * (c->s.head_dim / 2) + 127) / 128; }
+
+// rope_rows: the table's rows for the layers that follow; they start at row 0 unless the caller moves them
 dmtd_status launch_rope_table(dmtd_ctx *c, const int *pos0, int R) {
-  int half = c->s.head_dim / 2, n = R * half;
-  rope_table_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(pos0, R, half, c->inv_freq, c->rope_tab);
+  rope_table_kernel<<<rope_blocks(c, R), 128, 0, c->stream>>>(pos0, R, rope_table(c));
   LAUNCH_OK(c, "rope_table_kernel");
+  c->rope_rows = c->rope_tab;
   return DMTD_OK;
 }
 
+// x = (accumulate: +=) the embeddings of positions *pos0 .. *pos0 + R - 1; not accumulate: their rotary table as well
 dmtd_status launch_embed(dmtd_ctx *c, const int *pos0, int B, int R, float *x, bool accumulate) {
-  embed_kernel<<<B * R, 128, 0, c->stream>>>(c->embed, c->tokens, c->max_seq, pos0, R, x, c->s.hidden,
-                                             accumulate ? 1 : 0, c->dstate);
+  embed_kernel<<<B * R + (accumulate ? 0 : rope_blocks(c, R)), 128, 0, c->stream>>>(c->embed, c->tokens, c->max_seq, pos0, R, B * R, x,
+                                                                                    c->s.hidden, accumulate ? 1 : 0, c->dstate, rope_table(c));
   LAUNCH_OK(c, "embed_kernel");
+  if (!accumulate) c->rope_rows = c->rope_tab;
   return DMTD_OK;
 }
 
@@ -527,6 +546,20 @@ int slices_for(const dmtd_ctx *c, int B, int R, int pos_end) {
   return tc_attention_plan(c, B, R, (int)std::max(1ll, std::min<long long>(room, std::max(1, fused_merge)))).nsplit;
 }
 
+// fp32 weights, the few rows of a decode pass: every projection with the step in front of it.
+bool f32_fused_rows(const dmtd_ctx *c, int M) {
+  const dmtd_model_shape &s = c->s;
+  return !is_bf16(c) && M <= F32_FUSE_ROWS && (long long)M * std::max({s.hidden, s.intermediate, s.n_q_heads * s.head_dim}) <= F32_FUSE_FLOATS;
+}
+template <int IN>
+dmtd_status launch_gemv_f32_fused(dmtd_ctx *c, const PackedMat &W, const F32In &in, int M, float *out, int ldo, bool store) {
+  CUDA_TRY(c, launch_pdl(gemv_f32_fused_kernel<IN>, dim3(std::min(4 * c->n_sms, (W.N + 7) / 8)), dim3(256),
+                         (size_t)M * W.K * sizeof(float), c->stream, W, in, M, out, ldo, store ? 1 : 0));
+  LAUNCH_OK(c, "gemv_f32_fused_kernel");
+  return DMTD_OK;
+}
+F32In f32_norm_input(const dmtd_ctx *c, const float *x, const float *w) { return F32In{x, c->s.hidden, w, c->s.rms_eps, nullptr, nullptr, 0, 0}; }
+
 // One decoder layer (steps a2-a7) on x [B*R][hidden]; rows of sequence b sit at positions
 // *pos0 .. *pos0+R-1.  pos_end = host's value of *pos0 + R.
 dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos0, int pos_end) {
@@ -535,6 +568,14 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   int M = B * R, H = s.hidden, I = s.intermediate;
   // the tcgen05 path normalises while it writes its activation blocks
   const bool tc = lw.qkv_u.w && c->use_umma;
+  if (f32_fused_rows(c, M) && !flash_attention_ok(c, R)) {
+    const int nsplit = slices_for(c, B, R, pos_end);
+    TRY(launch_gemv_f32_fused<F32_NORM>(c, lw.qkv, f32_norm_input(c, x, lw.w_in), M, c->qkv, c->ldqkv, true));
+    TRY(launch_attention(c, l, B, R, pos0, nsplit, false));
+    TRY(launch_gemv_f32_fused<F32_SLICES>(c, lw.o, F32In{nullptr, 0, nullptr, 0.f, c->part_o, c->part_ml, nsplit, s.n_q_heads}, M, x, H, false));
+    TRY(launch_gemv_f32_fused<F32_NORM>(c, lw.gu, f32_norm_input(c, x, lw.w_post), M, c->gu, c->ldgu, true));
+    return launch_gemv_f32_fused<F32_SWIGLU>(c, lw.down, F32In{c->gu, c->ldgu, nullptr, 0.f, nullptr, nullptr, 0, 0}, M, x, H, false);
+  }
   if (tc) {
     TRY(launch_gemm_tc05(c, lw.qkv_u, norm_input(x, H, lw.w_in), M, c->qkv, c->ldqkv));
   } else {
@@ -592,10 +633,12 @@ SampleParams sample_params(const dmtd_ctx *c) {
   return sp;
 }
 
-// Step a9/a10: final norm, tied LM head, greedy pick, token feedback.
-dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits) {
+// Step a9/a10/a0: final norm, tied LM head, greedy pick, token feedback, the schedule's counters.
+dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits, int kind, int P) {
   const dmtd_model_shape &s = c->s;
-  if (c->embed_u.w && c->use_umma) {
+  if (f32_fused_rows(c, B)) {
+    TRY(launch_gemv_f32_fused<F32_NORM>(c, c->embed, f32_norm_input(c, c->x_up, c->w_final), B, c->logits, c->ldl, true));
+  } else if (c->embed_u.w && c->use_umma) {
     TRY(launch_gemm_tc05(c, c->embed_u, norm_input(c->x_up, s.hidden, c->w_final), B, c->logits, c->ldl));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
@@ -606,12 +649,10 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
   if (out_logits)
     CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (size_t)s.vocab * 4, c->logits, (size_t)c->ldl * 4, (size_t)s.vocab * 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
-  CUDA_TRY(c, launch_pdl(argmax_slices_kernel, dim3(B, ARGMAX_SLICES), dim3(256), (size_t)(0), c->stream,
-                          c->logits, c->ldl, s.vocab, c->pick_val, c->pick_idx, c->dstate, sample_params(c)));
-  LAUNCH_OK(c, "argmax_slices_kernel");
-  CUDA_TRY(c, launch_pdl(argmax_pick_kernel, dim3(B), dim3(32), (size_t)(0), c->stream,
-                          c->pick_val, c->pick_idx, ARGMAX_SLICES, c->tokens, c->max_seq, c->dstate, write_token ? 1 : 0, out_argmax));
-  LAUNCH_OK(c, "argmax_pick_kernel");
+  CUDA_TRY(c, launch_pdl(argmax_kernel, dim3(B, ARGMAX_SLICES), dim3(256), (size_t)(0), c->stream,
+                          c->logits, c->ldl, s.vocab, c->dstate, sample_params(c),
+                          PickParams{c->pick_val, c->pick_idx, c->pick_arrived, write_token ? c->tokens : nullptr, c->max_seq, out_argmax, kind, P}));
+  LAUNCH_OK(c, "argmax_kernel");
   return DMTD_OK;
 }
 
@@ -652,10 +693,23 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
-  // 16 query rows of 128 dimensions: a little over 48 KiB with the kernel's static arrays
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, float, 16>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __nv_bfloat16, 16>, dyn, 64 * 1024));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_kernel<128, __half, 16>, dyn, 64 * 1024));
+  // 16 query rows, 128 dimensions or new rows take the key-group kernel past 48 KiB
+  auto partial = [&](auto kv) -> dmtd_status {
+    using KVT = decltype(kv);
+    for (int rows : {8, 16}) {
+      CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<128, KVT, false>(rows, 1, 64).kernel, dyn, 64 * 1024));
+      for (int CH : {64, 128}) {
+        CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<64, KVT, false>(rows, 1, CH).kernel, dyn, 64 * 1024));
+        CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<64, KVT, true>(rows, 1, CH).kernel, dyn, 64 * 1024));
+      }
+    }
+    return DMTD_OK;
+  };
+  for (auto gemv : {gemv_f32_fused_kernel<F32_NORM>, gemv_f32_fused_kernel<F32_SWIGLU>, gemv_f32_fused_kernel<F32_SLICES>})
+    CUDA_TRY(c, cudaFuncSetAttribute(gemv, dyn, (int)(F32_FUSE_FLOATS * sizeof(float))));
+  TRY(partial(0.f));
+  TRY(partial(__nv_bfloat16{}));
+  TRY(partial(__half{}));
   return DMTD_OK;
 }
 
@@ -776,7 +830,6 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
     // output h_enc is kept until the thinking layers have seen the position
     const int Le = c->L_e;
     TRY(launch_embed(c, &c->dstate->newest, B, 1, c->x_up, false));
-    TRY(launch_rope_table(c, &c->dstate->newest, 1));
     for (int l = 0; l < Le; ++l) TRY(run_layer(c, l, c->x_up, B, 1, &c->dstate->newest, newest + 1));
     if (kind == 1) {
       // full pass: the pending rows' h_enc and the newest row's through the thinking layers
@@ -801,7 +854,6 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
     }
   } else if (kind == 1 && lo > 0) {
     TRY(launch_embed(c, &c->dstate->lo_len, B, R_lower, c->x_lo, false));
-    TRY(launch_rope_table(c, &c->dstate->lo_len, R_lower));
     for (int l = 0; l < lo; ++l) TRY(run_layer(c, l, c->x_lo, B, R_lower, &c->dstate->lo_len, c->h.n_known));
     CUDA_TRY(c, launch_pdl(select_last_kernel, dim3(B), dim3(256), (size_t)(0), c->stream,
                             c->x_lo, R_lower, H, c->x_up));
@@ -810,13 +862,10 @@ dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, i
   } else {
     TRY(launch_embed(c, &c->dstate->newest, B, 1, c->x_up, false));
   }
-  TRY(launch_rope_table(c, &c->dstate->newest, 1));
+  // the newest position's row is the last one of a full pass's table
+  if (kind == 1 && lo > 0) c->rope_rows = c->rope_tab + (size_t)(R_lower - 1) * (c->s.head_dim / 2);
   for (int l = lo; l < L; ++l) TRY(run_layer(c, l, c->x_up, B, 1, &c->dstate->newest, newest + 1));
-  TRY(run_head(c, B, write_token, out_argmax, out_logits));
-  CUDA_TRY(c, launch_pdl(advance_state_kernel, dim3(1), dim3(1), (size_t)(0), c->stream,
-                          c->dstate, kind, 0));
-  LAUNCH_OK(c, "advance_state_kernel");
-  return DMTD_OK;
+  return run_head(c, B, write_token, out_argmax, out_logits, kind, 0);
 }
 
 void host_advance(dmtd_ctx *c, int kind) {
@@ -1041,6 +1090,8 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   CTRY(dev_alloc(c, &c->logits, (size_t)max_batch * c->ldl));
   CTRY(dev_alloc(c, &c->pick_val, (size_t)max_batch * ARGMAX_SLICES));
   CTRY(dev_alloc(c, &c->pick_idx, (size_t)max_batch * ARGMAX_SLICES));
+  CTRY(dev_alloc(c, &c->pick_arrived, (size_t)max_batch + 1));
+  CCUDA(cudaMemsetAsync(c->pick_arrived, 0, ((size_t)max_batch + 1) * sizeof(unsigned int), c->stream));
   CTRY(dev_alloc(c, &c->part_o, (size_t)c->part_rows * s.n_q_heads * c->nsplit_max * D));
   CTRY(dev_alloc(c, &c->part_ml, (size_t)c->part_rows * s.n_q_heads * c->nsplit_max * 2));
   CTRY(dev_alloc(c, &c->rope_tab, (size_t)c->ws_rows * (D / 2)));
@@ -1107,7 +1158,6 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
     set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->scratch, p0);
     LAUNCH_OK(c, "set_int_kernel");
     TRY(launch_embed(c, &c->dstate->scratch, B, R, c->x_lo, false));
-    TRY(launch_rope_table(c, &c->dstate->scratch, R));
     for (int l = 0; l < L; ++l) {
       if (c->literal_sum && c->L_e > 0) {
         // Eq. 4's sum with h_enc in h_emb's place: keep the encoding layers' output, add it at the boundary
@@ -1132,13 +1182,10 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
   // n_known must read P when the head writes the token
   set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->n_known, P);
   LAUNCH_OK(c, "set_int_kernel");
-  TRY(run_head(c, B, forced_first == nullptr, out_token, out_logits));
+  TRY(run_head(c, B, forced_first == nullptr, out_token, out_logits, 0, P));
   if (forced_first)
     CUDA_TRY(c, cudaMemcpy2DAsync(c->tokens + P, (size_t)c->max_seq * 4, forced_first, 4, 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
-  CUDA_TRY(c, launch_pdl(advance_state_kernel, dim3(1), dim3(1), (size_t)(0), c->stream,
-                          c->dstate, 0, P));
-  LAUNCH_OK(c, "advance_state_kernel");
   c->h.n_known = P + 1; c->h.lo_len = P; c->h.up_len = P; c->h.cycle = 1;
   c->h.slot = 1 % c->tau; c->h.n_emitted = 1;
   c->prefilled = true;
@@ -1225,7 +1272,6 @@ dmtd_status dmtd_masked_forward(dmtd_ctx *c, const int32_t *tokens, int32_t B, i
     set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->scratch, p0);
     LAUNCH_OK(c, "set_int_kernel");
     TRY(launch_embed(c, &c->dstate->scratch, B, R, c->x_lo, false));                 // h_emb
-    TRY(launch_rope_table(c, &c->dstate->scratch, R));
     for (int l = 0; l < Le; ++l) TRY(run_layer(c, l, c->x_lo, B, R, &c->dstate->scratch, p0 + R));   // Eq. 1: h_enc
     copy_rows_kernel<<<256, 256, 0, c->stream>>>(c->x_lo, c->h_base, n4, 0);
     LAUNCH_OK(c, "copy_rows_kernel");
@@ -1449,12 +1495,12 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
     }
   } else {
-    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT>(std::min(R, RB) * G);
+    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, p.CH);
     e = cudaFuncSetAttribute(ap.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ap.smem);
     if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
-    ap.kernel<<<dim3(p.nsplit, nkv * n_rb, B), ATTN_WARPS * 32, ap.smem, stream>>>(
+    ap.kernel<<<dim3(p.nsplit, nkv * n_rb, B), ap.threads, ap.smem, stream>>>(
         q, ld, static_cast<const KVT *>(k), static_cast<const KVT *>(v), max_seq, nq, nkv, R, RB, p.CH, nullptr, pos0, part_o,
-        part_ml, p.nsplit);
+        part_ml, p.nsplit, AttnFuse{});
   }
   int n_rh = B * R * nq;
   e = launch_pdl(attn_merge_kernel<D>, dim3((n_rh + 3) / 4), dim3(128), 0, stream, part_o, part_ml, nsplit, n_rh, nq, out, ld);

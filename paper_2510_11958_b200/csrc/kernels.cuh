@@ -57,9 +57,25 @@ __global__ void to_float_kernel(const T *__restrict__ src, float *__restrict__ d
 // a1: embedding gather.  x[m][:] = E[token of row m]; row m = b*R + r sits at position
 // *pos0 + r of sequence b.
 // ------------------------------------------------------------------------------------
+// The blocks past the rows write the rotary table of the same positions (rope_table_kernel's).
+struct RopeTable {
+  const double *inv_freq;
+  float2 *table;
+  int half;
+};
+// cos/sin of pos * theta^(-2i/d), computed in double so that long contexts do not lose angle precision; entry idx of
+// the table [R][d/2] of (cos, sin).
+__device__ __forceinline__ void rope_entry(const RopeTable &T, int pos0, int R, int idx) {
+  if (idx >= R * T.half) return;
+  double s, c;
+  sincos((double)(pos0 + idx / T.half) * T.inv_freq[idx % T.half], &s, &c);
+  T.table[idx] = make_float2((float)c, (float)s);
+}
+// grid (rows + blocks of the table), 128 threads
 __global__ void embed_kernel(PackedMat E, const int *__restrict__ tokens, int max_seq,
-                             const int *__restrict__ pos0, int R, float *__restrict__ x, int ldx,
-                             int accumulate, DevState *st) {
+                             const int *__restrict__ pos0, int R, int n_rows, float *__restrict__ x, int ldx,
+                             int accumulate, DevState *st, RopeTable rope) {
+  if (blockIdx.x >= n_rows) return rope_entry(rope, *pos0, R, (blockIdx.x - n_rows) * blockDim.x + threadIdx.x);
   int m = blockIdx.x, b = m / R, r = m % R;
   int tok = tokens[(size_t)b * max_seq + *pos0 + r];
   if (tok < 0 || tok >= E.N) {
@@ -263,20 +279,160 @@ __global__ void gemv_f32_kernel(PackedMat W, const float *__restrict__ act, int 
   }
 }
 
+// The same for the few rows of a decode pass, together with the step in front of it: every block works the M activation
+// rows out in shared memory (a few KB) - RMSNorm, the SwiGLU gate, or the merge of the attention's key slices - and
+// multiplies its weight rows.  A layer of a small model is bound by the number of its launches and by the trips to memory
+// that follow one another in each: five launches instead of ten, and in each of them one trip for everything that is read
+// (the first weight row of a warp is requested before the kernel in front is waited for).  24 passes of the 4-layer fp32
+// test shape (hidden 256), one sequence: 2.00 ms with ten launches a layer, 1.34 so; 16 sequences: 5.72 and 4.92.
+// store: out = instead of out +=.
+enum { F32_NORM = 0, F32_SWIGLU = 1, F32_SLICES = 2 };
+constexpr int F32_FUSE_ROWS = 16, F32_FUSE_FLOATS = 12 * 1024;     // most rows, and rows x K (48 KB)
+constexpr int F32_AHEAD = 6;                                        // 128-value pieces of a row in flight
+struct F32In {
+  const float *act;               // F32_NORM: [M][lda]; F32_SWIGLU: gate | up, K apart
+  int lda;
+  const float *norm_w;
+  float eps;
+  const float *part_o, *part_ml;  // F32_SLICES: [(row * nq + head) * nsplit + slice][K / nq] and (max, sum)
+  int nsplit, nq;
+};
+template <int IN>
+__global__ void __launch_bounds__(256) gemv_f32_fused_kernel(PackedMat W, F32In in, int M, float *__restrict__ out, int ldo, int store) {
+  extern __shared__ __align__(16) float xs[];                       // [M][K]
+  __shared__ float ss_part[8][F32_FUSE_ROWS];                       // F32_NORM: sums of squares, by a row's warps
+  const int lane = threadIdx.x & 31, w8 = threadIdx.x >> 5, K = W.K;
+  const int warp = blockIdx.x * 8 + w8, n_warps = gridDim.x * 8;
+  const int row_warps = M >= 8 ? 1 : 8 / M, part = w8 % row_warps;  // warps that share an activation row
+  float4 w0[F32_AHEAD];
+#pragma unroll
+  for (int c = 0; c < F32_AHEAD; ++c) {
+    const int k = lane * 4 + 128 * c;
+    w0[c] = warp < W.N && k < K ? *reinterpret_cast<const float4 *>(W.wf + (size_t)warp * K + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  pdl_enter();
+  // lane i < 4: the value that row i's product is added to
+  const float old = !store && warp < W.N && lane < min(4, M) ? out[(size_t)lane * ldo + warp] : 0.f;
+  if (IN == F32_SLICES) {
+    // one warp per (row, head), as attn_merge_kernel; the first slices' outputs are requested with the (max, sum) pairs
+    constexpr int FIRST = 2;
+    const int D = K / in.nq;
+    for (int i = w8; i < M * in.nq; i += 8) {
+      const float2 *ml = reinterpret_cast<const float2 *>(in.part_ml) + (size_t)i * in.nsplit;
+      const float *po = in.part_o + (size_t)i * in.nsplit * D;
+      float2 v = lane < in.nsplit ? ml[lane] : make_float2(0.f, 0.f);
+      float first[FIRST][4];
+#pragma unroll
+      for (int s = 0; s < FIRST; ++s)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) first[s][e] = s < in.nsplit && lane + 32 * e < D ? po[s * D + lane + 32 * e] : 0.f;
+      float mx = v.y > 0.f ? v.x : -INFINITY;
+      for (int s = lane + 32; s < in.nsplit; s += 32) {
+        const float2 u = ml[s];
+        if (u.y > 0.f) mx = fmaxf(mx, u.x);
+      }
+      mx = warp_max(mx);
+      float l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};                    // D is 64 or 128: two or four values per lane
+      for (int s0 = 0; s0 < in.nsplit; s0 += 32) {
+        if (s0) v = s0 + lane < in.nsplit ? ml[s0 + lane] : make_float2(0.f, 0.f);
+        const float f = v.y > 0.f ? __expf(v.x - mx) : 0.f;
+        l += f * v.y;
+        unsigned live = __ballot_sync(0xffffffffu, v.y > 0.f);       // slices without keys hold nothing that may be used
+        if (s0 == 0) {
+#pragma unroll
+          for (int s = 0; s < FIRST; ++s)
+            if (live >> s & 1) {
+              const float fs = __shfl_sync(0xffffffffu, f, s);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o[e] += fs * first[s][e];
+            }
+          live &= ~0u << FIRST;
+        }
+        while (live) {
+          const int s = __ffs(live) - 1;
+          live &= live - 1;
+          const float fs = __shfl_sync(0xffffffffu, f, s);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (lane + 32 * e < D) o[e] += fs * po[(size_t)(s0 + s) * D + lane + 32 * e];
+        }
+      }
+      const float inv = 1.f / warp_sum(l);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (lane + 32 * e < D) xs[(size_t)i * D + lane + 32 * e] = o[e] * inv;
+    }
+  } else {
+    // RMSNorm: the rows times the gain, 1 / rms goes to the product; a row's warps take its 128-value pieces in turn
+    for (int m = w8 / row_warps; m < M; m += 8) {
+      const float *xr = in.act + (size_t)m * in.lda;
+      float ss = 0.f;
+#pragma unroll 4
+      for (int k = (part * 32 + lane) * 4; k < K; k += 128 * row_warps) {
+        float4 v = *reinterpret_cast<const float4 *>(xr + k);
+        const float4 u = *reinterpret_cast<const float4 *>((IN == F32_SWIGLU ? xr + K : in.norm_w) + k);
+        if (IN == F32_SWIGLU) {
+          v.x = v.x / (1.f + expf(-v.x)); v.y = v.y / (1.f + expf(-v.y));
+          v.z = v.z / (1.f + expf(-v.z)); v.w = v.w / (1.f + expf(-v.w));
+        } else {
+          ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        }
+        *reinterpret_cast<float4 *>(xs + (size_t)m * K + k) = make_float4(v.x * u.x, v.y * u.y, v.z * u.z, v.w * u.w);
+      }
+      if (IN == F32_NORM) {
+        ss = warp_sum(ss);
+        if (lane == 0) ss_part[part][m] = ss;
+      }
+    }
+  }
+  __syncthreads();
+  float row_scale = 1.f;                                            // lane m: of row m
+  if (IN == F32_NORM && lane < M) {
+    float ss = 0.f;
+    for (int i = 0; i < row_warps; ++i) ss += ss_part[i][lane];
+    row_scale = rsqrtf(ss / (float)K + in.eps);
+  }
+  for (int n = warp; n < W.N; n += n_warps) {
+    const float *wr = W.wf + (size_t)n * K;
+    for (int m0 = 0; m0 < M; m0 += 4) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      auto add = [&](const float4 &w, int k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (m0 + i < M) {
+            const float4 a = *reinterpret_cast<const float4 *>(xs + (size_t)(m0 + i) * K + k);
+            acc[i] += w.x * a.x + w.y * a.y + w.z * a.z + w.w * a.w;
+          }
+      };
+      int k = lane * 4;
+      if (n == warp) {
+#pragma unroll
+        for (int c = 0; c < F32_AHEAD; ++c, k += 128)
+          if (k < K) add(w0[c], k);
+      }
+      for (; k < K; k += 128) add(*reinterpret_cast<const float4 *>(wr + k), k);
+      float v = 0.f;                                                // lane i < 4: row m0 + i
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float t = warp_sum(acc[i]);
+        if (lane == i) v = t;
+      }
+      const float scale = __shfl_sync(0xffffffffu, row_scale, (m0 + lane) & 31);
+      if (lane < 4 && m0 + lane < M) {
+        float *o = out + (size_t)(m0 + lane) * ldo + n;
+        *o = v * scale + (store ? 0.f : n == warp && m0 == 0 ? old : *o);
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------
 // a3: per-head QK-norm, rotary embedding, KV append.
 // ------------------------------------------------------------------------------------
 
-// cos/sin of pos * theta^(-2i/d) for the R positions of this pass, computed in double so
-// that long contexts do not lose angle precision.  table [R][d/2] of (cos, sin).
-__global__ void rope_table_kernel(const int *__restrict__ pos0, int R, int half,
-                                  const double *__restrict__ inv_freq, float2 *__restrict__ table) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= R * half) return;
-  int r = idx / half, i = idx % half;
-  double s, c;
-  sincos((double)(*pos0 + r) * inv_freq[i], &s, &c);
-  table[idx] = make_float2((float)c, (float)s);
+// The table for the R positions of a call that embeds nothing.
+__global__ void rope_table_kernel(const int *__restrict__ pos0, int R, RopeTable T) {
+  rope_entry(T, *pos0, R, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <typename KVT> __device__ __forceinline__ KVT to_kv(float v);
@@ -339,13 +495,40 @@ __global__ void qk_norm_rope_append_kernel(float *__restrict__ qkv, int ldq, int
   }
 }
 
+// Step a3 inside an attention kernel: it reads the raw q | k | v rows of the QKV projection itself; every block
+// normalises and rotates its own query rows and the new K rows that fall into its keys (a few rows, recomputed by the
+// blocks that share them), and the block that owns a position appends its K and V rows to the cache.
+struct AttnFuse {
+  const float *w_qn, *w_kn;        // QK-norm weights [D]
+  const float2 *table;             // (cos, sin) of the pass's positions [R][D / 2]
+  float eps;
+};
+// QK-norm and rotary embedding of one head vector, v[j] = element lane + 32 j.
+template <int D>
+__device__ __forceinline__ void head_norm_rope(const float *w, const float2 *cs_row, float eps, int lane, float (&v)[D / 32]) {
+  constexpr int E = D / 32;
+  float ss = 0.f;
+#pragma unroll
+  for (int j = 0; j < E; ++j) ss += v[j] * v[j];
+  const float inv = rsqrtf(warp_sum(ss) / (float)D + eps);
+#pragma unroll
+  for (int j = 0; j < E; ++j) v[j] = v[j] * inv * w[lane + 32 * j];
+#pragma unroll
+  for (int j = 0; j < E / 2; ++j) {
+    const float2 cs = cs_row[lane + 32 * j];
+    const float a = v[j], b = v[j + E / 2];
+    v[j] = a * cs.x - b * cs.y;
+    v[j + E / 2] = b * cs.x + a * cs.y;
+  }
+}
+
 // ------------------------------------------------------------------------------------
 // a4: split-KV attention.  Each block handles one (sequence, kv head, block of RB new
 // positions, slice of CH keys): the G query heads of that kv head for those positions form
 // up to 16 query rows that share every key/value it reads.  Blocks write unnormalised
 // partial outputs with their running max and sum; attn_merge_kernel combines the slices.
 // ------------------------------------------------------------------------------------
-constexpr int ATTN_WARPS = 4;
+__host__ __device__ constexpr int attn_warps(int T) { return T == 1 ? 8 : 4; }       // warps of an attn_partial_kernel block
 constexpr int ATTN_QR = 16;       // query rows per block
 
 template <typename KVT> __device__ __forceinline__ void load8(const KVT *p, float (&f)[8]);
@@ -374,30 +557,35 @@ template <> __device__ __forceinline__ void load8<__half>(const __half *p, float
   }
 }
 // NQ: query rows the block is compiled for, 4, 8 or 16 (the scores, the probabilities and the outputs of all NQ rows are
-// worked out); the loads of eight keys are in flight at a time.  36 keys of one head, 2 query rows: 27 us with 16 rows
-// and one load at a time.
-template <int D, typename KVT, int NQ>
-__global__ void __launch_bounds__(ATTN_WARPS * 32)
+// worked out).  A warp takes 8 T keys at a time:
+//   T = 1, 8 warps, four lanes to a key: slices of 64 keys.  Bound by the trips to memory that follow one another, so K and V come in one, and
+//   the older keys (previous passes appended them) are requested before the kernel in front is waited for.
+//   T = 4, 4 warps, a lane to a key: longer slices.  Bound by instructions, so one softmax step serves 32 keys.
+// Isolated, 36 keys of one head and 2 query rows took 27 us with 16 rows and one load at a time, 11 us with T = 4 in 8-key
+// loads.  32 x 8192 keys, 8 kv heads of bf16 rows: 234 us with T = 4, 460 with T = 1.
+template <int D, typename KVT, int NQ, bool FUSED, int T>
+__global__ void __launch_bounds__(attn_warps(T) * 32)
 attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restrict__ kc,
                     const KVT *__restrict__ vc, int max_seq, int nq, int nkv, int R, int RB, int CH,
                     const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
-                    float *__restrict__ part_ml, int nsplit) {
-  pdl_enter();
-  constexpr int E = D / 32;
+                    float *__restrict__ part_ml, int nsplit, AttnFuse F) {
+  constexpr int E = D / 32, NC = D / 32, W = attn_warps(T), TK = 8 * T;   // V: dims lane * E ..; K: NC chunks of 8 dims per lane
   const int G = nq / nkv;
   const int split = blockIdx.x, n_rb = (R + RB - 1) / RB;
   const int kvh = blockIdx.y / n_rb, rb = blockIdx.y % n_rb, b = blockIdx.z;
   const int r0 = rb * RB, r1 = min(R, r0 + RB), nQ = (r1 - r0) * G;
+  // the position, and keys before it, are older than the last plainly launched kernel (the rotary table's)
   const int pos0 = pos0_ptr ? *pos0_ptr : pos0_val;
   const int j0 = split * CH, j1 = min(j0 + CH, pos0 + r1);      // keys [j0, j1); last row sees pos0+r1-1
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   __shared__ float q_s[NQ][D];
-  __shared__ float p_s[ATTN_WARPS][NQ][32];
-  __shared__ float red_m[ATTN_WARPS][NQ], red_l[ATTN_WARPS][NQ];
-  extern __shared__ __align__(16) float o_s[];                   // [ATTN_WARPS][NQ][D]
+  __shared__ __align__(16) float p_s[W][NQ][TK];
+  __shared__ float red_m[W][NQ], red_l[W][NQ];
+  extern __shared__ __align__(16) float o_s[];                   // [W][NQ][D]
 
   if (j0 >= j1) {                                                 // empty slice: mark and leave
+    pdl_enter();
     for (int qi = threadIdx.x; qi < nQ; qi += blockDim.x) {
       int r = r0 + qi / G, h = kvh * G + qi % G;
       size_t slot = ((size_t)(b * R + r) * nq + h) * nsplit + split;
@@ -407,20 +595,85 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     return;
   }
   const float scale = rsqrtf((float)D);
-  for (int idx = threadIdx.x; idx < NQ * D; idx += blockDim.x) {
-    int qi = idx / D, dd = idx % D;
-    float v = 0.f;
-    if (qi < nQ) {
-      int r = r0 + qi / G, h = kvh * G + qi % G;
-      v = qkv[(size_t)(b * R + r) * ldq + (size_t)h * D + dd] * scale;
+  const size_t head_off = ((size_t)b * nkv + kvh) * max_seq * D;
+  const KVT *kbase = kc + head_off, *vbase = vc + head_off;
+  KVT *const new_k = reinterpret_cast<KVT *>(o_s + W * NQ * D), *const new_v = new_k + (size_t)R * D;
+  auto k_row = [&](int j) { return FUSED && j >= pos0 ? new_k + (size_t)(j - pos0) * D : kbase + (size_t)j * D; };
+  auto v_row = [&](int j) { return FUSED && j >= pos0 ? new_v + (size_t)(j - pos0) * D : vbase + (size_t)j * D; };
+  float kf[NC][8], vf[8][E];
+  // T = 1: of the keys [jb, jb + 8) those in [lo, hi)
+  auto load_tile = [&](int jb, int lo, int hi) {
+    const int jk = jb + (lane >> 2);
+    if (jk >= lo && jk < hi) {
+      const KVT *k = k_row(jk);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) load8<KVT>(k + (c * 4 + (lane & 3)) * 8, kf[c]);
     }
-    q_s[qi][dd] = v;
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj)
+      if (jb + jj >= lo && jb + jj < hi) {
+        const KVT *v = v_row(jb + jj);
+#pragma unroll
+        for (int e = 0; e < E; ++e) vf[jj][e] = (float)v[lane * E + e];
+      }
+  };
+  if (T == 1) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) kf[c][e] = 0.f;
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj)
+#pragma unroll
+      for (int e = 0; e < E; ++e) vf[jj][e] = 0.f;
+    load_tile(j0 + warp * TK, j0, min(j1, pos0));
+  }
+  pdl_enter();
+
+  if (FUSED) {
+    // step a3 (see AttnFuse): the pass's rows r_lo .. r_hi - 1 sit at positions inside this slice
+    const int r_lo = max(0, j0 - pos0), r_hi = min(r1, j1 - pos0);
+    const int n_kv = 2 * max(0, r_hi - r_lo);
+    for (int task = warp; task < n_kv + NQ; task += W) {
+      const bool is_q = task >= n_kv;
+      const int qi = task - n_kv, r = is_q ? r0 + qi / G : r_lo + (task >> 1), is_v = !is_q && (task & 1);
+      float v[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = 0.f;
+      if (!is_q || qi < nQ) {
+        const int head = is_q ? kvh * G + qi % G : nq + (is_v ? nkv : 0) + kvh;
+        const float *src = qkv + (size_t)(b * R + r) * ldq + (size_t)head * D;
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = src[lane + 32 * e];
+        if (!is_v) head_norm_rope<D>(is_q ? F.w_qn : F.w_kn, F.table + (size_t)r * (D / 2), F.eps, lane, v);
+      }
+      if (is_q) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) q_s[qi][lane + 32 * e] = v[e] * scale;
+      } else {
+        KVT *cache = const_cast<KVT *>(is_v ? vbase : kbase) + (size_t)(pos0 + r) * D;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const KVT h = to_kv<KVT>(v[e]);
+          (is_v ? new_v : new_k)[(size_t)r * D + lane + 32 * e] = h;
+          if (r >= r0) cache[lane + 32 * e] = h;         // the row block that owns the position appends it
+        }
+      }
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < NQ * D; idx += blockDim.x) {
+      int qi = idx / D, dd = idx % D;
+      float v = 0.f;
+      if (qi < nQ) {
+        int r = r0 + qi / G, h = kvh * G + qi % G;
+        v = qkv[(size_t)(b * R + r) * ldq + (size_t)h * D + dd] * scale;
+      }
+      q_s[qi][dd] = v;
+    }
   }
   __syncthreads();
 
-  const KVT *kbase = kc + ((size_t)b * nkv + kvh) * max_seq * D;
-  const KVT *vbase = vc + ((size_t)b * nkv + kvh) * max_seq * D;
-  float m_run[NQ], l_run[NQ], o_acc[NQ][E];
+  float m_run[NQ], l_run[NQ], o_acc[NQ][E];                       // l_run: of this lane's own keys
 #pragma unroll
   for (int qi = 0; qi < NQ; ++qi) {
     m_run[qi] = -INFINITY; l_run[qi] = 0.f;
@@ -428,69 +681,88 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     for (int e = 0; e < E; ++e) o_acc[qi][e] = 0.f;
   }
 
-  for (int jb = j0 + warp * 32; jb < j1; jb += ATTN_WARPS * 32) {
-    const int j = jb + lane;
+  for (int jb = j0 + warp * TK; jb < j1; jb += W * TK) {
     float s[NQ];
+    auto dot8 = [](const float (&k)[8], const float *q) {
+      const float4 a = *reinterpret_cast<const float4 *>(q), b = *reinterpret_cast<const float4 *>(q + 4);
+      return k[0] * a.x + k[1] * a.y + k[2] * a.z + k[3] * a.w + k[4] * b.x + k[5] * b.y + k[6] * b.z + k[7] * b.w;
+    };
+    if constexpr (T == 1) {
+      if (jb != j0 + warp * TK) load_tile(jb, j0, min(j1, pos0));
+      if (jb + TK > pos0) load_tile(jb, pos0, j1);                // keys of this pass
 #pragma unroll
-    for (int qi = 0; qi < NQ; ++qi) s[qi] = 0.f;
-    if (j < j1) {
-      const KVT *kr = kbase + (size_t)j * D;
+      for (int qi = 0; qi < NQ; ++qi) {
+        s[qi] = 0.f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[qi] += dot8(kf[c], &q_s[qi][(c * 4 + (lane & 3)) * 8]);
+        s[qi] += __shfl_xor_sync(0xffffffffu, s[qi], 1);
+        s[qi] += __shfl_xor_sync(0xffffffffu, s[qi], 2);
+      }
+    } else {
+      const KVT *k = k_row(min(jb + lane, j1 - 1));
+#pragma unroll
+      for (int qi = 0; qi < NQ; ++qi) s[qi] = 0.f;
 #pragma unroll 4
       for (int c = 0; c < D / 8; ++c) {
-        float kf[8];
-        load8<KVT>(kr + c * 8, kf);
+        float kr[8];
+        load8<KVT>(k + c * 8, kr);
 #pragma unroll
-        for (int qi = 0; qi < NQ; ++qi) {
-          const float4 qa = *reinterpret_cast<const float4 *>(&q_s[qi][c * 8]);
-          const float4 qb = *reinterpret_cast<const float4 *>(&q_s[qi][c * 8 + 4]);
-          s[qi] += kf[0] * qa.x + kf[1] * qa.y + kf[2] * qa.z + kf[3] * qa.w + kf[4] * qb.x +
-                   kf[5] * qb.y + kf[6] * qb.z + kf[7] * qb.w;
-        }
+        for (int qi = 0; qi < NQ; ++qi) s[qi] += dot8(kr, &q_s[qi][c * 8]);
       }
     }
+    const int jt = T == 1 ? lane >> 2 : lane, j = jb + jt;
 #pragma unroll
     for (int qi = 0; qi < NQ; ++qi) {
       if (qi < nQ) {                                  // uniform across the warp
         const int pos = pos0 + r0 + qi / G;
-        const bool ok = (j < j1) && (j <= pos);
-        const float sv = ok ? s[qi] : -INFINITY;
-        const float m_new = fmaxf(m_run[qi], warp_max(sv));
+        const bool ok = j < j1 && j <= pos;
+        float mx = ok ? s[qi] : -INFINITY;
+#pragma unroll
+        for (int x = T == 1 ? 4 : 1; x < 32; x <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+        const float m_new = fmaxf(m_run[qi], mx);
         float p = 0.f, corr = 1.f;
         if (m_new > -INFINITY) {
           corr = __expf(m_run[qi] - m_new);           // exp(-inf) = 0 on the first block
-          p = ok ? __expf(sv - m_new) : 0.f;
+          p = ok ? __expf(s[qi] - m_new) : 0.f;
         }
-        l_run[qi] = l_run[qi] * corr + warp_sum(p);
+        l_run[qi] = l_run[qi] * corr + p;
         m_run[qi] = m_new;
 #pragma unroll
         for (int e = 0; e < E; ++e) o_acc[qi][e] *= corr;
-        p_s[warp][qi][lane] = p;
+        if (T > 1 || (lane & 3) == 0) p_s[warp][qi][jt] = p;
       }
     }
     __syncwarp();
-    const int n_here = min(32, j1 - jb);
+    const int n_here = min(TK, j1 - jb);
+#pragma unroll 1
     for (int j8 = 0; j8 < n_here; j8 += 8) {
-      float vf[8][E];
+      if (T > 1) {
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj) {                  // past the last key: its row again, with probability 0
-        const KVT *vr = vbase + (size_t)(jb + min(j8 + jj, n_here - 1)) * D + lane * E;
+        for (int jj = 0; jj < 8; ++jj) {                          // past the last key: its row again, with probability 0
+          const KVT *vr = v_row(jb + min(j8 + jj, n_here - 1)) + lane * E;
 #pragma unroll
-        for (int e = 0; e < E; ++e) vf[jj][e] = (float)vr[e];
+          for (int e = 0; e < E; ++e) vf[jj][e] = (float)vr[e];
+        }
       }
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) {
         if (qi < nQ) {
+          float p[8];
+          *reinterpret_cast<float4 *>(p) = *reinterpret_cast<const float4 *>(&p_s[warp][qi][j8]);
+          *reinterpret_cast<float4 *>(p + 4) = *reinterpret_cast<const float4 *>(&p_s[warp][qi][j8 + 4]);
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            const float p = p_s[warp][qi][j8 + jj];
+          for (int jj = 0; jj < 8; ++jj)
 #pragma unroll
-            for (int e = 0; e < E; ++e) o_acc[qi][e] += p * vf[jj][e];
-          }
+            for (int e = 0; e < E; ++e) o_acc[qi][e] += p[jj] * vf[jj][e];
         }
       }
     }
     __syncwarp();
   }
+#pragma unroll
+  for (int qi = 0; qi < NQ; ++qi)
+#pragma unroll
+    for (int x = T == 1 ? 4 : 1; x < 32; x <<= 1) l_run[qi] += __shfl_xor_sync(0xffffffffu, l_run[qi], x);
 
   // combine the warps of the block
 #pragma unroll
@@ -504,10 +776,10 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
     int qi = idx / D, dd = idx % D;
     float m = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < ATTN_WARPS; ++w) m = fmaxf(m, red_m[w][qi]);
+    for (int w = 0; w < W; ++w) m = fmaxf(m, red_m[w][qi]);
     float l = 0.f, o = 0.f;
 #pragma unroll
-    for (int w = 0; w < ATTN_WARPS; ++w) {
+    for (int w = 0; w < W; ++w) {
       float f = red_m[w][qi] > -INFINITY ? __expf(red_m[w][qi] - m) : 0.f;
       l += red_l[w][qi] * f;
       o += o_s[((size_t)w * NQ + qi) * D + dd] * f;
@@ -614,10 +886,10 @@ __global__ void masked_select_kernel(float *__restrict__ x, const float *__restr
 
 // ------------------------------------------------------------------------------------
 // a9 (second half): greedy pick, lowest index on ties; a10: feed the token back.
-// Two levels: ARGMAX_SLICES blocks per sequence each find the best of their slice of the
-// vocabulary, then one block per sequence picks among them.  The token goes to position
-// n_known of the token buffer unless a forced token already sits there (teacher forcing), and
-// to out_argmax if given.
+// ARGMAX_SLICES blocks per sequence each find the best of their slice of the vocabulary; the last of them to arrive
+// picks among the slices, and the last of all advances the schedule's counters: one launch where a block of its own for
+// each step took three.  The token goes to position n_known of the token buffer unless a forced token already sits
+// there (teacher forcing), and to out_argmax if given.
 // ------------------------------------------------------------------------------------
 constexpr int ARGMAX_SLICES = 64;       // 151 936 logits of one sequence: 10 us with 16 slices
 
@@ -635,9 +907,34 @@ __device__ __forceinline__ void argmax_block_reduce(float best, int bi, float *s
   }
 }
 
+// a0: schedule counters after a pass (Section 2.2).  kind: 0 = prefill of P rows, 1 = full
+// pass, 2 = decoding-layers-only pass.
+__device__ __forceinline__ void advance_state(DevState *st, int kind, int P) {
+  if (kind == 0) {
+    st->n_known = P + 1; st->lo_len = P; st->up_len = P; st->cycle = 1;
+    st->slot = 1 % st->tau; st->n_emitted = 1;
+  } else {
+    if (kind == 1) { st->lo_len = st->n_known; st->cycle += 1; }
+    st->up_len = st->n_known;
+    st->n_known += 1;
+    st->slot = (st->slot + 1) % st->tau;
+    st->n_emitted += 1;
+  }
+  st->newest = st->n_known - 1;
+}
+
+struct PickParams {
+  float *part_val;                // [sequences][ARGMAX_SLICES]
+  int *part_idx;
+  unsigned int *arrived;          // [sequences + 1], zero between launches
+  int *tokens;                    // null: the position holds its token already
+  int max_seq;
+  int *out_argmax;                // may be null
+  int kind, P;                    // for advance_state
+};
+
 // grid (sequences, ARGMAX_SLICES), 256 threads
-__global__ void argmax_slices_kernel(const float *__restrict__ logits, int ldl, int V, float *__restrict__ part_val,
-                                     int *__restrict__ part_idx, const DevState *__restrict__ st, SampleParams sp) {
+__global__ void argmax_kernel(const float *__restrict__ logits, int ldl, int V, DevState *st, SampleParams sp, PickParams pp) {
   pdl_enter();
   const int b = blockIdx.x, per = ((V + gridDim.y - 1) / gridDim.y + 3) & ~3;      // whole 16-byte loads
   const int i0 = blockIdx.y * per, i1 = min(V, i0 + per);
@@ -673,51 +970,31 @@ __global__ void argmax_slices_kernel(const float *__restrict__ logits, int ldl, 
   __shared__ float sv[256];
   __shared__ int si[256];
   argmax_block_reduce(best, bi, sv, si);
+  __shared__ bool last;
   if (threadIdx.x == 0) {
-    part_val[b * gridDim.y + blockIdx.y] = sv[0];
-    part_idx[b * gridDim.y + blockIdx.y] = si[0];
+    pp.part_val[b * gridDim.y + blockIdx.y] = sv[0];
+    pp.part_idx[b * gridDim.y + blockIdx.y] = si[0];
+    __threadfence();                                  // this block's pair, and its read of n_known, before its arrival
+    last = atomicInc(&pp.arrived[b], gridDim.y - 1) == gridDim.y - 1;
+    __threadfence();
   }
-}
-
-// grid (sequences), 32 threads
-__global__ void argmax_pick_kernel(const float *__restrict__ part_val, const int *__restrict__ part_idx, int n_slices,
-                                   int *__restrict__ tokens, int max_seq, const DevState *__restrict__ st, int write_token,
-                                   int *__restrict__ out_argmax) {
-  pdl_enter();
-  const int b = blockIdx.x;
-  float best = -INFINITY;
-  int bi = 0x7fffffff;
-  for (int i = threadIdx.x; i < n_slices; i += blockDim.x) {
-    float v = part_val[b * n_slices + i];
-    int ix = part_idx[b * n_slices + i];
+  __syncthreads();
+  if (!last) return;
+  best = -INFINITY;
+  bi = 0x7fffffff;
+  for (int i = threadIdx.x; i < gridDim.y; i += blockDim.x) {
+    const float v = __ldcg(&pp.part_val[b * gridDim.y + i]);
+    const int ix = __ldcg(&pp.part_idx[b * gridDim.y + i]);
     if (v > best || (v == best && ix < bi)) { best = v; bi = ix; }
   }
-  __shared__ float sv[32];
-  __shared__ int si[32];
   argmax_block_reduce(best, bi, sv, si);
   if (threadIdx.x == 0) {
-    int pick = si[0] == 0x7fffffff ? 0 : si[0];
-    if (write_token) tokens[(size_t)b * max_seq + st->n_known] = pick;
-    if (out_argmax) out_argmax[b] = pick;
+    const int pick = si[0] == 0x7fffffff ? 0 : si[0];
+    if (pp.tokens) pp.tokens[(size_t)b * pp.max_seq + position] = pick;
+    if (pp.out_argmax) pp.out_argmax[b] = pick;
+    __threadfence();
+    if (atomicInc(&pp.arrived[gridDim.x], gridDim.x - 1) == gridDim.x - 1) advance_state(st, pp.kind, pp.P);
   }
-}
-
-// a0: schedule counters after a pass (Section 2.2).  kind: 0 = prefill of P rows, 1 = full
-// pass, 2 = decoding-layers-only pass.
-__global__ void advance_state_kernel(DevState *st, int kind, int P) {
-  pdl_enter();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (kind == 0) {
-    st->n_known = P + 1; st->lo_len = P; st->up_len = P; st->cycle = 1;
-    st->slot = 1 % st->tau; st->n_emitted = 1;
-  } else {
-    if (kind == 1) { st->lo_len = st->n_known; st->cycle += 1; }
-    st->up_len = st->n_known;
-    st->n_known += 1;
-    st->slot = (st->slot + 1) % st->tau;
-    st->n_emitted += 1;
-  }
-  st->newest = st->n_known - 1;
 }
 
 __global__ void set_int_kernel(int *p, int v) { *p = v; }

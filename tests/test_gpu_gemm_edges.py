@@ -72,3 +72,27 @@ def test_gated_epilogue(dmtd, intermediate, n):
     eng = dmtd.Dmtd(shape, to_cuda(w), L_d=1, tau=2, max_batch=1, max_seq=n + 2, kv_dtype="f32")
     got = eng.masked_forward(torch.from_numpy(tokens).cuda(), 5).double().cpu().numpy()
     assert np.abs(got[0] - ref).max() < 1e-3
+
+
+@pytest.mark.parametrize("head_dim,B,tau,P", [
+    (64, 1, 1, 1),          # one row
+    (64, 4, 1, 130),        # full groups of 4 rows, key slices that end inside the new rows
+    (64, 3, 5, 61),         # 15 rows in the lower layers, 3 in the upper ones
+    (64, 16, 1, 9),         # the most rows
+    (64, 17, 1, 9),         # one more: the separate kernels
+    (64, 1, 15, 9),         # the most new positions of a sequence
+    (64, 1, 16, 9),         # one more: step a3 as a launch of its own
+    (128, 5, 3, 33),
+])
+def test_f32_decode_rows(dmtd, head_dim, B, tau, P):
+    """fp32 weights: projections together with the step in front of them, and the separate kernels past their limits."""
+    shape = SHAPES["tiny"].with_(head_dim=head_dim, hidden=260, intermediate=776, vocab=1003, n_layers=4)
+    w = make_weights(shape, seed=0, norm_jitter=0.1)
+    prompts = make_prompts(shape.vocab, B, P, seed=1).numpy()
+    forced = make_prompts(shape.vocab, B, 2 * tau + 2, seed=2).numpy()
+    ref_logits, ref_am, o = oracle_forced(shape, w, 2, tau, prompts, forced)
+    eng = dmtd.Dmtd(shape, to_cuda(w), L_d=2, tau=tau, max_batch=B, max_seq=P + forced.shape[1] + 1, kv_dtype="f32")
+    got_logits, got_am = gpu_forced(eng, prompts, forced)
+    err, _ = check_logits(got_logits, ref_logits, got_am, ref_am)
+    assert err < 1e-3       # as above; fp32 sums of fp32 products
+    assert eng.device_state() == o.state()

@@ -483,10 +483,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   }
 }
 
-// Activations [rows][lda] fp32 -> bf16 hi/lo units in the order of ActTiles.  One thread per unit: 8 values of k of a
-// row, both parts; neighbouring threads take neighbouring rows (consecutive 16-byte stores, 32-byte reads).
-// With `gated` the source rows hold gate and up values in turn and the activation is the SwiGLU gate silu(gate) * up
-// (step a6, second half), computed on the way; the source's first column then belongs to k block kb0.
+// 8 values of k of an activation row as its hi and lo units.
 __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, size_t lo_offset) {
   uint32_t hi[4], lo[4];
 #pragma unroll
@@ -498,30 +495,81 @@ __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, siz
   dst[lo_offset] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
-__global__ void act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T, uint4 *__restrict__ blocks,
-                                  int gated, int kb0) {
+// Activations [rows][lda] fp32 -> bf16 hi/lo units (8 values of k of a row, 16 bytes a part) in the order of ActTiles.
+// With GATED the source rows hold gate and up values in turn and the activation is the SwiGLU gate silu(gate) * up
+// (step a6, second half), computed on the way; the source's first column then belongs to k block kb0.
+// A warp takes a k block of four rows at a time: it reads whole rows of it (512 bytes in a row; every load in flight
+// before the first is used), and the lanes exchange their parts so that each stores a unit beside its neighbour row's.
+// No shared memory, so that the blocks become resident beside the GEMM in front.
+// Bound by the time of one trip to memory behind the next projection's first weights, which its blocks
+// request meanwhile: with a thread to a unit (its lanes' loads 32 rows apart, 16 bytes each) a block took 13.6 us at
+// 96 rows of the Qwen3-4B shape and 6 us at 32 (4 cycles of 32 sequences 21.3 ms, 20.3 so).
+constexpr int AB_ROWS = 4, AB_THREADS = 256;
+template <bool GATED>
+__global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T,
+                                                                uint4 *__restrict__ blocks, int kb0) {
+  // lanes of a row, 16-byte loads of a lane, and 32-bit registers of a part that a load becomes
+  constexpr int LANES = GATED ? 32 : 16, LOADS = AB_ROWS * LANES / 32, REGS = GATED ? 1 : 2;
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int total = (T.n_kb - kb0) * 8 * rows;
-  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
-    const int m = u % rows, kc = u / rows;
-    const float4 *src = reinterpret_cast<const float4 *>(act + (size_t)m * lda + (size_t)kc * (gated ? 16 : 8));
-    float f[8];
-    if (gated) {
+  const int lane = threadIdx.x & 31, col = lane % LANES, half = lane / LANES;
+  const int row_tiles = (rows + AB_ROWS - 1) / AB_ROWS, n_tiles = (T.n_kb - kb0) * row_tiles;
+  for (int tile = blockIdx.x * (AB_THREADS / 32) + (threadIdx.x >> 5); tile < n_tiles; tile += gridDim.x * (AB_THREADS / 32)) {
+    const int kb = tile / row_tiles, m0 = (tile % row_tiles) * AB_ROWS;
+    float4 v[LOADS];                                                 // load i: row m0 + i (32 / LANES) + half
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 v = src[j];
-        f[2 * j] = v.x / (1.f + expf(-v.x)) * v.y;
-        f[2 * j + 1] = v.z / (1.f + expf(-v.z)) * v.w;
-      }
-    } else {
-      const float4 a = src[0], b = src[1];
-      f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+    for (int i = 0; i < LOADS; ++i) {
+      const int m = m0 + i * (32 / LANES) + half;
+      v[i] = m < rows ? *reinterpret_cast<const float4 *>(act + (size_t)m * lda + (size_t)kb * LANES * 4 + col * 4)
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    store_hi_lo(f, blocks + T.unit(m, kb0 + (kc >> 3), kc & 7), T.lo_offset());
+    uint32_t hi[LOADS][REGS], lo[LOADS][REGS];
+    auto split = [](float a, float b, uint32_t &h, uint32_t &l) {
+      h = pack_bf16x2(a, b);
+      l = pack_bf16x2(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xffff0000u));
+    };
+#pragma unroll
+    for (int i = 0; i < LOADS; ++i) {
+      if (GATED) {
+        split(v[i].x / (1.f + expf(-v[i].x)) * v[i].y, v[i].z / (1.f + expf(-v[i].z)) * v[i].w, hi[i][0], lo[i][0]);
+      } else {
+        split(v[i].x, v[i].y, hi[i][0], lo[i][0]);
+        split(v[i].z, v[i].w, hi[i][REGS - 1], lo[i][REGS - 1]);
+      }
+    }
+    // the LOADS lanes of a unit hold a LOADS-th of it for each of LOADS rows: transposed, lane q of them holds row q's unit
+    auto transpose = [&](uint32_t (&x)[LOADS][REGS]) {
+#pragma unroll
+      for (int step = 1; step < LOADS; step <<= 1) {
+        const bool up = lane & step;
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i)
+          if (!(i & step)) {
+#pragma unroll
+            for (int r = 0; r < REGS; ++r) {
+              const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? x[i][r] : x[i + step][r], step);
+              if (up) x[i][r] = got;
+              else x[i + step][r] = got;
+            }
+          }
+      }
+    };
+    transpose(hi);
+    transpose(lo);
+    const int q = col & (LOADS - 1), m = m0 + q * (32 / LANES) + half;
+    if (m < rows) {
+      uint4 *dst = blocks + T.unit(m, kb0 + kb, col / LOADS);
+      if (GATED) {
+        dst[0] = make_uint4(hi[0][0], hi[1 % LOADS][0], hi[2 % LOADS][0], hi[3 % LOADS][0]);
+        dst[T.lo_offset()] = make_uint4(lo[0][0], lo[1 % LOADS][0], lo[2 % LOADS][0], lo[3 % LOADS][0]);
+      } else {
+        dst[0] = make_uint4(hi[0][0], hi[0][REGS - 1], hi[1][0], hi[1][REGS - 1]);
+        dst[T.lo_offset()] = make_uint4(lo[0][0], lo[0][REGS - 1], lo[1][0], lo[1][REGS - 1]);
+      }
+    }
   }
 }
 

@@ -96,3 +96,24 @@ def test_f32_decode_rows(dmtd, head_dim, B, tau, P):
     err, _ = check_logits(got_logits, ref_logits, got_am, ref_am)
     assert err < 1e-3       # as above; fp32 sums of fp32 products
     assert eng.device_state() == o.state()
+
+
+@pytest.mark.parametrize("B", [1, 3, 5, 33])
+def test_rows_from_unmerged_slices(dmtd, B):
+    """Captured passes launch the key slices of the whole cache: more than the O projection's activation blocks merge
+    on the way, so its rows come from a merge of their own (1 to 66 rows a pass)."""
+    shape = SHAPE.with_(n_layers=2, hidden=256, n_q_heads=16, n_kv_heads=4, head_dim=64)
+    w = make_weights(shape, seed=0, norm_jitter=0.1)
+    prompts = make_prompts(shape.vocab, B, 9, seed=1).numpy()
+    eng = dmtd.Dmtd(shape, to_cuda(w), L_d=1, tau=2, max_batch=B, max_seq=41 * 64, kv_dtype="f32")
+    eng.set_option("fused_pass", 0)
+    tokens = [eng.prefill(torch.from_numpy(prompts).cuda())[0][:, None]]
+    for _ in range(3):
+        rc, n, out = eng.decode_cycle(2)
+        tokens.append(out[:, :n].clone())
+    forced = torch.cat(tokens, 1).cpu().numpy()
+    ref_logits, ref_am, _ = oracle_forced(shape, w, 1, 2, prompts, forced)
+    srt = np.sort(ref_logits, -1)
+    clear = srt[..., -1] - srt[..., -2] > 2e-3       # logits within 1e-3, as above: picks may differ below twice that
+    assert clear.mean() > 0.8
+    assert (forced.T == ref_am)[clear].all()

@@ -348,7 +348,7 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   // as many stages as shared memory holds, two accumulators where tensor memory does.  (Half of both for decode launches,
   // so that the next projection's blocks become resident beside this one's and fetch their first weights, was no
   // faster at 8-32 rows and slower at 96: fewer stages are in flight while a launch streams.)
-  const int n_cols = P.T.split ? 2 * P.T.tile_rows : P.T.tile_rows, stage_bytes = TG_WBLOCK + P.T.tile_rows * 128;
+  const int n_cols = P.T.split ? 2 * P.T.tile_rows : P.T.tile_rows, stage_bytes = tg_stage_units(P.T.split) * (TG_WBLOCK + P.T.tile_rows * 128);
   P.stages = std::max(2, std::min(TG_MAX_STAGES, (TG_MAX_SMEM - TG_TAIL_BYTES) / stage_bytes));
   if (c->gemm_stages >= 2) P.stages = std::min(P.stages, c->gemm_stages);
   int cols = 32;

@@ -16,7 +16,7 @@
 //
 // Both operands are K-major in shared memory in the interleaved (no swizzle) canonical form: 8 rows x 16 bytes per
 // core matrix.  The weights are stored in global memory in exactly that order (16 KiB blocks, one per 128-row tile and
-// k block), the activations are written that way by the kernels below, so a pipeline stage is two bulk copies.
+// k block), the activations are written that way by the kernels below, so a pipeline stage is a few bulk copies.
 //
 // Persistent: one pair of blocks per two SMs.  The units of a launch (row-tile pairs x column tiles x k blocks) are cut
 // into equal shares whatever the shape is: the row-tile pairs that are not a multiple of the block pairs (all of them,
@@ -46,10 +46,14 @@ constexpr int TG_EPI_WARPS = 8;              // epilogue warps: two per quarter 
 constexpr int TG_THREADS = 64 + 32 * TG_EPI_WARPS;
 constexpr int TG_MAX_STAGES = 8;             // most pipeline stages of a block
 constexpr int TG_ROWS = 128;                 // weight rows per tile; a pair of blocks takes two tiles (MMA M = 256)
-constexpr int TG_KB = 64;                    // k per pipeline stage: four MMAs of K = 16 (per part)
+constexpr int TG_KB = 64;                    // k per unit: four MMAs of K = 16 (per part)
 constexpr int TG_WBLOCK = TG_ROWS * TG_KB * 2;      // 16384 bytes
 constexpr int TG_SPLIT_ROWS = 128;           // most rows of a column tile with hi and lo in columns of their own
 constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
+// k blocks of a pipeline stage.  Up to 128 rows: two; a stage costs its waits, its commit and its copies' issue whatever it
+// holds (4 cycles of 32 sequences of the Qwen3-4B shape: 20.26 ms with one, 20.12 with two).  More rows: one, the
+// activations of a stage are 32 KiB there.
+__host__ __device__ constexpr int tg_stage_units(bool split) { return split ? 2 : 1; }
 constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
 constexpr int TG_MAX_SMEM = 226 * 1024;      // dynamic shared memory of a block: it has its SM to itself
 enum { TG_ERR_WAIT = 4 };
@@ -184,12 +188,14 @@ struct TgCursor {
   int kb, ct, rt;            // k block, column tile, row-tile pair
   int left;                  // units left of the line; then 0
   int step;                  // row-tile pairs from one tile row to the next
-  __device__ __forceinline__ void next(int n_kb, int n_ct, int pair, int n_pairs) {
-    if (left > 0 && --left == 0) {
+  // units of the next stage: whole tiles and the line's parts end where a stage ends
+  __device__ __forceinline__ int units(int n_kb, int most) const { return min(min(most, n_kb - kb), left > 0 ? left : most); }
+  __device__ __forceinline__ void next(int n, int n_kb, int n_ct, int pair, int n_pairs) {
+    if (left > 0 && (left -= n) == 0) {
       kb = 0; ct = 0; rt = pair; step = n_pairs;
       return;
     }
-    if (++kb == n_kb) {
+    if ((kb += n) == n_kb) {
       kb = 0;
       if (++ct == n_ct) { ct = 0; rt += step; }
     }
@@ -241,7 +247,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int S = P.stages, n_kb = P.W.n_kb, tile_rows = P.T.tile_rows;
-  const uint32_t act_bytes = (uint32_t)tile_rows * 128, stage_bytes = TG_WBLOCK + act_bytes;
+  constexpr int KPS = tg_stage_units(SPLIT);
+  const uint32_t act_bytes = (uint32_t)tile_rows * 128, act_off = KPS * TG_WBLOCK, stage_bytes = act_off + KPS * act_bytes;
   unsigned char *const tail = tg_smem + (size_t)S * stage_bytes;
   const uint32_t full0 = smem_u32(tail), empty0 = full0 + 8 * TG_MAX_STAGES, acc_full0 = empty0 + 8 * TG_MAX_STAGES,
                  acc_empty0 = acc_full0 + 16;
@@ -265,17 +272,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   // can then request its first weight blocks while this grid's last blocks finish
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   TgCursor cur_w = start, cur_a = start;               // producer's positions (thread 0)
-  auto copy_w = [&](int st) {
+  auto copy_w = [&](int st, int n) {                   // the k blocks of a row tile follow one another
     bulk_g2s(smem_u32(tg_smem) + st * stage_bytes, P.W.w + ((size_t)(2 * cur_w.rt + rank) * n_kb + cur_w.kb) * (TG_WBLOCK / 16),
-             TG_WBLOCK, full0 + st * 8);
-    cur_w.next(n_kb, n_ct, pair, n_pairs);
+             n * TG_WBLOCK, full0 + st * 8);
+    cur_w.next(n, n_kb, n_ct, pair, n_pairs);
   };
-  auto copy_act = [&](int st) {
-    bulk_g2s(smem_u32(tg_smem) + st * stage_bytes + TG_WBLOCK,
-             P.act_blocks + (((size_t)cur_a.ct * n_kb + cur_a.kb) * 2 + rank) * P.T.units_per_sm(), act_bytes, full0 + st * 8);
-    cur_a.next(n_kb, n_ct, pair, n_pairs);
+  auto copy_act = [&](int st, int n) {
+    for (int u = 0; u < n; ++u)
+      bulk_g2s(smem_u32(tg_smem) + st * stage_bytes + act_off + u * act_bytes,
+               P.act_blocks + (((size_t)cur_a.ct * n_kb + cur_a.kb + u) * 2 + rank) * P.T.units_per_sm(), act_bytes, full0 + st * 8);
+    cur_a.next(n, n_kb, n_ct, pair, n_pairs);
   };
-  const int n_first = min(S, n_it);
+  int n_first = 0, issued_units = 0;                   // (thread 0) the stages requested before the activations are there
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full0 + s * 8, rank == 0 ? 2 : 1);       // this block's copies; on the first SM also the other's
@@ -298,9 +306,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   if (threadIdx.x == 0) {
     // the weight blocks of the first stages are requested before the other block is waited for: they touch this
     // block's barriers only, and eight copies take the issuing thread some thousand cycles
-    for (int i = 0; i < n_first; ++i) {
-      mbar_expect_tx(full0 + i * 8, stage_bytes);
-      copy_w(i);
+    for (; n_first < S && issued_units < n_it; ++n_first) {
+      const int n = cur_w.units(n_kb, KPS);
+      mbar_expect_tx(full0 + n_first * 8, n * (TG_WBLOCK + act_bytes));
+      copy_w(n_first, n);
+      issued_units += n;
     }
   }
   __syncwarp();
@@ -311,19 +321,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---- producer: two bulk copies per unit; the activation blocks only after the kernel that writes them has
+      // ---- producer: a bulk copy for a stage's weights and one for each unit's activations; the activation blocks only after the kernel that writes them has
       // completed and its writes are visible
       asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (int i = 0; i < n_first; ++i) copy_act(i);
+      for (int i = 0; i < n_first; ++i) copy_act(i, cur_a.units(n_kb, KPS));
       int st = 0, issued = n_first;
       uint32_t ph = 0;
       bool ok = true;
-      for (int i = n_first; i < n_it; ++i) {
+      while (issued_units < n_it) {
         ok = tg_wait(empty0 + st * 8, ph, P);
         if (!ok) break;
-        mbar_expect_tx(full0 + st * 8, stage_bytes);
-        copy_w(st);
-        copy_act(st);
+        const int n = cur_w.units(n_kb, KPS);
+        mbar_expect_tx(full0 + st * 8, n * (TG_WBLOCK + act_bytes));
+        copy_w(st, n);
+        copy_act(st, n);
+        issued_units += n;
         ++issued;
         if (++st == S) { st = 0; ph ^= 1; }
       }
@@ -340,44 +352,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     // ---- MMA issuer
     const int n_cols = SPLIT ? 2 * tile_rows : tile_rows;         // MMA N
     const uint32_t idesc = umma_instr_desc(2 * TG_ROWS, n_cols);
-    const uint32_t b_lbo = (uint32_t)(n_cols / 2) * 16, part_bytes = b_lbo * 8;
-    int kb = start.kb, st = 0, acc = 0;
-    uint32_t ph = 0, acc_ph = 1;                                      // the accumulators start free
+    const uint32_t b_lbo = (uint32_t)(n_cols / 2) * 16;
+    // what a unit costs is instructions in a row, so the descriptors and barriers of the stage are carried along
+    const uint64_t da0 = umma_smem_desc(smem_u32(tg_smem), (TG_ROWS / 8) * 128, 128),
+                   db0 = umma_smem_desc(smem_u32(tg_smem) + act_off, b_lbo, 128);
+    const uint64_t da_step = 2 * (TG_ROWS / 8) * 128 / 16, db_step = 2 * b_lbo / 16, part_step = b_lbo * 8 / 16;
+    const uint32_t st_step = stage_bytes / 16, full_end = full0 + 8 * S;
+    uint64_t da_st = da0, db_st = db0;
+    uint32_t full = full0, ph = 0, acc_ph = 1, d = tmem;              // the accumulators start free
+    int kb = start.kb, acc = 0;
     bool first = true, ok = true;
-    for (int i = 0; i < n_it; ++i) {
+    for (int i = 0; i < n_it;) {
       if (first) {
         ok = __all_sync(0xffffffffu, tg_wait(acc_empty0 + acc * 8, acc_ph, P));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      ok = __all_sync(0xffffffffu, tg_wait(full0 + st * 8, ph, P));
+      ok = __all_sync(0xffffffffu, mbar_try_wait(full, ph)) || __all_sync(0xffffffffu, tg_wait_slow(full, ph, P));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const bool last = ++kb == n_kb || i + 1 == n_part;
+      const int n = min(min(KPS, n_kb - kb), i < n_part ? n_part - i : KPS);
+      kb += n;
+      i += n;
+      const bool last = kb == n_kb || i == n_part;
       if (elect_one()) {
-        const uint32_t a_base = smem_u32(tg_smem) + st * stage_bytes, b_base = a_base + TG_WBLOCK;
-        const uint32_t d = tmem + acc * acc_cols;
-        uint64_t da = umma_smem_desc(a_base, (TG_ROWS / 8) * 128, 128), db = umma_smem_desc(b_base, b_lbo, 128);
-        const uint64_t da_step = 2 * (TG_ROWS / 8) * 128 / 16, db_step = 2 * b_lbo / 16, part_step = part_bytes / 16;
-        uint32_t accumulate = first ? 0u : 1u;
+        const uint32_t accumulate = first ? 0u : 1u;
 #pragma unroll
-        for (int kk = 0; kk < TG_KB / 16; ++kk) {
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-              "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-              : "memory");
-          accumulate = 1u;
-          if (!SPLIT)                                             // the lo part into the same columns
+        for (int u = 0; u < KPS; ++u) {
+          if (u && n == 1) break;
+          const uint64_t da = da_st + u * (TG_WBLOCK / 16), db = db_st + u * (act_bytes / 16);
+#pragma unroll
+          for (int kk = 0; kk < TG_KB / 16; ++kk) {
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                 " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                "l"(da), "l"(db + part_step), "r"(idesc), "r"(1u)
+                "l"(da + kk * da_step), "l"(db + kk * db_step), "r"(idesc), "r"(u || kk ? 1u : accumulate)
                 : "memory");
-          da += da_step;
-          db += db_step;
+            if (!SPLIT)                                           // the lo part into the same columns
+              asm volatile(
+                  "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                  " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                  "l"(da + kk * da_step), "l"(db + kk * db_step + part_step), "r"(idesc), "r"(1u)
+                  : "memory");
+          }
         }
-        umma_commit_pair(empty0 + st * 8);
+        umma_commit_pair(full + 8 * TG_MAX_STAGES);               // the stage's empty barrier
         if (last) umma_commit_pair(acc_full0 + acc * 8);
       }
       __syncwarp();
@@ -385,8 +404,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
       if (last) {
         kb = 0;
         if (++acc == P.n_acc) { acc = 0; acc_ph ^= 1; }
+        d = tmem + acc * acc_cols;
       }
-      if (++st == S) { st = 0; ph ^= 1; }
+      full += 8; da_st += st_step; db_st += st_step;
+      if (full == full_end) { full = full0; ph ^= 1; da_st = da0; db_st = db0; }
     }
     if (!ok && lane == 0) { *gave_up = 1; __threadfence_block(); }
   } else if (warp == 1) {
@@ -394,9 +415,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     if (lane == 0) {
       int st = 0;
       uint32_t ph = 0;
-      for (int i = 0; i < n_it; ++i) {
+      TgCursor cur = start;
+      for (int i = 0; i < n_it;) {
+        const int n = cur.units(n_kb, KPS);
         if (!tg_wait(full0 + st * 8, ph, P)) break;
         mbar_arrive_leader(full0 + st * 8);
+        cur.next(n, n_kb, n_ct, pair, n_pairs);
+        i += n;
         if (++st == S) { st = 0; ph ^= 1; }
       }
     }

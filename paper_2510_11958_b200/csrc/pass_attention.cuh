@@ -29,23 +29,8 @@ constexpr int PK_KROW = 320;                                  // bytes per K row
 constexpr int PK_VROW = 272;                                  // bytes per V row: 256 + 16, conflict-free ldmatrix
 constexpr int PK_QROW = 272;
 constexpr int PK_OROW = PK_D + 8;                             // floats per partial-output row, padded against bank conflicts
-// layout of the attention scratch (the activation staging area and the row staging area behind it)
-constexpr int PK_AT_KH = 0;                                   // K tile, hi parts [PK_TK][PK_KROW]
-constexpr int PK_AT_KL = PK_AT_KH + PK_TK * PK_KROW;          // second K tile (the standalone kernel's double buffer)
-constexpr int PK_AT_VH = PK_AT_KL + PK_TK * PK_KROW;          // V tile, hi parts [PK_TK][PK_VROW]
-constexpr int PK_AT_VL = PK_AT_VH + PK_TK * PK_VROW;          // second V tile
-constexpr int PK_AT_QH = PK_AT_VL + PK_TK * PK_VROW;          // Q tile [PK_QR][PK_QROW], hi then lo
-constexpr int PK_AT_QL = PK_AT_QH + PK_QR * PK_QROW;
-constexpr int PK_AT_NEW = PK_AT_QL + PK_QR * PK_QROW;         // K rows of the pass [4][128] floats, then V rows [4][128]
-constexpr int PK_AT_TILES_END = PK_AT_NEW + 2 * PK_MAX_ROWS * PK_D * 4;
-constexpr int PK_AT_OS = 0;                                   // after the tiles are consumed: [warps][16][PK_OROW] floats
-constexpr int PK_AT_RED = 90112;                              // running max [warps][16], then sum / merge factor [warps][16]
-constexpr int PK_AT_ROWS = PK_AT_RED + 2 * PK_WARPS * PK_QR * 4;   // the pass's q | k | v vectors of one kv head, fp32, per row
-constexpr int PK_AT_ROW_FLOATS = (PK_MAX_GROUP + 2) * PK_D;
-constexpr int PK_AT_END = PK_AT_ROWS + PK_MAX_ROWS * PK_AT_ROW_FLOATS * 4;
-static_assert(PK_AT_TILES_END <= PK_AT_RED && PK_WARPS * PK_QR * PK_OROW * 4 <= PK_AT_RED, "attention scratch overlaps");
-// The pass kernel keeps one tile of each kind, so its map of the same pieces is more compact (its
-// scratch is what the weight rings leave of the SM's shared memory):
+constexpr int PK_AT_ROW_FLOATS = (PK_MAX_GROUP + 2) * PK_D;   // the q | k | v vectors of one kv head and row
+// layout of the attention scratch (what the weight rings leave of the SM's shared memory): one tile of each kind
 constexpr int PK_PA_KH = 0;                                   // K tile [PK_TK][PK_KROW]
 constexpr int PK_PA_VH = PK_PA_KH + PK_TK * PK_KROW;          // V tile [PK_TK][PK_VROW]
 constexpr int PK_PA_QH = PK_PA_VH + PK_TK * PK_VROW;          // Q tile [PK_QR][PK_QROW], and a second one kept zero

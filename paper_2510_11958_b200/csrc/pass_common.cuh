@@ -28,11 +28,11 @@
 //    4 KiB chunk (shared-memory atomic, table look-ups, two divisions, slot records) sits
 //    between a slot becoming free and its next request, and the stream ran at half speed.
 //    Fixed per-warp shares keep that path to a few dozen instructions.
-//  * mma.sync issues once per 32 cycles per SM sub-partition here (the hmma sub-pipe counter of ncu):
-//    with two warps per sub-partition and two MMAs per atom that is 128 of the 150 cycles the weight
-//    loop takes per atom and warp - 2.3 times the SM's share of HBM, so the loop keeps up, and a ring
-//    filled during a barrier is drained at that rate.  It is too slow for attention with bf16 hi/lo
-//    pairs, which is why the fp32-cache attention stage uses FMAs.
+//  * with straight-line code per tile a round of the 8 warps' chunks (64 KiB) takes some 1060 cycles, 2.3 times the
+//    SM's share of HBM, so the loop keeps up, and a ring filled during a barrier is drained at that rate.  It is not
+//    bound by instructions or by mma.sync (one m16n8k16 per 8 cycles and sub-partition, 21 for a dependent one): all
+//    loads of a tile before its MMAs, more accumulators, an earlier or unfenced hand-over of the slot left it
+//    unchanged; 64 bytes a cycle is what the SM takes from L2.
 //  * the weight loop must stay short: with one atom per trip and the tile bookkeeping inside it
 //    (about 45 instructions per atom, each at its full latency with two warps per sub-partition) a
 //    warp took 260 cycles per atom, exactly the SM's share of HBM, and never waited for a chunk.

@@ -90,9 +90,7 @@ __device__ __noinline__ bool gemv_consume(const PassParams &P, const PackedMat &
     Bq[k] = make_uint4(0u, 0u, 0u, 0u);
     if (need_b && k < aps) Bq[k] = lds128(b_addr + k * 64);
   }
-  // PK_NACC accumulators taken in turn (measured: 2, 4, 8 and 16 give 0.65, 0.74, 0.76 and 0.83 us per 8-atom
-  // chunk: the loop is bound by the rate at which the SM takes mma.sync, about one m16n8k16 per 32 cycles and
-  // scheduler, not by the chain through an accumulator)
+  // PK_NACC accumulators taken in turn (2, 4, 8 and 16: 0.65, 0.74, 0.76 and 0.83 us per 8-atom chunk)
   float acc[PK_NACC][4];
 #pragma unroll
   for (int i = 0; i < PK_NACC; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;

@@ -252,8 +252,8 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *ctx, float temperature, uint64_t seed);
  *                       tensor cores; bf16 contexts whose hidden, query and intermediate sizes
  *                       are multiples of 64 hold the second weight copy it reads, which doubles
  *                       the weight memory of the context (default 1)
- *   "tcgen05_gemm_stages" n  pipeline stages of a block of that GEMM, 2..6; 0 = as many as
- *                       shared memory holds (default 0)
+ *   "tcgen05_gemm_stages" n  most pipeline stages of a block of that GEMM, 2..6 (shared memory holds 3 to 6);
+ *                       0 = as many as it holds, which is the fastest (default 0)
  *   "fused_qk_rope" 0/1 QK-norm, rotary embedding and the KV append (Section 3.1's Qwen3 block) inside
  *                       the decode attention kernels of the per-step path (chunks of fewer than 16 positions; not
  *                       an fp32 cache with head_dim 128) instead of a launch of their own (default 1)

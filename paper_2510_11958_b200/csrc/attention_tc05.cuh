@@ -20,7 +20,8 @@
 // (680 TFLOP/s); one sequence of 512 tokens (32 query and 8 kv heads): 18 us per layer, 69 us with the kernel
 // before this one, which ran the same tiles on mma.sync, each warp re-reading K and V from shared memory for 16 rows.
 //
-// Warps 0-3 load Q, run the softmax and store; warp 4 issues the MMAs; warp 5 copies K and V.  All waits bounded.
+// Warps 0-3 load Q, run the softmax and store; warp 4 issues the MMAs; warp 5 copies K and V.  Every barrier wait is bounded; the
+// tensor-memory allocation waits only for grids in front of this one (see pdl_enter in the kernel).
 #pragma once
 
 #include "gemm_tc05.cuh"
@@ -37,6 +38,8 @@ constexpr int AP_HALF = 128 * 128;               // bytes of one half (64 of the
 constexpr int AP_Q = 0, AP_K = 2 * AP_HALF, AP_V = 4 * AP_HALF, AP_BARS = 6 * AP_HALF;
 constexpr int AP_SMEM = AP_BARS + 64;
 constexpr int AP_TMEM_COLS = 256;                // S (P over it) and O
+static_assert(TG_MIN_SMEM + AP_SMEM + 2 * 1024 > 228 * 1024 && 2 * (TG_MIN_SMEM + 1024) > 228 * 1024,
+              "a GEMM block shares its SM with no other holder of tensor memory");
 constexpr float AP_LOG2E = 1.4426950408889634f;
 constexpr float AP_RESCALE_LOG2 = 8.f;           // a row's reference maximum may be this far (in powers of two) behind
 
@@ -129,9 +132,6 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
   const int G = P.nq / P.nkv, lgG = 31 - __clz(G), QB = AP_M >> lgG;  // G is a power of two (it divides 128); positions per block
   const int kvh = blockIdx.y, b = blockIdx.z;
   const int r0 = blockIdx.x * QB, r1 = min(P.R, r0 + QB);
-  pdl_enter();
-  const int pos0 = *P.pos0;
-  const int n_keys = pos0 + r1, n_tiles = (n_keys + AP_TK - 1) / AP_TK;     // the block's last position sees keys [0, pos0 + r1)
   const uint32_t smem = smem_u32(sc);
   // tile i completes phase i of every barrier
   const uint32_t bar_k = smem + AP_BARS, bar_v = bar_k + 8;           // K / V tile in shared memory
@@ -157,7 +157,12 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // The dependent grid (the O projection's GEMM) takes tensor memory before it waits for this one, and an allocation waits
+  // without a limit: this block lets it in only now that it holds its own columns.
+  pdl_enter();
   const uint32_t tmem_s = *tmem_slot, tmem_o = tmem_s + 128;
+  const int pos0 = *P.pos0;
+  const int n_keys = pos0 + r1, n_tiles = (n_keys + AP_TK - 1) / AP_TK;     // the block's last position sees keys [0, pos0 + r1)
 
   if (warp >= 5) {
     // ---- copies: K(i) once S(i - 1) is computed, V(i) once P V (i - 1) is

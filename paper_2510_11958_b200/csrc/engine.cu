@@ -355,8 +355,8 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   while (cols < n_cols) cols <<= 1;
   P.n_acc = 2 * cols <= 512 ? 2 : 1;
   P.tmem_cols = P.n_acc * cols;
-  CUDA_TRY(c, launch_pdl(gemm_tc05_for(P.T.split != 0, whole), dim3(2 * n_pairs), dim3(TG_THREADS), (size_t)P.stages * stage_bytes + TG_TAIL_BYTES,
-                         c->stream, P));
+  CUDA_TRY(c, launch_pdl(gemm_tc05_for(P.T.split != 0, whole), dim3(2 * n_pairs), dim3(TG_THREADS),
+                         (size_t)std::max(TG_MIN_SMEM, P.stages * stage_bytes + TG_TAIL_BYTES), c->stream, P));
   LAUNCH_OK(c, "gemm_tc05_kernel");
   return DMTD_OK;
 }

@@ -34,8 +34,9 @@
 // 8.8 -> 8.1 ms, of 32 x 1024 tokens 539 -> 469 ms.
 //
 // Warp roles: warp 0 issues the bulk copies, warp 1 issues the MMAs (first SM of the pair) or passes on to the first
-// SM that a stage has landed (second SM), warps 2-9 run the epilogue (each the 32 lanes of its quarter, every second 16 columns).  Every wait is
-// bounded and reports through an error word; tensor memory is freed on every path.
+// SM that a stage has landed (second SM), warps 2-9 run the epilogue (each the 32 lanes of its quarter, every second 16 columns).  Every barrier wait is
+// bounded and reports through an error word; tensor memory is freed on every path.  Its allocation waits without a limit,
+// so it is taken in the order of the stream: a block lets the grids behind it in only once it holds its own.
 #pragma once
 
 #include "pass_stream.cuh"
@@ -55,7 +56,9 @@ constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
 // activations of a stage are 32 KiB there.
 __host__ __device__ constexpr int tg_stage_units(bool split) { return split ? 2 : 1; }
 constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
-constexpr int TG_MAX_SMEM = 226 * 1024;      // dynamic shared memory of a block: it has its SM to itself
+// Dynamic shared memory of a block: it has its SM to itself, beside a block of the prefill attention (96 KiB) or another
+// GEMM's, which take tensor memory as well.  Two stages of narrow column tiles need less than the lower bound.
+constexpr int TG_MAX_SMEM = 226 * 1024, TG_MIN_SMEM = 136 * 1024;
 enum { TG_ERR_WAIT = 4 };
 enum { TG_ADD = 0, TG_STORE = 1, TG_SWIGLU = 2 };           // tiles dealt out whole: none; stored; gated
 
@@ -267,10 +270,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     start = TgCursor{0, 0, pair, 0, n_pairs};
   }
 
-  // the kernel after this one (the next projection's activation-block kernel, launched the same way) may become
-  // resident now; it waits for this grid's completion before it reads or writes anything, and the GEMM behind it
-  // can then request its first weight blocks while this grid's last blocks finish
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   TgCursor cur_w = start, cur_a = start;               // producer's positions (thread 0)
   auto copy_w = [&](int st, int n) {                   // the k blocks of a row tile follow one another
     bulk_g2s(smem_u32(tg_smem) + st * stage_bytes, P.W.w + ((size_t)(2 * cur_w.rt + rank) * n_kb + cur_w.kb) * (TG_WBLOCK / 16),
@@ -302,6 +301,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  // The kernel after this one (the next projection's activation-block kernel, launched the same way) may become
+  // resident now; it waits for this grid's completion before it reads or writes anything, and the GEMM behind it
+  // can then request its first weight blocks while this grid's last blocks finish.  Not before this block holds its
+  // tensor memory: a later grid that took the columns first would wait for this one, and an allocation has no limit.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   if (threadIdx.x == 0) {
     // the weight blocks of the first stages are requested before the other block is waited for: they touch this

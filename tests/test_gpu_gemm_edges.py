@@ -117,3 +117,20 @@ def test_rows_from_unmerged_slices(dmtd, B):
     clear = srt[..., -1] - srt[..., -2] > 2e-3       # logits within 1e-3, as above: picks may differ below twice that
     assert clear.mean() > 0.8
     assert (forced.T == ref_am)[clear].all()
+
+
+@pytest.mark.parametrize("n", [100, 128, 144, 208, 512])
+def test_stage_counts(dmtd, n):
+    """Every pipeline depth, with the prefill attention (16-bit cache) in front of the O projection: both hold tensor memory."""
+    w = to_cuda(make_weights(SHAPE, seed=0, norm_jitter=0.1))
+    prompt = torch.from_numpy(make_prompts(SHAPE.vocab, 1, n, seed=5).numpy()).cuda()
+    eng = dmtd.Dmtd(SHAPE, w, L_d=2, tau=3, max_batch=1, max_seq=n + 2, kv_dtype="f16")
+    logits = []
+    for stages in (0, 2, 3, 4, 5, 6):
+        eng.reset()
+        eng.set_option("tcgen05_gemm_stages", stages)
+        logits.append(eng.prefill(prompt, want_logits=True)[1].double())
+        eng.device_state()                                  # raises if a wait gave up
+    # the same products; the order of the reductions moves the last bit of single values of the fp16 cache (2^-11)
+    for got in logits[1:]:
+        assert (got - logits[0]).norm() <= 2 ** -11 * logits[0].norm()

@@ -142,7 +142,8 @@ dmtd_status dmtd_decode_forced(dmtd_ctx *ctx, const int32_t *forced, int32_t n,
  * of layers applied to some rows): layers [l0, l1) on hidden [B][R][hidden] fp32 (device,
  * in place), rows of each sequence at positions pos0 .. pos0+R-1, attending causally to the
  * context's KV cache (positions < pos0 must have been written in those layers) and writing
- * the rows' K and V into it.  Does not touch the schedule state.
+ * the rows' K and V into it.  Does not touch the schedule state.  `hidden` may begin on any float;
+ * off a 16-byte boundary it is copied to the workspace and back.
  * Errors: CAPACITY if pos0 + R > max_seq or B > max_batch. */
 dmtd_status dmtd_step_layers(dmtd_ctx *ctx, int32_t l0, int32_t l1, float *hidden, int32_t B,
                              int32_t R, int32_t pos0);

@@ -1248,7 +1248,12 @@ dmtd_status dmtd_step_layers(dmtd_ctx *c, int32_t l0, int32_t l1, float *hidden,
   set_int_kernel<<<1, 1, 0, c->stream>>>(&c->dstate->scratch, pos0);
   LAUNCH_OK(c, "set_int_kernel");
   TRY(launch_rope_table(c, &c->dstate->scratch, R));
-  for (int l = l0; l < l1; ++l) TRY(run_layer(c, l, hidden, B, R, &c->dstate->scratch, pos0 + R));
+  // the kernels read rows in 16-byte loads: rows that begin elsewhere are worked on in the workspace
+  float *const x = reinterpret_cast<uintptr_t>(hidden) % 16 ? c->x_lo : hidden;
+  const size_t bytes = (size_t)B * R * c->s.hidden * sizeof(float);
+  if (x != hidden) CUDA_TRY(c, cudaMemcpyAsync(x, hidden, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  for (int l = l0; l < l1; ++l) TRY(run_layer(c, l, x, B, R, &c->dstate->scratch, pos0 + R));
+  if (x != hidden) CUDA_TRY(c, cudaMemcpyAsync(hidden, x, bytes, cudaMemcpyDeviceToDevice, c->stream));
   return DMTD_OK;
 }
 

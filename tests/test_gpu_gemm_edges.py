@@ -134,3 +134,20 @@ def test_stage_counts(dmtd, n):
     # the same products; the order of the reductions moves the last bit of single values of the fp16 cache (2^-11)
     for got in logits[1:]:
         assert (got - logits[0]).norm() <= 2 ** -11 * logits[0].norm()
+
+
+@pytest.mark.parametrize("model", ["f32", "bf16"])
+@pytest.mark.parametrize("B,R", [(1, 1), (2, 2), (3, 2), (2, 20)])
+def test_step_layers_rows_off_a_16_byte_boundary(dmtd, model, B, R):
+    shape = SHAPES["tiny"] if model == "f32" else SHAPE.with_(n_layers=2)
+    eng = dmtd.Dmtd(shape, to_cuda(make_weights(shape, seed=0, norm_jitter=0.1)), L_d=1, tau=1, max_batch=B, max_seq=R + 1, kv_dtype="f32")
+    rows = torch.randn(B, R, shape.hidden, generator=torch.Generator().manual_seed(3)).cuda()
+    ref = eng.step_layers(0, 2, rows.clone(), 0)
+    for off in (1, 2, 3):
+        buf = torch.full((rows.numel() + 8,), 7.0, device="cuda")
+        view = buf[off:off + rows.numel()].view(rows.shape)
+        view.copy_(rows)
+        got = eng.step_layers(0, 2, view, 0)
+        # the same kernels on the same values: fp32 reductions in another order at most
+        assert (got - ref).abs().max() <= 1e-5 * max(1.0, ref.abs().max().item())
+        assert (buf[:off] == 7).all() and (buf[off + rows.numel():] == 7).all()

@@ -296,17 +296,26 @@ struct GemmInput {
   int nsplit = 0;                           // SLICES: the attention's key slices, merged on the way
   int kb0 = 0;                              // SWIGLU: the first k block that is not written yet
   uint4 *blocks = nullptr;                  // READY (and SWIGLU, for the rest): the blocks' own buffer
+  GateUpParts gu{};                         // SWIGLU: the parts of gate+up's cut tiles
+  // of the GEMM: outputs that do not depend on the order in which parts of tiles are added (see repeats)
+  enum Sums { ANY_ORDER, TWO_PARTS, UNCUT } sums = ANY_ORDER;
+  size_t part_stride = 0;                   // gate+up: its cut tiles' parts are stored this far apart
 };
+
+ActTiles projection_tiles(const dmtd_ctx *c, const UmmaMat &W, int M, bool uncut) {
+  return uncut ? act_tiles_uncut(M, W.n_kb, W.n_tiles / 2, c->n_sms / 2) : act_tiles_for(M, W.n_kb);
+}
 
 // out[m][n] (+)= sum_k W[n][k] act[m][k]: the kernel that writes the activation blocks, then the GEMM.  After a norm the
 // outputs are new: what the GEMM adds into is cleared beside the norm, the rest is stored (`whole`).  With `gated` the
 // matrix is gate+up and the gate's result goes to the down projection's activation blocks there; `out` takes the
 // values of the weight rows behind the tiles dealt out whole, [M][ldo] from row tg_whole_pairs * 256 on.
-dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in, int M, float *out, int ldo, uint4 *gated = nullptr) {
+dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in, int M, float *out, int ldo, uint4 *gated = nullptr,
+                             const ActTiles &gated_tiles = ActTiles{}) {
   GemmTcParams P{};
   P.W = W;
   P.rows = M;
-  P.T = act_tiles_for(M, W.n_kb);
+  P.T = projection_tiles(c, W, M, in.sums == GemmInput::UNCUT);
   P.out = out; P.ldo = ldo;
   P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
   uint4 *blocks = in.blocks ? in.blocks : c->act_blocks;
@@ -318,10 +327,12 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   const int whole = in.kind != GemmInput::NORM ? TG_ADD : gated ? TG_SWIGLU : W.n_tiles / 2 >= 4 * n_pairs ? TG_STORE : TG_ADD;
   P.rt_whole = tg_whole_pairs(W, whole, n_pairs);
   P.whole_units = P.rt_whole / n_pairs * P.T.n_ctiles * W.n_kb;
-  const int n_line = (W.n_tiles / 2 - P.rt_whole) * P.T.n_ctiles * W.n_kb;
-  P.line_q = n_line / n_pairs; P.line_r = n_line % n_pairs;
+  const int tiles = (W.n_tiles / 2 - P.rt_whole) * P.T.n_ctiles;
+  P.line = in.sums == GemmInput::TWO_PARTS ? tg_line_two(tiles, W.n_kb, n_pairs)
+                                           : tg_line(tiles, W.n_kb, in.sums == GemmInput::UNCUT ? tiles : n_pairs);
+  P.part_stride = in.part_stride;
   const int n_whole = P.rt_whole * 2 * TG_ROWS;                                   // weight rows dealt out whole
-  if (gated) { P.gated = gated; P.gated_kb = W.N / 2 / TG_KB; P.out_n0 = n_whole; }
+  if (gated) { P.gated = gated; P.gated_T = gated_tiles; P.out_n0 = n_whole; }
   // shares of the k blocks per group of rows: one wave of blocks (two per SM; every block reads its rows for their sums).
   // 1 / 2 / 4 per SM: batch 32 21.8 / 21.65 / 22.4 ms for 4 cycles, batch 3 23.11 / 23.06 / 23.05 for 6
   const int n_groups = (M + NAB_ROWS - 1) / NAB_ROWS, ky = std::max(1, std::min(W.n_kb, 2 * c->n_sms / n_groups));
@@ -330,9 +341,9 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
                            in.nsplit, c->s.n_q_heads, c->s.head_dim, M, P.T, blocks));
     LAUNCH_OK(c, "merge_act_blocks_kernel");
   } else if (in.kind == GemmInput::NORM) {
-    const int n_rest = std::max(0, W.N - n_whole);
+    const int n_rest = in.part_stride ? 0 : std::max(0, W.N - n_whole);
     ZeroArea zero{gated ? out : out + n_whole, M, n_rest, (size_t)ldo};
-    if (n_whole == 0) zero.cols = ldo;                                            // whole rows, padding included
+    if (n_whole == 0 && n_rest) zero.cols = ldo;                                          // whole rows, padding included
     const size_t zero_n = (size_t)zero.rows * zero.cols;
     const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
     CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
@@ -342,7 +353,7 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   } else if (in.kind != GemmInput::READY && in.kb0 < W.n_kb) {
     const int tiles = (W.n_kb - in.kb0) * ((M + AB_ROWS - 1) / AB_ROWS);
     CUDA_TRY(c, launch_pdl(in.kind == GemmInput::SWIGLU ? act_blocks_kernel<true> : act_blocks_kernel<false>,
-                           dim3(std::min((tiles + AB_THREADS / 32 - 1) / (AB_THREADS / 32), 8 * c->n_sms)), dim3(AB_THREADS), 0, c->stream, in.act, in.lda, M, P.T, blocks, in.kb0));
+                           dim3(std::min((tiles + AB_THREADS / 32 - 1) / (AB_THREADS / 32), 8 * c->n_sms)), dim3(AB_THREADS), 0, c->stream, in.act, in.lda, M, P.T, blocks, in.kb0, in.gu));
     LAUNCH_OK(c, "act_blocks_kernel");
   }
   // as many stages as shared memory holds, two accumulators where tensor memory does.  (Half of both for decode launches,
@@ -423,6 +434,31 @@ AttnDecodePlan tc_attention_plan(const dmtd_ctx *c, int B, int R, int max_slots)
   return attn_decode_plan(c->n_sms, B * s.n_kv_heads * n_rb, (c->max_seq + AD_UNIT - 1) / AD_UNIT, max_slots);
 }
 
+// Large chunks give the same bits every time, as no sum depends on the order in which blocks finish: QKV's tiles are in at most
+// two parts (onto zeroed outputs), O's and the down projection's are not cut, and the parts of the few row tiles of gate+up
+// that are cut keep to themselves until the gate sums them.  Where uncut tiles of more than 128 rows keep the block
+// pairs busy (Qwen3-4B shape: from 897 rows, 0.84 to 0.87 of their columns in use).  Four layers on 1024 rows take 1355 us
+// so and 1327 with every tile cut into equal parts, on 900 rows 1333 and 1279; the prefill of 32 x 1024 tokens 461.3 and
+// 457.0 ms.  (Parts summed in order by the last block to arrive: 1497 us; three buffers for the residual rows, one to a
+// part: 1430.)  Fewer rows, and decode passes, add their parts in any order.
+bool repeats(const dmtd_ctx *c, int M) {
+  if (!c->umma_ok || !c->use_umma || M <= TG_SPLIT_ROWS) return false;
+  const LayerDev &lw = c->layers[0];
+  const int n_pairs = c->n_sms / 2, n_ct = act_tiles_for(M, 1).n_ctiles;
+  auto uncut = [&](const UmmaMat &W) {
+    const int n_rt = W.n_tiles / 2;
+    if (n_rt > n_pairs) return false;
+    const int rows = act_tiles_uncut(M, W.n_kb, n_rt, n_pairs).tile_rows;
+    return rows > TG_SPLIT_ROWS && rows <= TG_TILE_ROWS && n_rt * M >= 0.8 * n_pairs * rows;
+  };
+  const int gu_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, n_pairs), gu_tiles = (lw.gu_u.n_tiles / 2 - gu_whole) * n_ct;
+  const TgLine gu = tg_line(gu_tiles, lw.gu_u.n_kb, n_pairs);
+  const size_t gu_parts = gu_tiles == 0 ? 0 : gu.q == 0 ? n_pairs : std::max(0, lw.gu_u.n_kb - 2) / gu.q + 2;
+  const size_t n_rest = std::max(0, lw.gu_u.N - gu_whole * 2 * TG_ROWS);
+  return lw.qkv_u.n_tiles / 2 * n_ct >= n_pairs && uncut(lw.o_u) && uncut(lw.down_u) &&
+         gu_parts * n_rest * M <= (size_t)c->ws_rows * c->ldgu;
+}
+
 template <int D, typename KVT>
 dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge, bool flash) {
   const dmtd_model_shape &s = c->s;
@@ -448,7 +484,7 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
       A.R = R; A.pos0 = pos0; A.out = c->act; A.ld = c->lda;
       if (!merge) {                         // straight into the O projection's activation blocks
         A.blocks = c->act_blocks;
-        A.T = act_tiles_for(M, s.n_q_heads * D / TG_KB);
+        A.T = projection_tiles(c, lw.o_u, M, repeats(c, M));
       }
       A.error = &c->dstate->error; A.wait_limit = kDeviceWaitLimitTicks;
       CUDA_TRY(c, launch_pdl(attn_prefill_kernel<Op>, dim3((R + QB - 1) / QB, s.n_kv_heads, B), dim3(AP_THREADS), (size_t)(AP_SMEM), c->stream,
@@ -576,8 +612,13 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     TRY(launch_gemv_f32_fused<F32_NORM>(c, lw.gu, f32_norm_input(c, x, lw.w_post), M, c->gu, c->ldgu, true));
     return launch_gemv_f32_fused<F32_SWIGLU>(c, lw.down, F32In{c->gu, c->ldgu, nullptr, 0.f, nullptr, nullptr, 0, 0}, M, x, H, false);
   }
+  const bool same_bits = tc && repeats(c, M);
+  auto with_sums = [&](GemmInput in, GemmInput::Sums sums) {
+    if (same_bits) in.sums = sums;
+    return in;
+  };
   if (tc) {
-    TRY(launch_gemm_tc05(c, lw.qkv_u, norm_input(x, H, lw.w_in), M, c->qkv, c->ldqkv));
+    TRY(launch_gemm_tc05(c, lw.qkv_u, with_sums(norm_input(x, H, lw.w_in), GemmInput::TWO_PARTS), M, c->qkv, c->ldqkv));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldqkv + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              x, H, lw.w_in, H, s.rms_eps, c->act, c->lda, c->qkv, c->ldqkv, c->ldqkv));
@@ -594,7 +635,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     GemmInput in;
     in.kind = flash ? GemmInput::READY : GemmInput::SLICES;
     in.nsplit = nsplit;
-    TRY(launch_gemm_tc05(c, lw.o_u, in, M, x, H));
+    TRY(launch_gemm_tc05(c, lw.o_u, with_sums(in, GemmInput::UNCUT), M, x, H));
   }
   else TRY(launch_gemv(c, lw.o, lw.o_u, c->act, c->lda, M, x, H));
   if (tc) {
@@ -606,12 +647,19 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     if (M > TG_SPLIT_ROWS) {
       const int n_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, c->n_sms / 2) * 2 * TG_ROWS, n_rest = std::max(0, 2 * I - n_whole);
       down.lda = std::max(4, n_rest); down.kb0 = n_whole / 2 / TG_KB; down.blocks = c->gated_blocks;
-      TRY(launch_gemm_tc05(c, lw.gu_u, norm_input(x, H, lw.w_post), M, c->gu, down.lda, c->gated_blocks));
+      GemmInput gu = norm_input(x, H, lw.w_post);
+      if (same_bits && n_rest) {
+        const ActTiles T = act_tiles_for(M, lw.gu_u.n_kb);
+        gu.part_stride = (size_t)M * down.lda;
+        down.gu = GateUpParts{tg_line((lw.gu_u.n_tiles / 2 - n_whole / (2 * TG_ROWS)) * T.n_ctiles, T.n_kb, c->n_sms / 2), T.n_ctiles, T.n_kb,
+                              T.tile_rows, gu.part_stride};
+      }
+      TRY(launch_gemm_tc05(c, lw.gu_u, gu, M, c->gu, down.lda, c->gated_blocks, projection_tiles(c, lw.down_u, M, same_bits)));
     } else {
       down.lda = c->ldgu;
       TRY(launch_gemm_tc05(c, lw.gu_u, norm_input(x, H, lw.w_post), M, c->gu, c->ldgu));
     }
-    TRY(launch_gemm_tc05(c, lw.down_u, down, M, x, H));
+    TRY(launch_gemm_tc05(c, lw.down_u, with_sums(down, GemmInput::UNCUT), M, x, H));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(M, (c->ldgu + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              x, H, lw.w_post, H, s.rms_eps, c->act, c->lda, c->gu, c->ldgu, c->ldgu));
@@ -639,7 +687,9 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
   if (f32_fused_rows(c, B)) {
     TRY(launch_gemv_f32_fused<F32_NORM>(c, c->embed, f32_norm_input(c, c->x_up, c->w_final), B, c->logits, c->ldl, true));
   } else if (c->embed_u.w && c->use_umma) {
-    TRY(launch_gemm_tc05(c, c->embed_u, norm_input(c->x_up, s.hidden, c->w_final), B, c->logits, c->ldl));
+    GemmInput in = norm_input(c->x_up, s.hidden, c->w_final);
+    if (kind == 0) in.sums = GemmInput::TWO_PARTS;      // the first token's logits repeat as a large chunk's rows do
+    TRY(launch_gemm_tc05(c, c->embed_u, in, B, c->logits, c->ldl));
   } else {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(B, (c->ldl + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
                              c->x_up, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act, c->lda, c->logits, c->ldl, c->ldl));
@@ -1098,9 +1148,10 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   c->pend_cap = std::max(1, c->part_rows / max_batch);
   CTRY(dev_alloc(c, &c->h_pend, (size_t)max_batch * c->pend_cap * H));
   CTRY(dev_alloc(c, &c->h_base, (size_t)c->ws_rows * H));
-  // activation blocks: hi and lo units of every row, the rows rounded up to whole column tiles
+  // activation blocks: hi and lo units of every row, the rows rounded up to whole column tiles (the last of them may be
+  // mostly empty)
   if (c->umma_ok) {
-    const size_t rows = (size_t)c->ws_rows + 16 * (c->ws_rows / TG_TILE_ROWS + 1);
+    const size_t rows = (size_t)c->ws_rows + 16 * (c->ws_rows / TG_SPLIT_ROWS + 1) + TG_TILE_ROWS;
     CTRY(dev_alloc(c, &c->act_blocks, rows * (c->lda / 8) * 2));
     CTRY(dev_alloc(c, &c->gated_blocks, rows * (I / 8) * 2));
   }

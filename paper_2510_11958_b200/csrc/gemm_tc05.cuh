@@ -100,6 +100,15 @@ inline ActTiles act_tiles_for(int rows, int n_kb) {
   return t;
 }
 
+// A line of units in equal parts: the first `pairs` block pairs take q units each, the first r of them one more.
+struct TgLine {
+  int q, r, pairs;
+  __host__ __device__ __forceinline__ int begin(int pair) const { return pair * q + (pair < r ? pair : r); }
+  __host__ __device__ __forceinline__ int size(int pair) const { return pair < pairs ? q + (pair < r ? 1 : 0) : 0; }
+  // the pair that holds unit u
+  __host__ __device__ __forceinline__ int holder(int u) const { return u < r * (q + 1) ? u / (q + 1) : r + (u - r * (q + 1)) / q; }
+};
+
 struct GemmTcParams {
   UmmaMat W;
   const uint4 *act_blocks;
@@ -109,10 +118,11 @@ struct GemmTcParams {
   int ldo;
   int rt_whole;              // row-tile pairs dealt out whole, a multiple of the block pairs: the first ones
   int whole_units;           // units of a block pair's whole tiles
-  int line_q, line_r;        // a block pair's part of the units of the others: line_q, one more for the first line_r pairs
+  TgLine line;               // the block pairs' parts of the units of the others
   int out_n0;                // first weight row of out's columns (TG_SWIGLU: out holds the remaining row-tile pairs only)
-  uint4 *gated;              // TG_SWIGLU: units of the next projection, in the tiles of T (k = half of the interleaved weight row)
-  int gated_kb;              // ... and its k blocks
+  uint4 *gated;              // TG_SWIGLU: units of the next projection (k = half of the interleaved weight row)
+  ActTiles gated_T;          // ... and their tiles
+  size_t part_stride;        // TG_SWIGLU: part i of a cut tile (counted along the line) is stored i * part_stride further; 0: added
   int stages;                // pipeline stages of a block, 2 .. TG_MAX_STAGES
   int n_acc, tmem_cols;      // accumulators in tensor memory (1 or 2), tmem_cols / n_acc columns apart
   int *error;
@@ -179,6 +189,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
 }
 __device__ __forceinline__ void red_add(float *p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+// `tiles` tiles of n_kb units each, cut into equal parts for n_pairs block pairs.
+inline TgLine tg_line(int tiles, int n_kb, int n_pairs) { return TgLine{tiles * n_kb / n_pairs, tiles * n_kb % n_pairs, n_pairs}; }
+// ... no tile in more than two parts: a sum onto zeroed outputs is then the same in either order.  Leaves block pairs idle
+// where there are fewer tiles than pairs.
+inline TgLine tg_line_two(int tiles, int n_kb, int n_pairs) {
+  return tg_line(tiles, n_kb, tiles >= n_pairs ? n_pairs : std::max(1, n_kb % 2 == 0 && 2 * tiles <= n_pairs ? 2 * tiles : tiles));
+}
+// Column tiles so narrow that every block pair takes one whole tile of n_rt row-tile pairs (or none): nothing is cut, every
+// output has one sum.
+inline ActTiles act_tiles_uncut(int rows, int n_kb, int n_rt, int n_pairs) {
+  ActTiles t = act_tiles_for(rows, n_kb);
+  const int most = std::max(1, n_pairs / n_rt);
+  t.tile_rows = ((rows + most - 1) / most + 15) / 16 * 16;
+  t.n_ctiles = (rows + t.tile_rows - 1) / t.tile_rows;
+  return t;
 }
 // Row-tile pairs dealt out whole: the largest multiple of the block pairs.
 inline int tg_whole_pairs(const UmmaMat &W, int whole, int n_pairs) {
@@ -260,7 +286,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
 
   // this pair's share of the units
   const int n_ct = SPLIT ? 1 : P.T.n_ctiles;
-  const int u0 = pair * P.line_q + min(pair, P.line_r), n_part = P.line_q + (pair < P.line_r ? 1 : 0);
+  const int u0 = P.line.begin(pair), n_part = P.line.size(pair);
   const int n_it = n_part + (WHOLE == TG_ADD ? 0 : P.whole_units);
   TgCursor start;
   if (n_part > 0) {
@@ -450,6 +476,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
       const uint32_t t_base = tmem + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols;
       const int c_first = warp < 6 ? 0 : 16;
       float *dst = P.out + (size_t)(m0 + c_first) * P.ldo + (n - (WHOLE == TG_SWIGLU ? P.out_n0 : 0));
+      const bool in_parts = WHOLE == TG_SWIGLU && !whole && P.part_stride;
+      if (in_parts) dst += (pair - P.line.holder(((this_rt - P.rt_whole) * n_ct + this_ct) * n_kb)) * P.part_stride;
 #pragma unroll 1
       for (int c0 = c_first; c0 < n_rows; c0 += 32) {
         uint32_t r[16];
@@ -468,15 +496,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
         } else if (WHOLE == TG_SWIGLU && whole) {
           uint4 hi, lo;
           swiglu_units(r, hi, lo);
-          const int col = c0 + 2 * ((lane >> 1) & 7) + (lane & 1), half = tile_rows / 2, sm = col >= half ? 1 : 0;
+          const int col = c0 + 2 * ((lane >> 1) & 7) + (lane & 1);
           if (col < n_rows) {
-            uint4 *u = P.gated + (((size_t)this_ct * P.gated_kb + 2 * this_rt + rank) * 2 + sm) * P.T.units_per_sm() +
-                       (2 * quarter + (lane >> 4)) * half + (col - sm * half);
+            uint4 *u = P.gated + P.gated_T.unit(m0 + col, 2 * this_rt + rank, 2 * quarter + (lane >> 4));
             u[0] = hi;
-            u[P.T.lo_offset()] = lo;
+            u[P.gated_T.lo_offset()] = lo;
           }
         } else {
-          if (whole) {
+          if (whole || in_parts) {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
               if (c0 + j < n_rows) dst[(size_t)j * P.ldo] = __uint_as_float(r[j]);
@@ -534,9 +561,20 @@ __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, siz
 // request meanwhile: with a thread to a unit (its lanes' loads 32 rows apart, 16 bytes each) a block took 13.6 us at
 // 96 rows of the Qwen3-4B shape and 6 us at 32 (4 cycles of 32 sequences 21.3 ms, 20.3 so).
 constexpr int AB_ROWS = 4, AB_THREADS = 256;
+// The parts that the cut tiles of gate+up were stored in; stride 0: one buffer that they were added into.
+struct GateUpParts {
+  TgLine line;
+  int n_ct, n_kb, tile_rows;
+  size_t stride;
+  // parts of the tile of k block kb (of the intermediate values: two of them to a row-tile pair) and row m
+  __device__ __forceinline__ int count(int kb, int m) const {
+    const int u = (kb / (TG_ROWS / TG_KB) * n_ct + m / tile_rows) * n_kb;
+    return line.holder(u + n_kb - 1) - line.holder(u) + 1;
+  }
+};
 template <bool GATED>
 __global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T,
-                                                                uint4 *__restrict__ blocks, int kb0) {
+                                                                uint4 *__restrict__ blocks, int kb0, GateUpParts parts) {
   // lanes of a row, 16-byte loads of a lane, and 32-bit registers of a part that a load becomes
   constexpr int LANES = GATED ? 32 : 16, LOADS = AB_ROWS * LANES / 32, REGS = GATED ? 1 : 2;
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
@@ -554,6 +592,26 @@ __global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *__r
       const int m = m0 + i * (32 / LANES) + half;
       v[i] = m < rows ? *reinterpret_cast<const float4 *>(act + (size_t)m * lda + (size_t)kb * LANES * 4 + col * 4)
                       : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (GATED && parts.stride) {
+      const int n = parts.count(kb, m0);                             // four rows lie in one tile
+      constexpr int AHEAD = 5;
+#pragma unroll 1
+      for (int p0 = 1; p0 < n; p0 += AHEAD) {
+        float4 u[AHEAD][LOADS];
+#pragma unroll
+        for (int p = 0; p < AHEAD; ++p)
+#pragma unroll
+          for (int i = 0; i < LOADS; ++i) {
+            const int m = min(m0 + i * (32 / LANES) + half, rows - 1);
+            u[p][i] = *reinterpret_cast<const float4 *>(act + min(p0 + p, n - 1) * parts.stride + (size_t)m * lda + (size_t)kb * LANES * 4 + col * 4);
+          }
+#pragma unroll
+        for (int p = 0; p < AHEAD; ++p)
+#pragma unroll
+          for (int i = 0; i < LOADS; ++i)
+            if (p0 + p < n) { v[i].x += u[p][i].x; v[i].y += u[p][i].y; v[i].z += u[p][i].z; v[i].w += u[p][i].w; }
+      }
     }
     uint32_t hi[LOADS][REGS], lo[LOADS][REGS];
     auto split = [](float a, float b, uint32_t &h, uint32_t &l) {

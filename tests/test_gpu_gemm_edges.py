@@ -151,3 +151,42 @@ def test_step_layers_rows_off_a_16_byte_boundary(dmtd, model, B, R):
         # the same kernels on the same values: fp32 reductions in another order at most
         assert (got - ref).abs().max() <= 1e-5 * max(1.0, ref.abs().max().item())
         assert (buf[:off] == 7).all() and (buf[off + rows.numel():] == 7).all()
+
+
+# projections of this size keep 74 block pairs busy with uncut tiles from 897 rows on
+WIDE = SHAPE.with_(n_layers=2, hidden=2560, n_q_heads=32, n_kv_heads=8, intermediate=9728, vocab=20000)
+
+
+@pytest.fixture(scope="module")
+def wide_weights():
+    return make_weights(WIDE, seed=0, device="cuda", norm_jitter=0.1)
+
+
+@pytest.mark.parametrize("B,P,kv", [
+    (1, 897, "f16"),
+    (2, 512, "f16"),
+    (3, 300, "f32"),        # 900 rows
+    (8, 256, "bf16"),       # two chunks
+])
+def test_large_prefill_repeats(dmtd, wide_weights, B, P, kv):
+    """Large chunks give the same bits again, cache and logits."""
+    prompt = torch.from_numpy(make_prompts(WIDE.vocab, B, P, seed=5).numpy()).cuda()
+    eng = dmtd.Dmtd(WIDE, wide_weights, L_d=1, tau=3, max_batch=B, max_seq=P + 1, kv_dtype=kv)
+    first = None
+    for _ in range(4):
+        eng.reset()
+        logits = eng.prefill(prompt, want_logits=True)[1]
+        if first is None:
+            first = logits.clone()
+        assert torch.equal(logits, first)
+
+
+@pytest.mark.parametrize("layers", [1, 2])
+@pytest.mark.parametrize("R", [897, 950, 1000])
+def test_large_chunk_against_small_ones(dmtd, wide_weights, layers, R):
+    eng = dmtd.Dmtd(WIDE, wide_weights, L_d=1, tau=1, max_batch=1, max_seq=R + 1, kv_dtype="f32")
+    rows = torch.randn(1, R, WIDE.hidden, generator=torch.Generator().manual_seed(3)).cuda()
+    got = eng.step_layers(0, layers, rows.clone(), 0)
+    ref = torch.cat([eng.step_layers(0, layers, rows[:, p:p + 200].clone(), p) for p in range(0, R, 200)], 1)
+    # sums of at most 9728 products in another order, activations within 2^-17 on both sides
+    assert (got - ref).abs().max() <= 1e-4 * max(1.0, ref.abs().max().item())

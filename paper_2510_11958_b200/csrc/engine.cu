@@ -343,7 +343,7 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   } else if (in.kind == GemmInput::NORM) {
     const int n_rest = in.part_stride ? 0 : std::max(0, W.N - n_whole);
     ZeroArea zero{gated ? out : out + n_whole, M, n_rest, (size_t)ldo};
-    if (n_whole == 0 && n_rest) zero.cols = ldo;                                          // whole rows, padding included
+    if (n_whole == 0 && n_rest && ldo - W.N < 16) zero.cols = ldo;                                          // whole rows, padding included
     const size_t zero_n = (size_t)zero.rows * zero.cols;
     const int n_zero = (int)std::min<size_t>((zero_n + 4095) / 4096, 2 * c->n_sms);
     CUDA_TRY(c, launch_pdl(norm_act_blocks_kernel, dim3(n_groups + (n_zero + ky - 1) / ky, ky), dim3(256), 0, c->stream,
@@ -707,23 +707,27 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
 }
 
 // The LM head over many positions (the scoring pass): final norm and tied head of n_seg segments of seg_rows rows,
-// segment i starting at row i * seg_stride of x; row m of them all to out[m][vocab].  One GEMM over all rows: a
+// segment i starting at row i * seg_stride of x; row m of them all to out + m * ldo.  One GEMM over all rows: a
 // head launch per position streams the whole head again (Qwen3-4B shape, 2 x 187 of 2 x 250 positions: 187 x 0.25 ms
 // of 59.1 ms a call; 13.4 ms now).
-dmtd_status run_head_rows(dmtd_ctx *c, const float *x, int n_seg, int seg_rows, int seg_stride, float *out) {
+dmtd_status run_head_rows(dmtd_ctx *c, const float *x, int n_seg, int seg_rows, int seg_stride, float *out, int ldo) {
   const dmtd_model_shape &s = c->s;
   const int M = n_seg * seg_rows;
   if (c->embed_u.w && c->use_umma) {
     GemmInput in = norm_input(x, s.hidden, c->w_final);
     in.seg_rows = seg_rows; in.seg_stride = seg_stride;
-    return launch_gemm_tc05(c, c->embed_u, in, M, out, s.vocab);
+    return launch_gemm_tc05(c, c->embed_u, in, M, out, ldo);
   }
+  // segments of one row are rows of a longer stride
+  int ldx = s.hidden;
+  if (seg_rows == 1) { ldx *= seg_stride; seg_rows = n_seg; n_seg = 1; }
   for (int i = 0; i < n_seg; ++i) {
     CUDA_TRY(c, launch_pdl(prep_norm_kernel, dim3(seg_rows, (s.vocab + PREP_ZERO_COLS - 1) / PREP_ZERO_COLS), dim3(256), (size_t)(0), c->stream,
-                             x + (size_t)i * seg_stride * s.hidden, s.hidden, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda, c->lda, out + (size_t)i * seg_rows * s.vocab, s.vocab, s.vocab));
+                             x + (size_t)i * seg_stride * s.hidden, ldx, c->w_final, s.hidden, s.rms_eps, c->act + (size_t)i * seg_rows * c->lda, c->lda,
+                             out + (size_t)i * seg_rows * ldo, ldo, s.vocab));
     LAUNCH_OK(c, "prep_norm_kernel");
   }
-  return launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, M, out, s.vocab);
+  return launch_gemv(c, c->embed, c->embed_u, c->act, c->lda, M, out, ldo);
 }
 
 // Kernels that need more than 48 KiB of dynamic shared memory must be told so once per device
@@ -1340,11 +1344,15 @@ dmtd_status dmtd_masked_forward(dmtd_ctx *c, const int32_t *tokens, int32_t B, i
     if (r0 >= R) continue;
     const float *x0 = c->x_lo + (size_t)r0 * H;
     float *out = out_logits + (size_t)(p0 + r0 - (P - 1)) * c->s.vocab;
+    const size_t V = c->s.vocab;
     if (R - r0 == (int)n_out) {
-      TRY(run_head_rows(c, x0, B, R - r0, R, out));                                  // all positions of all sequences
+      TRY(run_head_rows(c, x0, B, R - r0, R, out, V));                               // all positions of all sequences
+    } else if (R - r0 < B && n_out * V < (1ull << 31)) {
+      // fewer positions than sequences: position by position, as each launch streams the head (18 positions of 64 sequences
+      // in three chunks, 2 layers, 32000 tokens: a launch to a sequence 7.26 ms, to a position 2.23)
+      for (int r = 0; r < R - r0; ++r) TRY(run_head_rows(c, x0 + (size_t)r * H, B, 1, R, out + r * V, (int)(n_out * V)));
     } else {
-      for (int b = 0; b < B; ++b)
-        TRY(run_head_rows(c, x0 + (size_t)b * R * H, 1, R - r0, R, out + (size_t)b * n_out * c->s.vocab));
+      for (int b = 0; b < B; ++b) TRY(run_head_rows(c, x0 + (size_t)b * R * H, 1, R - r0, R, out + b * n_out * V, V));
     }
   }
   // the cache now holds this forward's K and V; the schedule state is untouched (still "no sequence")

@@ -30,6 +30,7 @@ def dmtd():
     (1, 5, 133),            # 129 rows in the head
     (1, 2, 257),            # two column tiles
     (3, 40, 400),           # several chunks of the workspace, four column tiles each
+    (70, 3, 17),            # 14 and 1 positions of two chunks: fewer than sequences, position by position
 ])
 def test_scoring_pass(dmtd, B, P, n):
     w = make_weights(SHAPE, seed=0, norm_jitter=0.1)

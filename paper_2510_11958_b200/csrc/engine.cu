@@ -416,10 +416,15 @@ AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R) {
                     : attn_partial_kernel<D, KVT, 16, FUSED, T>,
           warps * 32, (size_t)warps * nq * D * sizeof(float) + (FUSED ? 2 * (size_t)R * D * sizeof(KVT) : 0)};
 }
+// The form for slices of 64 keys (T = 1) takes more of an SM than the other and gains by latency alone: only for launches
+// whose blocks are resident at once, one to an SM with 16 query rows, two with 8, four with 4.  head_dim 64, fp16 cache,
+// against T = 4: 16 rows, 128 blocks 22 us (T = 4 31), 362 blocks 42 (31), 16384 blocks 1070 (670); 8 rows, 256 blocks 21
+// (25), 512 blocks 30 (25); 4 rows, 362 blocks 15 (17), 1024 blocks 29 (25).
 template <int D, typename KVT, bool FUSED>
-AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R, int CH) {
-  if constexpr (D == 64)                    // head_dim 128: only with "tensor_core_attention" off
-    if (CH <= 64) return attn_partial_for<D, KVT, FUSED, 1>(n_rows, R);
+AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R, int CH, long long n_blocks, int n_sms) {
+  const int nq = n_rows <= 4 ? 4 : n_rows <= 8 ? 8 : 16;
+  if constexpr (D == 64)                    // head_dim 128: only with "tc_attention" off
+    if (CH <= 64 && n_blocks * nq <= 16ll * n_sms) return attn_partial_for<D, KVT, FUSED, 1>(n_rows, R);
   return attn_partial_for<D, KVT, FUSED, 4>(n_rows, R);
 }
 
@@ -509,7 +514,8 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
     }
   } else {
     const AttnPartialKernel<KVT> ap =
-        fused_a3 ? attn_partial_for<D, KVT, D == 64>(std::min(R, RB) * G, R, c->CH) : attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, c->CH);
+        fused_a3 ? attn_partial_for<D, KVT, D == 64>(std::min(R, RB) * G, R, c->CH, (long long)nsplit * s.n_kv_heads * n_rb * B, c->n_sms)
+                 : attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, c->CH, (long long)nsplit * s.n_kv_heads * n_rb * B, c->n_sms);
     CUDA_TRY(c, launch_pdl(ap.kernel, dim3(nsplit, s.n_kv_heads * n_rb, B), dim3(ap.threads), ap.smem, c->stream, c->qkv, c->ldqkv,
                            kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, R, RB, c->CH, pos0, 0, c->part_o, c->part_ml, nsplit,
                            AttnFuse{lw.w_qn, lw.w_kn, c->rope_rows, s.rms_eps}));
@@ -751,11 +757,10 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   auto partial = [&](auto kv) -> dmtd_status {
     using KVT = decltype(kv);
     for (int rows : {8, 16}) {
-      CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<128, KVT, false>(rows, 1, 64).kernel, dyn, 64 * 1024));
-      for (int CH : {64, 128}) {
-        CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<64, KVT, false>(rows, 1, CH).kernel, dyn, 64 * 1024));
-        CUDA_TRY(c, cudaFuncSetAttribute(attn_partial_for<64, KVT, true>(rows, 1, CH).kernel, dyn, 64 * 1024));
-      }
+      const AttnPartialKernel<KVT> forms[] = {attn_partial_for<128, KVT, false, 4>(rows, 1), attn_partial_for<64, KVT, false, 1>(rows, 1),
+                                              attn_partial_for<64, KVT, false, 4>(rows, 1), attn_partial_for<64, KVT, true, 1>(rows, 1),
+                                              attn_partial_for<64, KVT, true, 4>(rows, 1)};
+      for (const AttnPartialKernel<KVT> &form : forms) CUDA_TRY(c, cudaFuncSetAttribute(form.kernel, dyn, 64 * 1024));
     }
     return DMTD_OK;
   };
@@ -1538,6 +1543,9 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
   const int G = nq / nkv, RB = std::max(1, ATTN_QR / G), n_rb = (R + RB - 1) / RB, ld = nq * D;
   int nsplit = p.nsplit;                    // slots per (row, head)
   cudaError_t e;
+  int dev = 0, n_sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return fail(nullptr, DMTD_ERR_CUDA, "attention: device query failed");
   if (D == PK_D) {
     if constexpr (std::is_same<KVT, float>::value) {
       e = cudaFuncSetAttribute(attn_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATTN_F32_SMEM);
@@ -1549,9 +1557,6 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
       e = cudaFuncSetAttribute(attn_decode_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
-      int dev = 0, n_sms = 0;
-      if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return fail(nullptr, DMTD_ERR_CUDA, "attention: device query failed");
       const AttnDecodePlan dp = attn_decode_plan(n_sms, B * nkv * n_rb, (pos0 + R + AD_UNIT - 1) / AD_UNIT, p.nsplit);
       nsplit = dp.nsplit;
       e = launch_pdl(attn_decode_kernel<Op, false>, dim3(dp.n_blocks), dim3(AD_THREADS), AD_SMEM, stream, q, ld, k, v, max_seq, nq, nkv, B,
@@ -1559,7 +1564,7 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
     }
   } else {
-    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, p.CH);
+    const AttnPartialKernel<KVT> ap = attn_partial_for<D, KVT, false>(std::min(R, RB) * G, R, p.CH, (long long)p.nsplit * nkv * n_rb * B, n_sms);
     e = cudaFuncSetAttribute(ap.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ap.smem);
     if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
     ap.kernel<<<dim3(p.nsplit, nkv * n_rb, B), ap.threads, ap.smem, stream>>>(

@@ -558,13 +558,14 @@ template <> __device__ __forceinline__ void load8<__half>(const __half *p, float
 }
 // NQ: query rows the block is compiled for, 4, 8 or 16 (the scores, the probabilities and the outputs of all NQ rows are
 // worked out).  A warp takes 8 T keys at a time:
-//   T = 1, 8 warps, four lanes to a key: slices of 64 keys.  Bound by the trips to memory that follow one another, so K and V come in one, and
+//   T = 1, 8 warps, four lanes to a key: slices of 64 keys of launches that are resident at once.  Bound by the trips to memory that follow one another, so K and V come in one, and
 //   the older keys (previous passes appended them) are requested before the kernel in front is waited for.
-//   T = 4, 4 warps, a lane to a key: longer slices.  Bound by instructions, so one softmax step serves 32 keys.
+//   T = 4, 4 warps, a lane to a key: longer slices, and more blocks than that.  Bound by instructions, so one softmax step
+//     serves 32 keys, and by the blocks an SM holds: four with 64 dimensions, three with 128.
 // Isolated, 36 keys of one head and 2 query rows took 27 us with 16 rows and one load at a time, 11 us with T = 4 in 8-key
 // loads.  32 x 8192 keys, 8 kv heads of bf16 rows: 234 us with T = 4, 460 with T = 1.
 template <int D, typename KVT, int NQ, bool FUSED, int T>
-__global__ void __launch_bounds__(attn_warps(T) * 32)
+__global__ void __launch_bounds__(attn_warps(T) * 32, T == 1 ? 1 : D == 64 ? 4 : 3)
 attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restrict__ kc,
                     const KVT *__restrict__ vc, int max_seq, int nq, int nkv, int R, int RB, int CH,
                     const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,

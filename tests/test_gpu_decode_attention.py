@@ -45,3 +45,29 @@ def test_attention_decode_pieces(dmtd, dtype, B, R, nq, nkv, n_keys):
     u = 2.0 ** -9 if dtype == torch.bfloat16 else 2.0 ** -12
     err = (out.double() - ref).abs().max().item()
     assert err <= 4 * u * max(1.0, ref.abs().max().item()), err
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,R,nq,nkv,n_keys", [
+    (1, 1, 4, 2, 1),            # one key
+    (1, 4, 16, 4, 2300),        # 16 query rows, 36 slices x 4 heads: 144 blocks
+    (1, 4, 16, 4, 2400),        # 152 blocks: more than one to an SM
+    (2, 1, 16, 2, 4100),        # 8 query rows, slices of 64 keys, two blocks to an SM and a few more
+    (3, 300, 8, 8, 310),        # many row blocks, the last of 12 rows
+    (2, 40, 16, 1, 129),        # 16 query heads per kv head
+])
+def test_attention_head_dim_64(dmtd, dtype, B, R, nq, nkv, n_keys):
+    D, G, pos0 = 64, nq // nkv, n_keys - R
+    g = torch.Generator(device="cuda").manual_seed(12)
+    q = torch.randn(B, R, nq, D, generator=g, device="cuda") * 2
+    k, v = (torch.randn(B, nkv, n_keys + 3, D, generator=g, device="cuda").to(dtype) for _ in range(2))
+    k[:, :, n_keys:] = float("nan")                          # nothing behind the last key may be used
+    v[:, :, n_keys:] = float("nan")
+    out = dmtd.attention_decode(q, k, v, pos0)
+    for b in range(B):
+        kd, vd = (x[b, :, :n_keys].double().repeat_interleave(G, 0) for x in (k, v))
+        s = torch.einsum("rhd,hkd->hrk", q[b].double(), kd) / D ** 0.5
+        hidden = torch.arange(n_keys, device="cuda")[None] > (pos0 + torch.arange(R, device="cuda"))[:, None]
+        ref = torch.einsum("hrk,hkd->rhd", torch.softmax(s.masked_fill(hidden, float("-inf")), -1), vd)
+        # fp32 throughout: scores of size below 16 to 2^-20, the exponential's two units in the last place
+        assert (out[b].double() - ref).abs().max() <= 2e-5 * max(1.0, ref.abs().max().item())

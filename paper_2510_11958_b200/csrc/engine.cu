@@ -391,8 +391,14 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   // layer's projections at 3 rows in 82 us against 58 (kernel times)
   if (U.w && c->use_umma) return launch_gemm_tc05(c, U, rows_input(act, lda), M, out, ldo);
   if (W.wf) {
-    CUDA_TRY(c, launch_pdl(gemv_f32_kernel, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream,
-                            W, act, lda, M, out, ldo));
+    // A launch of more than a few microseconds of arithmetic starts when everything in front is complete: as a dependent
+    // launch its blocks come to lie unevenly on the SMs, where the kernel in front still has blocks.  Layers of fp32 models,
+    // dependent against plain: 24 rows of hidden 256 (9 M products in gate+up) 163 us against 175, 12 rows of 512 (19 M) 167
+    // against 179, 24 rows of 512 (38 M) 313 against 292, 32 rows of 1024 (201 M) 699 against 638.
+    if ((long long)M * W.N * W.K <= (32ll << 20))
+      CUDA_TRY(c, launch_pdl(gemv_f32_kernel, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream, W, act, lda, M, out, ldo, 1));
+    else
+      gemv_f32_kernel<<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo, 0);
     LAUNCH_OK(c, "gemv_f32_kernel");
     return DMTD_OK;
   }
@@ -600,6 +606,14 @@ dmtd_status launch_gemv_f32_fused(dmtd_ctx *c, const PackedMat &W, const F32In &
   LAUNCH_OK(c, "gemv_f32_fused_kernel");
   return DMTD_OK;
 }
+// Every block of the O projection would merge all key slices again: more than 8192 values of them (of slices that hold keys; a
+// captured pass keeps what held when it was captured) are merged by a kernel of their own.  Four layers of fp32 models, merged
+// in front of the product against apart: 2048 values 82 us against 92, 4096 to 8192 within 5 % of each other, 32768 1.34 times
+// as long, 327680 (4 rows of 16 heads x 128, 40 slices) 942 us against 360.
+bool merge_apart(const dmtd_ctx *c, int M, int nsplit, int pos_end) {
+  const int keys = tc_decode_attention(c) ? AD_UNIT : c->CH, live = std::min(nsplit, (pos_end + keys - 1) / keys);
+  return (long long)M * c->s.n_q_heads * c->s.head_dim * live > 8192;
+}
 F32In f32_norm_input(const dmtd_ctx *c, const float *x, const float *w) { return F32In{x, c->s.hidden, w, c->s.rms_eps, nullptr, nullptr, 0, 0}; }
 
 // One decoder layer (steps a2-a7) on x [B*R][hidden]; rows of sequence b sit at positions
@@ -613,8 +627,10 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   if (f32_fused_rows(c, M) && !flash_attention_ok(c, R)) {
     const int nsplit = slices_for(c, B, R, pos_end);
     TRY(launch_gemv_f32_fused<F32_NORM>(c, lw.qkv, f32_norm_input(c, x, lw.w_in), M, c->qkv, c->ldqkv, true));
-    TRY(launch_attention(c, l, B, R, pos0, nsplit, false));
-    TRY(launch_gemv_f32_fused<F32_SLICES>(c, lw.o, F32In{nullptr, 0, nullptr, 0.f, c->part_o, c->part_ml, nsplit, s.n_q_heads}, M, x, H, false));
+    const bool apart = merge_apart(c, M, nsplit, pos_end);
+    TRY(launch_attention(c, l, B, R, pos0, nsplit, apart));
+    if (apart) TRY(launch_gemv(c, lw.o, lw.o_u, c->act, c->lda, M, x, H));
+    else TRY(launch_gemv_f32_fused<F32_SLICES>(c, lw.o, F32In{nullptr, 0, nullptr, 0.f, c->part_o, c->part_ml, nsplit, s.n_q_heads}, M, x, H, false));
     TRY(launch_gemv_f32_fused<F32_NORM>(c, lw.gu, f32_norm_input(c, x, lw.w_post), M, c->gu, c->ldgu, true));
     return launch_gemv_f32_fused<F32_SWIGLU>(c, lw.down, F32In{c->gu, c->ldgu, nullptr, 0.f, nullptr, nullptr, 0, 0}, M, x, H, false);
   }

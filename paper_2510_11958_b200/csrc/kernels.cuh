@@ -251,10 +251,11 @@ gemv_bf16_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
   }
 }
 
-// Projection, fp32 weights (small verification models only): one warp per output row.
+// Projection, fp32 weights (small verification models only): one warp per output row.  early: launched with programmatic
+// stream serialisation.
 __global__ void gemv_f32_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
-                                float *__restrict__ out, int ldo) {
-  pdl_enter();
+                                float *__restrict__ out, int ldo, int early) {
+  if (early) pdl_enter();
   int lane = threadIdx.x & 31;
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
   for (int n = warp; n < W.N; n += n_warps) {

@@ -191,3 +191,20 @@ def test_large_chunk_against_small_ones(dmtd, wide_weights, layers, R):
     ref = torch.cat([eng.step_layers(0, layers, rows[:, p:p + 200].clone(), p) for p in range(0, R, 200)], 1)
     # sums of at most 9728 products in another order, activations within 2^-17 on both sides
     assert (got - ref).abs().max() <= 1e-4 * max(1.0, ref.abs().max().item())
+
+
+@pytest.mark.parametrize("P,B,tau", [
+    (500, 1, 4),        # 4 rows x 4 heads x 64 x 8 slices: the most that the O projection merges itself
+    (513, 1, 4),        # one slice more
+    (130, 11, 1),       # 11 rows, 3 slices
+])
+def test_f32_slices_merged_apart(dmtd, P, B, tau):
+    shape = SHAPES["tiny"].with_(n_layers=2, vocab=500)
+    w = make_weights(shape, seed=0, norm_jitter=0.1)
+    prompts = make_prompts(shape.vocab, B, P, seed=1).numpy()
+    forced = make_prompts(shape.vocab, B, tau + 2, seed=2).numpy()
+    ref_logits, ref_am, o = oracle_forced(shape, w, 1, tau, prompts, forced)
+    eng = dmtd.Dmtd(shape, to_cuda(w), L_d=1, tau=tau, max_batch=B, max_seq=P + forced.shape[1] + 1, kv_dtype="f32")
+    got_logits, got_am = gpu_forced(eng, prompts, forced)
+    err, _ = check_logits(got_logits, ref_logits, got_am, ref_am)
+    assert err < 1e-3       # fp32 sums of fp32 products, as above

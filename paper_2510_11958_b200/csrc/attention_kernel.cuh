@@ -244,9 +244,9 @@ struct AttnShares {
 // part_o / part_ml: `nsplit` slots per (row, head); the pieces of an item take slots 0, 1, ...; the rest are marked empty.
 template <class Op, bool FUSED = false>
 __global__ void __launch_bounds__(AD_THREADS, 2)
-attn_decode_kernel(const float *__restrict__ qkv, int ldq, const void *__restrict__ kc, const void *__restrict__ vc, int max_seq,
-                   int nq, int nkv, int B, int R, int RB, const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
-                   float *__restrict__ part_ml, int nsplit, AttnFuse F = AttnFuse{nullptr, nullptr, nullptr, 0.f}) {
+attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, int max_seq,
+                   int nq, int nkv, int B, int R, int RB, const int *__restrict__ pos0_ptr, int pos0_val, float *part_o,
+                   float *part_ml, int nsplit, AttnFuse F = AttnFuse{nullptr, nullptr, nullptr, 0.f}) {
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int G = nq / nkv, n_rb = (R + RB - 1) / RB;
@@ -462,9 +462,9 @@ using StepF32Map = AttnF32Map<64>;
 constexpr int ATTN_F32_SMEM = StepF32Map::NEW;           // K and V tile, Q, partial scores, running max / sum / rescale factor
 
 __global__ void __launch_bounds__(PK_THREADS, 2)
-attn_f32_kernel(const float *__restrict__ qkv, int ldq, const float *__restrict__ kc, const float *__restrict__ vc, int max_seq,
-                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
-                float *__restrict__ part_ml, int nsplit) {
+attn_f32_kernel(const float *qkv, int ldq, const float *kc, const float *vc, int max_seq,
+                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, int pos0_val, float *part_o,
+                float *part_ml, int nsplit) {
   pdl_enter();
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

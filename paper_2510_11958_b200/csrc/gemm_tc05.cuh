@@ -573,8 +573,8 @@ struct GateUpParts {
   }
 };
 template <bool GATED>
-__global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *__restrict__ act, int lda, int rows, ActTiles T,
-                                                                uint4 *__restrict__ blocks, int kb0, GateUpParts parts) {
+__global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *act, int lda, int rows, ActTiles T,
+                                                                uint4 *blocks, int kb0, GateUpParts parts) {
   // lanes of a row, 16-byte loads of a lane, and 32-bit registers of a part that a load becomes
   constexpr int LANES = GATED ? 32 : 16, LOADS = AB_ROWS * LANES / 32, REGS = GATED ? 1 : 2;
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
@@ -683,7 +683,7 @@ struct RowSegments {
 // squares.  What a thread's first unit needs is requested beside the rows, so that the whole costs one trip to memory
 // (as two, and with the rows' loads in small batches, 5.5 us a launch instead of 4.5).  part: 8 floats of shared memory.
 __device__ __forceinline__ void norm_group(const float *x, int ldx, RowSegments seg, const float *__restrict__ w, float eps, int rows_all,
-                                           int K, const ActTiles &T, uint4 *__restrict__ blocks, int m0, int kb_lo, int kb_hi, float *part,
+                                           int K, const ActTiles &T, uint4 *blocks, int m0, int kb_lo, int kb_hi, float *part,
                                            int tid) {
   const int warp = tid >> 5, lane = tid & 31;
   // unit = (k block, k chunk of 8, row of the group): this thread writes the row's hi and lo parts
@@ -730,9 +730,9 @@ __device__ __forceinline__ void norm_group(const float *x, int ldx, RowSegments 
   }
 }
 
-__global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *__restrict__ x, int ldx, RowSegments seg,
+__global__ void __launch_bounds__(256) norm_act_blocks_kernel(const float *x, int ldx, RowSegments seg,
                                                               const float *__restrict__ w, float eps, int rows_all, int K,
-                                                              ActTiles T, uint4 *__restrict__ blocks, int n_groups,
+                                                              ActTiles T, uint4 *blocks, int n_groups,
                                                               ZeroArea zero_area) {
   // the GEMM that follows may be scheduled already: it waits for this grid before it reads the blocks
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -770,8 +770,8 @@ constexpr int MAB_MAX_SLOTS = 2048;            // (rows of a group) x heads x sl
 // sum (one thread per row and head, into wgt), then the merged values.  A thread's first unit has its first slices
 // requested beside the weights' inputs: one trip to memory for up to four slices.
 constexpr int MERGE_AHEAD = 4;
-__device__ __forceinline__ void merge_group(const float *__restrict__ part_o, const float *__restrict__ part_ml, int nsplit, int nq, int D,
-                                            int rows_all, const ActTiles &T, uint4 *__restrict__ blocks, int m0, int kb_lo, int kb_hi,
+__device__ __forceinline__ void merge_group(const float *part_o, const float *part_ml, int nsplit, int nq, int D,
+                                            int rows_all, const ActTiles &T, uint4 *blocks, int m0, int kb_lo, int kb_hi,
                                             float *wgt, int tid) {
   const int r = tid % NAB_ROWS, c = (tid / NAB_ROWS) % 8, m = m0 + r, total = (kb_hi - kb_lo) * 8 * NAB_ROWS;
   const bool row_ok = m < rows_all;
@@ -833,9 +833,9 @@ __device__ __forceinline__ void merge_group(const float *__restrict__ part_o, co
     store_hi_lo(f, blocks + T.unit(m, kb_lo + u / (NAB_ROWS * 8), c), T.lo_offset());
   }
 }
-__global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml,
+__global__ void __launch_bounds__(256) merge_act_blocks_kernel(const float *part_o, const float *part_ml,
                                                                int nsplit, int nq, int D, int rows_all, ActTiles T,
-                                                               uint4 *__restrict__ blocks) {
+                                                               uint4 *blocks) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ... and this grid may itself have started before the kernel before it has finished (the GEMM of the previous
   // projection lets its dependents in at once): nothing is read or written before that kernel is complete

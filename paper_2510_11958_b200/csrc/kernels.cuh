@@ -12,6 +12,9 @@ namespace dmtd {
 // resident now (it does the same, or touches nothing but weights and the cache rows of earlier passes before it waits);
 // nothing is read or written here before the kernels in front are complete.  Kernels without it are launched
 // plainly: they start when everything before them is complete.
+// What an earlier grid of such a chain writes (activations, partial results, the cache) changes while this one is
+// running: such parameters are not __restrict__, which would allow loads that assume the opposite or are moved in front of
+// the wait.  Weights, norm gains and the rotary table are.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -73,7 +76,7 @@ __device__ __forceinline__ void rope_entry(const RopeTable &T, int pos0, int R, 
 }
 // grid (rows + blocks of the table), 128 threads
 __global__ void embed_kernel(PackedMat E, const int *__restrict__ tokens, int max_seq,
-                             const int *__restrict__ pos0, int R, int n_rows, float *__restrict__ x, int ldx,
+                             const int *__restrict__ pos0, int R, int n_rows, float *x, int ldx,
                              int accumulate, DevState *st, RopeTable rope) {
   if (blockIdx.x >= n_rows) return rope_entry(rope, *pos0, R, (blockIdx.x - n_rows) * blockDim.x + threadIdx.x);
   int m = blockIdx.x, b = m / R, r = m % R;
@@ -110,9 +113,9 @@ __global__ void embed_kernel(PackedMat E, const int *__restrict__ tokens, int ma
 // PREP_ZERO_COLS columns of its row's accumulator, the first block of a row also does the norm.
 // ------------------------------------------------------------------------------------
 constexpr int PREP_ZERO_COLS = 4096;
-__global__ void prep_norm_kernel(const float *__restrict__ x, int ldx, const float *__restrict__ w,
-                                 int K, float eps, float *__restrict__ act, int lda,
-                                 float *__restrict__ zero_buf, int zero_ld, int zero_cols) {
+__global__ void prep_norm_kernel(const float *x, int ldx, const float *__restrict__ w,
+                                 int K, float eps, float *act, int lda,
+                                 float *zero_buf, int zero_ld, int zero_cols) {
   pdl_enter();
   const int m = blockIdx.x;
   if (zero_buf) {
@@ -143,8 +146,8 @@ __global__ void prep_norm_kernel(const float *__restrict__ x, int ldx, const flo
 }
 
 // act[m][i] = silu(g) * u with g = gu[m][i], u = gu[m][I + i]  (the SwiGLU gate).
-__global__ void prep_swiglu_kernel(const float *__restrict__ gu, int ldgu, int I,
-                                   float *__restrict__ act, int lda) {
+__global__ void prep_swiglu_kernel(const float *gu, int ldgu, int I,
+                                   float *act, int lda) {
   pdl_enter();
   int m = blockIdx.y;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -166,8 +169,8 @@ __global__ void prep_swiglu_kernel(const float *__restrict__ gu, int ldgu, int I
 // ------------------------------------------------------------------------------------
 template <int NT>
 __global__ void __launch_bounds__(GEMV_THREADS)
-gemv_bf16_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
-                 float *__restrict__ out, int ldo) {
+gemv_bf16_kernel(PackedMat W, const float *act, int lda, int M,
+                 float *out, int ldo) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int KS = W.aps * 32;
@@ -253,8 +256,8 @@ gemv_bf16_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
 
 // Projection, fp32 weights (small verification models only): one warp per output row.  early: launched with programmatic
 // stream serialisation.
-__global__ void gemv_f32_kernel(PackedMat W, const float *__restrict__ act, int lda, int M,
-                                float *__restrict__ out, int ldo, int early) {
+__global__ void gemv_f32_kernel(PackedMat W, const float *act, int lda, int M,
+                                float *out, int ldo, int early) {
   if (early) pdl_enter();
   int lane = threadIdx.x & 31;
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
@@ -299,7 +302,7 @@ struct F32In {
   int nsplit, nq;
 };
 template <int IN>
-__global__ void __launch_bounds__(256) gemv_f32_fused_kernel(PackedMat W, F32In in, int M, float *__restrict__ out, int ldo, int store) {
+__global__ void __launch_bounds__(256) gemv_f32_fused_kernel(PackedMat W, F32In in, int M, float *out, int ldo, int store) {
   extern __shared__ __align__(16) float xs[];                       // [M][K]
   __shared__ float ss_part[8][F32_FUSE_ROWS];                       // F32_NORM: sums of squares, by a row's warps
   const int lane = threadIdx.x & 31, w8 = threadIdx.x >> 5, K = W.K;
@@ -447,11 +450,11 @@ template <> __device__ __forceinline__ __half to_kv<__half>(float v) { return __
 // and rotated in place (fp32); k is normalised, rotated and stored in the cache; v is stored.
 // qkv [M][ldq] = (q | k | v) per row.  Cache layout [b][kv head][max_seq][D].
 template <int D, typename KVT>
-__global__ void qk_norm_rope_append_kernel(float *__restrict__ qkv, int ldq, int nq, int nkv, int R,
+__global__ void qk_norm_rope_append_kernel(float *qkv, int ldq, int nq, int nkv, int R,
                                            const float *__restrict__ w_qn, const float *__restrict__ w_kn,
                                            float eps, const float2 *__restrict__ table,
-                                           const int *__restrict__ pos0, KVT *__restrict__ kc,
-                                           KVT *__restrict__ vc, int max_seq) {
+                                           const int *__restrict__ pos0, KVT *kc,
+                                           KVT *vc, int max_seq) {
   pdl_enter();
   constexpr int E = D / 32;                 // values per lane; value j pairs with j + E/2
   int lane = threadIdx.x & 31;
@@ -567,10 +570,10 @@ template <> __device__ __forceinline__ void load8<__half>(const __half *p, float
 // loads.  32 x 8192 keys, 8 kv heads of bf16 rows: 234 us with T = 4, 460 with T = 1.
 template <int D, typename KVT, int NQ, bool FUSED, int T>
 __global__ void __launch_bounds__(attn_warps(T) * 32, T == 1 ? 1 : D == 64 ? 4 : 3)
-attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restrict__ kc,
-                    const KVT *__restrict__ vc, int max_seq, int nq, int nkv, int R, int RB, int CH,
-                    const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
-                    float *__restrict__ part_ml, int nsplit, AttnFuse F) {
+attn_partial_kernel(const float *qkv, int ldq, const KVT *kc,
+                    const KVT *vc, int max_seq, int nq, int nkv, int R, int RB, int CH,
+                    const int *__restrict__ pos0_ptr, int pos0_val, float *part_o,
+                    float *part_ml, int nsplit, AttnFuse F) {
   constexpr int E = D / 32, NC = D / 32, W = attn_warps(T), TK = 8 * T;   // V: dims lane * E ..; K: NC chunks of 8 dims per lane
   const int G = nq / nkv;
   const int split = blockIdx.x, n_rb = (R + RB - 1) / RB;
@@ -795,8 +798,8 @@ attn_partial_kernel(const float *__restrict__ qkv, int ldq, const KVT *__restric
 
 // One warp per (row, head): act[m][h*D + :] = sum_s w_s o_s / sum_s w_s l_s, w_s = exp(m_s - max m).
 template <int D>
-__global__ void attn_merge_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml,
-                                  int nsplit, int n_rows_heads, int nq, float *__restrict__ act, int lda) {
+__global__ void attn_merge_kernel(const float *part_o, const float *part_ml,
+                                  int nsplit, int n_rows_heads, int nq, float *act, int lda) {
   pdl_enter();
   constexpr int E = D / 32;
   int lane = threadIdx.x & 31;
@@ -829,7 +832,7 @@ __global__ void attn_merge_kernel(const float *__restrict__ part_o, const float 
 // a8: the lower->upper boundary of a full pass.  Only the newest row of each sequence goes
 // on into the decoding layers (Section 2.2); the refill rows' outputs are dropped.
 // ------------------------------------------------------------------------------------
-__global__ void select_last_kernel(const float *__restrict__ x_lo, int R, int H, float *__restrict__ x_up) {
+__global__ void select_last_kernel(const float *x_lo, int R, int H, float *x_up) {
   pdl_enter();
   int b = blockIdx.x;
   const float *src = x_lo + ((size_t)b * R + (R - 1)) * H;
@@ -843,7 +846,7 @@ __global__ void select_last_kernel(const float *__restrict__ x_lo, int R, int H,
 // (pending row = position - lo_len) and fed to them at the next full pass.
 // ------------------------------------------------------------------------------------
 // pend[b][newest - lo_len][:] = x_up[b][:]
-__global__ void save_pending_kernel(const float *__restrict__ x_up, float *__restrict__ pend, int pend_cap, int H,
+__global__ void save_pending_kernel(const float *x_up, float *__restrict__ pend, int pend_cap, int H,
                                     const DevState *st) {
   const int b = blockIdx.x, r = st->newest - st->lo_len;
   if (r < 0 || r >= pend_cap) return;
@@ -852,8 +855,8 @@ __global__ void save_pending_kernel(const float *__restrict__ x_up, float *__res
 }
 
 // x_lo[b][r][:] = pend[b][r][:] for r < R - 1, x_up[b][:] for the newest row r = R - 1
-__global__ void gather_pending_kernel(const float *__restrict__ pend, int pend_cap, const float *__restrict__ x_up, int R, int H,
-                                      float *__restrict__ x_lo) {
+__global__ void gather_pending_kernel(const float *__restrict__ pend, int pend_cap, const float *x_up, int R, int H,
+                                      float *x_lo) {
   const int b = blockIdx.x / R, r = blockIdx.x % R;
   const float *src = r < R - 1 ? pend + ((size_t)b * pend_cap + r) * H : x_up + (size_t)b * H;
   float *dst = x_lo + (size_t)blockIdx.x * H;
@@ -876,7 +879,7 @@ __global__ void copy_rows_kernel(const float *__restrict__ src, float *__restric
 // p0 + r; at a mask position (inside the prompt, or (p - (P-1)) mod tau == 0: the anchors of
 // Section 2.2) the decoding layers read h_think (x), or base + h_think with the literal sum of
 // Eq. 4; elsewhere they read base (h_emb, or h_enc when encoding layers are reused).
-__global__ void masked_select_kernel(float *__restrict__ x, const float *__restrict__ base, int R, int H, int p0, int P,
+__global__ void masked_select_kernel(float *x, const float *__restrict__ base, int R, int H, int p0, int P,
                                      int tau, int literal_sum) {
   const int r = blockIdx.x % R, p = p0 + r;
   const bool m = p < P || (p - (P - 1)) % tau == 0;
@@ -936,7 +939,7 @@ struct PickParams {
 };
 
 // grid (sequences, ARGMAX_SLICES), 256 threads
-__global__ void argmax_kernel(const float *__restrict__ logits, int ldl, int V, DevState *st, SampleParams sp, PickParams pp) {
+__global__ void argmax_kernel(const float *logits, int ldl, int V, DevState *st, SampleParams sp, PickParams pp) {
   pdl_enter();
   const int b = blockIdx.x, per = ((V + gridDim.y - 1) / gridDim.y + 3) & ~3;      // whole 16-byte loads
   const int i0 = blockIdx.y * per, i1 = min(V, i0 + per);

@@ -193,7 +193,7 @@ def measure_workload(eng, wl, shape, prompts, tau, K, W, replicas, want_tau1=Tru
 
 
 def roofline_of(shape, wl, tau, res, K, peak, peak_src):
-    """The roofline object of one measured workload (see the design doc for the byte model)."""
+    """The roofline object of one measured workload (bytes_per_cycle is its byte model)."""
     kvb = 4 if wl.kv_dtype == "f32" else 2
     cyc_bytes = bytes_per_cycle(shape, wl.L_d, tau, wl.batch, res["mean_ctx"], kv_bytes=kvb)
     cyc_bytes_bf16kv = bytes_per_cycle(shape, wl.L_d, tau, wl.batch, res["mean_ctx"], kv_bytes=2)

@@ -272,9 +272,10 @@ dmtd_status dmtd_get_kv(dmtd_ctx *ctx, int32_t layer, void **k, void **v);
 dmtd_status dmtd_debug_set_error_word(dmtd_ctx *ctx, int32_t word);
 
 /* Device memory the context holds, by purpose.  A bf16 context whose hidden, query and
- * intermediate sizes are multiples of 64 keeps its weights twice: as the atom stream the
- * pass kernel reads (passes of up to 4 rows) and as the 16 KiB blocks
- * the tcgen05 GEMM reads (everything else): 2 x 8.04 GB for the Qwen3-4B shape.
+ * intermediate sizes are multiples of 64 keeps its weights twice: as the atom stream that the
+ * pass kernel (passes of up to 4 rows of a context with max_batch <= 4), the embedding gather and
+ * the kernels of "tcgen05_gemm" 0 read, and as the 16 KiB blocks the tcgen05 GEMM reads
+ * (everything else): 2 x 8.04 GB for the Qwen3-4B shape.
  * With DMTD_WEIGHT_COPIES=1 in the environment at create only the first is kept. */
 typedef struct {
   size_t weight_stream_bytes, weight_block_bytes, kv_cache_bytes, workspace_bytes;

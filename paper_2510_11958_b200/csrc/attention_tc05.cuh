@@ -56,22 +56,6 @@ struct AttnPrefillParams {
   long long wait_limit;
 };
 
-__device__ __noinline__ bool ap_wait_slow(uint32_t bar, uint32_t parity, int *error, long long limit) {
-  const long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
-    const long long dt = clock64() - t0;
-    if (dt > (1 << 20) && (dt > limit || *reinterpret_cast<volatile int *>(error) >= TG_ERR_WAIT)) {
-      atomicMax(error, TG_ERR_WAIT);
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool ap_wait(uint32_t bar, uint32_t parity, const AttnPrefillParams &P) {
-  return mbar_try_wait(bar, parity) || ap_wait_slow(bar, parity, P.error, P.wait_limit);
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -185,14 +169,14 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     };
     bool ok = true;
     for (int i = 0; i < n_tiles && ok; ++i) {
-      if (i > 0) ok = ap_wait(bar_s, (i - 1) & 1, P);
+      if (i > 0) ok = tg_wait(bar_s, (i - 1) & 1, P);
       if (!ok) break;
       fetch(kb, i * AP_TK, smem + AP_K);
       if (i > 0) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");          // long done when P V (i - 1) is
         fence_proxy_async();
         mbar_arrive(bar_k);
-        ok = ap_wait(bar_o, (i - 1) & 1, P);
+        ok = tg_wait(bar_o, (i - 1) & 1, P);
         if (!ok) break;
         fetch(vb, i * AP_TK, smem + AP_V);
       } else {
@@ -211,10 +195,10 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     constexpr uint32_t fmt = std::is_same<typename Op::T, __half>::value ? 0u : 1u;       // A and B of one type
     const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
     const uint32_t idesc_pv = idesc | (1u << 16);                                         // B is N-major
-    bool ok = __all_sync(0xffffffffu, ap_wait(bar_q, 0, P));
+    bool ok = __all_sync(0xffffffffu, tg_wait(bar_q, 0, P));
     for (int i = 0; i < n_tiles && ok; ++i) {
-      ok = __all_sync(0xffffffffu, ap_wait(bar_k, i & 1, P));
-      if (i > 0) ok = __all_sync(0xffffffffu, ok && ap_wait(bar_o, (i - 1) & 1, P));      // P lies over S
+      ok = __all_sync(0xffffffffu, tg_wait(bar_k, i & 1, P));
+      if (i > 0) ok = __all_sync(0xffffffffu, ok && tg_wait(bar_o, (i - 1) & 1, P));      // P lies over S
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (elect_one()) {
@@ -232,7 +216,7 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_s) : "memory");
       }
       __syncwarp();
-      ok = __all_sync(0xffffffffu, ap_wait(bar_v, i & 1, P) && ap_wait(bar_p, i & 1, P));
+      ok = __all_sync(0xffffffffu, tg_wait(bar_v, i & 1, P) && tg_wait(bar_p, i & 1, P));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (elect_one()) {
@@ -274,7 +258,7 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
     float m_ref = -INFINITY, l = 0.f;                                 // reference maximum (times log2 e) and running sum
     bool ok = true;
     for (int i = 0; i < n_tiles; ++i) {
-      ok = __all_sync(0xffffffffu, ap_wait(bar_s, i & 1, P));
+      ok = __all_sync(0xffffffffu, tg_wait(bar_s, i & 1, P));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // keys of the tile this row sees: [0, lim); only the block's last tiles are cut
@@ -304,7 +288,7 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
         const bool grow = mx > m_ref + AP_RESCALE_LOG2;
         if (grow) { alpha = exp2_approx(m_ref - mx); m_ref = mx; l *= alpha; }
         if (__any_sync(0xffffffffu, grow)) {
-          ok = __all_sync(0xffffffffu, ap_wait(bar_o, (i - 1) & 1, P));
+          ok = __all_sync(0xffffffffu, tg_wait(bar_o, (i - 1) & 1, P));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
@@ -355,7 +339,7 @@ __global__ void __launch_bounds__(AP_THREADS, 2) attn_prefill_kernel(const __gri
       l += l0 + l1;
     }
     // ---- O / l: fp32 rows, or hi and lo units of the O projection's activations
-    if (ok && n_tiles > 0) ok = __all_sync(0xffffffffu, ap_wait(bar_o, (n_tiles - 1) & 1, P)) && !*gave_up;
+    if (ok && n_tiles > 0) ok = __all_sync(0xffffffffu, tg_wait(bar_o, (n_tiles - 1) & 1, P)) && !*gave_up;
     if (ok) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const float inv = 1.f / l;

@@ -1078,12 +1078,13 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   // every pass outside the pass kernel uses it
   c->umma_ok = s.weight_dtype == DMTD_BF16 && H % TG_KB == 0 && QD % TG_KB == 0 && I % TG_KB == 0;
   // DMTD_WEIGHT_COPIES=1 in the environment keeps only the atom stream (half the weight memory):
-  // every projection then runs on the mma.sync kernels, the prefill included (slower from 5 rows up)
+  // every projection then runs on the mma.sync kernels, the prefill included (slower at every row count)
   if (const char *e = getenv("DMTD_WEIGHT_COPIES")) if (atoi(e) == 1) c->umma_ok = false;
   c->layers.resize(s.n_layers);
-  // k-slab width of the packed matrices: contexts small enough for the pass kernel (which stages
-  // only the slabs a block's share touches, and gains from short ones) get 256-wide slabs;
-  // larger batches run the per-step GEMV, which is faster with 1280-wide slabs
+  // k-slab width of the packed matrices: contexts small enough for the pass kernel (which stages only the slabs a block's
+  // share touches, and gains from short ones) get 256-wide slabs; in larger ones the layers' streams are read by the
+  // mma.sync GEMV alone, which is faster with 1280-wide slabs (without the block copy, or with "tcgen05_gemm" off), and
+  // the head's by the embedding gather
   const int aps = max_batch <= PK_MAX_ROWS ? 8 : 40;
   for (int l = 0; l < s.n_layers; ++l) {
     const dmtd_layer_weights &lw = w->layers[l];

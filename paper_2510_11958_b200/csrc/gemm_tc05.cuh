@@ -144,21 +144,22 @@ __device__ __forceinline__ uint32_t umma_instr_desc(int m, int n) {
 // Bounded wait.  The error word (another block gave up) is looked at only after the wait has lasted half a
 // millisecond: a read of global memory inside the spin takes a microsecond under load, which made every wait that
 // long (head at 8 rows 2.2 TB/s instead of 6).
-__device__ __noinline__ bool tg_wait_slow(uint32_t bar, uint32_t parity, const GemmTcParams &P) {
+__device__ __noinline__ bool tg_wait_slow(uint32_t bar, uint32_t parity, int *error, long long limit) {
   const long long t0 = clock64();
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
       if (mbar_try_wait(bar, parity)) return true;
     const long long dt = clock64() - t0;
-    if (dt > (1 << 20) && (dt > P.wait_limit || *reinterpret_cast<volatile int *>(P.error) >= TG_ERR_WAIT)) {
-      atomicMax(P.error, TG_ERR_WAIT);
+    if (dt > (1 << 20) && (dt > limit || *reinterpret_cast<volatile int *>(error) >= TG_ERR_WAIT)) {
+      atomicMax(error, TG_ERR_WAIT);
       return false;
     }
   }
 }
-__device__ __forceinline__ bool tg_wait(uint32_t bar, uint32_t parity, const GemmTcParams &P) {
-  return mbar_try_wait(bar, parity) || tg_wait_slow(bar, parity, P);
+template <class Params>
+__device__ __forceinline__ bool tg_wait(uint32_t bar, uint32_t parity, const Params &P) {
+  return mbar_try_wait(bar, parity) || tg_wait_slow(bar, parity, P.error, P.wait_limit);
 }
 // Arrive on the barrier at the same place in the first SM of the pair.  Without a scope: what is handed over is the
 // completion of bulk copies and of tensor-memory loads, not this thread's stores, and an arrive that releases at
@@ -398,7 +399,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      ok = __all_sync(0xffffffffu, mbar_try_wait(full, ph)) || __all_sync(0xffffffffu, tg_wait_slow(full, ph, P));
+      ok = __all_sync(0xffffffffu, mbar_try_wait(full, ph)) || __all_sync(0xffffffffu, tg_wait_slow(full, ph, P.error, P.wait_limit));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int n = min(min(KPS, n_kb - kb), i < n_part ? n_part - i : KPS);

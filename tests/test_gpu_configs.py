@@ -24,7 +24,7 @@ from helpers import LOGIT_ATOL, check_logits, gpu_forced, oracle_forced, to_cuda
 
 pytestmark = pytest.mark.gpu
 
-# Measured on the 36-layer model (readings): a bf16 KV cache alone moves the logits by
+# Measured on the 36-layer model: a bf16 KV cache alone moves the logits by
 # about 0.06 at full depth, which is why the workloads whose logits are held to 2e-2 keep an fp32
 # cache.  The bound asserted below is that measurement with head-room, so that a kernel fault in the
 # bf16 attention path (errors of order 1) cannot hide behind it.

@@ -462,9 +462,9 @@ using StepF32Map = AttnF32Map<64>;
 constexpr int ATTN_F32_SMEM = StepF32Map::NEW;           // K and V tile, Q, partial scores, running max / sum / rescale factor
 
 __global__ void __launch_bounds__(PK_THREADS, 2)
-attn_f32_kernel(const float *qkv, int ldq, const float *kc, const float *vc, int max_seq,
-                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, int pos0_val, float *part_o,
-                float *part_ml, int nsplit) {
+attn_f32_kernel(const float *qkv, int ldq, const float *__restrict__ kc, const float *__restrict__ vc, int max_seq,
+                int nq, int nkv, int R, int RB, int CH, const int *__restrict__ pos0_ptr, int pos0_val, float *__restrict__ part_o,
+                float *__restrict__ part_ml, int nsplit) {
   pdl_enter();
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -487,7 +487,7 @@ attn_f32_kernel(const float *qkv, int ldq, const float *kc, const float *vc, int
     const float *src = qkv + (size_t)(b * R + r0 + qi / G) * ldq + (size_t)(kvh * G + qi % G) * PK_D;
     float *dst = reinterpret_cast<float *>(sc + StepF32Map::Q) + qi * PK_D;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) dst[lane + 32 * j] = src[lane + 32 * j] * scale;
+    for (int j = 0; j < 4; ++j) dst[lane + 32 * j] = __ldcg(src + lane + 32 * j) * scale;
   }
   float *const m_run = reinterpret_cast<float *>(sc + StepF32Map::STAT), *const l_run = m_run + PK_QR;
   if ((int)threadIdx.x < PK_QR) { m_run[threadIdx.x] = -INFINITY; l_run[threadIdx.x] = 0.f; }

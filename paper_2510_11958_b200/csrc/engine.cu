@@ -396,9 +396,9 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
     // dependent against plain: 24 rows of hidden 256 (9 M products in gate+up) 163 us against 175, 12 rows of 512 (19 M) 167
     // against 179, 24 rows of 512 (38 M) 313 against 292, 32 rows of 1024 (201 M) 699 against 638.
     if ((long long)M * W.N * W.K <= (32ll << 20))
-      CUDA_TRY(c, launch_pdl(gemv_f32_kernel, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream, W, act, lda, M, out, ldo, 1));
+      CUDA_TRY(c, launch_pdl(gemv_f32_kernel<true>, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream, W, act, lda, M, out, ldo));
     else
-      gemv_f32_kernel<<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo, 0);
+      gemv_f32_kernel<false><<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo);
     LAUNCH_OK(c, "gemv_f32_kernel");
     return DMTD_OK;
   }

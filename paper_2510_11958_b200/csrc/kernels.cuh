@@ -14,7 +14,8 @@ namespace dmtd {
 // plainly: they start when everything before them is complete.
 // What an earlier grid of such a chain writes (activations, partial results, the cache) changes while this one is
 // running: such parameters are not __restrict__, which would allow loads that assume the opposite or are moved in front of
-// the wait.  Weights, norm gains and the rotary table are.
+// the wait.  Weights, norm gains and the rotary table are; where a buffer is read by volatile instructions only (asynchronous
+// copies, __ldcg), which keep their order to the wait, it may be.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -254,11 +255,13 @@ gemv_bf16_kernel(PackedMat W, const float *act, int lda, int M,
   }
 }
 
-// Projection, fp32 weights (small verification models only): one warp per output row.  early: launched with programmatic
-// stream serialisation.
+// Projection, fp32 weights (small verification models only): one warp per output row.  EARLY: launched with programmatic
+// stream serialisation; otherwise the activations are complete before it starts and are read as constants (3 % of a layer
+// of hidden 1024 at 64 rows and more).
+template <bool EARLY>
 __global__ void gemv_f32_kernel(PackedMat W, const float *act, int lda, int M,
-                                float *out, int ldo, int early) {
-  if (early) pdl_enter();
+                                float *out, int ldo) {
+  if (EARLY) pdl_enter();
   int lane = threadIdx.x & 31;
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
   for (int n = warp; n < W.N; n += n_warps) {
@@ -270,7 +273,8 @@ __global__ void gemv_f32_kernel(PackedMat W, const float *act, int lda, int M,
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           if (m0 + i < M) {
-            float4 a = *reinterpret_cast<const float4 *>(act + (size_t)(m0 + i) * lda + k);
+            const float4 *ap = reinterpret_cast<const float4 *>(act + (size_t)(m0 + i) * lda + k);
+            const float4 a = EARLY ? *ap : __ldg(ap);
             acc[i] += w.x * a.x + w.y * a.y + w.z * a.z + w.w * a.w;
           }
       }

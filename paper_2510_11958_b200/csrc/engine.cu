@@ -321,10 +321,12 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
   uint4 *blocks = in.blocks ? in.blocks : c->act_blocks;
   P.act_blocks = blocks;
   const int n_pairs = c->n_sms / 2;
-  // Tiles dealt out whole: gate+up where it gates, and matrices of many rounds of tiles (the head).  With one round (gate+up
-  // of a decode pass) the part of a tile in front of it costs an epilogue more than the clearing it saves: batch 32
-  // 23.3 ms for 4 cycles instead of 22.8, batch 3 24.3 instead of 24.0 for 6.
-  const int whole = in.kind != GemmInput::NORM ? TG_ADD : gated ? TG_SWIGLU : W.n_tiles / 2 >= 4 * n_pairs ? TG_STORE : TG_ADD;
+  // Tiles dealt out whole: gate+up where it gates, and matrices of two rounds of tiles and more (the head).  With one round (gate+up
+  // of a decode pass) the part of a tile in front of it costs an epilogue more than the clearing it saves.  A pass of one
+  // layer and a head of 1 / 2 / 4 / 6 rounds, stored against added: 32 rows 110.6 / 125.2 / 156.0 / 186.8 us against 108.9 / 125.3 /
+  // 158.8 / 190.5, 8 rows 96.0 / 109.7 / 139.1 / 168.3 against 95.8 / 110.3 / 140.1 / 169.7, 96 rows 153.2 / 170.3 / 206.2 / 239.7
+  // against 155.6 / 174.7 / 213.8 / 255.1.
+  const int whole = in.kind != GemmInput::NORM ? TG_ADD : gated ? TG_SWIGLU : W.n_tiles / 2 >= 2 * n_pairs ? TG_STORE : TG_ADD;
   P.rt_whole = tg_whole_pairs(W, whole, n_pairs);
   P.whole_units = P.rt_whole / n_pairs * P.T.n_ctiles * W.n_kb;
   const int tiles = (W.n_tiles / 2 - P.rt_whole) * P.T.n_ctiles;

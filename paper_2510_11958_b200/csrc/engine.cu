@@ -469,7 +469,7 @@ bool repeats(const dmtd_ctx *c, int M) {
   const size_t gu_parts = gu_tiles == 0 ? 0 : gu.q == 0 ? n_pairs : std::max(0, lw.gu_u.n_kb - 2) / gu.q + 2;
   const size_t n_rest = std::max(0, lw.gu_u.N - gu_whole * 2 * TG_ROWS);
   return lw.qkv_u.n_tiles / 2 * n_ct >= n_pairs && uncut(lw.o_u) && uncut(lw.down_u) &&
-         gu_parts * n_rest * M <= (size_t)c->ws_rows * c->ldgu;
+         (gu_tiles >= n_pairs || gu_parts * n_rest * M <= (size_t)c->ws_rows * c->ldgu);
 }
 
 template <int D, typename KVT>
@@ -672,11 +672,11 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
       const int n_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, c->n_sms / 2) * 2 * TG_ROWS, n_rest = std::max(0, 2 * I - n_whole);
       down.lda = std::max(4, n_rest); down.kb0 = n_whole / 2 / TG_KB; down.blocks = c->gated_blocks;
       GemmInput gu = norm_input(x, H, lw.w_post);
-      if (same_bits && n_rest) {
-        const ActTiles T = act_tiles_for(M, lw.gu_u.n_kb);
+      const ActTiles T = act_tiles_for(M, lw.gu_u.n_kb);
+      const int tiles = (lw.gu_u.n_tiles / 2 - n_whole / (2 * TG_ROWS)) * T.n_ctiles;       // cut ones
+      if (same_bits && tiles > 0 && tiles < c->n_sms / 2) {       // (a tile for every block pair: two parts at most, as QKV's)
         gu.part_stride = (size_t)M * down.lda;
-        down.gu = GateUpParts{tg_line((lw.gu_u.n_tiles / 2 - n_whole / (2 * TG_ROWS)) * T.n_ctiles, T.n_kb, c->n_sms / 2), T.n_ctiles, T.n_kb,
-                              T.tile_rows, gu.part_stride};
+        down.gu = GateUpParts{tg_line(tiles, T.n_kb, c->n_sms / 2), T.n_ctiles, T.n_kb, T.tile_rows, gu.part_stride};
       }
       TRY(launch_gemm_tc05(c, lw.gu_u, gu, M, c->gu, down.lda, c->gated_blocks, projection_tiles(c, lw.down_u, M, same_bits)));
     } else {

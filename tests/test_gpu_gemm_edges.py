@@ -193,6 +193,22 @@ def test_large_chunk_against_small_ones(dmtd, wide_weights, layers, R):
     assert (got - ref).abs().max() <= 1e-4 * max(1.0, ref.abs().max().item())
 
 
+@pytest.mark.parametrize("intermediate", [
+    6400,       # gate+up in 50 row-tile pairs: none dealt out whole, its tiles in two parts at most
+    9472,       # 74: all dealt out whole
+])
+def test_large_chunk_repeats_at_other_widths(dmtd, intermediate):
+    shape = WIDE.with_(n_layers=1, intermediate=intermediate, vocab=600)
+    eng = dmtd.Dmtd(shape, make_weights(shape, seed=0, device="cuda", norm_jitter=0.1), L_d=1, tau=1, max_batch=1, max_seq=951, kv_dtype="f16")
+    rows = torch.randn(1, 950, shape.hidden, generator=torch.Generator().manual_seed(3)).cuda()
+    first = eng.step_layers(0, 1, rows.clone(), 0)
+    for _ in range(3):
+        assert torch.equal(eng.step_layers(0, 1, rows.clone(), 0), first)
+    ref = torch.cat([eng.step_layers(0, 1, rows[:, p:p + 200].clone(), p) for p in range(0, 950, 200)], 1)
+    # as above; the fp16 cache rounds K and V of sums in another order (2^-11), the query and the probabilities too
+    assert (first - ref).abs().max() <= 2e-3 * max(1.0, ref.abs().max().item())
+
+
 @pytest.mark.parametrize("P,B,tau", [
     (500, 1, 4),        # 4 rows x 4 heads x 64 x 8 slices: the most that the O projection merges itself
     (513, 1, 4),        # one slice more

@@ -354,7 +354,7 @@ dmtd_status launch_gemm_tc05(dmtd_ctx *c, const UmmaMat &W, const GemmInput &in,
     LAUNCH_OK(c, "norm_act_blocks_kernel");
   } else if (in.kind != GemmInput::READY && in.kb0 < W.n_kb) {
     const int tiles = (W.n_kb - in.kb0) * ((M + AB_ROWS - 1) / AB_ROWS);
-    CUDA_TRY(c, launch_pdl(in.kind == GemmInput::SWIGLU ? act_blocks_kernel<true> : act_blocks_kernel<false>,
+    CUDA_TRY(c, launch_pdl(in.gu.stride ? act_blocks_kernel<true, true> : in.kind == GemmInput::SWIGLU ? act_blocks_kernel<true> : act_blocks_kernel<false>,
                            dim3(std::min((tiles + AB_THREADS / 32 - 1) / (AB_THREADS / 32), 8 * c->n_sms)), dim3(AB_THREADS), 0, c->stream, in.act, in.lda, M, P.T, blocks, in.kb0, in.gu));
     LAUNCH_OK(c, "act_blocks_kernel");
   }

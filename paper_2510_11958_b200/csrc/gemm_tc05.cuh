@@ -499,7 +499,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
           swiglu_units(r, hi, lo);
           const int col = c0 + 2 * ((lane >> 1) & 7) + (lane & 1);
           if (col < n_rows) {
-            uint4 *u = P.gated + P.gated_T.unit(m0 + col, 2 * this_rt + rank, 2 * quarter + (lane >> 4));
+            const int kb = 2 * this_rt + rank, c = 2 * quarter + (lane >> 4), half = tile_rows / 2, sm = col >= half ? 1 : 0;
+            uint4 *u = P.gated + (P.gated_T.tile_rows != tile_rows
+                                      ? P.gated_T.unit(m0 + col, kb, c)
+                                      : (((size_t)this_ct * P.gated_T.n_kb + kb) * 2 + sm) * P.T.units_per_sm() + c * half + (col - sm * half));
             u[0] = hi;
             u[P.gated_T.lo_offset()] = lo;
           }
@@ -562,7 +565,9 @@ __device__ __forceinline__ void store_hi_lo(const float (&f)[8], uint4 *dst, siz
 // request meanwhile: with a thread to a unit (its lanes' loads 32 rows apart, 16 bytes each) a block took 13.6 us at
 // 96 rows of the Qwen3-4B shape and 6 us at 32 (4 cycles of 32 sequences 21.3 ms, 20.3 so).
 constexpr int AB_ROWS = 4, AB_THREADS = 256;
-// The parts that the cut tiles of gate+up were stored in; stride 0: one buffer that they were added into.
+// The parts that the cut tiles of gate+up were stored in (stride 0: one buffer that they were added into).  A form of its own:
+// with the registers of its loads in flight fewer blocks become resident beside the GEMM in front (4 cycles of 32 sequences:
+// 20.7 ms with one form for both, 20.45 with two).
 struct GateUpParts {
   TgLine line;
   int n_ct, n_kb, tile_rows;
@@ -573,7 +578,7 @@ struct GateUpParts {
     return line.holder(u + n_kb - 1) - line.holder(u) + 1;
   }
 };
-template <bool GATED>
+template <bool GATED, bool PARTS = false>
 __global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *act, int lda, int rows, ActTiles T,
                                                                 uint4 *blocks, int kb0, GateUpParts parts) {
   // lanes of a row, 16-byte loads of a lane, and 32-bit registers of a part that a load becomes
@@ -594,7 +599,7 @@ __global__ void __launch_bounds__(AB_THREADS) act_blocks_kernel(const float *act
       v[i] = m < rows ? *reinterpret_cast<const float4 *>(act + (size_t)m * lda + (size_t)kb * LANES * 4 + col * 4)
                       : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (GATED && parts.stride) {
+    if (PARTS) {
       const int n = parts.count(kb, m0);                             // four rows lie in one tile
       constexpr int AHEAD = 5;
 #pragma unroll 1

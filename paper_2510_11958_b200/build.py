@@ -12,7 +12,7 @@ LIB = os.path.join(HERE, "libdmtd_b200.so")
 SOURCES = ["engine.cu"]
 HEADERS = ["common.cuh", "kernels.cuh", "pass_common.cuh", "pass_stream.cuh", "pass_prologues.cuh",
            "pass_attention.cuh", "pass_attention_f32.cuh", "pass_kernel.cuh", "attention_kernel.cuh", "attention_tc05.cuh",
-           "gemm_tc05.cuh"]
+           "gemm_tc05.cuh", "small_pass.cuh"]
 
 
 def _stale() -> bool:

@@ -21,6 +21,7 @@
 #include "attention_kernel.cuh"
 #include "gemm_tc05.cuh"
 #include "attention_tc05.cuh"
+#include "small_pass.cuh"
 
 using namespace dmtd;
 
@@ -101,6 +102,8 @@ struct dmtd_ctx {
   int *pick_idx = nullptr;
   unsigned int *pick_arrived = nullptr;
   long long *pass_timing = nullptr;         // profiling builds only
+
+  bool small_ok = false;                    // the model fits small_pass_kernel
 
   // graphs: [kind 1 = full, 2 = upper-only]
   cudaGraphExec_t graph_exec[3] = {nullptr, nullptr, nullptr};
@@ -894,6 +897,90 @@ dmtd_status enqueue_pass_fused(dmtd_ctx *c, int kind, int R_lower, bool write_to
   return DMTD_OK;
 }
 
+// ---------------------------------------------------------------------------- small fp32 models
+
+// Can passes of this model run as one launch of one cluster (small_pass_kernel)?
+dmtd_status setup_small(dmtd_ctx *c) {
+  const dmtd_model_shape &s = c->s;
+  c->small_ok = false;
+  if (is_bf16(c) || s.kv_dtype != DMTD_F32 || s.head_dim != SP_D || s.n_layers > SP_MAX_LAYERS ||
+      !small_pass_fits(s.hidden, s.intermediate, s.n_q_heads, s.n_kv_heads, s.vocab))
+    return DMTD_OK;
+  const auto kernel = small_pass_kernel;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return DMTD_OK;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(SP_CTAS); cfg.blockDim = dim3(SP_THREADS); cfg.dynamicSmemBytes = SP_SMEM;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = SP_CTAS; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return DMTD_OK; }
+  c->small_ok = clusters >= 1;
+  return DMTD_OK;
+}
+
+// ... and a pass of this kind?  At most eight rows, and as many cached keys to a block (a slice of a kv head) as it walks in
+// the time that the launches of the other form take.  Cycles of the 4-layer test shape (hidden 256), launches against one
+// cluster, us: 1 sequence, 3 passes, context 16 / 600 / 1800 / 7000 (875 keys to a block) 159 / 190 / 232 / 298 against 96 /
+// 105 / 121 / 199; 2 sequences (6 rows), context 1800 (450 keys) 239 against 183, 7000 (1750 keys) 328 against 371; 4 sequences, 2 passes,
+// 1800 (900 keys) 194 against 190; 8 sequences, 1 pass, 600 keys 130 against 122, 1800 keys 157 against 200.
+bool small_pass_ok(const dmtd_ctx *c, int kind, int R_lower) {
+  if (!c->small_ok || !c->use_fused || c->literal_sum || c->L_e > 0) return false;
+  const dmtd_model_shape &s = c->s;
+  const int R = kind == 1 && s.n_layers > c->L_d ? R_lower : 1, G = s.n_q_heads / s.n_kv_heads, M = c->B * R, items = c->B * s.n_kv_heads;
+  if (M > SP_MAX_ROWS || R * G > SP_MAX_ROWS || items > SP_CTAS) return false;
+  if (c->h.n_known / (SP_CTAS / items) > (M <= 4 ? 900 : 500)) return false;
+  return small_pass_smem(small_pass_map(s.hidden, s.intermediate, s.n_q_heads, s.n_kv_heads, s.n_layers, c->B, R)) <= SP_SMEM;
+}
+
+// n passes from here to the end of the cycle at most, as one launch.
+dmtd_status enqueue_small(dmtd_ctx *c, int n, bool write_token, int *out_argmax, float *out_logits, int *out_tokens) {
+  const dmtd_model_shape &s = c->s;
+  const bool full = c->h.slot == 0;
+  SmallParams P{};
+  for (int l = 0; l < s.n_layers; ++l) {
+    const LayerDev &ld = c->layers[l];
+    P.layers[l] = SmallLayer{ld.qkv.wf, ld.o.wf, ld.gu.wf, ld.down.wf, ld.w_in, ld.w_post, ld.w_qn, ld.w_kn,
+                             static_cast<float *>(c->kc) + (size_t)l * c->kv_layer_elems, static_cast<float *>(c->vc) + (size_t)l * c->kv_layer_elems};
+  }
+  P.embed = c->embed.wf; P.w_final = c->w_final; P.inv_freq = c->inv_freq;
+  P.n_layers = s.n_layers; P.lo = s.n_layers - c->L_d; P.B = c->B;
+  P.full = full ? 1 : 0;
+  P.lower = full && P.lo > 0 ? 1 : 0;
+  P.R = full && P.lo > 0 ? c->h.n_known - c->h.lo_len : 1;
+  P.n_passes = n;
+  P.ns = SP_CTAS / (c->B * s.n_kv_heads);
+  P.H = s.hidden; P.I = s.intermediate; P.nq = s.n_q_heads; P.nkv = s.n_kv_heads; P.vocab = s.vocab; P.max_seq = c->max_seq;
+  P.eps = s.rms_eps; P.write_token = write_token ? 1 : 0;
+  P.tokens = c->tokens; P.st = c->dstate; P.out_logits = out_logits; P.out_argmax = out_argmax; P.out_tokens = out_tokens; P.tau = c->tau;
+  P.sample = sample_params(c);
+  P.map = small_pass_map(s.hidden, s.intermediate, s.n_q_heads, s.n_kv_heads, s.n_layers, P.B, P.R);
+  P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(SP_CTAS); cfg.blockDim = dim3(SP_THREADS); cfg.dynamicSmemBytes = small_pass_smem(P.map); cfg.stream = c->stream;
+  cudaLaunchAttribute attr[2]{};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = SP_CTAS; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  CUDA_TRY(c, cudaLaunchKernelEx(&cfg, small_pass_kernel, P));
+  c->launches += 1;
+  return DMTD_OK;
+}
+
+// The passes of at most n that the next launch of small_pass_kernel takes (0: none): to the end of the cycle.
+int small_passes(const dmtd_ctx *c, int n) {
+  const int kind = c->h.slot == 0 ? 1 : 2, R = c->h.n_known - c->h.lo_len;
+  if (!small_pass_ok(c, kind, R)) return 0;
+  return std::min(std::min(n, c->tau - c->h.slot), SP_MAX_POSITIONS - R);
+}
+
 // One pass of the decode stage (Section 2.2).  kind 1: full pass - the R = n_known - lo_len
 // pending rows through the lower layers (refill), the newest row through the decoding
 // layers.  kind 2: the newest token's embedding through the decoding layers only.
@@ -1185,6 +1272,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   }
   CTRY(configure_kernels(c));
   CTRY(setup_fused(c));
+  CTRY(setup_small(c));
   CTRY(dmtd_reset(c));
   CCUDA(cudaStreamSynchronize(c->stream));   // repacking done: the caller may free its weights
 #undef CTRY
@@ -1278,16 +1366,25 @@ dmtd_status dmtd_decode_cycle(dmtd_ctx *c, int32_t max_new, int32_t *out_tokens,
   CHECK_NOT_FAILED(c);
   if (!c->prefilled) return fail(c, DMTD_ERR_STATE, "decode_cycle: no prefill yet");
   const int first = c->h.n_known;
-  int n = 0;
+  int n = 0, n_written = 0;                   // tokens; of them already in out_tokens
   dmtd_status rc = DMTD_OK;
   while (n < max_new) {
     if (c->h.n_known + 1 > c->max_seq) { rc = fail(c, DMTD_ERR_CAPACITY, "decode_cycle: position %d does not fit max_seq=%d", c->h.n_known, c->max_seq); break; }
-    rc = run_greedy_pass(c);
-    if (rc != DMTD_OK) break;                // the passes that were enqueued still count
-    ++n;
+    const int together = small_passes(c, std::min(max_new - n, c->max_seq - c->h.n_known));
+    if (together > 0) {
+      rc = enqueue_small(c, together, true, nullptr, nullptr, n == 0 ? out_tokens : nullptr);
+      if (rc != DMTD_OK) break;
+      if (n == 0) n_written = together;
+      for (int i = 0; i < together; ++i) host_advance(c, c->h.slot == 0 ? 1 : 2);
+      n += together;
+    } else {
+      rc = run_greedy_pass(c);
+      if (rc != DMTD_OK) break;              // the passes that were enqueued still count
+      ++n;
+    }
     if (c->h.slot == 0) break;     // the cycle is complete
   }
-  if (out_tokens && n > 0) {
+  if (out_tokens && n > n_written) {
     gather_tokens_kernel<<<c->B, 32, 0, c->stream>>>(c->tokens, c->max_seq, first, n, c->tau, out_tokens);
     LAUNCH_OK(c, "gather_tokens_kernel");
   }
@@ -1308,6 +1405,13 @@ dmtd_status dmtd_decode_forced(dmtd_ctx *c, const int32_t *forced, int32_t n, fl
                                 c->B, cudaMemcpyDeviceToDevice, c->stream));
   const size_t BV = (size_t)c->B * c->s.vocab;
   for (int i = 0; i < n; ++i) {
+    const int together = small_passes(c, n - i);
+    if (together > 0) {
+      TRY(enqueue_small(c, together, false, out_argmax ? out_argmax + (size_t)i * c->B : nullptr, out_logits ? out_logits + (size_t)i * BV : nullptr, nullptr));
+      for (int k = 0; k < together; ++k) host_advance(c, c->h.slot == 0 ? 1 : 2);
+      i += together - 1;
+      continue;
+    }
     int kind = c->h.slot == 0 ? 1 : 2;
     TRY(enqueue_pass(c, kind, c->h.n_known - c->h.lo_len, false, out_argmax ? out_argmax + (size_t)i * c->B : nullptr,
                      out_logits ? out_logits + (size_t)i * BV : nullptr));

@@ -225,12 +225,13 @@ dmtd_status vec_to_float(dmtd_ctx *c, float **out, const void *src, int n) {
 }
 
 // Second copy of a (fused) matrix in the block order of the tcgen05 GEMM; in_turn: the rows of the sources (of equal
-// size) one after the other instead of source after source.
-dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs, const int *Ns, int n_src, bool in_turn = false) {
+// size) one after the other instead of source after source.  K is filled up with zeros to whole k blocks, the rows to
+// `rows` of them.
+dmtd_status pack_umma(dmtd_ctx *c, UmmaMat *out, int K, const void *const *srcs, const int *Ns, int n_src, bool in_turn = false, int rows = 0) {
   int N = 0;
   for (int i = 0; i < n_src; ++i) N += Ns[i];
   UmmaMat m{};
-  m.N = N; m.K = K; m.n_tiles = (N + 2 * TG_ROWS - 1) / (2 * TG_ROWS) * 2; m.n_kb = K / TG_KB;
+  m.N = N = std::max(N, rows); m.K = K; m.n_tiles = (N + 2 * TG_ROWS - 1) / (2 * TG_ROWS) * 2; m.n_kb = (K + TG_KB - 1) / TG_KB;
   uint4 *dst = nullptr;
   size_t units = (size_t)m.n_tiles * m.n_kb * (TG_WBLOCK / 16);
   c->mem_kind = 1;
@@ -672,7 +673,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
     down.kind = GemmInput::SWIGLU;
     down.act = c->gu;
     if (M > TG_SPLIT_ROWS) {
-      const int n_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, c->n_sms / 2) * 2 * TG_ROWS, n_rest = std::max(0, 2 * I - n_whole);
+      const int n_whole = tg_whole_pairs(lw.gu_u, TG_SWIGLU, c->n_sms / 2) * 2 * TG_ROWS, n_rest = std::max(0, lw.gu_u.N - n_whole);
       down.lda = std::max(4, n_rest); down.kb0 = n_whole / 2 / TG_KB; down.blocks = c->gated_blocks;
       GemmInput gu = norm_input(x, H, lw.w_post);
       const ActTiles T = act_tiles_for(M, lw.gu_u.n_kb);
@@ -1162,10 +1163,14 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   CCUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, c->device));
   const dmtd_model_shape &s = c->s;
   const int H = s.hidden, D = s.head_dim, QD = s.n_q_heads * D, KVD = s.n_kv_heads * D, I = s.intermediate;
+  const int I_pad = (I + TG_KB - 1) / TG_KB * TG_KB;
 
   // weights; every bf16 context whose dimensions fit also gets the copy the tcgen05 GEMM reads:
   // every pass outside the pass kernel uses it
-  c->umma_ok = s.weight_dtype == DMTD_BF16 && H % TG_KB == 0 && QD % TG_KB == 0 && I % TG_KB == 0;
+  // (An intermediate size between two multiples of 64 is filled up: gate and up rows of zeros give the down projection's
+  // last k block zeros.  6 layers of hidden 640, intermediate 1824, on the mma.sync kernels against these, us: prefill of 8 / 130 / 2000 tokens
+  // 270 / 878 / 10237 against 234 / 290 / 1195; a cycle of three passes for 5 / 16 / 64 sequences 493 / 739 / 2011 against 351 / 361 / 488.)
+  c->umma_ok = s.weight_dtype == DMTD_BF16 && H % TG_KB == 0 && QD % TG_KB == 0;
   // DMTD_WEIGHT_COPIES=1 in the environment keeps only the atom stream (half the weight memory):
   // every projection then runs on the mma.sync kernels, the prefill included (slower at every row count)
   if (const char *e = getenv("DMTD_WEIGHT_COPIES")) if (atoi(e) == 1) c->umma_ok = false;
@@ -1195,7 +1200,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
     if (c->umma_ok) {
       CTRY(pack_umma(c, &ld.qkv_u, H, qkv_src, qkv_n, 3));
       CTRY(pack_umma(c, &ld.o_u, QD, o_src, o_n, 1));
-      CTRY(pack_umma(c, &ld.gu_u, H, gu_src, gu_n, 2, true));        // gate and up of one index side by side: the epilogue gates
+      CTRY(pack_umma(c, &ld.gu_u, H, gu_src, gu_n, 2, true, 2 * I_pad));      // gate and up of one index side by side: the epilogue gates
       CTRY(pack_umma(c, &ld.down_u, I, d_src, d_n, 1));
     }
     CTRY(vec_to_float(c, &ld.w_in, lw.input_norm, H));
@@ -1233,8 +1238,8 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   *c->h_error = 0;
 
   // workspace
-  c->lda = std::max(H, std::max(QD, I));
-  c->ldqkv = QD + 2 * KVD; c->ldgu = 2 * I; c->ldl = (s.vocab + 15) / 16 * 16;
+  c->lda = std::max(H, std::max(QD, c->umma_ok ? I_pad : I));
+  c->ldqkv = QD + 2 * KVD; c->ldgu = 2 * (c->umma_ok ? I_pad : I); c->ldl = (s.vocab + 15) / 16 * 16;
   // Keys per slice of the split-KV attention: enough slices that a decode step of max_batch
   // sequences fills the SMs about four times over, and no more (every slice costs a block its
   // set-up, a partial result and a share of the merge); whole 64-key tiles.
@@ -1268,7 +1273,7 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   if (c->umma_ok) {
     const size_t rows = (size_t)c->ws_rows + 16 * (c->ws_rows / TG_SPLIT_ROWS + 1) + TG_TILE_ROWS;
     CTRY(dev_alloc(c, &c->act_blocks, rows * (c->lda / 8) * 2));
-    CTRY(dev_alloc(c, &c->gated_blocks, rows * (I / 8) * 2));
+    CTRY(dev_alloc(c, &c->gated_blocks, rows * (I_pad / 8) * 2));
   }
   CTRY(configure_kernels(c));
   CTRY(setup_fused(c));
@@ -1495,7 +1500,7 @@ dmtd_status dmtd_prefill_host(dmtd_ctx *c, const int32_t *prompt_host, int32_t B
   if (B > c->max_batch || P + 1 > c->max_seq) return fail(c, DMTD_ERR_CAPACITY, "prefill_host: sizes exceed capacity");
   // stage the prompt at the tail of the act workspace (unused until the first layer runs)
   int *stage = reinterpret_cast<int *>(c->gu);
-  if ((size_t)B * P > (size_t)c->ws_rows * c->ldgu) return fail(c, DMTD_ERR_CAPACITY, "prefill_host: prompt larger than staging space");
+  if ((size_t)B * P > (size_t)c->ws_rows * 2 * c->s.intermediate) return fail(c, DMTD_ERR_CAPACITY, "prefill_host: prompt larger than staging space");
   CUDA_TRY(c, cudaMemcpyAsync(stage, prompt_host, (size_t)B * P * 4, cudaMemcpyHostToDevice, c->stream));
   // the token buffer copy inside dmtd_prefill reads `stage` before any layer writes gu
   TRY(dmtd_prefill(c, stage, B, P, nullptr, nullptr, nullptr));

@@ -58,6 +58,15 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Two products at once: a += x * y by halves.
+__device__ __forceinline__ void fma_f32x2(float2 &a, float2 x, float2 y) {
+  uint64_t r;
+  asm("{\n .reg .b64 a, x, y;\n mov.b64 a, {%1, %2};\n mov.b64 x, {%3, %4};\n mov.b64 y, {%5, %6};\n fma.rn.f32x2 %0, x, y, a;\n}\n"
+      : "=l"(r)
+      : "f"(a.x), "f"(a.y), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+}
+
 // Split an fp32 value into two bf16 terms hi + lo (|error| <= 2^-17 |x|): tensor-core
 // operands must be bf16, and a single rounding of the activations would exceed the logit
 // tolerance after 36 layers.

@@ -397,15 +397,17 @@ dmtd_status launch_gemv(dmtd_ctx *c, const PackedMat &W, const UmmaMat &U, const
   // layer's projections at 3 rows in 82 us against 58 (kernel times)
   if (U.w && c->use_umma) return launch_gemm_tc05(c, U, rows_input(act, lda), M, out, ldo);
   if (W.wf) {
-    // A launch of more than a few microseconds of arithmetic starts when everything in front is complete: as a dependent
-    // launch its blocks come to lie unevenly on the SMs, where the kernel in front still has blocks.  Layers of fp32 models,
-    // dependent against plain: 24 rows of hidden 256 (9 M products in gate+up) 163 us against 175, 12 rows of 512 (19 M) 167
-    // against 179, 24 rows of 512 (38 M) 313 against 292, 32 rows of 1024 (201 M) 699 against 638.
-    if ((long long)M * W.N * W.K <= (32ll << 20))
-      CUDA_TRY(c, launch_pdl(gemv_f32_kernel<true>, dim3(2 * c->n_sms), dim3(256), (size_t)(0), c->stream, W, act, lda, M, out, ldo));
-    else
-      gemv_f32_kernel<false><<<2 * c->n_sms, 256, 0, c->stream>>>(W, act, lda, M, out, ldo);
-    LAUNCH_OK(c, "gemv_f32_kernel");
+    auto launch = [&](auto kernel, int bm, int bn, int threads, int smem) {
+      return launch_pdl(kernel, dim3((W.N + bn - 1) / bn, (M + bm - 1) / bm), dim3(threads), (size_t)smem, c->stream, W, act, lda, M, out, ldo);
+    };
+    // Small tiles up to 64 rows, large ones where they give every SM three blocks.  Layers of fp32 models, us, 16 / 32 / 64 wide
+    // tiles: hidden 256, 64 rows 50 / 56 / 110, 192 rows 67 / 62 / 112, 1000 rows 213 / 137 / 156; hidden 1024, 64 rows 132 / 158 /
+    // 385, 96 rows 208 / 186 / 375, 512 rows 645 / 543 / 555, 1000 rows 1249 / 1022 / 915.
+    const long long large = (long long)((W.N + 63) / 64) * ((M + 63) / 64);
+    if (M <= 64) CUDA_TRY(c, launch(gemm_f32_kernel<16, 16, 8>, 16, 16, 128, gemm_f32_smem<16, 16, 8>()));
+    else if (large < 3ll * c->n_sms) CUDA_TRY(c, launch(gemm_f32_kernel<32, 32, 4>, 32, 32, 256, gemm_f32_smem<32, 32, 4>()));
+    else CUDA_TRY(c, launch(gemm_f32_kernel<64, 64, 1>, 64, 64, 256, gemm_f32_smem<64, 64, 1>()));
+    LAUNCH_OK(c, "gemm_f32_kernel");
     return DMTD_OK;
   }
   if (M <= 4) return launch_gemv_nt<1>(c, W, act, lda, M, out, ldo);
@@ -768,6 +770,9 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<4>, dyn, 100 * 1024));
   for (int whole : {TG_ADD, TG_STORE, TG_SWIGLU})
     for (bool split : {false, true}) CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_for(split, whole), dyn, TG_MAX_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<16, 16, 8>, dyn, gemm_f32_smem<16, 16, 8>()));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<64, 64, 1>, dyn, gemm_f32_smem<64, 64, 1>()));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<32, 32, 4>, dyn, gemm_f32_smem<32, 32, 4>()));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16>, dyn, AD_SMEM));

@@ -255,34 +255,104 @@ gemv_bf16_kernel(PackedMat W, const float *act, int lda, int M,
   }
 }
 
-// Projection, fp32 weights (small verification models only): one warp per output row.  EARLY: launched with programmatic
-// stream serialisation; otherwise the activations are complete before it starts and are read as constants (3 % of a layer
-// of hidden 1024 at 64 rows and more).
-template <bool EARLY>
-__global__ void gemv_f32_kernel(PackedMat W, const float *act, int lda, int M,
-                                float *out, int ldo) {
-  if (EARLY) pdl_enter();
-  int lane = threadIdx.x & 31;
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
-  for (int n = warp; n < W.N; n += n_warps) {
-    const float *wr = W.wf + (size_t)n * W.K;
-    for (int m0 = 0; m0 < M; m0 += 4) {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int k = lane * 4; k < W.K; k += 128) {
-        float4 w = *reinterpret_cast<const float4 *>(wr + k);
+// Projection, fp32 weights (small verification models only), more rows than a decode pass of a few sequences has:
+// out[m][n] += sum_k W[n][k] act[m][k] by tiles of BM activation rows x BN weight rows.  A thread holds 4 x 4 outputs; KG sets
+// of threads share a tile, each a part of every piece of k, and add their sums at the end.  Both operands come as they lie
+// (k fastest) by asynchronous copies, two pieces of 32 KG values in flight; four floats of padding to a row keep the 16-byte reads
+// free of bank conflicts.  Bound by fp32 arithmetic at prefill sizes (two products per instruction, fma.f32x2), by the trips
+// to memory of its few blocks at decode sizes, hence the small tiles with four thread sets.
+// Measured, a layer with its other kernels, against one warp to a weight row, which read every activation row from L1 for each
+// of them: hidden 256, 32 / 512 / 1000 rows 97 / 1090 / 2054 us -> 48 / 86 / 137; hidden 1024, 12 / 1000 rows 122 / 6892 -> 83 / 915.
+// Sums over 128 values of k at a time, then of those sums: no further from fp64 than the lane-wise sums before.
+constexpr int GF_PAD = 4;
+template <int BM, int BN, int KG>
+constexpr int gemm_f32_smem() { return 2 * (BM + BN) * (32 * KG + GF_PAD) * 4; }
+template <int BM, int BN, int KG>
+__global__ void __launch_bounds__(BM * BN / 16 * KG) gemm_f32_kernel(PackedMat W, const float *act, int lda, int M, float *out, int ldo) {
+  constexpr int SET = BM * BN / 16, THREADS = SET * KG, BK = 32 * KG, LD = BK + GF_PAD, STAGE = (BM + BN) * LD;
+  extern __shared__ __align__(16) float gf_smem[];
+  const int tid = threadIdx.x, kg = tid / SET, tx = tid % SET % (BN / 4), ty = tid % SET / (BN / 4);
+  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM, K = W.K;
+  const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(gf_smem);
+  // rows [first, first + ROWS) of the stage: values k0 .. k0 + BK - 1 of the rows of `src` from row0 on; zeros past the end
+  auto fetch_rows = [&](const float *src, size_t ld, int row0, int n_rows, int first, int rows, int k0, int stage) {
+    for (int i = tid; i < rows * (BK / 4); i += THREADS) {
+      const int r = i / (BK / 4), k = k0 + i % (BK / 4) * 4;
+      const bool ok = row0 + r < n_rows && k < K;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem0 + (stage * STAGE + (first + r) * LD + i % (BK / 4) * 4) * 4),
+                   "l"(src + (ok ? (size_t)(row0 + r) * ld + k : 0)), "r"(ok ? 16 : 0)
+                   : "memory");
+    }
+  };
+  auto fetch_w = [&](int k0, int stage) { fetch_rows(W.wf, K, n0, W.N, BM, BN, k0, stage); };
+  auto fetch_act = [&](int k0, int stage) { fetch_rows(act, lda, m0, M, 0, BM, k0, stage); };
+  fetch_w(0, 0);                            // weights: before the kernel in front is complete
+  pdl_enter();
+  fetch_act(0, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  float sum[4][4];
+  float2 acc[4][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (m0 + i < M) {
-            const float4 *ap = reinterpret_cast<const float4 *>(act + (size_t)(m0 + i) * lda + k);
-            const float4 a = EARLY ? *ap : __ldg(ap);
-            acc[i] += w.x * a.x + w.y * a.y + w.z * a.z + w.w * a.w;
-          }
-      }
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float v = warp_sum(acc[i]);
-        if (lane == 0 && m0 + i < M) out[(size_t)(m0 + i) * ldo + n] += v;
-      }
+    for (int j = 0; j < 4; ++j) { sum[i][j] = 0.f; acc[i][j] = make_float2(0.f, 0.f); }
+  const int n_pieces = (K + BK - 1) / BK;
+#pragma unroll 1
+  for (int p = 0; p < n_pieces; ++p) {
+    if (p + 1 < n_pieces) { fetch_w((p + 1) * BK, (p + 1) & 1); fetch_act((p + 1) * BK, (p + 1) & 1); }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    const float *a_s = gf_smem + (p & 1) * STAGE + kg * 32, *b_s = a_s + BM * LD;
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4 *>(a_s + (ty + i * (BM / 4)) * LD + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4 *>(b_s + (tx + j * (BN / 4)) * LD + k);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          fma_f32x2(acc[i][j], make_float2(a[i].x, a[i].y), make_float2(b[j].x, b[j].y));
+          fma_f32x2(acc[i][j], make_float2(a[i].z, a[i].w), make_float2(b[j].z, b[j].w));
+        }
+    }
+    if ((p & 3) == 3 || p + 1 == n_pieces) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { sum[i][j] += acc[i][j].x + acc[i][j].y; acc[i][j] = make_float2(0.f, 0.f); }
+    }
+    __syncthreads();                        // the stage is free
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (KG > 1) {
+    // the other sets' sums, through the stages' memory
+    if (kg > 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gf_smem[((kg - 1) * 16 + i * 4 + j) * SET + tid % SET] = sum[i][j];
+    }
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int g = 0; g < KG - 1; ++g)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sum[i][j] += gf_smem[(g * 16 + i * 4 + j) * SET + tid];
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int m = m0 + ty + i * (BM / 4);
+    if (m >= M) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int n = n0 + tx + j * (BN / 4);
+      if (n < W.N) out[(size_t)m * ldo + n] += sum[i][j];
     }
   }
 }

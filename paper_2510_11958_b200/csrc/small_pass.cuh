@@ -269,17 +269,9 @@ __device__ __forceinline__ void sp_advance(SmallCursor &cur) {
   if (cur.dst >= smem_u32(sp_smem) + SP_FIXED_BYTES + SP_RING_BYTES) cur.dst -= SP_RING_BYTES;
 }
 
-// Two products at once: a += x * y by halves.
-__device__ __forceinline__ void sp_fma2(float2 &a, float2 x, float2 y) {
-  uint64_t r;
-  asm("{\n .reg .b64 a, x, y;\n mov.b64 a, {%1, %2};\n mov.b64 x, {%3, %4};\n mov.b64 y, {%5, %6};\n fma.rn.f32x2 %0, x, y, a;\n}\n"
-      : "=l"(r)
-      : "f"(a.x), "f"(a.y), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
-}
 __device__ __forceinline__ void sp_fma4(float2 &a, const float4 &x, const float4 &y) {
-  sp_fma2(a, make_float2(x.x, x.y), make_float2(y.x, y.y));
-  sp_fma2(a, make_float2(x.z, x.w), make_float2(y.z, y.w));
+  fma_f32x2(a, make_float2(x.x, x.y), make_float2(y.x, y.y));
+  fma_f32x2(a, make_float2(x.z, x.w), make_float2(y.z, y.w));
 }
 
 // The activation rows of a step: row m at x + m * ld; NORM steps normalise them (RMSNorm, 1 / rms goes to the product).
@@ -553,7 +545,7 @@ __device__ __forceinline__ void sp_attention(const SmallParams &P, uint32_t &pha
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const float pj = __shfl_sync(0xffffffffu, p[e], jj * 4);
-              sp_fma2(o[q0 + e], make_float2(pj, pj), now.v[jj]);
+              fma_f32x2(o[q0 + e], make_float2(pj, pj), now.v[jj]);
             }
         }
       }

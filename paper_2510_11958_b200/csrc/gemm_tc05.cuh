@@ -55,6 +55,15 @@ constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
 // holds (4 cycles of 32 sequences of the Qwen3-4B shape: 20.26 ms with one, 20.12 with two).  More rows: one, the
 // activations of a stage are 32 KiB there.
 __host__ __device__ constexpr int tg_stage_units(bool split) { return split ? 2 : 1; }
+// Decode launches: the ring's first round, requested before the activations are there, is asked for as fast as HBM delivers
+// it and not at once: two stages (64 KiB an SM, HBM's bandwidth times its latency and a little more), then one every TG_PACE
+// cycles (32 KiB for 148 SMs: 0.75 us).  With 192 KiB an SM outstanding, the few reads between two projections (the norms' and
+// gates' kernels, the keys) waited some 4 us in the L2's queues: a projection had its activations 8 us after the end of
+// the one in front.  4 layers and the head, context 64 to 700, 1 / 3 / 16 sequences, us: all at once 355 / 386 / 393; a stage every 600 cycles
+// 352 / 377 / 384, 1000 344 / 368 / 376, 1400 343 / 366 / 375, 2000 355 / 374 / 388.  (Asking L2 for the next projection's first
+// weights at the end of a launch: 2 % without pacing, nothing beside it.  Activations converted by warps of the GEMM instead of
+// kernels in front: as fast at 1 to 3 rows, slower above.)
+constexpr int TG_PACE_FREE = 2, TG_PACE = 1200;
 constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
 // Dynamic shared memory of a block: it has its SM to itself, beside a block of the prefill attention (96 KiB) or another
 // GEMM's, which take tensor memory as well.  Two stages of narrow column tiles need less than the lower bound.
@@ -337,7 +346,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
   if (threadIdx.x == 0) {
     // the weight blocks of the first stages are requested before the other block is waited for: they touch this
     // block's barriers only, and eight copies take the issuing thread some thousand cycles
-    for (; n_first < S && issued_units < n_it; ++n_first) {
+    for (; n_first < (SPLIT ? min(S, TG_PACE_FREE) : S) && issued_units < n_it; ++n_first) {
       const int n = cur_w.units(n_kb, KPS);
       mbar_expect_tx(full0 + n_first * 8, n * (TG_WBLOCK + act_bytes));
       copy_w(n_first, n);
@@ -354,8 +363,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     if (lane == 0) {
       // ---- producer: a bulk copy for a stage's weights and one for each unit's activations; the activation blocks only after the kernel that writes them has
       // completed and its writes are visible
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (int i = 0; i < n_first; ++i) copy_act(i, cur_a.units(n_kb, KPS));
+      if (SPLIT) {
+        // the rest of the ring's first round at the pace of HBM; the activations of this round are copied by an epilogue warp
+        long long t = clock64();
+        for (; n_first < S && issued_units < n_it; ++n_first) {
+          while (clock64() - t < TG_PACE) {}
+          t = clock64();
+          const int n = cur_w.units(n_kb, KPS);
+          mbar_expect_tx(full0 + n_first * 8, n * (TG_WBLOCK + act_bytes));
+          copy_w(n_first, n);
+          issued_units += n;
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int i = 0; i < n_first; ++i) cur_a.next(cur_a.units(n_kb, KPS), n_kb, n_ct, pair, n_pairs);
+      } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int i = 0; i < n_first; ++i) copy_act(i, cur_a.units(n_kb, KPS));
+      }
       int st = 0, issued = n_first;
       uint32_t ph = 0;
       bool ok = true;
@@ -458,6 +482,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TG_THREADS, 1) gemm_
     }
   } else {
     // ---- epilogue: thread = weight row (lane of tensor memory), registers = columns
+    if (SPLIT && warp == 2) {
+      // the activations of the ring's first round, while the producer is still asking for its weights
+      if (lane == 0) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int i = 0, units = 0; i < S && units < n_it; ++i) {
+          const int n = cur_a.units(n_kb, KPS);
+          copy_act(i, n);
+          units += n;
+        }
+      }
+      __syncwarp();
+    }
     const int quarter = warp & 3;
     int acc = 0, kb = start.kb, ct = start.ct, rt = start.rt, left = n_part;
     uint32_t ph = 0;

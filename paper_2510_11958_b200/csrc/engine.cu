@@ -88,6 +88,7 @@ struct dmtd_ctx {
 
   // options
   bool use_graph = true, literal_sum = false, use_fused = true, use_tc_attention = true;
+  bool choose_fused = true;                 // the pass kernel only where it is the faster one (until the option is set)
   bool fuse_qk_rope = true;                 // QK-norm, RoPE and the KV append inside the tensor-core attention kernel
   float temperature = 0.f;                  // > 0: tokens are drawn from softmax(logits / temperature); 0: greedy
   uint64_t sample_seed = 0;
@@ -866,10 +867,19 @@ dmtd_status setup_fused(dmtd_ctx *c) {
   return DMTD_OK;
 }
 
+// One sequence of a model with large layers.  Cycles of 1 to 4 passes, the pass kernel's time over the per-step kernels': one
+// sequence, context 64 to 3000, hidden 640 (7 MB a layer) 1.25 to 1.07, 1024 1.18 to 1.04, 1536 1.12 to 1.02, 2048 (100 MB)
+// 1.09 to 1.01, 2560 (202 MB) 1.03, and over 36 layers (7 cycles at 512 to 2500) 0.985; two sequences of 2560 1.05, three
+// 1.08 to 1.11, four 1.11 to 1.18.
+bool pass_kernel_faster(const dmtd_ctx *c) {
+  const LayerDev &l = c->layers[0];
+  return c->B == 1 && packed_atoms(l.qkv) + packed_atoms(l.o) + packed_atoms(l.gu) + packed_atoms(l.down) >= (128 << 10);      // 1 KiB atoms
+}
 bool fused_pass_ok(const dmtd_ctx *c, int kind, int R_lower) {
   if (!c->fused_ok || !c->use_fused || c->literal_sum || c->L_e > 0) return false;
   const int lo = c->s.n_layers - c->L_d;
   const int R = (kind == 1 && lo > 0) ? R_lower : 1;
+  if (c->choose_fused && !pass_kernel_faster(c)) return false;
   return c->B * R <= PK_MAX_ROWS && R * (c->s.n_q_heads / c->s.n_kv_heads) <= PK_QR &&
          c->B * R * c->s.hidden <= PK_XS_FLOATS;
 }
@@ -1582,7 +1592,7 @@ dmtd_status dmtd_set_option(dmtd_ctx *c, const char *name, int64_t value) {
   if (value != 0 && value != 1) return fail(c, DMTD_ERR_INVALID_ARG, "option %s takes 0 or 1", name);
   if (!strcmp(name, "cuda_graph")) { c->use_graph = value != 0; return DMTD_OK; }
   if (!strcmp(name, "literal_sum")) { c->literal_sum = value != 0; drop_graphs(c); return DMTD_OK; }
-  if (!strcmp(name, "fused_pass")) { c->use_fused = value != 0; return DMTD_OK; }
+  if (!strcmp(name, "fused_pass")) { c->use_fused = value != 0; c->choose_fused = false; return DMTD_OK; }
   if (!strcmp(name, "fused_qk_rope")) { c->fuse_qk_rope = value != 0; drop_graphs(c); return DMTD_OK; }
   if (!strcmp(name, "tcgen05_gemm")) { c->use_umma = value != 0; drop_graphs(c); return DMTD_OK; }
   if (!strcmp(name, "tc_attention")) { c->use_tc_attention = value != 0; drop_graphs(c); return DMTD_OK; }

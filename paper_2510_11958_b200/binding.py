@@ -276,8 +276,12 @@ class Dmtd:
         return n.value
 
 
-def _kv_code(t):
-    return {torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}[t.dtype]
+_KV_CODE = {torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}
+
+
+def _current_stream():
+    """The current device's current stream, as a number."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def attention_decode(q, k, v, pos0, scratch=None):
@@ -288,7 +292,8 @@ def attention_decode(q, k, v, pos0, scratch=None):
     `scratch` is a cuda uint8 tensor of at least attention_scratch_bytes(...) bytes; one is
     allocated through torch if none is given.
     """
-    dll = load_library()
+    # (a short sequence's attention is a few microseconds on the device: plain numbers for the pointers, no objects around them)
+    dll = _dll or load_library()
     assert q.is_cuda and q.dtype == torch.float32 and q.is_contiguous()
     assert k.is_cuda and v.is_cuda and k.is_contiguous() and v.is_contiguous() and k.dtype == v.dtype
     B, R, nq, D = q.shape
@@ -297,9 +302,8 @@ def attention_decode(q, k, v, pos0, scratch=None):
         need = dll.dmtd_attention_scratch_bytes(B, R, nq, D, pos0 + R)
         scratch = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
     out = torch.empty_like(q)
-    rc = dll.dmtd_attention_decode(_ptr(q), _ptr(k), _ptr(v), _kv_code(k), B, R, nq, nkv, D, max_seq, pos0,
-                                   _ptr(scratch), scratch.numel(), _ptr(out),
-                                   C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    rc = dll.dmtd_attention_decode(q.data_ptr(), k.data_ptr(), v.data_ptr(), _KV_CODE[k.dtype], B, R, nq, nkv, D, max_seq, pos0,
+                                   scratch.data_ptr(), scratch.numel(), out.data_ptr(), _current_stream())
     if rc:
         raise DmtdError(rc, dll.dmtd_last_error(None).decode())
     return out
@@ -322,8 +326,8 @@ def attention_decode_static(q, k, v, pos0, out):
     assert k.is_cuda and v.is_cuda and k.is_contiguous() and v.is_contiguous() and k.dtype == v.dtype
     B, R, nq, D = q.shape
     _, nkv, max_seq, _ = k.shape
-    rc = dll.dmtd_attention_decode_static(_ptr(q), _ptr(k), _ptr(v), _kv_code(k), B, R, nq, nkv, D, max_seq, pos0,
-                                          _ptr(out), C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    rc = dll.dmtd_attention_decode_static(q.data_ptr(), k.data_ptr(), v.data_ptr(), _KV_CODE[k.dtype], B, R, nq, nkv, D, max_seq, pos0,
+                                          out.data_ptr(), _current_stream())
     if rc:
         raise DmtdError(rc, dll.dmtd_last_error(None).decode())
     return out

@@ -4,6 +4,7 @@
 // results of the key slices are merged by attn_merge_kernel or by the O projection's activation-block kernel.
 #pragma once
 
+#include "gemm_tc05.cuh"
 #include "kernels.cuh"
 #include "pass_attention_f32.cuh"
 
@@ -22,8 +23,8 @@ namespace dmtd {
 //  * Rows are 256 dense bytes; 16-byte part c of row r lies at part c ^ f(r) of its half row, f(r) = (r & 1) * 4 +
 //    (r >> 1 & 3): free of bank conflicts for the copies, for the 16-byte operand loads of K and for ldmatrix on V.
 // Measured, attention with its merge, against the kernel before it (64-key tiles of the whole block, two barriers per
-// tile, slices of fixed length): 8 sequences x 16387 keys, 12 query rows per kv head, 159.8 -> 96.1 us (537 MB of K and V:
-// 5.6 TB/s, the kernel alone above 6); a layer step of 64 sequences x 8192 keys, 4 query rows, 507 -> 399 us.
+// tile, slices of fixed length): 8 sequences x 16387 keys, 12 query rows per kv head, 159.8 -> 87.9 us, as clusters 81.3 (537 MB of K
+// and V: 6.6 TB/s); a layer step of 64 sequences x 8192 keys, 4 query rows, 507 -> 381 us.
 constexpr int AD_WARPS = 4;
 constexpr int AD_THREADS = AD_WARPS * 32;
 constexpr int AD_KEYS = 16;                                   // keys per warp tile
@@ -239,14 +240,43 @@ struct AttnShares {
   __device__ __forceinline__ int holder(int u) const { return (int)((((long long)u + 1) * n_blocks - 1) / total); }
 };
 
+// Loads from the shared memory of another block of the cluster (addresses of the cluster's window).
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_cluster2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+constexpr int AD_MAX_CLUSTER = 8;
+
+// Where the form of a model's layer puts its results: the O projection's activation blocks.
+struct AttnBlocks {
+  uint4 *blocks;
+  ActTiles T;
+};
+
+// CLUSTER: one cluster to an item, its units cut into equal pieces for the cluster's blocks, which merge their results through
+// distributed shared memory: into `part_o` = out [B*R][nq][128], or, the fused form, into the O projection's activation
+// blocks.  One launch, no partial results in memory.  (Merging by the last block of an item to arrive at a counter in
+// memory instead: a layer of 8 sequences 2 us slower than with the merge as a launch of its own.)  See attn_cluster_ranks.
 // qkv [B*R][ldq]: FUSED: the raw q | k | v rows of the QKV projection (AttnFuse); else q heads already normalised and
 // rotated (not scaled) and K and V of the new rows already in the cache.  Cache [b][kv head][max_seq][128], 16 bit.
 // part_o / part_ml: `nsplit` slots per (row, head); the pieces of an item take slots 0, 1, ...; the rest are marked empty.
-template <class Op, bool FUSED = false>
+template <class Op, bool FUSED = false, bool CLUSTER = false>
 __global__ void __launch_bounds__(AD_THREADS, 2)
 attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, int max_seq,
                    int nq, int nkv, int B, int R, int RB, const int *__restrict__ pos0_ptr, int pos0_val, float *part_o,
-                   float *part_ml, int nsplit, AttnFuse F = AttnFuse{nullptr, nullptr, nullptr, 0.f}) {
+                   float *part_ml, int nsplit, AttnFuse F = AttnFuse{nullptr, nullptr, nullptr, 0.f},
+                   AttnBlocks O = AttnBlocks{nullptr, ActTiles{}}) {
   extern __shared__ __align__(1024) unsigned char sc[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int G = nq / nkv, n_rb = (R + RB - 1) / RB;
@@ -261,20 +291,26 @@ attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, in
   sh.per_item = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
   sh.total = (long long)B * nkv * n_rb * sh.per_item;
   sh.n_blocks = (int)min((long long)gridDim.x, sh.total);             // no empty shares: pieces of an item are consecutive blocks
-  if ((int)blockIdx.x >= sh.n_blocks) {
+  int n_ranks = 1, rank = 0;
+  if (CLUSTER) {
+    asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n_ranks));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  }
+  if (!CLUSTER && (int)blockIdx.x >= sh.n_blocks) {
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");    // this grid's end stands for the end of those before it
     return;
   }
-  const int u_end = sh.begin(blockIdx.x + 1);
+  const int u_item = CLUSTER ? (int)blockIdx.x / n_ranks * sh.per_item : 0;
+  const int u_end = CLUSTER ? u_item + sh.per_item * (rank + 1) / n_ranks : sh.begin(blockIdx.x + 1);
   const uint32_t ring = smem_u32(sc + AD_RING) + warp * AD_STAGES * AD_SLOT, q_t = smem_u32(sc + AD_Q);
   float *const o_s = reinterpret_cast<float *>(sc + AD_OS), *const red_m = reinterpret_cast<float *>(sc + AD_RED);
   float *const red_l = red_m + AD_WARPS * PK_QR;
   const float scale = rsqrtf((float)PK_D);
 
-  for (int u = sh.begin(blockIdx.x); u < u_end;) {
+  for (int u = CLUSTER ? u_item + sh.per_item * rank / n_ranks : sh.begin(blockIdx.x); CLUSTER || u < u_end;) {
     // one piece: units [t0, t1) of an item
-    const int item = u / sh.per_item, t0 = u - item * sh.per_item, t1 = min(sh.per_item, t0 + u_end - u);
-    const int piece = blockIdx.x - sh.holder(item * sh.per_item);
+    const int item = CLUSTER ? (int)blockIdx.x / n_ranks : u / sh.per_item, t0 = u - item * sh.per_item, t1 = min(sh.per_item, t0 + u_end - u);
+    const int piece = CLUSTER ? 0 : blockIdx.x - sh.holder(item * sh.per_item);
     u += t1 - t0;
     const int rb = item % n_rb, kvh = (item / n_rb) % nkv, b = item / n_rb / nkv;
     const int r0 = rb * RB, r1 = min(R, r0 + RB), nQ = (r1 - r0) * G;
@@ -416,9 +452,10 @@ attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, in
         l += red_l[w * PK_QR + qi] * f;
         red_l[w * PK_QR + qi] = f;
       }
+      if (CLUSTER) reinterpret_cast<float2 *>(sc + AD_RING + PK_QR * PK_D * 4)[qi] = make_float2(m, l);          // (the ring is free)
       const size_t slot = ((size_t)(b * R + r0 + qi / G) * nq + kvh * G + qi % G) * nsplit + piece;
-      *reinterpret_cast<float2 *>(part_ml + slot * 2) = make_float2(m, l);
-      if (t1 == sh.per_item)                                            // the item's last piece
+      if (!CLUSTER) *reinterpret_cast<float2 *>(part_ml + slot * 2) = make_float2(m, l);
+      if (!CLUSTER && t1 == sh.per_item)                                // the item's last piece
         for (int e = piece + 1; e < nsplit; ++e) *reinterpret_cast<float2 *>(part_ml + (slot + e - piece) * 2) = make_float2(-INFINITY, 0.f);
     }
     __syncthreads();
@@ -433,8 +470,61 @@ attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, in
           acc.x += v.x * f; acc.y += v.y * f; acc.z += v.z * f; acc.w += v.w * f;
         }
       }
+      if (CLUSTER) {
+        reinterpret_cast<float4 *>(sc + AD_RING)[idx] = acc;
+        continue;
+      }
       const size_t slot = ((size_t)(b * R + r0 + qi / G) * nq + kvh * G + qi % G) * nsplit + piece;
       *reinterpret_cast<float4 *>(part_o + slot * PK_D + d4 * 4) = acc;
+    }
+    if (CLUSTER) {
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      // a thread to PER values of a query row: 4 of the output, or 8 (a unit) of the blocks
+      constexpr int PER = FUSED ? 8 : 4, V = PER / 4;
+      for (int idx = rank * AD_THREADS + threadIdx.x; idx < nQ * (PK_D / PER); idx += n_ranks * AD_THREADS) {
+        const int qi = idx / (PK_D / PER), row = b * R + r0 + qi / G, head = kvh * G + qi % G;
+        const uint32_t o_a = smem_u32(sc + AD_RING) + idx * PER * 4, ml_a = smem_u32(sc + AD_RING + PK_QR * PK_D * 4) + qi * 8;
+        float2 ml[AD_MAX_CLUSTER];
+        float4 o[AD_MAX_CLUSTER][V];
+        float m = -INFINITY;
+#pragma unroll
+        for (int s = 0; s < AD_MAX_CLUSTER; ++s)
+          if (s < n_ranks) {
+            ml[s] = ld_cluster2(cluster_address(ml_a, s));
+#pragma unroll
+            for (int i = 0; i < V; ++i) o[s][i] = ld_cluster4(cluster_address(o_a + i * 16, s));
+          }
+#pragma unroll
+        for (int s = 0; s < AD_MAX_CLUSTER; ++s)
+          if (s < n_ranks && ml[s].y > 0.f) m = fmaxf(m, ml[s].x);
+        float l = 0.f, f[PER];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) f[i] = 0.f;
+#pragma unroll
+        for (int s = 0; s < AD_MAX_CLUSTER; ++s)
+          if (s < n_ranks && ml[s].y > 0.f) {
+            const float w = __expf(ml[s].x - m);
+            l += ml[s].y * w;
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+              f[4 * i] += o[s][i].x * w; f[4 * i + 1] += o[s][i].y * w;
+              f[4 * i + 2] += o[s][i].z * w; f[4 * i + 3] += o[s][i].w * w;
+            }
+          }
+        const float inv = 1.f / l;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) f[i] *= inv;
+        if constexpr (FUSED) {
+          const int k = head * PK_D + idx % (PK_D / PER) * PER;
+          store_hi_lo(f, O.blocks + O.T.unit(row, k / TG_KB, k % TG_KB / 8), O.T.lo_offset());
+        } else {
+          reinterpret_cast<float4 *>(part_o)[((size_t)row * nq + head) * (PK_D / 4) + idx % (PK_D / 4)] = make_float4(f[0], f[1], f[2], f[3]);
+        }
+      }
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");       // no block leaves while another reads from it
+      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      break;
     }
     __syncthreads();                                                    // outputs, factors and query rows consumed
   }

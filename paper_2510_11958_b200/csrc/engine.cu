@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -269,6 +270,20 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same for a grid of clusters of `ranks` blocks.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int ranks, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr[2]{};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ranks; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 int gemv_smem_bytes(const PackedMat &W, int NT) {
   int KS = W.aps * 32;
   int row_bytes = ((KS * 2) % 128 == 64) ? KS * 2 : KS * 2 + 64;
@@ -446,6 +461,52 @@ AttnPartialKernel<KVT> attn_partial_for(int n_rows, int R, int CH, long long n_b
 // Does the attention of R new rows per sequence run on attn_decode_kernel?
 bool tc_decode_attention(const dmtd_ctx *c) { return c->use_tc_attention && c->s.head_dim == PK_D && c->s.kv_dtype != DMTD_F32; }
 
+// Clusters of 2, 4 and 8 attention blocks that the device holds at once (a cluster lies in one GPC).
+int attn_cluster_room(int device, int ranks) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> room[kDevices][4];
+  const int i = ranks == 2 ? 1 : ranks == 4 ? 2 : 3;
+  if (device < 0 || device >= kDevices) return 0;
+  int n = room[device][i].load(std::memory_order_relaxed);
+  if (n == 0) {
+    const auto kernel = attn_decode_kernel<OpBf16, true, true>;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ranks); cfg.blockDim = dim3(AD_THREADS); cfg.dynamicSmemBytes = AD_SMEM;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = ranks; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    room[device][i].store(n > 0 ? n : -1, std::memory_order_relaxed);
+  }
+  return std::max(0, n);
+}
+// Blocks of a cluster to an item (sequence, kv head, row block) of `units` 64-key units where the attention runs as one launch of
+// clusters; 0: equal shares for one wave of blocks, and a launch behind them that merges.  As many blocks to an item as are
+// resident at once; clusters of 8 up to 3/2 blocks per SM (with 32 of them a layer of 16 sequences and 2 kv heads took 5 us
+// longer than without clusters: eight free places in one GPC come late).  More items than resident blocks go by ones, but
+// for a wave and a few blocks more, which would wait for a second one.  Attention alone, 32 query and 8 kv heads, equal
+// shares and merge against clusters, us: 1 x 64 / 1000 / 4000 / 16000 keys 4.9 / 8.3 / 15.0 / 24.0 against 3.9 / 5.2 / 8.7 / 24.0, 8 x 1000 14.3
+// against 10.4, 32 x 1000 28.9 against 24.2, 8 x 16387 (3 rows) 87.9 against 81.3, 64 x 4000 156.9 against 154.4; 4 layers and the head, 3 / 16 /
+// 32 sequences 355 / 373 / 408 against 345 / 358 / 396.
+int attn_cluster_ranks(int device, int n_sms, int items, int units) {
+  int ranks = 1;
+  while (ranks < AD_MAX_CLUSTER && ranks < units && items <= attn_cluster_room(device, 2 * ranks) && (ranks < 4 || 16 * items <= 3 * n_sms)) ranks *= 2;
+  const int slots = 2 * n_sms, over = items % slots;
+  if (items > slots && items < 4 * slots && over > 0 && over < slots / 4) return 0;
+  return ranks;
+}
+// ... for R new rows per sequence in a layer, up to position pos_end (a captured pass: up to the context's last).
+int attention_ranks(const dmtd_ctx *c, int B, int R, int pos_end) {
+  if (!tc_decode_attention(c) || !c->fuse_qk_rope || R > AD_MAX_NEW || !c->use_umma || !c->umma_ok) return 0;
+  const int RB = std::max(1, ATTN_QR / (c->s.n_q_heads / c->s.n_kv_heads)), n_rb = (R + RB - 1) / RB;
+  return attn_cluster_ranks(c->device, c->n_sms, B * c->s.n_kv_heads * n_rb, ((c->capturing ? c->max_seq : pos_end) + AD_UNIT - 1) / AD_UNIT);
+}
+
 // Its blocks and slots: as many slots as the partial results' buffer holds (and, up to four rows at a time, the merge
 // inside the O projection's activation-block kernel).
 AttnDecodePlan tc_attention_plan(const dmtd_ctx *c, int B, int R, int max_slots) {
@@ -480,7 +541,7 @@ bool repeats(const dmtd_ctx *c, int M) {
 }
 
 template <int D, typename KVT>
-dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge, bool flash) {
+dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge, bool flash, int ranks) {
   const dmtd_model_shape &s = c->s;
   int M = B * R, heads = s.n_q_heads + 2 * s.n_kv_heads, G = s.n_q_heads / s.n_kv_heads;
   KVT *kc = static_cast<KVT *>(c->kc) + (size_t)layer * c->kv_layer_elems;
@@ -522,10 +583,18 @@ dmtd_status launch_attention_t(dmtd_ctx *c, int layer, int B, int R, const int *
                              c->part_ml, nsplit));
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
+      const AttnFuse fuse{lw.w_qn, lw.w_kn, c->rope_rows, s.rms_eps};
+      if (ranks > 0) {
+        CUDA_TRY(c, launch_cluster(attn_decode_kernel<Op, true, true>, dim3(B * s.n_kv_heads * n_rb * ranks), dim3(AD_THREADS), AD_SMEM, c->stream, ranks,
+                                   c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, 0, nullptr, nullptr, 1, fuse,
+                                   AttnBlocks{c->act_blocks, projection_tiles(c, lw.o_u, M, repeats(c, M))}));
+        LAUNCH_OK(c, "attn_decode_kernel");
+        return DMTD_OK;
+      }
       const int n_blocks = tc_attention_plan(c, B, R, nsplit).n_blocks;
       CUDA_TRY(c, launch_pdl(fused_a3 ? attn_decode_kernel<Op, true> : attn_decode_kernel<Op, false>, dim3(n_blocks), dim3(AD_THREADS),
                              AD_SMEM, c->stream, c->qkv, c->ldqkv, kc, vc, c->max_seq, s.n_q_heads, s.n_kv_heads, B, R, RB, pos0, 0,
-                             c->part_o, c->part_ml, nsplit, AttnFuse{lw.w_qn, lw.w_kn, c->rope_rows, s.rms_eps}));
+                             c->part_o, c->part_ml, nsplit, fuse, AttnBlocks{nullptr, ActTiles{}}));
     }
   } else {
     const AttnPartialKernel<KVT> ap =
@@ -557,15 +626,15 @@ int chunk_positions(const dmtd_ctx *c, int B) {
 }
 
 dmtd_status launch_attention(dmtd_ctx *c, int layer, int B, int R, const int *pos0, int nsplit, bool merge = true,
-                             bool flash = false) {
+                             bool flash = false, int ranks = 0) {
   const int kv = c->s.kv_dtype;
   if (c->s.head_dim == 128)
-    return kv == DMTD_BF16 ? launch_attention_t<128, __nv_bfloat16>(c, layer, B, R, pos0, nsplit, merge, flash)
-         : kv == DMTD_F16 ? launch_attention_t<128, __half>(c, layer, B, R, pos0, nsplit, merge, flash)
-                          : launch_attention_t<128, float>(c, layer, B, R, pos0, nsplit, merge, flash);
-  return kv == DMTD_BF16 ? launch_attention_t<64, __nv_bfloat16>(c, layer, B, R, pos0, nsplit, merge, flash)
-       : kv == DMTD_F16 ? launch_attention_t<64, __half>(c, layer, B, R, pos0, nsplit, merge, flash)
-                        : launch_attention_t<64, float>(c, layer, B, R, pos0, nsplit, merge, flash);
+    return kv == DMTD_BF16 ? launch_attention_t<128, __nv_bfloat16>(c, layer, B, R, pos0, nsplit, merge, flash, ranks)
+         : kv == DMTD_F16 ? launch_attention_t<128, __half>(c, layer, B, R, pos0, nsplit, merge, flash, ranks)
+                          : launch_attention_t<128, float>(c, layer, B, R, pos0, nsplit, merge, flash, ranks);
+  return kv == DMTD_BF16 ? launch_attention_t<64, __nv_bfloat16>(c, layer, B, R, pos0, nsplit, merge, flash, ranks)
+       : kv == DMTD_F16 ? launch_attention_t<64, __half>(c, layer, B, R, pos0, nsplit, merge, flash, ranks)
+                        : launch_attention_t<64, float>(c, layer, B, R, pos0, nsplit, merge, flash, ranks);
 }
 
 RopeTable rope_table(const dmtd_ctx *c) { return RopeTable{c->inv_freq, c->rope_tab, c->s.head_dim / 2}; }
@@ -661,10 +730,11 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   // on the tcgen05 path the O projection's activation blocks come from the prefill attention itself, or from the
   // kernel that merges the key slices
   const bool fuse_merge = tc && (flash || NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS);
-  TRY(launch_attention(c, l, B, R, pos0, nsplit, !fuse_merge, flash));
-  if (fuse_merge) {
+  const int ranks = tc && !flash ? attention_ranks(c, B, R, pos_end) : 0;       // > 0: the attention kernel merges, too
+  TRY(launch_attention(c, l, B, R, pos0, nsplit, !fuse_merge && ranks == 0, flash, ranks));
+  if (fuse_merge || ranks > 0) {
     GemmInput in;
-    in.kind = flash ? GemmInput::READY : GemmInput::SLICES;
+    in.kind = flash || ranks > 0 ? GemmInput::READY : GemmInput::SLICES;
     in.nsplit = nsplit;
     TRY(launch_gemm_tc05(c, lw.o_u, with_sums(in, GemmInput::UNCUT), M, x, H));
   }
@@ -771,14 +841,20 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemv_bf16_kernel<4>, dyn, 100 * 1024));
   for (int whole : {TG_ADD, TG_STORE, TG_SWIGLU})
     for (bool split : {false, true}) CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc05_for(split, whole), dyn, TG_MAX_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<16, 16, 8>, dyn, gemm_f32_smem<16, 16, 8>()));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<64, 64, 1>, dyn, gemm_f32_smem<64, 64, 1>()));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<32, 32, 4>, dyn, gemm_f32_smem<32, 32, 4>()));
+  if (!is_bf16(c)) {
+    CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<16, 16, 8>, dyn, gemm_f32_smem<16, 16, 8>()));
+    CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<64, 64, 1>, dyn, gemm_f32_smem<64, 64, 1>()));
+    CUDA_TRY(c, cudaFuncSetAttribute(gemm_f32_kernel<32, 32, 4>, dyn, gemm_f32_smem<32, 32, 4>()));
+    for (auto gemv : {gemv_f32_fused_kernel<F32_NORM>, gemv_f32_fused_kernel<F32_SWIGLU>, gemv_f32_fused_kernel<F32_SLICES>})
+      CUDA_TRY(c, cudaFuncSetAttribute(gemv, dyn, (int)(F32_FUSE_FLOATS * sizeof(float))));
+  }
   CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16, true>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true>, dyn, AD_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16, true, true>, dyn, AD_SMEM));
+  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true, true>, dyn, AD_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
   CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
   // 16 query rows, 128 dimensions or new rows take the key-group kernel past 48 KiB
@@ -792,8 +868,6 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
     }
     return DMTD_OK;
   };
-  for (auto gemv : {gemv_f32_fused_kernel<F32_NORM>, gemv_f32_fused_kernel<F32_SWIGLU>, gemv_f32_fused_kernel<F32_SLICES>})
-    CUDA_TRY(c, cudaFuncSetAttribute(gemv, dyn, (int)(F32_FUSE_FLOATS * sizeof(float))));
   TRY(partial(0.f));
   TRY(partial(__nv_bfloat16{}));
   TRY(partial(__half{}));
@@ -977,15 +1051,7 @@ dmtd_status enqueue_small(dmtd_ctx *c, int n, bool write_token, int *out_argmax,
   P.sample = sample_params(c);
   P.map = small_pass_map(s.hidden, s.intermediate, s.n_q_heads, s.n_kv_heads, s.n_layers, P.B, P.R);
   P.error = &c->dstate->error; P.wait_limit = kDeviceWaitLimitTicks;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(SP_CTAS); cfg.blockDim = dim3(SP_THREADS); cfg.dynamicSmemBytes = small_pass_smem(P.map); cfg.stream = c->stream;
-  cudaLaunchAttribute attr[2]{};
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = SP_CTAS; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 2;
-  CUDA_TRY(c, cudaLaunchKernelEx(&cfg, small_pass_kernel, P));
+  CUDA_TRY(c, launch_cluster(small_pass_kernel, dim3(SP_CTAS), dim3(SP_THREADS), small_pass_smem(P.map), c->stream, SP_CTAS, P));
   c->launches += 1;
   return DMTD_OK;
 }
@@ -1698,12 +1764,23 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
           part_ml, p.nsplit);
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
+      const int items = B * nkv * n_rb, units = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
+      const int ranks = attn_cluster_ranks(dev, n_sms, items, units);
+      if (ranks > 0) {
+        const auto kernel = attn_decode_kernel<Op, false, true>;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);
+        if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
+        e = launch_cluster(kernel, dim3(items * ranks), dim3(AD_THREADS), AD_SMEM, stream, ranks, q, ld, k, v, max_seq, nq, nkv, B, R, RB, nullptr, pos0,
+                           out, nullptr, 1, AttnFuse{}, AttnBlocks{nullptr, ActTiles{}});
+        if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
+        return DMTD_OK;
+      }
       e = cudaFuncSetAttribute(attn_decode_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: %s", cudaGetErrorString(e));
       const AttnDecodePlan dp = attn_decode_plan(n_sms, B * nkv * n_rb, (pos0 + R + AD_UNIT - 1) / AD_UNIT, p.nsplit);
       nsplit = dp.nsplit;
       e = launch_pdl(attn_decode_kernel<Op, false>, dim3(dp.n_blocks), dim3(AD_THREADS), AD_SMEM, stream, q, ld, k, v, max_seq, nq, nkv, B,
-                     R, RB, nullptr, pos0, part_o, part_ml, nsplit, AttnFuse{});
+                     R, RB, nullptr, pos0, part_o, part_ml, nsplit, AttnFuse{}, AttnBlocks{nullptr, ActTiles{}});
       if (e != cudaSuccess) return fail(nullptr, DMTD_ERR_CUDA, "attention: launch failed: %s", cudaGetErrorString(e));
     }
   } else {

@@ -237,10 +237,11 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *ctx, float temperature, uint64_t seed);
  *   "cuda_graph"   0/1  replay captured CUDA graphs for whole passes (default 1)
  *   "literal_sum"  0/1  upper-layer input of a full pass = embedding + lower-stack output, the
  *                       literal sum of Eq. 4, instead of the lower-stack output alone (default 0)
- *   "fused_pass"   0/1  run each decode pass as one persistent kernel where the model and batch
- *                       allow it (bf16 weights, head_dim 128, at most 4 rows per pass; small fp32
- *                       models: one cluster); 0 = always the per-step kernels.  Until it is set,
- *                       whichever is the faster for the model and the batch
+ *   "fused_pass"   0/1  1 = run each decode pass as one persistent kernel where the model and batch
+ *                       allow it (bf16 weights, head_dim 128, at most 4 rows per pass), 0 = always
+ *                       the per-step kernels.  Until it is set: one kernel for bf16 models with
+ *                       an fp32 cache or without block-ordered weights, the per-step kernels, which
+ *                       are the faster ones, for other bf16 models; small fp32 models: one cluster
  *   "encoding_layers" x  the ExDy variant (Section 2.1, the paragraph after Eq. 4; Section 3.3): the
  *                       short passes run the first x encoding layers as well as the last L_d
  *                       decoding layers, the decoding layers read the encoding layers' output

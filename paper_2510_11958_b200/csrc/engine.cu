@@ -88,8 +88,8 @@ struct dmtd_ctx {
   int pend_cap = 0;
 
   // options
-  bool use_graph = true, literal_sum = false, use_fused = true, use_tc_attention = true;
-  bool choose_fused = true;                 // the pass kernel only where it is the faster one (until the option is set)
+  bool use_graph = true, literal_sum = false, use_tc_attention = true;
+  int pass_option = -1;                     // the option "fused_pass", once it is set
   bool fuse_qk_rope = true;                 // QK-norm, RoPE and the KV append inside the tensor-core attention kernel
   float temperature = 0.f;                  // > 0: tokens are drawn from softmax(logits / temperature); 0: greedy
   uint64_t sample_seed = 0;
@@ -848,15 +848,15 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
     for (auto gemv : {gemv_f32_fused_kernel<F32_NORM>, gemv_f32_fused_kernel<F32_SWIGLU>, gemv_f32_fused_kernel<F32_SLICES>})
       CUDA_TRY(c, cudaFuncSetAttribute(gemv, dyn, (int)(F32_FUSE_FLOATS * sizeof(float))));
   }
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16, true>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpBf16, true, true>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<OpF16, true, true>, dyn, AD_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpBf16>, dyn, AP_SMEM));
-  CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<OpF16>, dyn, AP_SMEM));
+  // (only the kernels of the context's cache type: the first touch of a kernel loads it)
+  auto attention = [&](auto op) -> dmtd_status {
+    using Op = decltype(op);
+    CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<Op>, dyn, AD_SMEM));
+    CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<Op, true>, dyn, AD_SMEM));
+    CUDA_TRY(c, cudaFuncSetAttribute(attn_decode_kernel<Op, true, true>, dyn, AD_SMEM));
+    CUDA_TRY(c, cudaFuncSetAttribute(attn_prefill_kernel<Op>, dyn, AP_SMEM));
+    return DMTD_OK;
+  };
   // 16 query rows, 128 dimensions or new rows take the key-group kernel past 48 KiB
   auto partial = [&](auto kv) -> dmtd_status {
     using KVT = decltype(kv);
@@ -868,10 +868,16 @@ dmtd_status configure_kernels(dmtd_ctx *c) {
     }
     return DMTD_OK;
   };
-  TRY(partial(0.f));
-  TRY(partial(__nv_bfloat16{}));
-  TRY(partial(__half{}));
-  return DMTD_OK;
+  if (c->s.kv_dtype == DMTD_F32) {
+    CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel, dyn, ATTN_F32_SMEM));
+    return partial(0.f);
+  }
+  if (c->s.kv_dtype == DMTD_BF16) {
+    TRY(attention(OpBf16{}));
+    return partial(__nv_bfloat16{});
+  }
+  TRY(attention(OpF16{}));
+  return partial(__half{});
 }
 
 // ---------------------------------------------------------------------------- fused pass
@@ -941,19 +947,17 @@ dmtd_status setup_fused(dmtd_ctx *c) {
   return DMTD_OK;
 }
 
-// One sequence of a model with large layers.  Cycles of 1 to 4 passes, the pass kernel's time over the per-step kernels': one
-// sequence, context 64 to 3000, hidden 640 (7 MB a layer) 1.25 to 1.07, 1024 1.18 to 1.04, 1536 1.12 to 1.02, 2048 (100 MB)
-// 1.09 to 1.01, 2560 (202 MB) 1.03, and over 36 layers (7 cycles at 512 to 2500) 0.985; two sequences of 2560 1.05, three
-// 1.08 to 1.11, four 1.11 to 1.18.
-bool pass_kernel_faster(const dmtd_ctx *c) {
-  const LayerDev &l = c->layers[0];
-  return c->B == 1 && packed_atoms(l.qkv) + packed_atoms(l.o) + packed_atoms(l.gu) + packed_atoms(l.down) >= (128 << 10);      // 1 KiB atoms
-}
+// The pass kernel runs where the option asks for it, and unasked where the per-step path lacks the block-ordered weights or the
+// tensor-core attention (an fp32 cache): with both, a launch per step is faster at every size, since its rings fill at HBM's pace
+// and the attention merges by cluster.  Cycles of 1 to 4 passes, the pass kernel's time over the per-step kernels': one sequence,
+// context 64 to 3000, hidden 640 (7 MB a layer) 1.25 to 1.07, 1024 1.18 to 1.04, 2048 (100 MB) 1.09 to 1.01, 2560 (202 MB) 1.03
+// to 1.05, over 36 layers 1.01 at 550 positions and 1.03 at 2500 (8 cycles 25.2 / 26.65 ms against 24.95 / 25.7); two sequences
+// of 2560 1.05, three 1.08 to 1.11, four 1.11 to 1.18.
 bool fused_pass_ok(const dmtd_ctx *c, int kind, int R_lower) {
-  if (!c->fused_ok || !c->use_fused || c->literal_sum || c->L_e > 0) return false;
+  const bool asked = c->pass_option >= 0 ? c->pass_option != 0 : !(c->umma_ok && c->use_umma && tc_decode_attention(c) && c->fuse_qk_rope);
+  if (!c->fused_ok || !asked || c->literal_sum || c->L_e > 0) return false;
   const int lo = c->s.n_layers - c->L_d;
   const int R = (kind == 1 && lo > 0) ? R_lower : 1;
-  if (c->choose_fused && !pass_kernel_faster(c)) return false;
   return c->B * R <= PK_MAX_ROWS && R * (c->s.n_q_heads / c->s.n_kv_heads) <= PK_QR &&
          c->B * R * c->s.hidden <= PK_XS_FLOATS;
 }
@@ -1020,7 +1024,7 @@ dmtd_status setup_small(dmtd_ctx *c) {
 // 105 / 121 / 199; 2 sequences (6 rows), context 1800 (450 keys) 239 against 183, 7000 (1750 keys) 328 against 371; 4 sequences, 2 passes,
 // 1800 (900 keys) 194 against 190; 8 sequences, 1 pass, 600 keys 130 against 122, 1800 keys 157 against 200.
 bool small_pass_ok(const dmtd_ctx *c, int kind, int R_lower) {
-  if (!c->small_ok || !c->use_fused || c->literal_sum || c->L_e > 0) return false;
+  if (!c->small_ok || c->pass_option == 0 || c->literal_sum || c->L_e > 0) return false;
   const dmtd_model_shape &s = c->s;
   const int R = kind == 1 && s.n_layers > c->L_d ? R_lower : 1, G = s.n_q_heads / s.n_kv_heads, M = c->B * R, items = c->B * s.n_kv_heads;
   if (M > SP_MAX_ROWS || R * G > SP_MAX_ROWS || items > SP_CTAS) return false;
@@ -1658,7 +1662,7 @@ dmtd_status dmtd_set_option(dmtd_ctx *c, const char *name, int64_t value) {
   if (value != 0 && value != 1) return fail(c, DMTD_ERR_INVALID_ARG, "option %s takes 0 or 1", name);
   if (!strcmp(name, "cuda_graph")) { c->use_graph = value != 0; return DMTD_OK; }
   if (!strcmp(name, "literal_sum")) { c->literal_sum = value != 0; drop_graphs(c); return DMTD_OK; }
-  if (!strcmp(name, "fused_pass")) { c->use_fused = value != 0; c->choose_fused = false; return DMTD_OK; }
+  if (!strcmp(name, "fused_pass")) { c->pass_option = (int)value; return DMTD_OK; }
   if (!strcmp(name, "fused_qk_rope")) { c->fuse_qk_rope = value != 0; drop_graphs(c); return DMTD_OK; }
   if (!strcmp(name, "tcgen05_gemm")) { c->use_umma = value != 0; drop_graphs(c); return DMTD_OK; }
   if (!strcmp(name, "tc_attention")) { c->use_tc_attention = value != 0; drop_graphs(c); return DMTD_OK; }

@@ -48,15 +48,27 @@ __device__ __forceinline__ uint32_t ad_part(int row, int part) {
   return (uint32_t)(row * 256 + ((part & 8) | ((part & 7) ^ (((row & 1) << 2) | ((row >> 1) & 3)))) * 16);
 }
 
+// The score that a tile's probabilities are taken relative to, exp(s - level): the tile's own largest, whose probability then
+// is 1 and loses nothing when the probabilities are rounded to 16 bits for the product with V, but not more than AD_BELOW
+// below the largest so far, so that sums stay within exp(AD_BELOW) of their usual size (tiles further down hardly count).
+// With the running maximum alone the rounding loss grew with the tiles to a warp: 32 query and 8 kv heads, 1 x 1000 keys,
+// bf16, error against fp64 1.91e-3 with one tile to a warp and 1.95e-3 with two.
+constexpr float AD_BELOW = 4.f;
+__device__ __forceinline__ float attn_level(float &top, float tile_max) {
+  top = fmaxf(top, tile_max);
+  return fmaxf(tile_max, top - AD_BELOW);
+}
+
 // One warp tile (16 keys, K at k_t, V at v_t) against up to 8 query rows, operands swapped: the keys are the M axis of
 // S^T = K Q^T and the 128 output dimensions the M axis of O^T = V^T P^T, the query rows the 8 columns (with the rows on
 // the M axis an m16 tile would be half padding or more).  Thread (g, t) holds columns (query rows) 2t, 2t + 1 of rows
 // g and g + 8.  lim[e]: keys this lane's query row 2t + e sees, counted from the tile's first key.
 struct AttnAccS {
-  float m_run[2], l_part[2];       // per query row 2t, 2t + 1: running max, this lane's share of the running sum
+  float m_run[2], l_part[2];       // per query row 2t, 2t + 1: level of the sums, this lane's share of the running sum
+  float top[2];                    // ... the largest score
   float o[8][4];                   // O^T: m-tile dt = dimensions 16 dt .. + 15
   __device__ __forceinline__ void clear() {
-    m_run[0] = m_run[1] = -INFINITY;
+    m_run[0] = m_run[1] = top[0] = top[1] = -INFINITY;
     l_part[0] = l_part[1] = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
@@ -88,7 +100,7 @@ __device__ __forceinline__ void attn_tile_swap(AttnAccS &A, uint32_t k_t, uint32
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-    const float m_new = fmaxf(A.m_run[hq], mx);
+    const float m_new = attn_level(A.top[hq], mx);
     corr[hq] = m_new > -INFINITY ? __expf(A.m_run[hq] - m_new) : 1.f;
     A.m_run[hq] = m_new;
   }
@@ -118,10 +130,10 @@ __device__ __forceinline__ void attn_tile_swap(AttnAccS &A, uint32_t k_t, uint32
 // The same with 9 to 16 query rows, on the M axis: thread (g, t) holds rows g, g + 8 and keys (dimensions) 2t, 2t + 1 of
 // every 8.  lim[h]: keys row g + 8 h sees.
 struct AttnAccW {
-  float m_run[2], l_part[2];
+  float m_run[2], l_part[2], top[2];
   float o[16][4];
   __device__ __forceinline__ void clear() {
-    m_run[0] = m_run[1] = -INFINITY;
+    m_run[0] = m_run[1] = top[0] = top[1] = -INFINITY;
     l_part[0] = l_part[1] = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
@@ -161,7 +173,7 @@ __device__ __forceinline__ void attn_tile_rows(AttnAccW &A, uint32_t k_t, uint32
     float mx = fmaxf(fmaxf(c[0][2 * hr], c[0][2 * hr + 1]), fmaxf(c[1][2 * hr], c[1][2 * hr + 1]));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float m_new = fmaxf(A.m_run[hr], mx);
+    const float m_new = attn_level(A.top[hr], mx);
     corr[hr] = m_new > -INFINITY ? __expf(A.m_run[hr] - m_new) : 1.f;
     A.m_run[hr] = m_new;
   }
@@ -193,7 +205,7 @@ __device__ __forceinline__ void attn_tile_rows(AttnAccW &A, uint32_t k_t, uint32
   }
 }
 
-// The warps' running max, sum and unnormalised output go to shared memory as [warp][query row][dimension].
+// The warps' level, sum and unnormalised output go to shared memory as [warp][query row][dimension].
 __device__ __forceinline__ void attn_acc_store(AttnAccS &A, float *o_s, float *red_m, float *red_l, int nQ) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -438,7 +450,7 @@ attn_decode_kernel(const float *qkv, int ldq, const void *kc, const void *vc, in
       attn_acc_store(A, o_s, red_m, red_l, nQ);
     }
     __syncthreads();
-    // per query row: the piece's max and sum, and the factor each warp's share is scaled by (a warp without keys: 0)
+    // per query row: the piece's largest level and its sum, and the factor each warp's share is scaled by (a warp without keys: 0)
     if ((int)threadIdx.x < nQ) {
       const int qi = threadIdx.x;
       float m = -INFINITY;

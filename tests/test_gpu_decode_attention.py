@@ -47,6 +47,33 @@ def test_attention_decode_pieces(dmtd, dtype, B, R, nq, nkv, n_keys):
     assert err <= 4 * u * max(1.0, ref.abs().max().item()), err
 
 
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("R,n_keys", [(1, 1000), (4, 1000), (1, 8000), (4, 2052)])
+def test_largest_probability_of_a_tile_is_not_rounded(dmtd, dtype, R, n_keys):
+    """Every 16 keys one that counts, with a value of its own: its weight carries no 16-bit rounding, whatever number of
+    tiles a warp walks."""
+    nq, nkv, D, pos0 = 32, 8, 128, n_keys - R
+    g = torch.Generator(device="cuda").manual_seed(13)
+    q = torch.zeros(1, R, nq, D, device="cuda")              # exact in 16 bits once it is scaled by 1 / sqrt(D)
+    q[..., 0] = torch.tensor([1.0, -1.0, 0.5, -0.75], device="cuda").repeat(nkv)
+    q[..., 1] = 1.0
+    k, v = (torch.zeros(1, nkv, n_keys, D, device="cuda") for _ in range(2))
+    tiles = n_keys // 16
+    k[..., 1] = -40.0                                        # exp(-40): below the bound
+    k[:, :, :tiles * 16:16, 1] = 0.0
+    k[:, :, :tiles * 16:16, 0] = torch.randint(-96, 97, (1, nkv, tiles), generator=g, device="cuda") / 64.0
+    t = torch.arange(tiles, device="cuda")
+    v[:, :, t * 16, t % D] = 1.0
+    out = dmtd.attention_decode(q * D ** 0.5, k.to(dtype), v.to(dtype), pos0)
+    s = torch.einsum("brhd,bhkd->bhrk", q.double(), k.double().repeat_interleave(nq // nkv, 1))
+    hidden = torch.arange(n_keys, device="cuda")[None] > (pos0 + torch.arange(R, device="cuda"))[:, None]
+    p = torch.softmax(s.masked_fill(hidden, float("-inf")), -1)
+    ref = torch.einsum("bhrk,bhkd->brhd", p, v.double().repeat_interleave(nq // nkv, 1))
+    seen = ref > 1e-12
+    # fp32: exponentials of at most 4 to 2^-21 or two, a factor of as much per tile of a warp's chain (8000 keys: 16)
+    assert ((out.double() - ref).abs() / ref)[seen].max() <= 2e-5
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("B,R,nq,nkv,n_keys", [
     (1, 1, 4, 2, 1),            # one key

@@ -1769,7 +1769,8 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
     } else {
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
       const int items = B * nkv * n_rb, units = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
-      const int ranks = attn_cluster_ranks(dev, n_sms, items, units);
+      // the clusters store whole float4; results that begin elsewhere go through the merge kernel, which stores single values
+      const int ranks = reinterpret_cast<uintptr_t>(out) % 16 ? 0 : attn_cluster_ranks(dev, n_sms, items, units);
       if (ranks > 0) {
         const auto kernel = attn_decode_kernel<Op, false, true>;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);

@@ -74,6 +74,32 @@ def test_largest_probability_of_a_tile_is_not_rounded(dmtd, dtype, R, n_keys):
     assert ((out.double() - ref).abs() / ref)[seen].max() <= 2e-5
 
 
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("R,n_keys", [(1, 40), (3, 1000)])
+def test_results_off_a_16_byte_boundary(dmtd, dtype, R, n_keys):
+    """q and out are float arrays of the caller: views into larger buffers begin at any float."""
+    B, nq, nkv, D, pos0 = 2, 8, 2, 128, n_keys - R
+    g = torch.Generator(device="cuda").manual_seed(14)
+    k, v = (torch.randn(B, nkv, n_keys, D, generator=g, device="cuda").to(dtype) for _ in range(2))
+    n = B * R * nq * D
+    q_room = torch.randn(n + 8, generator=g, device="cuda")
+    want = dmtd.attention_decode(q_room[:n].reshape(B, R, nq, D), k, v, pos0)
+    dll, code = dmtd.load_library(), {torch.float16: 2, torch.bfloat16: 1}[dtype]
+    scratch = torch.empty(dll.dmtd_attention_scratch_bytes(B, R, nq, D, n_keys), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    u = 2.0 ** -9 if dtype == torch.bfloat16 else 2.0 ** -12            # the probabilities' rounding, on both sides
+    for off in (1, 2, 3):
+        q = torch.empty(n + 8, device="cuda")[off:off + n].view(B, R, nq, D).copy_(q_room[:n].view(B, R, nq, D))
+        room = torch.full((2, n + 8), 7.0, device="cuda")
+        dmtd.attention_decode_static(q, k, v, pos0, room[0, off:off + n].view(B, R, nq, D))
+        out = room[1, off:off + n]
+        assert dll.dmtd_attention_decode(q.data_ptr(), k.data_ptr(), v.data_ptr(), code, B, R, nq, nkv, D, n_keys, pos0,
+                                         scratch.data_ptr(), scratch.numel(), out.data_ptr(), stream) == 0
+        for row in room:
+            assert (row[off:off + n].view_as(want) - want).abs().max() <= 4 * u * max(1.0, want.abs().max().item())
+            assert (row[:off] == 7.0).all() and (row[off + n:] == 7.0).all()
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("B,R,nq,nkv,n_keys", [
     (1, 1, 4, 2, 1),            # one key

@@ -488,23 +488,31 @@ int attn_cluster_room(int device, int ranks) {
 // Blocks of a cluster to an item (sequence, kv head, row block) of `units` 64-key units where the attention runs as one launch of
 // clusters; 0: equal shares for one wave of blocks, and a launch behind them that merges.  As many blocks to an item as are
 // resident at once; clusters of 8 up to 3/2 blocks per SM (with 32 of them a layer of 16 sequences and 2 kv heads took 5 us
-// longer than without clusters: eight free places in one GPC come late).  More items than resident blocks go by ones, but
-// for a wave and a few blocks more, which would wait for a second one.  Attention alone, 32 query and 8 kv heads, equal
+// longer than without clusters: eight free places in one GPC come late).  Attention alone, 32 query and 8 kv heads, equal
 // shares and merge against clusters, us: 1 x 64 / 1000 / 4000 / 16000 keys 4.9 / 8.3 / 15.0 / 24.0 against 3.9 / 5.2 / 8.7 / 24.0, 8 x 1000 14.3
-// against 10.4, 32 x 1000 28.9 against 24.2, 8 x 16387 (3 rows) 87.9 against 81.3, 64 x 4000 156.9 against 154.4; 4 layers and the head, 3 / 16 /
-// 32 sequences 355 / 373 / 408 against 345 / 358 / 396.
-int attn_cluster_ranks(int device, int n_sms, int items, int units) {
+// against 10.4, 32 x 1000 28.9 against 24.2, 8 x 16387 (3 rows) 87.9 against 81.3; 4 layers and the head, 3 / 16 / 32 sequences
+// 355 / 373 / 408 against 345 / 358 / 396.
+// More items than resident blocks: one block each, or equal shares.  Alone, ones up to three waves (two with few keys), but for a few
+// items more than whole waves, which wait for another one; 128 / 300 / 1000 / 4000 keys, ones' time over equal shares': 320 items 0.80
+// / 1.07 / 1.02 / 1.00, 512 0.95 / 0.95 / 0.97 / 0.98, 640 1.10 / 1.02 / 1.00 / 0.98, 832 1.02 / 1.01 / 0.99 / 0.98, 1040 1.09 / 1.02 / 1.00 / 1.01, 2000 1.16
+// / 1.04 / 1.01.  In a layer, whose next launch waits for the last wave, only for short items in a well filled second wave; the
+// whole layer, one row: 320 items 1.03 / 1.05 / 1.11 / 1.18, 384 1.03 / 1.01 / 1.04 / 1.09, 512 0.99 / 1.00 / 1.02 /
+// 0.99 (three rows 0.98 / 0.98 / 1.01 / 1.01), 592 1.00, 640 1.05 / 1.05 / 1.07 / 1.08, 832 1.01 / 1.02 / 1.03 / 1.00, 1280 1.06 / 1.05 / 1.07 / 1.03.
+int attn_cluster_ranks(int device, int n_sms, int items, int units, bool in_layer) {
+  const int slots = 2 * n_sms, over = items % slots;
+  if (items > slots) {
+    if (in_layer) return 2 * items > 3 * slots && items <= 2 * slots && units <= 8 ? 1 : 0;
+    return (over > 0 && over < slots / 4) || items > (units > 4 ? 3 : 2) * slots ? 0 : 1;
+  }
   int ranks = 1;
   while (ranks < AD_MAX_CLUSTER && ranks < units && items <= attn_cluster_room(device, 2 * ranks) && (ranks < 4 || 16 * items <= 3 * n_sms)) ranks *= 2;
-  const int slots = 2 * n_sms, over = items % slots;
-  if (items > slots && items < 4 * slots && over > 0 && over < slots / 4) return 0;
   return ranks;
 }
 // ... for R new rows per sequence in a layer, up to position pos_end (a captured pass: up to the context's last).
 int attention_ranks(const dmtd_ctx *c, int B, int R, int pos_end) {
   if (!tc_decode_attention(c) || !c->fuse_qk_rope || R > AD_MAX_NEW || !c->use_umma || !c->umma_ok) return 0;
   const int RB = std::max(1, ATTN_QR / (c->s.n_q_heads / c->s.n_kv_heads)), n_rb = (R + RB - 1) / RB;
-  return attn_cluster_ranks(c->device, c->n_sms, B * c->s.n_kv_heads * n_rb, ((c->capturing ? c->max_seq : pos_end) + AD_UNIT - 1) / AD_UNIT);
+  return attn_cluster_ranks(c->device, c->n_sms, B * c->s.n_kv_heads * n_rb, ((c->capturing ? c->max_seq : pos_end) + AD_UNIT - 1) / AD_UNIT, true);
 }
 
 // Its blocks and slots: as many slots as the partial results' buffer holds (and, up to four rows at a time, the merge
@@ -1770,7 +1778,7 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
       const int items = B * nkv * n_rb, units = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
       // the clusters store whole float4; results that begin elsewhere go through the merge kernel, which stores single values
-      const int ranks = reinterpret_cast<uintptr_t>(out) % 16 ? 0 : attn_cluster_ranks(dev, n_sms, items, units);
+      const int ranks = reinterpret_cast<uintptr_t>(out) % 16 ? 0 : attn_cluster_ranks(dev, n_sms, items, units, false);
       if (ranks > 0) {
         const auto kernel = attn_decode_kernel<Op, false, true>;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);

@@ -29,6 +29,8 @@ def dmtd():
     (8, 2, 70, 1, 200),          # 140 items
     (8, 2, 148, 1, 70),          # 296 items: a block each
     (8, 2, 150, 1, 70),          # 300 items: a few more than resident blocks
+    (8, 2, 250, 1, 70),          # 500 items: a block each
+    (8, 2, 300, 1, 70),          # 600 items: a few more than two waves
 ])
 def test_layer(dmtd, kv, nq, nkv, B, R, pos0):
     shape = SHAPES["mid"].with_(n_layers=1, hidden=256, intermediate=256, n_q_heads=nq, n_kv_heads=nkv, vocab=64)
@@ -50,3 +52,24 @@ def test_layer(dmtd, kv, nq, nkv, B, R, pos0):
     # query and probabilities rounded to 16 bits on both sides, the latter against other maxima: 2^-9 (bf16) or 2^-12 each
     tol = 4e-3 if kv == "bf16" else 5e-4
     assert (out[0] - out[2]).abs().max() <= tol * max(1.0, out[2].abs().max().item())
+
+
+def test_more_items_than_resident_blocks(dmtd):
+    """A layer takes a block to an item, and no launch that merges, up to one wave, and for short items in a well filled
+    second one; otherwise equal shares and a merge, which are faster there."""
+    shape = SHAPES["mid"].with_(n_layers=1, hidden=256, intermediate=256, vocab=64)
+    eng = dmtd.Dmtd(shape, to_cuda(make_weights(shape, seed=3)), L_d=1, tau=1, max_batch=600, max_seq=700, kv_dtype="f16")
+    wave = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+
+    def launches(items, pos0):
+        B = items // shape.n_kv_heads
+        x = torch.zeros(B, 1, shape.hidden, device="cuda")
+        n0 = eng.launch_count()
+        eng.step_layers(0, 1, x, pos0)
+        # more than 128 rows: gate+up and down run differently; the number of launches is the same up to there and from there
+        return eng.launch_count() - n0
+
+    one_launch = launches(wave, 600)
+    assert launches(wave * 9 // 5, 200) == one_launch
+    for items, pos0 in [(wave + 60, 200), (wave * 9 // 5, 600), (wave * 5 // 2, 200), (wave * 4, 64)]:
+        assert launches(items, pos0) == one_launch + 1

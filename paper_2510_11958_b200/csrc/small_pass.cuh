@@ -17,7 +17,9 @@
 //  * The passes of a cycle are one launch: the first may be a full one (R rows per sequence through the lower layers), the
 //    others are short.  The picked token never leaves the cluster between them.
 //  * A buffer is overwritten at the earliest by outputs that another block could only compute from this block's outputs of
-//    the step that read it, so every barrier has one phase per layer and no buffer needs a second copy.
+//    the step that read it, so every barrier has one phase per layer and no buffer needs a second copy.  A barrier says
+//    nothing about this block's other warps (a block's own slices may be complete by one warp's outputs): what a block writes
+//    for itself, the attention's merged rows, goes where no warp reads since the last __syncthreads.
 //  * What a step costs is the length of a warp's chain of instructions: 8 warps (two to a scheduler), shares without
 //    remainders (small_pass_fits), index arithmetic once per launch.  With 16 warps and
 //    general shares a step took 4500 cycles.
@@ -52,7 +54,8 @@ struct SmallLayer {
 struct SmallMap {
   int xs;          // residual rows [M][H]
   int qkv;         // [M][(nq + 2 nkv) 64]
-  int wide;        // gated rows [M][I]; before that the attention's warps' outputs, then its merged rows [M][nq 64]
+  int merged;      // the attention's merged rows [M][nq 64], where qkv was
+  int wide;        // gated rows [M][I]; before that the attention's warps' outputs
   int part_o;      // partial results of the key slices [row][head][slice][64]
   int part_ml;     // ... their (max, sum) pairs
   int q;           // query rows [8][64], normalised, rotated, scaled
@@ -434,7 +437,7 @@ __device__ __forceinline__ void sp_load_tile(SmallTile &t, const float *kc, cons
 }
 
 // Steps a3 and a4: a block takes a kv head of a sequence and a slice of its keys; the partial results of the slices go to
-// every block.  Then their merge, into `wide`.  The last slice takes the pass's own rows.
+// every block.  Then their merge, over the projection's rows.  The last slice takes the pass's own rows.
 __device__ __forceinline__ void sp_attention(const SmallParams &P, uint32_t &phases, int layer, const SmallItem &T, int b, int kvh, int slice) {
   constexpr int D = SP_D, D4 = D / 4;
   float *const f = sp_floats();
@@ -600,7 +603,7 @@ __device__ __forceinline__ void sp_attention(const SmallParams &P, uint32_t &pha
   }
   // the merge
   sp_wait(P, SP_BAR_PART, phases, (uint32_t)(M * P.nq * ns * (D + 2) * 4));
-  float4 *const att = reinterpret_cast<float4 *>(f + map.wide);
+  float4 *const att = reinterpret_cast<float4 *>(f + map.merged);         // (not over the warps' outputs: other warps may still read them)
   for (int i = threadIdx.x; i < M * P.nq * D4; i += SP_THREADS) {
     const int rh = i / D4, d4 = i % D4;
     const float2 *ml = reinterpret_cast<const float2 *>(f + map.part_ml) + rh * ns;
@@ -638,7 +641,7 @@ __device__ __forceinline__ void sp_layer(const SmallParams &P, SmallCursor &cur,
   for (int n = 0; n < n_qkv; n += 4)
     sp_batch<SP_QKV, MR>(P, cur, H, X, n == 0, scale, M, map.qkv + share * n_qkv + n, ldq, rbase, rbars + 8 * SP_BAR_QKV);
   sp_attention(P, phases, layer, T, b, kvh, slice);
-  const SmallX A{f + map.wide, QD, M, nullptr};
+  const SmallX A{f + map.merged, QD, M, nullptr};
   const int at_h = map.xs + x_off + share * n_h;
 #pragma unroll 1
   for (int n = 0; n < n_h; n += 2) sp_batch<SP_O, MR>(P, cur, QD, A, false, scale, M, at_h + n, x_ld, rbase, rbars + 8 * SP_BAR_O);
@@ -828,8 +831,8 @@ inline SmallMap small_pass_map(int H, int I, int nq, int nkv, int n_layers, int 
   int at = 0;
   auto take = [&](int n) { const int r = at; at += (n + 31) / 32 * 32; return r; };
   m.xs = take(M * H);
-  m.qkv = take(M * (nq + 2 * nkv) * SP_D);
-  m.wide = take(std::max({M * I, M * nq * SP_D, SP_WARPS * SP_MAX_ROWS * SP_D}));
+  m.qkv = m.merged = take(M * (nq + 2 * nkv) * SP_D);
+  m.wide = take(std::max(M * I, SP_WARPS * SP_MAX_ROWS * SP_D));
   m.part_o = take(M * nq * ns * SP_D);
   m.part_ml = take(M * nq * ns * 2);
   m.q = take(SP_MAX_ROWS * SP_D);

@@ -86,3 +86,19 @@ def test_small_pass(dmtd, weights, name, L_d, tau, B, P, sample):
         assert (am[clear] == ref_am[clear]).all()
     if not sample and clear.all():
         assert (toks == ref_toks).all()
+
+
+def test_same_bits_every_time(dmtd, weights):
+    """No buffer is written while a warp may still read it: repeated passes give the same logits, bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    for B, tau, P in ((1, 3, 90), (1, 4, 500), (2, 4, 40)):
+        eng = dmtd.Dmtd(SHAPE, weights["tiny"], L_d=2, tau=tau, max_batch=B, max_seq=P + 5 * tau, kv_dtype="f32")
+        prompt = torch.randint(0, SHAPE.vocab, (B, P), generator=g, dtype=torch.int32, device="cuda")
+        forced = torch.randint(0, SHAPE.vocab, (B, 4 * tau), generator=g, dtype=torch.int32, device="cuda")
+        want = None
+        for _ in range(40):
+            eng.reset()
+            eng.prefill(prompt)
+            logits, _ = eng.decode_forced(forced)
+            want = logits if want is None else want
+            assert torch.equal(logits, want)

@@ -97,7 +97,7 @@ enum { SP_QKV = 0, SP_O, SP_GU, SP_DOWN, SP_HEAD };
 // A warp's share of a matrix, as its producer walks it: groups of four parts of a thread, one 128-value piece of four rows
 // or two pieces of two rows.
 struct __align__(16) SmallWalk {
-  uint32_t first;            // bytes from the matrix to the share
+  size_t first;              // bytes from the matrix to the share (a head may be larger than 4 GiB)
   uint32_t o1, o2, o3;       // from a group's first part to the others
   uint32_t step, skip;       // to the next group of a batch of rows; from the end of a batch to the next one
   int pieces, batches;       // groups of a batch; batches
@@ -204,20 +204,21 @@ __device__ __forceinline__ void sp_wait(const SmallParams &P, int which, uint32_
 }
 
 // The rows of a head share, a multiple of four: all of them for a warp before the vocabulary's end.
-__device__ __forceinline__ int sp_head_share(int vocab) { return ((vocab + SP_SHARES - 1) / SP_SHARES + 3) & ~3; }
-__device__ __forceinline__ SmallWalk sp_walk(const SmallParams &P, int kind, int warp) {
-  const int share = blockIdx.x * SP_WARPS + warp;
+__host__ __device__ __forceinline__ int sp_head_share(int vocab) { return ((vocab + SP_SHARES - 1) / SP_SHARES + 3) & ~3; }
+__host__ __device__ __forceinline__ SmallWalk sp_walk(const SmallParams &P, int kind, int share) {
   int K = P.H, first, n;     // values of a row; first row, rows (pairs for gate+up)
   if (kind == SP_HEAD) {
     const int per = sp_head_share(P.vocab);
-    first = share * per; n = max(0, min(per, P.vocab - first));
+    first = share * per;
+    n = first >= P.vocab ? 0 : P.vocab - first < per ? P.vocab - first : per;
   } else {
     n = (kind == SP_QKV ? (P.nq + 2 * P.nkv) * SP_D : kind == SP_GU ? P.I : P.H) / SP_SHARES;
     if (kind == SP_O) K = P.nq * SP_D;
     if (kind == SP_DOWN) K = P.I;
     first = share * n;
   }
-  const uint32_t row = K * 4, up = (uint32_t)P.I * row, at = (uint32_t)first * row;
+  const uint32_t row = K * 4, up = (uint32_t)P.I * row;
+  const size_t at = (size_t)first * row;
   if (kind == SP_O || kind == SP_DOWN) return SmallWalk{at, row, 512, row + 512, 1024, row, K / 256, n / 2};
   if (kind == SP_GU) return SmallWalk{at, up, row, up + row, 512, row, K / 128, n / 2};
   return SmallWalk{at, row, 2 * row, 3 * row, 512, 3 * row, K / 128, n / 4};
@@ -693,7 +694,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) small_pass_kernel(const __grid_
     F.gave_up = 0;
     fence_mbar_init();
   }
-  if (threadIdx.x < 5 * SP_WARPS) F.walk[threadIdx.x / SP_WARPS][threadIdx.x % SP_WARPS] = sp_walk(P, threadIdx.x / SP_WARPS, threadIdx.x % SP_WARPS);
+  if (threadIdx.x < 5 * SP_WARPS) F.walk[threadIdx.x / SP_WARPS][threadIdx.x % SP_WARPS] = sp_walk(P, threadIdx.x / SP_WARPS, blockIdx.x * SP_WARPS + threadIdx.x % SP_WARPS);
   if ((int)threadIdx.x < P.n_layers) {
     const SmallLayer &L = P.layers[threadIdx.x];
     F.w[threadIdx.x][SP_QKV] = L.qkv; F.w[threadIdx.x][SP_O] = L.o; F.w[threadIdx.x][SP_GU] = L.gu; F.w[threadIdx.x][SP_DOWN] = L.down;

@@ -1,5 +1,5 @@
 """Shared memory of the cluster pass for small fp32 models, as the library's own host code lays it out: buffers that are in use
-at the same time lie apart.  Runs without a GPU."""
+at the same time lie apart; and where the warps' shares of a matrix lie.  Runs without a GPU."""
 import os
 import subprocess
 
@@ -12,6 +12,13 @@ PROBE = r"""
 #include "small_pass.cuh"
 int main(int argc, char **argv) {
   int a[7];
+  if (argc == 4) {
+    dmtd::SmallParams P{};
+    P.H = atoi(argv[1]); P.vocab = atoi(argv[2]);
+    const dmtd::SmallWalk w = dmtd::sp_walk(P, dmtd::SP_HEAD, atoi(argv[3]));
+    printf("%zu %d\n", (size_t)w.first, w.batches);
+    return 0;
+  }
   for (int i = 0; i < 7; ++i) a[i] = atoi(argv[i + 1]);
   const dmtd::SmallMap m = dmtd::small_pass_map(a[0], a[1], a[2], a[3], a[4], a[5], a[6]);
   printf("%d %d %d %d %d %d %d\n", m.xs, m.qkv, m.merged, m.wide, m.part_o, m.total, dmtd::SP_WARPS * dmtd::SP_MAX_ROWS * dmtd::SP_D);
@@ -43,3 +50,15 @@ def test_buffers_in_use_at_once_lie_apart(probe, H, I, nq, nkv, L, B, R):
     # merged rows may take the place of the projection's rows, which no warp reads any more, but not reach past them
     assert not (qkv <= merged < wide) or merged + M * nq * 64 <= qkv + M * (nq + 2 * nkv) * 64
     assert spans[-1][1] <= total
+
+
+@pytest.mark.parametrize("H,vocab", [(256, 1024), (256, 1028), (1024, 1 << 20), (1024, (1 << 21) + 4)])
+def test_shares_of_the_head(probe, H, vocab):
+    """Four-row batches of 128 warps, one share after the other, also past 4 GiB."""
+    at = 0
+    for share in range(128):
+        first, batches = map(int, subprocess.run([str(probe), str(H), str(vocab), str(share)], check=True, capture_output=True,
+                                                 text=True).stdout.split())
+        assert batches == 0 or first == at
+        at += batches * 4 * H * 4
+    assert at == vocab * H * 4

@@ -1068,10 +1068,15 @@ dmtd_status enqueue_small(dmtd_ctx *c, int n, bool write_token, int *out_argmax,
   return DMTD_OK;
 }
 
-// The passes of at most n that the next launch of small_pass_kernel takes (0: none): to the end of the cycle.
+// The passes of at most n that the next launch of small_pass_kernel takes (0: none): to the end of the cycle.  Unasked only
+// for models that gain by it.
 int small_passes(const dmtd_ctx *c, int n) {
   const int kind = c->h.slot == 0 ? 1 : 2, R = c->h.n_known - c->h.lo_len;
   if (!small_pass_ok(c, kind, R)) return 0;
+  const dmtd_model_shape &s = c->s;
+  if (c->pass_option < 0 && small_pass_gain(s.hidden, s.intermediate, s.n_q_heads, s.n_kv_heads, s.vocab, s.n_layers, c->L_d, c->B, c->tau,
+                                            small_pass_ok(c, 1, c->tau)) <= 0.f)
+    return 0;
   return std::min(std::min(n, c->tau - c->h.slot), SP_MAX_POSITIONS - R);
 }
 

@@ -119,6 +119,24 @@ constexpr int SP_FIXED_BYTES = (int)((sizeof(SmallFixed) + 127) / 128 * 128);
 inline bool small_pass_fits(int H, int I, int nq, int nkv, int vocab) {
   return H % (2 * SP_SHARES) == 0 && I % (2 * SP_SHARES) == 0 && (nq + 2 * nkv) * SP_D % (4 * SP_SHARES) == 0 && nq * SP_D % 256 == 0 && vocab % 4 == 0;
 }
+// us that a cycle of this form gains on a launch per step (captured), for B sequences; whole: the full pass runs so, too.
+// Sixteen SMs stream the weights where the other form has 148, so the form pays by the launches of small layers and
+// loses by bytes and by rows of the head, the more so the more activation rows each of them is multiplied with.  The
+// figures are fitted to cycles of 25 fp32 shapes (hidden 256 to 1024, layers of 3 to 50 MB, 1 to 12 of them, vocabularies of
+// 1024 to 151936) at 1 to 8 rows; one launch / captured steps, us: hidden 256, 4 layers of 3.1 MB, 3 passes, vocabulary 1024 97
+// / 163, 16384 145 / 182, 32768 195 / 198, 65536 306 / 241, 151936 576 / 382; two sequences 131 / 185, 206 / 202, 289 / 227, 474 /
+// 271, 913 / 412; 4 layers, 1 pass, vocabulary 1024, layers of 12.6 MB (hidden 512) 69 / 85, four sequences 119 / 119; of 50 MB
+// (hidden 1024) 166 / 175.  Where only the short passes run so, changing over costs a cycle some 18 us: layers of 12.6 MB, two
+// sequences, 251 / 233, of 31 MB 418 / 349.
+inline float small_pass_gain(int H, int I, int nq, int nkv, int vocab, int n_layers, int L_d, int B, int tau, bool whole) {
+  struct Rows { float pass, layer, layer_mb, head_rows; };       // a pass's ends, a layer; less per MB of a layer, per 1000 rows of the head
+  const auto rows = [](int m) { return m == 1 ? Rows{8.f, 5.4f, 0.09f, 0.6f} : m <= 4 ? Rows{5.f, 6.2f, 0.5f, 1.1f} : Rows{4.f, 8.f, 0.9f, 1.5f}; };
+  const float mb = 4e-6f * H * ((2.f * nq + 2 * nkv) * SP_D + 3.f * I);
+  const auto layers = [&](int n, const Rows &r) { return n * (r.layer - r.layer_mb * mb); };
+  const Rows one = rows(B);
+  const float top = one.pass + layers(L_d, one) - one.head_rows * 1e-3f * vocab;         // what every pass has
+  return tau * top + (whole ? layers(n_layers - L_d, rows(B * tau)) : -top - 18.f);
+}
 __device__ __forceinline__ uint32_t sp_mapa(uint32_t addr, int cta) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));

@@ -1,5 +1,5 @@
 """Shared memory of the cluster pass for small fp32 models, as the library's own host code lays it out: buffers that are in use
-at the same time lie apart; and where the warps' shares of a matrix lie.  Runs without a GPU."""
+at the same time lie apart; where the warps' shares of a matrix lie; for which models the form is chosen.  Runs without a GPU."""
 import os
 import subprocess
 
@@ -11,7 +11,12 @@ PROBE = r"""
 #include <cstdlib>
 #include "small_pass.cuh"
 int main(int argc, char **argv) {
-  int a[7];
+  int a[10];
+  if (argc == 11) {
+    for (int i = 0; i < 10; ++i) a[i] = atoi(argv[i + 1]);
+    printf("%f\n", dmtd::small_pass_gain(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[9] != 0));
+    return 0;
+  }
   if (argc == 4) {
     dmtd::SmallParams P{};
     P.H = atoi(argv[1]); P.vocab = atoi(argv[2]);
@@ -62,3 +67,22 @@ def test_shares_of_the_head(probe, H, vocab):
         assert batches == 0 or first == at
         at += batches * 4 * H * 4
     assert at == vocab * H * 4
+
+
+# cycles as measured, us: one launch, captured launches per step
+MEASURED = [
+    # H, I, nq, nkv, vocab, layers, L_d, B, tau, the full pass by the cluster, times
+    (256, 768, 4, 2, 1024, 4, 2, 1, 3, 1, 97, 163), (256, 768, 4, 2, 1024, 4, 4, 8, 1, 1, 95, 118), (256, 768, 4, 2, 1024, 12, 6, 2, 3, 0, 404, 457),
+    (256, 768, 4, 2, 16384, 4, 2, 1, 3, 1, 145, 182), (256, 768, 4, 2, 65536, 4, 2, 1, 3, 1, 306, 241), (256, 768, 4, 2, 151936, 4, 4, 1, 1, 1, 200, 145),
+    (256, 768, 4, 2, 151936, 4, 2, 2, 3, 1, 913, 412), (256, 768, 4, 2, 32768, 4, 4, 4, 1, 1, 116, 103), (256, 768, 4, 2, 32768, 4, 4, 8, 1, 1, 179, 151),
+    (256, 768, 4, 2, 32768, 1, 1, 1, 1, 1, 52, 44), (256, 768, 4, 2, 8192, 1, 1, 1, 1, 1, 27, 34),
+    (512, 1536, 8, 4, 1024, 4, 2, 1, 3, 1, 162, 192), (512, 1536, 8, 4, 1024, 4, 2, 2, 3, 0, 251, 233), (512, 1536, 8, 4, 32768, 4, 2, 1, 3, 1, 319, 301),
+    (512, 512, 4, 2, 1024, 4, 2, 2, 3, 0, 172, 184), (512, 2048, 8, 8, 1024, 4, 2, 2, 3, 0, 304, 274),
+    (1024, 3072, 16, 8, 1024, 4, 4, 1, 1, 1, 166, 175), (1024, 3072, 16, 8, 32768, 4, 4, 1, 1, 1, 246, 235), (1024, 1024, 4, 2, 1024, 4, 2, 2, 3, 0, 278, 243),
+]
+
+
+@pytest.mark.parametrize("case", MEASURED, ids=lambda c: "-".join(map(str, c[:10])))
+def test_chosen_where_it_is_the_faster_form(probe, case):
+    gain = float(subprocess.run([str(probe)] + [str(x) for x in case[:10]], check=True, capture_output=True, text=True).stdout)
+    assert (gain > 0) == (case[10] < case[11]), gain

@@ -240,8 +240,10 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *ctx, float temperature, uint64_t seed);
  *   "fused_pass"   0/1  1 = run each decode pass as one persistent kernel where the model and batch
  *                       allow it (bf16 weights, head_dim 128, at most 4 rows per pass), 0 = always
  *                       the per-step kernels.  Until it is set: one kernel for bf16 models with
- *                       an fp32 cache or without block-ordered weights, the per-step kernels, which
- *                       are the faster ones, for other bf16 models; small fp32 models: one cluster
+ *                       an fp32 cache or without block-ordered weights, and for passes that are
+ *                       not replayed (decode_forced) of one sequence of a model with large layers;
+ *                       the per-step kernels, which are the faster ones, for other passes of bf16
+ *                       models; small fp32 models: one cluster where that is faster
  *   "encoding_layers" x  the ExDy variant (Section 2.1, the paragraph after Eq. 4; Section 3.3): the
  *                       short passes run the first x encoding layers as well as the last L_d
  *                       decoding layers, the decoding layers read the encoding layers' output

@@ -960,9 +960,17 @@ dmtd_status setup_fused(dmtd_ctx *c) {
 // and the attention merges by cluster.  Cycles of 1 to 4 passes, the pass kernel's time over the per-step kernels': one sequence,
 // context 64 to 3000, hidden 640 (7 MB a layer) 1.25 to 1.07, 1024 1.18 to 1.04, 2048 (100 MB) 1.09 to 1.01, 2560 (202 MB) 1.03
 // to 1.05, over 36 layers 1.01 at 550 positions and 1.03 at 2500 (8 cycles 25.2 / 26.65 ms against 24.95 / 25.7); two sequences
-// of 2560 1.05, three 1.08 to 1.11, four 1.11 to 1.18.
-bool fused_pass_ok(const dmtd_ctx *c, int kind, int R_lower) {
-  const bool asked = c->pass_option >= 0 ? c->pass_option != 0 : !(c->umma_ok && c->use_umma && tc_decode_attention(c) && c->fuse_qk_rope);
+// of 2560 1.05, three 1.08 to 1.11, four 1.11 to 1.18.  That is with captured passes.  Passes launched one by one (given tokens, "cuda_graph"
+// off) take 5 to 10 % longer, and one sequence of a model with large layers is faster on the pass kernel; its time over theirs, one
+// sequence: 10 MB a layer 1.06 to 1.11, 31 MB 1.01 to 1.08, 71 MB 1.00 to 1.04, 101 MB 0.95 to 1.00, 202 MB 0.96 to 0.99 (36 layers 0.945);
+// two sequences of 202 MB 0.99 to 1.03, three 1.03 to 1.04.
+bool fused_pass_ok(const dmtd_ctx *c, int kind, int R_lower, bool captured) {
+  bool asked = c->pass_option > 0;
+  if (c->pass_option < 0) {
+    const LayerDev &l = c->layers[0];
+    const bool per_step = c->umma_ok && c->use_umma && tc_decode_attention(c) && c->fuse_qk_rope;
+    asked = !per_step || (!captured && c->B == 1 && packed_atoms(l.qkv) + packed_atoms(l.o) + packed_atoms(l.gu) + packed_atoms(l.down) >= (96 << 10));   // 1 KiB atoms
+  }
   if (!c->fused_ok || !asked || c->literal_sum || c->L_e > 0) return false;
   const int lo = c->s.n_layers - c->L_d;
   const int R = (kind == 1 && lo > 0) ? R_lower : 1;
@@ -1086,7 +1094,7 @@ int small_passes(const dmtd_ctx *c, int n) {
 dmtd_status enqueue_pass(dmtd_ctx *c, int kind, int R_lower, bool write_token, int *out_argmax, float *out_logits) {
   const int B = c->B, L = c->s.n_layers, lo = L - c->L_d, H = c->s.hidden;
   const int newest = c->h.n_known - 1;
-  if (!c->capturing && fused_pass_ok(c, kind, R_lower))
+  if (!c->capturing && fused_pass_ok(c, kind, R_lower, false))
     return enqueue_pass_fused(c, kind, R_lower, write_token, out_argmax, out_logits);
   if (c->L_e > 0) {
     // ExDy: the newest token's embedding goes through the encoding layers in every pass; their
@@ -1199,10 +1207,10 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind) {
 dmtd_status run_greedy_pass(dmtd_ctx *c) {
   int kind = c->h.slot == 0 ? 1 : 2;
   int R_lower = c->h.n_known - c->h.lo_len;
-  bool steady = (kind == 2) || (R_lower == c->tau);
-  if (fused_pass_ok(c, kind, R_lower)) {
+  const bool captured = c->use_graph && (kind == 2 || R_lower == c->tau);
+  if (fused_pass_ok(c, kind, R_lower, captured)) {
     TRY(enqueue_pass_fused(c, kind, R_lower, true, nullptr, nullptr));
-  } else if (c->use_graph && steady) {
+  } else if (captured) {
     if (c->graph_B != c->B || c->graph_tau != c->tau) { drop_graphs(c); c->graph_B = c->B; c->graph_tau = c->tau; }
     if (!c->graph_exec[kind]) TRY(capture_pass(c, kind));
     CUDA_TRY(c, cudaGraphLaunch(c->graph_exec[kind], c->stream));

@@ -330,6 +330,27 @@ def test_fused_pass_kernel_teacher_forced(dmtd, name, L_d, tau, B, P, n_new, kv)
     assert np.abs(res[1][0] - res[0][0]).max() < 5e-3
 
 
+@pytest.mark.parametrize("hidden,intermediate,one_kernel", [(2560, 9728, True), (1024, 3072, False)])
+def test_passes_launched_one_by_one_take_the_faster_form(dmtd, hidden, intermediate, one_kernel):
+    """Passes with given tokens are not replayed: one sequence runs them on the pass kernel where the layers are large."""
+    shape = SHAPES["mid"].with_(n_layers=2, hidden=hidden, intermediate=intermediate, n_q_heads=16, n_kv_heads=4, vocab=1024)
+    wc = to_cuda(make_weights(shape, seed=0, norm_jitter=0.1))
+    prompt = make_prompts(shape.vocab, 1, 40, seed=1).cuda()
+    forced = make_prompts(shape.vocab, 1, 6, seed=2).cuda()
+    res = {}
+    for fused in (None, 1, 0):
+        eng = _engine(dmtd, shape, wc, 1, 3, 1, 64, kv_dtype="f16")
+        if fused is not None:
+            eng.set_option("fused_pass", fused)
+        eng.prefill(prompt)
+        l0 = eng.launch_count()
+        logits, _ = eng.decode_forced(forced)
+        res[fused] = (logits, eng.launch_count() - l0)
+    assert res[1][1] < res[0][1]
+    assert res[None][1] == res[1 if one_kernel else 0][1]
+    assert (res[None][0] - res[0][0]).abs().max() < 5e-3
+
+
 def test_fused_pass_kernel_free_running(dmtd):
     shape = SHAPES["mid"]
     w = make_weights(shape, seed=0, norm_jitter=0.1)

@@ -1203,6 +1203,31 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind) {
   return DMTD_OK;
 }
 
+// The graph of a kind of pass for the batch and cycle length at hand.
+dmtd_status ready_graph(dmtd_ctx *c, int kind) {
+  if (c->graph_B != c->B || c->graph_tau != c->tau) { drop_graphs(c); c->graph_B = c->B; c->graph_tau = c->tau; }
+  return c->graph_exec[kind] ? DMTD_OK : capture_pass(c, kind);
+}
+
+// Behind a prefill, while the device works on it: the passes of few rows are captured before the first one is asked for (the host
+// takes 0.3 to 1.5 ms for each).  A failure here is left for the pass itself to meet.
+void capture_ahead(dmtd_ctx *c) {
+  if (!c->use_graph || !c->fused_ok || c->B > PK_MAX_ROWS || c->literal_sum || c->L_e > 0) return;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(c->stream, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
+  for (int kind = 1; kind <= (c->tau > 1 ? 2 : 1); ++kind) {
+    if (fused_pass_ok(c, kind, c->tau, true)) continue;
+    const bool is_new = c->graph_B != c->B || c->graph_tau != c->tau || !c->graph_exec[kind];
+    if (ready_graph(c, kind) != DMTD_OK || (is_new && cudaGraphUpload(c->graph_exec[kind], c->capture_stream) != cudaSuccess)) {
+      cudaGetLastError();
+      return;
+    }
+  }
+}
+
 // Run the next pass of the schedule in greedy mode.
 dmtd_status run_greedy_pass(dmtd_ctx *c) {
   int kind = c->h.slot == 0 ? 1 : 2;
@@ -1211,8 +1236,7 @@ dmtd_status run_greedy_pass(dmtd_ctx *c) {
   if (fused_pass_ok(c, kind, R_lower, captured)) {
     TRY(enqueue_pass_fused(c, kind, R_lower, true, nullptr, nullptr));
   } else if (captured) {
-    if (c->graph_B != c->B || c->graph_tau != c->tau) { drop_graphs(c); c->graph_B = c->B; c->graph_tau = c->tau; }
-    if (!c->graph_exec[kind]) TRY(capture_pass(c, kind));
+    TRY(ready_graph(c, kind));
     CUDA_TRY(c, cudaGraphLaunch(c->graph_exec[kind], c->stream));
     c->launches += c->graph_nodes[kind];
   } else {
@@ -1467,6 +1491,7 @@ dmtd_status dmtd_prefill(dmtd_ctx *c, const int32_t *prompt, int32_t B, int32_t 
   c->h.n_known = P + 1; c->h.lo_len = P; c->h.up_len = P; c->h.cycle = 1;
   c->h.slot = 1 % c->tau; c->h.n_emitted = 1;
   c->prefilled = true;
+  capture_ahead(c);
   return DMTD_OK;
 }
 

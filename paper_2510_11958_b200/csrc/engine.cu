@@ -93,6 +93,7 @@ struct dmtd_ctx {
   bool fuse_qk_rope = true;                 // QK-norm, RoPE and the KV append inside the tensor-core attention kernel
   float temperature = 0.f;                  // > 0: tokens are drawn from softmax(logits / temperature); 0: greedy
   uint64_t sample_seed = 0;
+  SampleParams *dsample = nullptr;          // device copy, written in stream order
 
   // fused pass kernel: one persistent launch per pass
   bool fused_ok = false;
@@ -790,6 +791,12 @@ SampleParams sample_params(const dmtd_ctx *c) {
   return sp;
 }
 
+dmtd_status write_sample_params(dmtd_ctx *c) {
+  set_sample_kernel<<<1, 1, 0, c->stream>>>(c->dsample, sample_params(c));
+  LAUNCH_OK(c, "set_sample_kernel");
+  return DMTD_OK;
+}
+
 // Step a9/a10/a0: final norm, tied LM head, greedy pick, token feedback, the schedule's counters.
 dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits, int kind, int P) {
   const dmtd_model_shape &s = c->s;
@@ -809,7 +816,7 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
     CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (size_t)s.vocab * 4, c->logits, (size_t)c->ldl * 4, (size_t)s.vocab * 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
   CUDA_TRY(c, launch_pdl(argmax_kernel, dim3(B, ARGMAX_SLICES), dim3(256), (size_t)(0), c->stream,
-                          c->logits, c->ldl, s.vocab, c->dstate, sample_params(c),
+                          c->logits, c->ldl, s.vocab, c->dstate, c->dsample,
                           PickParams{c->pick_val, c->pick_idx, c->pick_arrived, write_token ? c->tokens : nullptr, c->max_seq, out_argmax, kind, P}));
   LAUNCH_OK(c, "argmax_kernel");
   return DMTD_OK;
@@ -1364,6 +1371,8 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   }
   CTRY(dev_alloc(c, &c->tokens, (size_t)max_batch * max_seq));
   CTRY(dev_alloc(c, &c->dstate, 1));
+  CTRY(dev_alloc(c, &c->dsample, 1));
+  CTRY(write_sample_params(c));
   CCUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->h_error), sizeof(int), cudaHostAllocDefault));
   *c->h_error = 0;
 
@@ -1689,8 +1698,7 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *c, float temperature, uint64_t seed) {
   if (!c) return DMTD_ERR_INVALID_ARG;
   if (!(temperature >= 0.f) || std::isinf(temperature)) return fail(c, DMTD_ERR_INVALID_ARG, "set_sampling: temperature must be finite and >= 0");
   c->temperature = temperature; c->sample_seed = seed;
-  drop_graphs(c);                           // the captured passes carry the old parameters
-  return DMTD_OK;
+  return write_sample_params(c);
 }
 
 dmtd_status dmtd_set_option(dmtd_ctx *c, const char *name, int64_t value) {

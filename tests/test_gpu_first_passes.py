@@ -40,3 +40,44 @@ def test_first_cycles_of_a_context(dmtd):
         later += [_timed(lambda: eng.decode_cycle(3)) for _ in range(10)]
         assert eng.device_state() == eng.state()
     assert min(first) < 1.4 * min(later), (min(first), min(later))
+
+
+def test_cycles_after_set_sampling(dmtd):
+    """Captured passes read the temperature and the seed from memory: a program that sets them for every request does not wait
+    for another capture.  (It took 1.6 times as long as a later cycle.)"""
+    shape = SHAPES["mid"]
+    eng = dmtd.Dmtd(shape, to_cuda(make_weights(shape, seed=0, norm_jitter=0.1)), L_d=2, tau=3, max_batch=1, max_seq=400, kv_dtype="f16")
+    eng.prefill(make_prompts(shape.vocab, 1, 200, seed=1).cuda())
+    while eng.state()["slot"]:
+        eng.decode_cycle(3)
+    after, later = [], []
+    for seed in range(8):
+        eng.set_sampling(0.8, seed)
+        after.append(_timed(lambda: eng.decode_cycle(3)))
+        later += [_timed(lambda: eng.decode_cycle(3)) for _ in range(5)]
+    assert min(after) < 1.3 * min(later), (min(after), min(later))
+
+
+@pytest.mark.parametrize("B", [1, 6])
+def test_sampling_changes_between_captured_cycles(dmtd, B):
+    """Greedy, sampled, another seed, greedy again: the tokens of replayed passes are those of passes launched one by one."""
+    shape = SHAPES["mid"]
+    w = to_cuda(make_weights(shape, seed=0, norm_jitter=0.1))
+    prompt = make_prompts(shape.vocab, B, 20, seed=1).cuda()
+    toks = []
+    for graph in (1, 0):
+        eng = dmtd.Dmtd(shape, w, L_d=2, tau=3, max_batch=B, max_seq=100, kv_dtype="f32")
+        eng.set_option("fused_pass", 0)
+        eng.set_option("cuda_graph", graph)
+        eng.prefill(prompt)
+        while eng.state()["slot"]:
+            eng.decode_cycle(3)
+        out = []
+        for setting in (None, (0.7, 5), (0.7, 6), (1.3, 6), (0.0, 0)):
+            if setting:
+                eng.set_sampling(*setting)
+            out += [eng.decode_cycle(3)[2].clone() for _ in range(2)]
+        toks.append(torch.cat(out, 1))
+    assert torch.equal(*toks)
+    runs = toks[0].view(B, 5, 6)
+    assert not torch.equal(runs[:, 1], runs[:, 2]) and not torch.equal(runs[:, 2], runs[:, 3])

@@ -57,10 +57,11 @@ def _kv_views(eng, layer, B, nkv, max_seq, D):
 
 
 def test_config2_full_depth_prompt_512_teacher_forced(dmtd):
-    """Config 2 at its own sizes: 36 layers, full vocabulary, 512-token prompt, the persistent pass
-    kernel on every decode pass, with the fp16 KV cache the benchmark workload uses and with an fp32
-    one.  97 tokens: the prefill's and 96 decode passes (32 whole cycles), logits of every pass
-    against the oracle."""
+    """Config 2 at its own sizes: 36 layers, full vocabulary, 512-token prompt, with the fp16 KV cache
+    the benchmark workload uses (a launch per step, and the persistent pass kernel on every pass) and
+    with an fp32 one (pass kernel).  97 tokens: the prefill's and 96 decode passes (32 whole cycles),
+    logits of every pass against the oracle.  Then the replayed passes that the benchmark times: the
+    tokens of 32 free-running cycles are what the logits of the same tokens, given, say."""
     shape = SHAPES["qwen3_4b"]
     P, n_new, L_d, tau = 512, 97, 8, 3
     w = make_weights(shape, seed=0)
@@ -69,15 +70,32 @@ def test_config2_full_depth_prompt_512_teacher_forced(dmtd):
     ref_logits, ref_am, o = oracle_forced(shape, w, L_d, tau, prompts, forced)
     wc = to_cuda(w)
     del w
-    for kv in ("f16", "f32"):
+    for kv, fused in (("f16", 0), ("f16", 1), ("f32", 1)):
         eng = dmtd.Dmtd(shape, wc, L_d=L_d, tau=tau, max_batch=1, max_seq=P + n_new + 1, kv_dtype=kv)
+        eng.set_option("fused_pass", fused)
         l0 = eng.launch_count()
         got_logits, got_am = gpu_forced(eng, prompts, forced)
+        launches = eng.launch_count() - l0
         err, clear = check_logits(got_logits, ref_logits, got_am, ref_am)
         assert eng.device_state() == o.state()
-        print(f"config 2, {n_new - 1} decode passes, {kv} cache: max|dlogit|={err:.2e}, clear-margin steps {clear:.0%}, "
-              f"launches {eng.launch_count() - l0}")
+        assert (launches < 20 * n_new) == bool(fused)
+        print(f"config 2, {n_new - 1} decode passes, {kv} cache, {'pass kernel' if fused else 'per-step'}: "
+              f"max|dlogit|={err:.2e}, clear-margin steps {clear:.0%}, launches {launches}")
         eng.close()
+    eng = dmtd.Dmtd(shape, wc, L_d=L_d, tau=tau, max_batch=1, max_seq=P + n_new + 1, kv_dtype="f16")
+    tok, _ = eng.prefill(torch.from_numpy(prompts).cuda())
+    toks, l0 = [tok.view(1, 1)], eng.launch_count()
+    while sum(t.shape[1] for t in toks) < n_new:
+        _, n, out = eng.decode_cycle(n_new - sum(t.shape[1] for t in toks))
+        toks.append(out[:, :n].clone())
+    assert eng.launch_count() - l0 > 20 * n_new                  # a launch per step
+    toks = torch.cat(toks, 1)
+    eng.reset()
+    logits, _ = gpu_forced(eng, prompts, toks.cpu().numpy())
+    srt = np.sort(logits, -1)
+    clear = (srt[..., -1] - srt[..., -2] > 5e-2).T
+    assert clear.any() and (logits.argmax(-1).T[clear] == toks.cpu().numpy()[clear]).all()
+    eng.close()
 
 
 def test_full_depth_bf16_kv_cache_measured_bound(dmtd):

@@ -351,18 +351,24 @@ def test_passes_launched_one_by_one_take_the_faster_form(dmtd, hidden, intermedi
     assert (res[None][0] - res[0][0]).abs().max() < 5e-3
 
 
-def test_fused_pass_kernel_free_running(dmtd):
+@pytest.mark.parametrize("fused", [1, 0])
+def test_fused_pass_kernel_free_running(dmtd, fused):
+    """Free-running cycles with a 16-bit cache, on the pass kernel and as replayed launches per step."""
     shape = SHAPES["mid"]
     w = make_weights(shape, seed=0, norm_jitter=0.1)
     B, P, n_new, L_d, tau = 1, 33, 19, 2, 3
     prompts = make_prompts(shape.vocab, B, P, seed=1).numpy()
     toks, logits, states, _ = oracle_greedy(shape, w, L_d, tau, prompts, n_new)
     eng = _engine(dmtd, shape, to_cuda(w), L_d, tau, B, P + n_new + 1)
+    eng.set_option("fused_pass", fused)
     tok, _ = eng.prefill(torch.from_numpy(prompts).cuda())
     got = [tok.cpu().numpy()]
     k = 1
     while len(got) < n_new:
+        l0 = eng.launch_count()
         rc, n, out = eng.decode_cycle(n_new - len(got))
+        # the pass kernel: a launch per pass and one that gathers the tokens
+        assert (eng.launch_count() - l0 == n + 1) == bool(fused)
         out = out.cpu().numpy()
         got += [out[:, i] for i in range(n)]
         assert eng.device_state() == states[k]

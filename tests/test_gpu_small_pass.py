@@ -80,11 +80,15 @@ def test_small_pass(dmtd, weights, name, L_d, tau, B, P, sample):
     assert launches < ref_launches
     for got, want in [(logits, ref)] + list(zip(kv, ref_kv)):
         assert (got - want).abs().max() <= RTOL * want.abs().max().clamp(min=1.0)
+    if sample:
+        # a draw goes the other way only where two perturbed logits lie within RTOL of each other: at these seeds none do
+        assert torch.equal(am, ref_am) and torch.equal(toks, ref_toks)
+        assert (am != ref.argmax(-1)).any()                 # and they are draws
+        return
     srt = ref.sort(-1).values
-    if not sample:
-        clear = srt[..., -1] - srt[..., -2] > 1e-3
-        assert (am[clear] == ref_am[clear]).all()
-    if not sample and clear.all():
+    clear = srt[..., -1] - srt[..., -2] > 1e-3
+    assert (am[clear] == ref_am[clear]).all()
+    if clear.all():
         assert (toks == ref_toks).all()
 
 

@@ -55,14 +55,15 @@ constexpr int TG_TILE_ROWS = 256;            // most rows of a column tile
 // holds (4 cycles of 32 sequences of the Qwen3-4B shape: 20.26 ms with one, 20.12 with two).  More rows: one, the
 // activations of a stage are 32 KiB there.
 __host__ __device__ constexpr int tg_stage_units(bool split) { return split ? 2 : 1; }
-// Decode launches: the ring's first round, requested before the activations are there, is asked for as fast as HBM delivers
+// Decode launches: the ring's first round, requested before the activations are there, is asked for about as fast as HBM delivers
 // it and not at once: two stages (64 KiB an SM, HBM's bandwidth times its latency and a little more), then one every TG_PACE
-// cycles (32 KiB for 148 SMs: 0.75 us).  With 192 KiB an SM outstanding, the few reads between two projections (the norms' and
-// gates' kernels, the keys) waited some 4 us in the L2's queues: a projection had its activations 8 us after the end of
-// the one in front.  4 layers and the head, context 64 to 700, 1 / 3 / 16 sequences, us: all at once 355 / 386 / 393; a stage every 600 cycles
-// 352 / 377 / 384, 1000 344 / 368 / 376, 1400 343 / 366 / 375, 2000 355 / 374 / 388.  (Asking L2 for the next projection's first
-// weights at the end of a launch: 2 % without pacing, nothing beside it.  Activations converted by warps of the GEMM instead of
-// kernels in front: as fast at 1 to 3 rows, slower above.)
+// cycles.  (32 KiB for 148 SMs take HBM 0.74 us at its copy rate; 1200 cycles are 0.61 us at 1965 MHz and 0.75 us at 1600 MHz.)  With
+// 192 KiB an SM outstanding, the few reads between two projections (the norms' and gates' kernels, the keys) waited some 4 us in
+// the L2's queues: a projection had its activations 8 us after the end of the one in front.  A cycle of three passes, 4 layers and
+// the head, context 512 to 1400, 1965 MHz, 1 / 3 / 16 sequences, us, a stage every 600 cycles 823 / 830 / 895, 1000 805 / 815 / 881, 1200
+// 802 / 814 / 882, 1400 805 / 819 / 888, 2000 832 / 847 / 915; all at once 3 to 5 % longer than 1000.  (Asking L2 for the next projection's
+// first weights at the end of a launch: 2 % without pacing, nothing beside it.  Activations converted by warps of the GEMM
+// instead of kernels in front: as fast at 1 to 3 rows, slower above.)
 constexpr int TG_PACE_FREE = 2, TG_PACE = 1200;
 constexpr int TG_TAIL_BYTES = 16 * TG_MAX_STAGES + 48;     // barriers, tensor-memory address, flag
 // Dynamic shared memory of a block: it has its SM to itself, beside a block of the prefill attention (96 KiB) or another

@@ -34,6 +34,9 @@ thread_local std::string g_create_error;
 // it gives up and reports through the context's error word: about a second of SM clock.
 constexpr long long kDeviceWaitLimitTicks = 2000000000ll;
 
+// Captured passes that a context keeps: both kinds for four batches or cycle lengths in turn.
+constexpr int kMaxGraphs = 8;
+
 struct LayerDev {
   PackedMat qkv, o, gu, down;
   UmmaMat qkv_u{}, o_u{}, gu_u{}, down_u{};     // second copy for the tcgen05 GEMM (contexts with many rows)
@@ -108,10 +111,10 @@ struct dmtd_ctx {
 
   bool small_ok = false;                    // the model fits small_pass_kernel
 
-  // graphs: [kind 1 = full, 2 = upper-only]
-  cudaGraphExec_t graph_exec[3] = {nullptr, nullptr, nullptr};
-  int graph_nodes[3] = {0, 0, 0};
-  int graph_B = 0, graph_tau = 0;
+  // captured passes: kind 1 = full (of tau pending rows), 2 = upper-only (any tau; 0 here)
+  struct PassGraph { int kind, B, tau, nodes; cudaGraphExec_t exec; int64_t used; };
+  std::vector<PassGraph> graphs;            // at most kMaxGraphs
+  int64_t graph_uses = 0;
   bool capturing = false;
 
   int64_t launches = 0;
@@ -1180,8 +1183,8 @@ dmtd_status device_error_status(dmtd_ctx *c, int word) {
   } while (0)
 
 void drop_graphs(dmtd_ctx *c) {
-  for (int k = 0; k < 3; ++k)
-    if (c->graph_exec[k]) { cudaGraphExecDestroy(c->graph_exec[k]); c->graph_exec[k] = nullptr; }
+  for (const auto &g : c->graphs) cudaGraphExecDestroy(g.exec);
+  c->graphs.clear();
 }
 
 // Capture a steady-state pass (R_lower = tau) into a graph.  Positions come from the device
@@ -1203,17 +1206,31 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind) {
   c->launches = before;
   if (st != DMTD_OK) { if (graph) cudaGraphDestroy(graph); return st; }
   if (e != cudaSuccess) return fail(c, DMTD_ERR_CUDA, "end capture: %s", cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&c->graph_exec[kind], graph, 0);
+  cudaGraphExec_t exec = nullptr;
+  e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return fail(c, DMTD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-  c->graph_nodes[kind] = nodes;
+  if ((int)c->graphs.size() == kMaxGraphs) {
+    const auto oldest = std::min_element(c->graphs.begin(), c->graphs.end(), [](const auto &a, const auto &b) { return a.used < b.used; });
+    cudaGraphExecDestroy(oldest->exec);      // (one that still runs is released when it has)
+    c->graphs.erase(oldest);
+  }
+  c->graphs.push_back({kind, c->B, kind == 1 ? c->tau : 0, nodes, exec, 0});
   return DMTD_OK;
 }
 
-// The graph of a kind of pass for the batch and cycle length at hand.
-dmtd_status ready_graph(dmtd_ctx *c, int kind) {
-  if (c->graph_B != c->B || c->graph_tau != c->tau) { drop_graphs(c); c->graph_B = c->B; c->graph_tau = c->tau; }
-  return c->graph_exec[kind] ? DMTD_OK : capture_pass(c, kind);
+// The graph of a kind of pass for the batch and cycle length at hand; captured: it is a new one.
+dmtd_status ready_graph(dmtd_ctx *c, int kind, const dmtd_ctx::PassGraph **out, bool *captured = nullptr) {
+  const int tau = kind == 1 ? c->tau : 0;
+  auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const auto &g) { return g.kind == kind && g.B == c->B && g.tau == tau; });
+  if (captured) *captured = it == c->graphs.end();
+  if (it == c->graphs.end()) {
+    TRY(capture_pass(c, kind));
+    it = c->graphs.end() - 1;
+  }
+  it->used = ++c->graph_uses;
+  *out = &*it;
+  return DMTD_OK;
 }
 
 // Behind a prefill, while the device works on it: the passes of few rows are captured before the first one is asked for (the host
@@ -1227,8 +1244,9 @@ void capture_ahead(dmtd_ctx *c) {
   }
   for (int kind = 1; kind <= (c->tau > 1 ? 2 : 1); ++kind) {
     if (fused_pass_ok(c, kind, c->tau, true)) continue;
-    const bool is_new = c->graph_B != c->B || c->graph_tau != c->tau || !c->graph_exec[kind];
-    if (ready_graph(c, kind) != DMTD_OK || (is_new && cudaGraphUpload(c->graph_exec[kind], c->capture_stream) != cudaSuccess)) {
+    const dmtd_ctx::PassGraph *g = nullptr;
+    bool is_new = false;
+    if (ready_graph(c, kind, &g, &is_new) != DMTD_OK || (is_new && cudaGraphUpload(g->exec, c->capture_stream) != cudaSuccess)) {
       cudaGetLastError();
       return;
     }
@@ -1243,9 +1261,10 @@ dmtd_status run_greedy_pass(dmtd_ctx *c) {
   if (fused_pass_ok(c, kind, R_lower, captured)) {
     TRY(enqueue_pass_fused(c, kind, R_lower, true, nullptr, nullptr));
   } else if (captured) {
-    TRY(ready_graph(c, kind));
-    CUDA_TRY(c, cudaGraphLaunch(c->graph_exec[kind], c->stream));
-    c->launches += c->graph_nodes[kind];
+    const dmtd_ctx::PassGraph *g = nullptr;
+    TRY(ready_graph(c, kind, &g));
+    CUDA_TRY(c, cudaGraphLaunch(g->exec, c->stream));
+    c->launches += g->nodes;
   } else {
     TRY(enqueue_pass(c, kind, R_lower, true, nullptr, nullptr));
   }

@@ -81,3 +81,35 @@ def test_sampling_changes_between_captured_cycles(dmtd, B):
     assert torch.equal(*toks)
     runs = toks[0].view(B, 5, 6)
     assert not torch.equal(runs[:, 1], runs[:, 2]) and not torch.equal(runs[:, 2], runs[:, 3])
+
+
+def test_cycle_lengths_and_batches_in_turn(dmtd):
+    """A program that changes the cycle length between cycles, or the batch between requests, does not wait for another capture;
+    more of them than a context keeps are captured again, and every cycle's tokens are those of passes launched one by one."""
+    shape = SHAPES["mid"]
+    w = to_cuda(make_weights(shape, seed=0, norm_jitter=0.1))
+    tokens = {}
+    for graph in (1, 0):
+        eng = dmtd.Dmtd(shape, w, L_d=2, tau=3, max_batch=6, max_seq=300, kv_dtype="f32")
+        eng.set_option("fused_pass", 0)
+        eng.set_option("cuda_graph", graph)
+        out, turns, steady = [], [], []
+        for B in (1, 2, 6, 1):
+            eng.reset()
+            eng.set_tau(3)
+            eng.prefill(make_prompts(shape.vocab, B, 30, seed=1).cuda())
+            while eng.state()["slot"]:
+                eng.decode_cycle(3)
+            for tau in (3, 2, 4, 5, 3, 2, 3, 2):
+                eng.set_tau(tau)
+                buf = torch.zeros(B, tau, dtype=torch.int32, device="cuda")
+                turns.append((tau, _timed(lambda: eng.decode_cycle(tau, out_tokens=buf))))
+                out.append(buf.flatten().clone())
+            assert eng.device_state() == eng.state()
+        for _ in range(6):
+            steady.append(_timed(lambda: eng.decode_cycle(2)))
+        tokens[graph] = torch.cat(out)
+        if graph:
+            # the last request's (one sequence) last cycles of two passes: captured earlier
+            assert min(t for tau, t in turns[-4:] if tau == 2) < 1.4 * min(steady)
+    assert torch.equal(tokens[0], tokens[1])

@@ -279,9 +279,17 @@ class Dmtd:
 _KV_CODE = {torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}
 
 
+try:
+    # The stream as a number without an object around it: 0.15 us instead of 3.2, in a call of some eight microseconds.
+    # Not part of torch's interface.
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream, _cuda_getDevice as _device
+except ImportError:
+    _raw_stream = None
+
+
 def _current_stream():
     """The current device's current stream, as a number."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
 
 
 def attention_decode(q, k, v, pos0, scratch=None):

@@ -252,12 +252,7 @@ struct AttnShares {
   __device__ __forceinline__ int holder(int u) const { return (int)((((long long)u + 1) * n_blocks - 1) / total); }
 };
 
-// Loads from the shared memory of another block of the cluster (addresses of the cluster's window).
-__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
+// Loads from the shared memory of another block of the cluster (cluster_address).
 __device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");

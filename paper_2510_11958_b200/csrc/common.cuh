@@ -58,6 +58,13 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Where address `addr` of this block's shared memory lies in block `rank` of the cluster, in the cluster's window.
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
 // Two products at once: a += x * y by halves.
 __device__ __forceinline__ void fma_f32x2(float2 &a, float2 x, float2 y) {
   uint64_t r;

@@ -137,12 +137,7 @@ inline float small_pass_gain(int H, int I, int nq, int nkv, int vocab, int n_lay
   const float top = one.pass + layers(L_d, one) - one.head_rows * 1e-3f * vocab;         // what every pass has
   return tau * top + (whole ? layers(n_layers - L_d, rows(B * tau)) : -top - 18.f);
 }
-__device__ __forceinline__ uint32_t sp_mapa(uint32_t addr, int cta) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
-  return r;
-}
-// Store into a block's shared memory (addresses of the cluster's window); its bytes are counted on the barrier there.
+// Store into a block's shared memory (cluster_address); its bytes are counted on the barrier there.
 __device__ __forceinline__ void sp_send8(uint32_t dst, uint64_t v, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst), "l"(v), "r"(bar) : "memory");
 }
@@ -612,9 +607,9 @@ __device__ __forceinline__ void sp_attention(const SmallParams &P, uint32_t &pha
       const uint32_t dst = base + (map.part_o + T.slot * D + d4 * 4) * 4, dst_ml = base + (map.part_ml + T.slot * 2) * 4;
 #pragma unroll 2
       for (int c = T.to; c < T.to + T.n_to; ++c) {
-        const uint32_t bar = sp_mapa(bars + 8 * SP_BAR_PART, c);
-        sp_send4(sp_mapa(dst, c), o, bar);
-        if (d4 == c) sp_send2(sp_mapa(dst_ml, c), m, l, bar);              // (every block's pair from another thread)
+        const uint32_t bar = cluster_address(bars + 8 * SP_BAR_PART, c);
+        sp_send4(cluster_address(dst, c), o, bar);
+        if (d4 == c) sp_send2(cluster_address(dst_ml, c), m, l, bar);              // (every block's pair from another thread)
       }
     }
   } else {
@@ -755,7 +750,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) small_pass_kernel(const __grid_
   }
   // the block's kv head and key slice, and where this lane sends its outputs
   const int item = cta / P.ns, slice = cta - item * P.ns, item_b = item / P.nkv, item_h = item - item_b * P.nkv;
-  const uint32_t rbars = sp_mapa(bars, lane & 15), rbase = rbars + (uint32_t)(SP_FIXED_BYTES + SP_RING_BYTES);
+  const uint32_t rbars = cluster_address(bars, lane & 15), rbase = rbars + (uint32_t)(SP_FIXED_BYTES + SP_RING_BYTES);
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 
   uint32_t phases = 0;
@@ -804,7 +799,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) small_pass_kernel(const __grid_
         const int i2 = F.pick_idx[w][b];
         if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
       }
-      sp_send8(sp_mapa(smem_u32(&F.pick[b][cta]), t), (uint64_t)__float_as_uint(v) | (uint64_t)(unsigned)i << 32, sp_mapa(bars + 8 * SP_BAR_PICK, t));
+      sp_send8(cluster_address(smem_u32(&F.pick[b][cta]), t), (uint64_t)__float_as_uint(v) | (uint64_t)(unsigned)i << 32, cluster_address(bars + 8 * SP_BAR_PICK, t));
     }
     __syncwarp();
     sp_wait(P, SP_BAR_PICK, phases, (uint32_t)(B * SP_CTAS * 8));

@@ -112,7 +112,7 @@ struct dmtd_ctx {
   bool small_ok = false;                    // the model fits small_pass_kernel
 
   // captured passes: kind 1 = full (of tau pending rows), 2 = upper-only (any tau; 0 here)
-  struct PassGraph { int kind, B, tau, nodes; cudaGraphExec_t exec; int64_t used; };
+  struct PassGraph { int kind, B, tau, forms, nodes; cudaGraphExec_t exec; int64_t used; };
   std::vector<PassGraph> graphs;            // at most kMaxGraphs
   int64_t graph_uses = 0;
   bool capturing = false;
@@ -502,7 +502,13 @@ int attn_cluster_room(int device, int ranks) {
 // / 1.04 / 1.01.  In a layer, whose next launch waits for the last wave, only for short items in a well filled second wave; the
 // whole layer, one row: 320 items 1.03 / 1.05 / 1.11 / 1.18, 384 1.03 / 1.01 / 1.04 / 1.09, 512 0.99 / 1.00 / 1.02 /
 // 0.99 (three rows 0.98 / 0.98 / 1.01 / 1.01), 592 1.00, 640 1.05 / 1.05 / 1.07 / 1.08, 832 1.01 / 1.02 / 1.03 / 1.00, 1280 1.06 / 1.05 / 1.07 / 1.03.
-int attn_cluster_ranks(int device, int n_sms, int items, int units, bool in_layer) {
+// Few long items: the clusters leave places free, and where a block's piece is longer than an equal share by more than the merge's
+// launch costs, shares are faster.  Layer, 8 kv heads, one row, clusters' time over equal shares', 8000 / 16000 / 32768 keys: 8 items (8 blocks each)
+// 1.03 / 1.09 / 1.19, 16 0.97 / 1.00 / 1.05, 24 0.96 / 0.98 / 0.99, 32 (4 each) 0.99 / 1.07 / 1.12, 64 0.98 / 0.99; three rows 1.04 / 1.12 / 1.23, 0.95 / 1.00 /
+// 1.08, 0.94 / 0.96 / 0.98, 0.99 / 1.08 / 1.18, 0.96 / 0.98: the lines cross at about 18 units of 64 keys more.  Alone, with caches read for the first
+// time, 8 items 0.82 / 1.01 / 1.22 (65536 keys 1.46), 16 0.84 / 0.99 / 1.05, 32 0.94 / 1.07 / 1.05, 2 items (2 kv heads) 0.78 / 1.12 / 1.61: at about 27.
+// `longest`: the units that the lengths at hand give, where `units` stands for a captured pass's longest context.
+int attn_cluster_ranks(int device, int n_sms, int items, int units, int longest, bool in_layer) {
   const int slots = 2 * n_sms, over = items % slots;
   if (items > slots) {
     if (in_layer) return 2 * items > 3 * slots && items <= 2 * slots && units <= 8 ? 1 : 0;
@@ -510,13 +516,16 @@ int attn_cluster_ranks(int device, int n_sms, int items, int units, bool in_laye
   }
   int ranks = 1;
   while (ranks < AD_MAX_CLUSTER && ranks < units && items <= attn_cluster_room(device, 2 * ranks) && (ranks < 4 || 16 * items <= 3 * n_sms)) ranks *= 2;
-  return ranks;
+  const long long free_places = slots - (long long)items * ranks;                  // longest / ranks - longest * items / slots > 18 or 27
+  return longest * free_places > (in_layer ? 18ll : 27ll) * ranks * slots ? 0 : ranks;
 }
-// ... for R new rows per sequence in a layer, up to position pos_end (a captured pass: up to the context's last).
-int attention_ranks(const dmtd_ctx *c, int B, int R, int pos_end) {
+// ... for R new rows per sequence in a layer, up to position pos_end.  A captured pass is replayed at other positions: its pieces are
+// those of the context's last one, and the choice between the forms is part of what it is kept under (attention_forms).
+int attention_ranks(const dmtd_ctx *c, int B, int R, int pos_end, bool captured) {
   if (!tc_decode_attention(c) || !c->fuse_qk_rope || R > AD_MAX_NEW || !c->use_umma || !c->umma_ok) return 0;
   const int RB = std::max(1, ATTN_QR / (c->s.n_q_heads / c->s.n_kv_heads)), n_rb = (R + RB - 1) / RB;
-  return attn_cluster_ranks(c->device, c->n_sms, B * c->s.n_kv_heads * n_rb, ((c->capturing ? c->max_seq : pos_end) + AD_UNIT - 1) / AD_UNIT, true);
+  return attn_cluster_ranks(c->device, c->n_sms, B * c->s.n_kv_heads * n_rb, ((captured ? c->max_seq : pos_end) + AD_UNIT - 1) / AD_UNIT,
+                            (pos_end + AD_UNIT - 1) / AD_UNIT, true);
 }
 
 // Its blocks and slots: as many slots as the partial results' buffer holds (and, up to four rows at a time, the merge
@@ -742,7 +751,7 @@ dmtd_status run_layer(dmtd_ctx *c, int l, float *x, int B, int R, const int *pos
   // on the tcgen05 path the O projection's activation blocks come from the prefill attention itself, or from the
   // kernel that merges the key slices
   const bool fuse_merge = tc && (flash || NAB_ROWS * s.n_q_heads * nsplit <= MAB_MAX_SLOTS);
-  const int ranks = tc && !flash ? attention_ranks(c, B, R, pos_end) : 0;       // > 0: the attention kernel merges, too
+  const int ranks = tc && !flash ? attention_ranks(c, B, R, pos_end, c->capturing) : 0;       // > 0: the attention kernel merges, too
   TRY(launch_attention(c, l, B, R, pos0, nsplit, !fuse_merge && ranks == 0, flash, ranks));
   if (fuse_merge || ranks > 0) {
     GemmInput in;
@@ -1189,7 +1198,7 @@ void drop_graphs(dmtd_ctx *c) {
 
 // Capture a steady-state pass (R_lower = tau) into a graph.  Positions come from the device
 // counters and the attention grid covers max_seq, so one graph serves the whole generation.
-dmtd_status capture_pass(dmtd_ctx *c, int kind) {
+dmtd_status capture_pass(dmtd_ctx *c, int kind, int forms) {
   cudaGraph_t graph = nullptr;
   int64_t before = c->launches;
   if (!c->capture_stream) CUDA_TRY(c, cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking));
@@ -1215,17 +1224,24 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind) {
     cudaGraphExecDestroy(oldest->exec);      // (one that still runs is released when it has)
     c->graphs.erase(oldest);
   }
-  c->graphs.push_back({kind, c->B, kind == 1 ? c->tau : 0, nodes, exec, 0});
+  c->graphs.push_back({kind, c->B, kind == 1 ? c->tau : 0, forms, nodes, exec, 0});
   return DMTD_OK;
+}
+
+// Which of a pass's attention launches take equal shares at the position at hand (they change at most once as a context grows).
+int attention_forms(const dmtd_ctx *c, int kind) {
+  const auto shares = [&](int R) { return attention_ranks(c, c->B, R, c->h.n_known, true) == 0; };
+  return (shares(1) ? 1 : 0) | (kind == 1 && shares(c->tau) ? 2 : 0);
 }
 
 // The graph of a kind of pass for the batch and cycle length at hand; captured: it is a new one.
 dmtd_status ready_graph(dmtd_ctx *c, int kind, const dmtd_ctx::PassGraph **out, bool *captured = nullptr) {
-  const int tau = kind == 1 ? c->tau : 0;
-  auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const auto &g) { return g.kind == kind && g.B == c->B && g.tau == tau; });
+  const int tau = kind == 1 ? c->tau : 0, forms = attention_forms(c, kind);
+  auto it = std::find_if(c->graphs.begin(), c->graphs.end(),
+                         [&](const auto &g) { return g.kind == kind && g.B == c->B && g.tau == tau && g.forms == forms; });
   if (captured) *captured = it == c->graphs.end();
   if (it == c->graphs.end()) {
-    TRY(capture_pass(c, kind));
+    TRY(capture_pass(c, kind, forms));
     it = c->graphs.end() - 1;
   }
   it->used = ++c->graph_uses;
@@ -1843,7 +1859,7 @@ dmtd_status attention_launch_t(const float *q, const void *k, const void *v, int
       using Op = typename std::conditional<std::is_same<KVT, __half>::value, OpF16, OpBf16>::type;
       const int items = B * nkv * n_rb, units = (pos0 + R + AD_UNIT - 1) / AD_UNIT;
       // the clusters store whole float4; results that begin elsewhere go through the merge kernel, which stores single values
-      const int ranks = reinterpret_cast<uintptr_t>(out) % 16 ? 0 : attn_cluster_ranks(dev, n_sms, items, units, false);
+      const int ranks = reinterpret_cast<uintptr_t>(out) % 16 ? 0 : attn_cluster_ranks(dev, n_sms, items, units, units, false);
       if (ranks > 0) {
         const auto kernel = attn_decode_kernel<Op, false, true>;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);

@@ -73,3 +73,36 @@ def test_more_items_than_resident_blocks(dmtd):
     assert launches(wave * 9 // 5, 200) == one_launch
     for items, pos0 in [(wave + 60, 200), (wave * 9 // 5, 600), (wave * 5 // 2, 200), (wave * 4, 64)]:
         assert launches(items, pos0) == one_launch + 1
+
+
+def test_few_long_items(dmtd):
+    """Where clusters leave places free, long items take equal shares and a merge; the passes of a context that grows past the
+    line are captured for either side, and their tokens are those of passes launched one by one."""
+    shape = SHAPES["mid"].with_(n_layers=2, hidden=256, intermediate=256, vocab=512)
+    w = to_cuda(make_weights(shape, seed=3, norm_jitter=0.1))
+    places = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    items, ranks = shape.n_kv_heads, 8
+    # the first number of 64-key units that is more than 18 of them longer in a block of a cluster than in an equal share
+    line = 18 * ranks * places // (places - items * ranks) + 1
+    keys = (line - 1) * 64                                    # the last context of fewer units
+    toks = []
+    for graph in (1, 0):
+        eng = dmtd.Dmtd(shape, w, L_d=1, tau=3, max_batch=1, max_seq=keys + 60, kv_dtype="f16")
+        eng.set_option("fused_pass", 0)
+        eng.set_option("cuda_graph", graph)
+        g = torch.Generator(device="cuda").manual_seed(5)
+        eng.prefill(torch.randint(0, shape.vocab, (1, keys - 20), generator=g, dtype=torch.int32, device="cuda"))
+        while eng.state()["slot"]:
+            eng.decode_cycle(3)
+        counts, out = [], []
+        for _ in range(12):
+            before, n0 = eng.state()["n_known"], eng.launch_count()
+            out.append(eng.decode_cycle(3)[2].clone())
+            counts.append((before, eng.launch_count() - n0))
+        assert eng.device_state() == eng.state()
+        short = {n for p, n in counts if p + 2 <= keys}
+        far = {n for p, n in counts if p > keys}
+        # a merge in each of the cycle's four layers
+        assert len(short) == 1 and far == {short.pop() + 4}
+        toks.append(torch.cat(out, 1))
+    assert torch.equal(*toks)

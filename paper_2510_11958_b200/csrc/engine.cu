@@ -96,7 +96,6 @@ struct dmtd_ctx {
   bool fuse_qk_rope = true;                 // QK-norm, RoPE and the KV append inside the tensor-core attention kernel
   float temperature = 0.f;                  // > 0: tokens are drawn from softmax(logits / temperature); 0: greedy
   uint64_t sample_seed = 0;
-  SampleParams *dsample = nullptr;          // device copy, written in stream order
 
   // fused pass kernel: one persistent launch per pass
   bool fused_ok = false;
@@ -112,7 +111,13 @@ struct dmtd_ctx {
   bool small_ok = false;                    // the model fits small_pass_kernel
 
   // captured passes: kind 1 = full (of tau pending rows), 2 = upper-only (any tau; 0 here)
-  struct PassGraph { int kind, B, tau, forms, nodes; cudaGraphExec_t exec; int64_t used; };
+  struct PassGraph {
+    int kind, B, tau, forms, nodes;
+    cudaGraphExec_t exec;
+    cudaGraph_t graph;                      // (owns the node below)
+    cudaGraphNode_t pick;                   // argmax_kernel: the pass's last launch
+    int64_t used;
+  };
   std::vector<PassGraph> graphs;            // at most kMaxGraphs
   int64_t graph_uses = 0;
   bool capturing = false;
@@ -803,12 +808,6 @@ SampleParams sample_params(const dmtd_ctx *c) {
   return sp;
 }
 
-dmtd_status write_sample_params(dmtd_ctx *c) {
-  set_sample_kernel<<<1, 1, 0, c->stream>>>(c->dsample, sample_params(c));
-  LAUNCH_OK(c, "set_sample_kernel");
-  return DMTD_OK;
-}
-
 // Step a9/a10/a0: final norm, tied LM head, greedy pick, token feedback, the schedule's counters.
 dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, float *out_logits, int kind, int P) {
   const dmtd_model_shape &s = c->s;
@@ -828,7 +827,7 @@ dmtd_status run_head(dmtd_ctx *c, int B, bool write_token, int *out_argmax, floa
     CUDA_TRY(c, cudaMemcpy2DAsync(out_logits, (size_t)s.vocab * 4, c->logits, (size_t)c->ldl * 4, (size_t)s.vocab * 4, B,
                                   cudaMemcpyDeviceToDevice, c->stream));
   CUDA_TRY(c, launch_pdl(argmax_kernel, dim3(B, ARGMAX_SLICES), dim3(256), (size_t)(0), c->stream,
-                          c->logits, c->ldl, s.vocab, c->dstate, c->dsample,
+                          c->logits, c->ldl, s.vocab, c->dstate, sample_params(c),
                           PickParams{c->pick_val, c->pick_idx, c->pick_arrived, write_token ? c->tokens : nullptr, c->max_seq, out_argmax, kind, P}));
   LAUNCH_OK(c, "argmax_kernel");
   return DMTD_OK;
@@ -1191,9 +1190,37 @@ dmtd_status device_error_status(dmtd_ctx *c, int word) {
       return fail((c), (c)->device_failure, "the context reported a device-side error earlier; call dmtd_reset"); \
   } while (0)
 
+void destroy_graph(const dmtd_ctx::PassGraph &g) {
+  cudaGraphExecDestroy(g.exec);              // (one that still runs is released when it has)
+  cudaGraphDestroy(g.graph);
+}
 void drop_graphs(dmtd_ctx *c) {
-  for (const auto &g : c->graphs) cudaGraphExecDestroy(g.exec);
+  for (const auto &g : c->graphs) destroy_graph(g);
   c->graphs.clear();
+}
+
+// Captured passes carry the sampling parameters as an argument of their last launch: a change replaces it (a few microseconds; another
+// capture takes 0.15 to 0.7 ms.  Parameters read from memory instead cost the pick of 32 sequences 3.4 us a pass: with them as
+// arguments the generator's keys are worked out once for a warp).
+void update_sampling(dmtd_ctx *c) {
+  SampleParams sp = sample_params(c);
+  for (const auto &g : c->graphs) {
+    cudaKernelNodeParams p{};
+    bool ok = cudaGraphKernelNodeGetParams(g.pick, &p) == cudaSuccess;
+    if (ok) {
+      void *args[] = {p.kernelParams[0], p.kernelParams[1], p.kernelParams[2], p.kernelParams[3], &sp, p.kernelParams[5]};
+      static_assert(std::is_same<decltype(&argmax_kernel), void (*)(const float *, int, int, DevState *, SampleParams, PickParams)>::value, "args");
+      p.func = reinterpret_cast<void *>(argmax_kernel);
+      p.kernelParams = args;
+      p.extra = nullptr;
+      ok = cudaGraphExecKernelNodeSetParams(g.exec, g.pick, &p) == cudaSuccess;
+    }
+    if (!ok) {                               // captured again when it is next needed
+      cudaGetLastError();
+      drop_graphs(c);
+      return;
+    }
+  }
 }
 
 // Capture a steady-state pass (R_lower = tau) into a graph.  Positions come from the device
@@ -1208,6 +1235,13 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind, int forms) {
   c->stream = c->capture_stream;
   c->capturing = true;
   dmtd_status st = enqueue_pass(c, kind, c->tau, true, nullptr, nullptr);
+  cudaGraphNode_t pick = nullptr;
+  {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t *last = nullptr;
+    size_t n_last = 0;
+    if (cudaStreamGetCaptureInfo(c->capture_stream, &status, nullptr, nullptr, &last, &n_last) == cudaSuccess && n_last == 1) pick = last[0];
+  }
   e = cudaStreamEndCapture(c->capture_stream, &graph);
   c->capturing = false;
   c->stream = user_stream;
@@ -1217,14 +1251,16 @@ dmtd_status capture_pass(dmtd_ctx *c, int kind, int forms) {
   if (e != cudaSuccess) return fail(c, DMTD_ERR_CUDA, "end capture: %s", cudaGetErrorString(e));
   cudaGraphExec_t exec = nullptr;
   e = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) return fail(c, DMTD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGraphDestroy(graph);
+    return fail(c, DMTD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+  }
   if ((int)c->graphs.size() == kMaxGraphs) {
     const auto oldest = std::min_element(c->graphs.begin(), c->graphs.end(), [](const auto &a, const auto &b) { return a.used < b.used; });
-    cudaGraphExecDestroy(oldest->exec);      // (one that still runs is released when it has)
+    destroy_graph(*oldest);
     c->graphs.erase(oldest);
   }
-  c->graphs.push_back({kind, c->B, kind == 1 ? c->tau : 0, forms, nodes, exec, 0});
+  c->graphs.push_back({kind, c->B, kind == 1 ? c->tau : 0, forms, nodes, exec, graph, pick, 0});
   return DMTD_OK;
 }
 
@@ -1406,8 +1442,6 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   }
   CTRY(dev_alloc(c, &c->tokens, (size_t)max_batch * max_seq));
   CTRY(dev_alloc(c, &c->dstate, 1));
-  CTRY(dev_alloc(c, &c->dsample, 1));
-  CTRY(write_sample_params(c));
   CCUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->h_error), sizeof(int), cudaHostAllocDefault));
   *c->h_error = 0;
 
@@ -1733,7 +1767,8 @@ dmtd_status dmtd_set_sampling(dmtd_ctx *c, float temperature, uint64_t seed) {
   if (!c) return DMTD_ERR_INVALID_ARG;
   if (!(temperature >= 0.f) || std::isinf(temperature)) return fail(c, DMTD_ERR_INVALID_ARG, "set_sampling: temperature must be finite and >= 0");
   c->temperature = temperature; c->sample_seed = seed;
-  return write_sample_params(c);
+  update_sampling(c);
+  return DMTD_OK;
 }
 
 dmtd_status dmtd_set_option(dmtd_ctx *c, const char *name, int64_t value) {

@@ -1013,9 +1013,8 @@ struct PickParams {
 };
 
 // grid (sequences, ARGMAX_SLICES), 256 threads
-__global__ void argmax_kernel(const float *logits, int ldl, int V, DevState *st, const SampleParams *sample, PickParams pp) {
+__global__ void argmax_kernel(const float *logits, int ldl, int V, DevState *st, SampleParams sp, PickParams pp) {
   pdl_enter();
-  const SampleParams sp = *sample;                   // (in memory: captured passes stay valid when it changes)
   const int b = blockIdx.x, per = ((V + gridDim.y - 1) / gridDim.y + 3) & ~3;      // whole 16-byte loads
   const int i0 = blockIdx.y * per, i1 = min(V, i0 + per);
   const float *z = logits + (size_t)b * ldl;
@@ -1078,7 +1077,6 @@ __global__ void argmax_kernel(const float *logits, int ldl, int V, DevState *st,
 }
 
 __global__ void set_int_kernel(int *p, int v) { *p = v; }
-__global__ void set_sample_kernel(SampleParams *p, SampleParams v) { *p = v; }
 
 // out[b][i] = tokens[b][first + i], i < n  (the tokens a decode call produced)
 __global__ void gather_tokens_kernel(const int *__restrict__ tokens, int max_seq, int first, int n,

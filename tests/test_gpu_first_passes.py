@@ -43,8 +43,8 @@ def test_first_cycles_of_a_context(dmtd):
 
 
 def test_cycles_after_set_sampling(dmtd):
-    """Captured passes read the temperature and the seed from memory: a program that sets them for every request does not wait
-    for another capture.  (It took 1.6 times as long as a later cycle.)"""
+    """A new temperature and seed go into the captured passes: a program that sets them for every request does not wait for
+    another capture.  (It took 1.6 times as long as a later cycle.)"""
     shape = SHAPES["mid"]
     eng = dmtd.Dmtd(shape, to_cuda(make_weights(shape, seed=0, norm_jitter=0.1)), L_d=2, tau=3, max_batch=1, max_seq=400, kv_dtype="f16")
     eng.prefill(make_prompts(shape.vocab, 1, 200, seed=1).cuda())

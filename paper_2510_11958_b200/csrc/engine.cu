@@ -1285,8 +1285,9 @@ dmtd_status ready_graph(dmtd_ctx *c, int kind, const dmtd_ctx::PassGraph **out, 
   return DMTD_OK;
 }
 
-// Behind a prefill, while the device works on it: the passes of few rows are captured before the first one is asked for (the host
-// takes 0.3 to 1.5 ms for each).  A failure here is left for the pass itself to meet.
+// The passes of few rows are captured before the first one is asked for: while the context is created, for its largest batch, and
+// behind a prefill of another batch or cycle length, while the device works on it (the host takes 0.2 to 1.5 ms for each pass).  A
+// failure here is left for the pass itself to meet.
 void capture_ahead(dmtd_ctx *c) {
   if (!c->use_graph || !c->fused_ok || c->B > PK_MAX_ROWS || c->literal_sum || c->L_e > 0) return;
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusActive;
@@ -1486,6 +1487,9 @@ dmtd_status dmtd_create(const dmtd_model_shape *shape, int32_t L_d, int32_t tau,
   CTRY(configure_kernels(c));
   CTRY(setup_fused(c));
   CTRY(setup_small(c));
+  c->B = max_batch; c->h.n_known = 1;        // the batch that a context of few sequences most often has
+  capture_ahead(c);
+  c->B = 0;
   CTRY(dmtd_reset(c));
   CCUDA(cudaStreamSynchronize(c->stream));   // repacking done: the caller may free its weights
 #undef CTRY

@@ -62,6 +62,7 @@ def main():
     eng = bd.Dmtd(shape, w, L_d=wl.L_d, tau=wl.tau, max_batch=wl.batch, max_seq=wl.prompt_len + 64,
                   kv_dtype=args.kv or wl.kv_dtype)
     del w
+    eng.set_option("fused_pass", 1)                      # the kernel that is stamped; replayed passes are launches per step unasked
     for kv in args.option:
         name, value = kv.split("=")
         eng.set_option(name, int(value))

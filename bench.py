@@ -148,6 +148,12 @@ NCU_TRAFFIC_RATIO = {
     # layer and head shapes, and its traffic grows with the bytes streamed
     ("qwen3_4b_l4_b1", "fused"): 1.0053,
     ("qwen3_4b_b1", "fused"): 1.0053,
+    # profiles/per_step_kernels_qwen3_4b_decode_launch_lists.md: all launches of a cycle on the 4-layer model, 3.9829 GB for
+    # 3.9656 GB at one sequence, 5.2752 GB for 5.0297 GB at 32
+    ("qwen3_4b_l4_b1", "per_step"): 1.0043,
+    ("qwen3_4b_b1", "per_step"): 1.0043,
+    ("qwen3_4b_l4_b32", "per_step"): 1.0488,
+    ("qwen3_4b_b32", "per_step"): 1.0488,
 }
 
 
